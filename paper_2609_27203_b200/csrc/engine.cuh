@@ -509,8 +509,9 @@ inline KeyTags sort_reduce(Ctx* c, int sr, DevBuf& k0, DevBuf& t0, DevBuf& k1, D
   // neighbours (a stable sort: rows end up ordered by (low, top), each key's candidates in their arrival order, so a
   // floating-point oplus sees them as the full sort would show them); the groups, far fewer than the candidates,
   // are then put in key order by a stable sort on the top bits.
+  // Candidates ordered by all of their key bits need no sort at all.
   const bool top_presorted = presorted_top > 0 && presorted_top < nbits && !want_head_pos && defer_slot < 0;
-  sort_pairs<K>(c, ka, ta, kb, tb, n, top_presorted ? nbits - presorted_top : nbits);
+  if (presorted_top < nbits) sort_pairs<K>(c, ka, ta, kb, tb, n, top_presorted ? nbits - presorted_top : nbits);
   const bool sorted_in_0 = (void*)ka == k0.p;
   KeyTags out = reduce_by_key<K>(c, sr, ka, ta, (uint32_t)n, sorted_in_0 ? &k1 : &k0, sorted_in_0 ? &t1 : &t0, want_head_pos, defer_slot);
   k0.reset(); t0.reset(); k1.reset(); t1.reset();

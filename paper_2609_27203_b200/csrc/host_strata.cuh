@@ -52,6 +52,11 @@ void stratum_recursive_additive(Ctx* c, const std::vector<int>& comp, const std:
   for (int p : comp) drop_current(*c->rels[p]);
   std::vector<KeyTags> delta(c->rels.size());
   for (int64_t round = 0;; ++round) {
+    if (round == 1) {
+      // closure-shaped rules over small rows: every row's remaining rounds in one launch
+      std::vector<RowSumRule> row_rules;
+      if (row_sums_applies(c, comp, rs, row_rules)) { row_sums_rounds(c, *c->rels[comp[0]], row_rules, delta[comp[0]]); return; }
+    }
     if (round >= c->max_iter) fail(XLOG_ERR_CONVERGENCE_FAILURE, "iteration cap reached before the fixpoint (cyclic derivations under a non-idempotent oplus never end)");
     ++c->r_iterations;
     std::vector<std::pair<int, KeyTags>> produced;
@@ -81,6 +86,16 @@ void stratum_recursive_additive(Ctx* c, const std::vector<int>& comp, const std:
       KeyTags& u = pr.second;
       if (u.n == 0) continue;
       derived += u.n;
+      if (H.n == 0) {                                       // nothing to merge with: I is Delta
+        KeyTags copy; copy.n = u.n;
+        copy.keys = DevBuf(c, (size_t)u.n * H.key_bytes); copy.tags = DevBuf(c, (size_t)u.n * 4);
+        XLOG_CUDA(cudaMemcpyAsync(copy.keys.p, u.keys.p, (size_t)u.n * H.key_bytes, cudaMemcpyDeviceToDevice, c->stream));
+        XLOG_CUDA(cudaMemcpyAsync(copy.tags.p, u.tags.p, (size_t)u.n * 4, cudaMemcpyDeviceToDevice, c->stream));
+        c->r_new += u.n;
+        set_current(H, std::move(copy));
+        delta[pr.first] = std::move(u);
+        continue;
+      }
       MergeResult m;
       DISPATCH_K(H.key_bytes, m = merge<K>(c, H.sr, u.keys.as<K>(), u.tags.as<float>(), u.n, -1, (const K*)H.keys(), H.tags(), H.n, false, false));
       c->r_new += m.n_new; c->r_improved += (int64_t)u.n - m.n_new;
