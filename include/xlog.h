@@ -141,7 +141,8 @@ xlog_status xlog_relation_read(xlog_ctx* ctx, xlog_rel rel, int32_t* const* cols
                                int64_t capacity, int64_t* n_out, xlog_memspace space);
 
 /* Zero-copy DEVICE pointers to the stored columns (Section "Zero-copy
- * interoperability"); borrowed, valid until the relation next changes. */
+ * interoperability"); borrowed, valid until the relation next changes.  The store keeps packed keys; the column
+ * view is built when it is first asked for.  xlog_relation_read into DEVICE memory does not need it. */
 xlog_status xlog_relation_view(xlog_ctx* ctx, xlog_rel rel, const int32_t** cols /*[arity]*/, const float** tags, int64_t* n);
 
 /* ---- rules: a compiled conjunctive plan ---------------------------------------

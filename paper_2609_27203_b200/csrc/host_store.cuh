@@ -53,6 +53,20 @@ void ensure_soa(Ctx* c, Relation& R) {
   R.soa_valid = true;
 }
 
+// The current contents into device columns and tags of the caller's (null: not wanted), in stored order.
+void read_out(Ctx* c, Relation& R, int32_t* const* cols, float* tags) {
+  if (R.n == 0) return;
+  ReadOut out{};
+  uintptr_t low = (uintptr_t)R.keys() | (uintptr_t)R.tags() | (uintptr_t)tags;
+  for (int i = 0; i < R.arity; ++i) { out.c[i] = cols ? cols[i] : nullptr; low |= (uintptr_t)out.c[i]; }
+  out.t = tags;
+  c->note_bytes = (int64_t)R.n * (R.key_bytes + 4 * (R.arity + 2));
+  if ((low & 15u) == 0)
+    DISPATCH_K(R.key_bytes, XLOG_LAUNCH(c, (k_read_out<K, true>), grid_for((R.n + 3) / 4, 256), 256, 0, (const K*)R.keys(), (const float*)R.tags(), (int64_t)R.n, R.layout, R.dicts(), out));
+  else
+    DISPATCH_K(R.key_bytes, XLOG_LAUNCH(c, (k_read_out<K, false>), grid_for(R.n, 256), 256, 0, (const K*)R.keys(), (const float*)R.tags(), (int64_t)R.n, R.layout, R.dicts(), out));
+}
+
 // Repack the loaded facts under a wider layout (derived tuples need more bits than the facts).
 void relayout_facts(Ctx* c, Relation& R, const KeyLayout& L) {
   if (same_layout(R.layout, L)) return;

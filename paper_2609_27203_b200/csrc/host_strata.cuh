@@ -215,7 +215,6 @@ void run_fixpoint(Ctx* c) {
     if (!recursive) stratum_once(c, comp[0], rs); else stratum_recursive(c, comp, rs);
     for (int p : comp) c->stratum_done[p] = 1;
   }
-  for (Relation* R : c->rels) if (R->is_head) ensure_soa(c, *R);
   sync_ctrl(c);
   c->poisoned = false;
   c->evaluated = true;

@@ -3,6 +3,8 @@
 // boundary detection then per-group reduction) and the merge-path set difference / union
 // with tag improvement (`dedup`, `set_ops`; Algorithm 1 lines 8-9).
 #pragma once
+#include <string.h>
+
 #include "common.cuh"
 
 namespace xlog {
@@ -79,6 +81,55 @@ __global__ void __launch_bounds__(256) k_unpack(const K* __restrict__ keys, int6
         const int32_t code = key_col<K>(L, k, c);
         cols.c[c][i] = D.n[c] ? D.v[c][min((uint32_t)code, D.n[c] - 1)] : code;
       }
+  }
+}
+
+// A relation copied out in one pass: the packed keys unpacked straight into the caller's columns, the tags beside them (any
+// of the destinations may be null).  Bound by memory: 8-byte keys and three columns are 24 bytes a row each way, against 44 for
+// unpacking into the store's own columns and copying those.  Four rows per thread and 16-byte accesses where every pointer
+// allows it (VEC).  Triangle join with 4.2 M rows 318 -> 271 us per evaluation and read, four-cycle join with 16.8 M rows
+// 2605 -> 2466, reachability with 54 M rows 9174 -> 8996.
+struct ReadOut { int32_t* c[kMaxArity]; float* t; };
+template <typename K, bool VEC>
+__global__ void __launch_bounds__(256) k_read_out(const K* __restrict__ keys, const float* __restrict__ tags, int64_t n, KeyLayout L, DictSet D, ReadOut out) {
+  constexpr int R = VEC ? 4 : 1;
+  const int64_t groups = (n + R - 1) / R;
+  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < groups; g += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = g * R;
+    const bool whole = VEC && i + R <= n;
+    K k[R];
+    float t[R];
+    if (whole) {
+      const uint4* src = reinterpret_cast<const uint4*>(keys + i);
+      uint4 v[R * sizeof(K) / 16 + (VEC ? 0 : 1)];
+#pragma unroll
+      for (int j = 0; j < (int)(R * sizeof(K) / 16); ++j) v[j] = __ldcs(src + j);
+      memcpy(k, v, sizeof(k));
+      if (out.t) { const float4 f = __ldcs(reinterpret_cast<const float4*>(tags + i)); memcpy(t, &f, sizeof(float) * R); }
+    } else {
+#pragma unroll
+      for (int j = 0; j < R; ++j) if (i + j < n) { k[j] = keys[i + j]; t[j] = tags[i + j]; } else { k[j] = 0; t[j] = 0.f; }
+    }
+#pragma unroll
+    for (int c = 0; c < kMaxArity; ++c)
+      if (c < L.arity && out.c[c]) {
+        int32_t v[R];
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+          const int32_t code = key_col<K>(L, k[j], c);
+          v[j] = D.n[c] ? D.v[c][min((uint32_t)code, D.n[c] - 1)] : code;
+        }
+        if (whole) { int4 q; memcpy(&q, v, sizeof(int32_t) * R); __stcs(reinterpret_cast<int4*>(out.c[c] + i), q); }
+        else
+#pragma unroll
+          for (int j = 0; j < R; ++j) if (i + j < n) out.c[c][i + j] = v[j];
+      }
+    if (out.t) {
+      if (whole) { float4 q; memcpy(&q, t, sizeof(float) * R); __stcs(reinterpret_cast<float4*>(out.t + i), q); }
+      else
+#pragma unroll
+        for (int j = 0; j < R; ++j) if (i + j < n) out.t[i + j] = t[j];
+    }
   }
 }
 
