@@ -4,6 +4,7 @@
 #include "host_mirror.cuh"
 #include "row_fixpoint.cuh"
 #include "row_sums.cuh"
+#include "sparse_rows.cuh"
 
 namespace xlog {
 namespace {
@@ -208,7 +209,7 @@ void stratum_row_fixpoint(Ctx* c, const std::vector<int>& comp, const std::vecto
 constexpr int kRowSumMaxBits = 27;
 
 bool row_sums_applies(Ctx* c, const std::vector<int>& comp, const std::vector<const RuleC*>& rs, std::vector<RowSumRule>& rules) {
-  if ((c->flags & XLOG_FLAG_NO_ROW_FIXPOINT) || comp.size() != 1) return false;
+  if ((c->flags & (XLOG_FLAG_NO_ROW_FIXPOINT | XLOG_FLAG_NO_TAG_MIRROR)) || comp.size() != 1) return false;
   const Relation& H = *c->rels[comp[0]];
   if (H.arity != 2 || H.key_bytes != 4 || H.dict_n[1] || H.layout.shift[1] != 0) return false;
   if (H.layout.shift[0] > kRowMaxBits || H.layout.total_bits > kRowSumMaxBits) return false;
@@ -280,6 +281,124 @@ void row_sums_rounds(Ctx* c, Relation& H, const std::vector<RowSumRule>& rules, 
   XLOG_LAUNCH(c, (k_mirror_full_emit<uint32_t>), tiles, kMirBlock, 0, (const int4*)table.as<int4>(), nquads, kMirrorEmptyMin, (const uint32_t*)sums.as<uint32_t>(), H.layout,
               H.layout, full.keys.as<uint32_t>(), full.tags.as<float>());
   set_current(H, std::move(full));
+}
+
+// ---- row-local fixpoint of short rows (sparse_rows.cuh) --------------------------------------------------------------------
+constexpr int kSlotSparse = 48;            // the kSpTotals control words (after the deferred counts of a component of one head)
+static_assert(kSlotSparse + kSpTotals <= kSlotResState, "control words overlap");
+// Worth trying when the rows are many (each is worked on by a few lanes) and their values of c too many for dense rows.  A try
+// that fails costs the launch until an eighth of the rows have outgrown the first table: tens of microseconds.
+constexpr int64_t kSparseMinRows = 4096, kSparseMaxRows = (int64_t)1 << 22;
+
+bool sparse_rows_applies(Ctx* c, const std::vector<int>& comp, const std::vector<const RuleC*>& rs, JoinSpec& S, int& r_rel) {
+  if (c->flags & (XLOG_FLAG_NO_ROW_FIXPOINT | XLOG_FLAG_NO_TAG_MIRROR | XLOG_FLAG_NO_RESIDENT_LOOP | XLOG_FLAG_NO_GRAPH | XLOG_FLAG_NO_GROUPED_JOIN)) return false;
+  if (comp.size() != 1) return false;
+  const Relation& H = *c->rels[comp[0]];
+  if (H.sr != XLOG_SR_MAXPLUS && H.sr != XLOG_SR_MINPLUS) return false;
+  if (H.arity != 2 || H.dict_n[1] || H.layout.shift[1] != 0 || H.layout.shift[0] <= kRowMaxBits || H.cur_owned) return false;
+  if ((int64_t)H.col_max[0] + 1 < kSparseMinRows || (int64_t)H.col_max[0] + 1 > kSparseMaxRows) return false;
+  int over = 0;
+  for (const RuleC* r : rs) {
+    int pos = -1, in = 0;
+    for (int j = 0; j < r->plan.n_atoms; ++j) if (r->plan.atoms[j].rel == comp[0]) { ++in; pos = j; }
+    if (in == 0) continue;
+    if (in != 1 || ++over != 1 || !closure_rule(c, r, pos, S)) return false;
+    r_rel = r->plan.atoms[1 - pos].rel;
+  }
+  return over == 1;
+}
+
+template <typename K, int SINK, int G, int T>
+void launch_sparse_tier(Ctx* c, SparseRows& P, int tier, uint32_t rows, uint32_t max_queued) {
+  constexpr size_t smem = sizeof(SparseRow<T>) * (kSparseBlock / G);
+  static_assert(smem <= (224u << 10), "table too long");
+  P.tier = tier; P.max_in = rows; P.max_queued = max_queued;
+  XLOG_CUDA(cudaFuncSetAttribute(k_sparse_rows<K, SINK, G, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const unsigned per_sm = (unsigned)std::max<size_t>(std::min<size_t>((226u << 10) / (smem + 1024), 8), 1);
+  const unsigned grid = (unsigned)std::min<uint64_t>(((uint64_t)rows + kSparseBlock / G - 1) / (kSparseBlock / G), (uint64_t)kSMs * per_sm);
+  XLOG_LAUNCH(c, (k_sparse_rows<K, SINK, G, T>), grid, kSparseBlock, smem, P);
+}
+// The tiers: lanes per row and slots per table.  Measured on 300,000 rows of 17 tuples (us for all tiers): 4 lanes and 32 slots
+// 613, 2 and 32 777, 8 and 32 739, 4 and 64 677: a longer first table costs rows in flight, wider groups cost lanes that idle.
+template <typename K, int SINK>
+void launch_sparse_tiers(Ctx* c, SparseRows& P, uint32_t* q0, uint32_t* q1) {
+  const uint32_t n = P.n_rows;
+  P.rows_in = nullptr; P.rows_out = q0;
+  launch_sparse_tier<K, SINK, 4, 32>(c, P, 0, n, n / 8 + 1024);
+  P.rows_in = q0; P.rows_out = q1;
+  launch_sparse_tier<K, SINK, 8, 128>(c, P, 1, n / 8 + 1024, n / 64 + 128);
+  P.rows_in = q1; P.rows_out = nullptr;
+  launch_sparse_tier<K, SINK, 32, (int)kSparseLongest>(c, P, 2, n / 64 + 128, 0);
+}
+
+// The rounds after the seed round: H holds the relation, (dkeys, dtags, dn) its delta.  False: some row is too long, or the
+// staging area too small; nothing has changed.
+bool sparse_rows_rounds(Ctx* c, Relation& H, const JoinSpec& S, uint32_t r_rows, const void* dkeys, const float* dtags, uint32_t dn) {
+  const int c_bits = H.layout.shift[0];
+  const uint32_t n_rows = (uint32_t)H.col_max[0] + 1;
+  const uint32_t max_q0 = n_rows / 8 + 1024, max_q1 = n_rows / 64 + 128;
+  const size_t fixed = (size_t)n_rows * 44 + (size_t)r_rows * 16 + (size_t)(max_q0 + max_q1) * 4 + (1u << 20);
+  if (fixed > c->arena.largest_free() / 2) return false;
+  const bool same = dn == H.n;              // the delta is a subset of the relation: of one size, they are the same rows
+  DevBuf rec(c, (size_t)n_rows * 16), rec_run(c, (size_t)n_rows * 8), drec(c, same ? 8 : (size_t)n_rows * 8), adj(c, (size_t)r_rows * 16), row_pos(c, (size_t)n_rows * 4),
+      row_len(c, (size_t)n_rows * 4), row_off(c, (size_t)n_rows * 4), q0(c, (size_t)max_q0 * 4), q1(c, (size_t)max_q1 * 4);
+  const size_t free_bytes = c->arena.largest_free();
+  const uint64_t cap = std::min<uint64_t>(free_bytes / 24, (uint64_t)kSortMaxN);      // 8 bytes staged and up to 12 in the relation
+  DevBuf st_c(c, cap * 4), st_t(c, cap * 4);
+  zero_ctrl(c, kSlotSparse, kSpTotals);
+  const uint32_t domain = (uint32_t)std::min<int64_t>(S.inner_domain, 0xffffffffll);
+  XLOG_CUDA(cudaMemsetAsync(rec.p, 0, (size_t)n_rows * 16, c->stream));
+  XLOG_LAUNCH(c, k_sparse_adj, grid_for(r_rows, 256), 256, 0, S.inner_col[0], S.inner_tag, r_rows, S.inner_off, domain, adj.as<uint4>());
+  DISPATCH_K(H.key_bytes, XLOG_LAUNCH(c, (k_sparse_records<K>), grid_for(H.n, 256), 256, 0, (const K*)H.keys(), (const float*)H.tags(), H.n, c_bits, S.inner_off, domain,
+                                       rec.as<uint4>(), rec_run.as<uint2>(), (uint2*)nullptr));
+  if (!same) {
+    XLOG_CUDA(cudaMemsetAsync(drec.p, 0, (size_t)n_rows * 8, c->stream));
+    DISPATCH_K(H.key_bytes, XLOG_LAUNCH(c, (k_sparse_records<K>), grid_for(dn, 256), 256, 0, (const K*)dkeys, dtags, dn, c_bits, S.inner_off, domain, (uint4*)nullptr,
+                                         (uint2*)nullptr, drec.as<uint2>()));
+  }
+  SparseRows P{};
+  P.keys = H.keys(); P.tags = H.tags(); P.dkeys = dkeys; P.dtags = dtags;
+  P.rec = rec.as<uint4>(); P.rec_run = rec_run.as<uint2>(); P.drec = same ? nullptr : drec.as<uint2>();
+  P.n_rows = n_rows; P.c_bits = c_bits; P.z_max = H.layout.mask[1];
+  P.max_rounds = (uint32_t)std::min<int64_t>(c->max_iter - 1, 0x7fffffff);
+  P.off = S.inner_off; P.domain = domain; P.adj = adj.as<uint4>();
+  P.row_pos = row_pos.as<uint32_t>(); P.row_len = row_len.as<uint32_t>();
+  P.st_c = st_c.as<uint32_t>(); P.st_t = st_t.as<float>(); P.st_cap = (uint32_t)cap;
+  P.totals = (unsigned long long*)(c->d_ctrl + kSlotSparse); P.err = ctrl_u32(c, kSlotErr);
+  const bool is_max = H.sr == XLOG_SR_MAXPLUS;
+  DISPATCH_K(H.key_bytes, {
+    if (is_max) launch_sparse_tiers<K, kSinkMax>(c, P, q0.as<uint32_t>(), q1.as<uint32_t>());
+    else launch_sparse_tiers<K, kSinkMin>(c, P, q0.as<uint32_t>(), q1.as<uint32_t>());
+  });
+  const unsigned tiles = (n_rows + kScanTile - 1) / kScanTile;
+  DevBuf sums(c, (size_t)tiles * 4);
+  XLOG_LAUNCH(c, (k_scan_tile_sums<uint32_t, uint32_t>), tiles, kScanBlock, 0, (const uint32_t*)row_len.as<uint32_t>(), (int64_t)n_rows, sums.as<uint32_t>());
+  XLOG_LAUNCH(c, (k_scan_spine<uint32_t>), 1, 1024, 0, sums.as<uint32_t>(), (int64_t)tiles, ctrl_u32(c, kSlotA));
+  XLOG_LAUNCH(c, (k_scan_apply<uint32_t, uint32_t>), tiles, kScanBlock, 0, (const uint32_t*)row_len.as<uint32_t>(), (int64_t)n_rows, (const uint32_t*)sums.as<uint32_t>(),
+              row_off.as<uint32_t>());
+  sync_ctrl(c);
+  const uint64_t* w = c->h_ctrl + kSlotSparse;
+  if (w[kSpStatus]) return false;
+  c->r_candidates += (int64_t)w[kSpCandidates];
+  c->r_unique += (int64_t)w[kSpUnique];
+  c->r_new += (int64_t)w[kSpNew];
+  c->r_improved += (int64_t)(w[kSpChanged] - w[kSpNew]);
+  c->r_iterations += (int64_t)w[kSpRounds];
+  if (w[kSpCapped]) fail(XLOG_ERR_CONVERGENCE_FAILURE, "iteration cap reached before the fixpoint");
+  KeyTags full;
+  full.n = (uint32_t)c->h_ctrl[kSlotA];
+  full.keys = DevBuf(c, (size_t)std::max(full.n, 1u) * H.key_bytes);
+  full.tags = DevBuf(c, (size_t)std::max(full.n, 1u) * 4);
+  c->note_bytes = (int64_t)full.n * (12 + H.key_bytes);
+  DISPATCH_K(H.key_bytes, XLOG_LAUNCH(c, (k_sparse_emit<K>), grid_for((uint64_t)n_rows * 8, 256), 256, 0, (const uint32_t*)row_pos.as<uint32_t>(), (const uint32_t*)row_len.as<uint32_t>(),
+                                       (const uint32_t*)row_off.as<uint32_t>(), n_rows, c_bits, (const uint32_t*)st_c.as<uint32_t>(), (const float*)st_t.as<float>(),
+                                       full.keys.as<K>(), full.tags.as<float>()));
+  set_current(H, std::move(full));
+  if (c->flags & XLOG_FLAG_CHECK_INVARIANTS) {
+    DISPATCH_K(H.key_bytes, XLOG_LAUNCH(c, (k_check_sorted<K>), grid_for(H.n, 256), 256, 0, (const K*)H.keys(), (int64_t)H.n, ctrl_u32(c, kSlotErr)));
+    sync_ctrl(c);
+  }
+  return true;
 }
 
 }  // namespace

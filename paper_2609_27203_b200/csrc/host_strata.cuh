@@ -120,10 +120,28 @@ void stratum_recursive(Ctx* c, const std::vector<int>& comp, const std::vector<c
     if (r->kind == 3 || r->kind == 4 || r->kind == 6) fail(XLOG_ERR_UNSUPPORTED, "triangle or four-cycle rule inside a recursive component");
   }
   if (additive) { stratum_recursive_additive(c, comp, rs); return; }
-  if (mirror_applies(c, comp, rs)) { stratum_recursive_mirror(c, comp[0], rs); return; }
-  if (mirror_multi_applies(c, comp, rs)) { stratum_recursive_mirror_multi(c, comp, rs); return; }
+  JoinSpec row_spec;
+  int row_rel = -1;
+  const bool try_rows = sparse_rows_applies(c, comp, rs, row_spec, row_rel);      // after the seed round: short rows, each to the end on its own
+  if (!try_rows) {
+    if (mirror_applies(c, comp, rs)) { stratum_recursive_mirror(c, comp[0], rs); return; }
+    if (mirror_multi_applies(c, comp, rs)) { stratum_recursive_mirror_multi(c, comp, rs); return; }
+  }
+  const int64_t before[5] = {c->r_candidates, c->r_unique, c->r_new, c->r_improved, c->r_iterations};
   std::vector<KeyTags> delta(c->rels.size());
   for (int64_t round = 0;; ++round) {
+    if (round == 1 && try_rows) {
+      Relation& H = *c->rels[comp[0]];
+      const KeyTags& d = delta[comp[0]];
+      if (sparse_rows_rounds(c, H, row_spec, c->rels[row_rel]->n, d.keys.p, d.tags.as<float>(), d.n)) return;
+      if (mirror_applies(c, comp, rs)) {                     // some row is long: over the mirror instead, from the start
+        delta.clear();
+        drop_current(H);
+        c->r_candidates = before[0]; c->r_unique = before[1]; c->r_new = before[2]; c->r_improved = before[3]; c->r_iterations = before[4];
+        stratum_recursive_mirror(c, comp[0], rs);
+        return;
+      }
+    }
     if (round >= c->max_iter) fail(XLOG_ERR_CONVERGENCE_FAILURE, "iteration cap reached before the fixpoint");
     ++c->r_iterations;
     // evaluate every head against the same state, then absorb
@@ -148,7 +166,7 @@ void stratum_recursive(Ctx* c, const std::vector<int>& comp, const std::vector<c
         }
       }
       if (vs.empty()) continue;
-      const int slot = produced.size() < 8 ? 32 + 4 * (int)produced.size() : -1;
+      const int slot = H.n && produced.size() < 8 ? 32 + 4 * (int)produced.size() : -1;      // a relation that is still empty takes the list as it is
       produced.emplace_back(h, evaluate(c, H, vs, nullptr, H.layout, false, slot));
     }
     for (int p : comp) delta[p] = KeyTags();
@@ -160,6 +178,16 @@ void stratum_recursive(Ctx* c, const std::vector<int>& comp, const std::vector<c
       Relation& H = *c->rels[produced[i].first];
       KeyTags& u = produced[i].second;
       if (u.n == 0) continue;
+      if (H.n == 0) {                                       // nothing to merge with: the relation and its delta are the list
+        KeyTags copy; copy.n = u.n;
+        copy.keys = DevBuf(c, (size_t)u.n * H.key_bytes); copy.tags = DevBuf(c, (size_t)u.n * 4);
+        XLOG_CUDA(cudaMemcpyAsync(copy.keys.p, u.keys.p, (size_t)u.n * H.key_bytes, cudaMemcpyDeviceToDevice, c->stream));
+        XLOG_CUDA(cudaMemcpyAsync(copy.tags.p, u.tags.p, (size_t)u.n * 4, cudaMemcpyDeviceToDevice, c->stream));
+        merged[i].n_new = u.n;
+        merged[i].full = std::move(copy);
+        merged[i].delta = std::move(u);                     // (the count stays behind for the loop below)
+        continue;
+      }
       if (!H.cur_owned && H.n_facts) {
         // first derivation into a relation that holds facts: work on a private copy
         KeyTags copy; copy.n = H.n_facts;
