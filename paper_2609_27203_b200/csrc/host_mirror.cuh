@@ -8,6 +8,7 @@
 #include "group_join.cuh"
 #include "mirror.cuh"
 #include "resident.cuh"
+#include "res_cluster.cuh"
 
 namespace xlog {
 namespace {
@@ -136,15 +137,48 @@ void resident_count(Ctx* c, Resident& R, const JoinSpec& S, size_t v) {
               R.tickets.as<uint32_t>() + v, ctrl_u32(c, kSlotErr), c->spin_limit);
 }
 
+// Small rounds inside a thread-block cluster (res_cluster.cuh): one rule, in the linear-key form with one looked-up column, over
+// a key space whose mirror fits the shared memory of the cluster.
+bool res_cluster_applies(const std::vector<JoinSpec>& specs, int bits) {
+  return specs.size() == 1 && specs[0].fast && specs[0].has_inner && specs[0].inner_free == 1 && !specs[0].times && bits >= kRcMinBits && bits <= kRcMaxBits;
+}
+// The largest key the columns' bounds allow ends the key space; whole bitmap words for every CTA.
+uint32_t res_cluster_slots(const Relation& H) {
+  uint32_t last = 0;
+  for (int k = 0; k < H.arity; ++k) last |= (uint32_t)H.col_max[k] << H.layout.shift[k];
+  const uint32_t per = 32u * kRcCtas;
+  return (uint32_t)std::min<uint64_t>(((uint64_t)last + per) / per * per, (uint64_t)1 << H.layout.total_bits);
+}
+template <int SINK>
+void launch_res_cluster(Ctx* c, const JoinSpec& S, const ResCluster& P) {
+  const size_t smem = res_cluster_smem(P.slots);
+  XLOG_CUDA(cudaFuncSetAttribute(k_res_cluster<SINK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)res_cluster_smem(1u << kRcMaxBits)));
+  if (c->flags & XLOG_FLAG_PROFILE) prof_begin(c, "k_res_cluster");
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kRcCtas); cfg.blockDim = dim3(kRcBlock); cfg.dynamicSmemBytes = smem; cfg.stream = c->stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = kRcCtas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  XLOG_CUDA(cudaLaunchKernelEx(&cfg, k_res_cluster<SINK>, S, P));
+  check_launch(c, "k_res_cluster");
+}
+
 // One round's launches.  Nothing here allocates, copies or waits: the same calls are either captured into the WHILE
 // body or issued directly (host-driven rounds, used when launches are being timed one by one).
-void resident_body(Ctx* c, Resident& R, const std::vector<JoinSpec>& specs, bool is_max, const MirrorArgs& mr, uint32_t bm_quads, unsigned ch_tiles,
+void resident_body(Ctx* c, Resident& R, const std::vector<JoinSpec>& specs, const Relation& H, bool is_max, const MirrorArgs& mr, uint32_t bm_quads, unsigned ch_tiles,
                    cudaGraphConditionalHandle handle, int use_handle) {
   ResState* st = res_state(c);
   uint32_t* err = ctrl_u32(c, kSlotErr);
   const uint32_t* dk = R.dkeys.as<uint32_t>();
   const ResScratch sc{R.scan_status.as<unsigned long long>(), R.scan_tiles_cap, R.tickets.as<uint32_t>()};
   const bool fused = specs.size() == 1;                  // the count of the next round rides on the emit kernel; the first round's is launched before the loop
+  const int bits = H.layout.total_bits;
+  if (res_cluster_applies(specs, bits)) {
+    const uint32_t slots = res_cluster_slots(H);
+    const ResCluster P{slots, R.table.as<int32_t>(), R.bitmap.as<uint32_t>(), R.present.as<uint32_t>(), dk, R.dtags.as<float>(), st, mr.n_new, std::min(mr.key_max, slots - 1), err};
+    if (is_max) launch_res_cluster<kSinkMax>(c, specs[0], P); else launch_res_cluster<kSinkMin>(c, specs[0], P);
+  }
   for (size_t v = 0; v < specs.size(); ++v) {
     const JoinSpec& S = specs[v];
     if (!fused) resident_count(c, R, S, v);
@@ -192,7 +226,8 @@ ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*
   XLOG_LAUNCH(c, k_res_init, 1, 1024, 0, res_state(c), sc, (uint32_t)specs.size(), n_delta, budget, R.max_tiles, (unsigned long long)new_seen);
   const MirrorArgs& mr = mr_host;
   const bool fused = specs.size() == 1;
-  if (fused) resident_count(c, R, specs[0], 0);          // the first round's count; every later one rides on the emit kernel
+  const bool in_cluster = res_cluster_applies(specs, H.layout.total_bits) && n_delta > 0 && n_delta <= kRcMaxRows;      // the cluster kernel takes the first round and counts it itself
+  if (fused && !in_cluster) resident_count(c, R, specs[0], 0);          // the first round's count; every later one rides on the emit kernel
   const int64_t l0 = c->launches;
   const bool use_graph = !(c->flags & (XLOG_FLAG_PROFILE | XLOG_FLAG_NO_GRAPH));
   ResState out{};
@@ -204,6 +239,7 @@ ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*
     std::vector<char> sig;
     for (const JoinSpec& S : specs) sig_add(sig, S);
     sig_add(sig, mr.table); sig_add(sig, mr.changed); sig_add(sig, mr.n_new); sig_add(sig, mr.key_max); sig_add(sig, mr.err); sig_add(sig, R.present.p);
+    if (res_cluster_applies(specs, H.layout.total_bits)) sig_add(sig, res_cluster_slots(H));
     sig_add(sig, is_max); sig_add(sig, bm_quads); sig_add(sig, ch_tiles); sig_add(sig, c->d_ctrl); sig_add(sig, c->spin_limit);
     if (!R.exec || sig != R.sig) {
       if (R.exec) { cudaGraphExecDestroy(R.exec); R.exec = nullptr; }
@@ -227,7 +263,7 @@ ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*
       c->stream = c->capture_stream;
       const int64_t b0 = c->launches;
       try {
-        resident_body(c, R, specs, is_max, mr, bm_quads, ch_tiles, handle, 1);
+        resident_body(c, R, specs, H, is_max, mr, bm_quads, ch_tiles, handle, 1);
       } catch (...) {
         c->stream = caller;
         cudaGraph_t dummy = nullptr;
@@ -242,7 +278,7 @@ ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*
     }
     XLOG_CUDA(cudaGraphLaunch(R.exec, c->stream));
     read_state();
-    c->launches = l0 + R.body_launches * (int64_t)out.rounds + (out.status == kResOverflow && !fused ? R.body_launches : 0);
+    c->launches = l0 + R.body_launches * (int64_t)out.bodies;
   } else {
     unsigned long long seen = 0;
     uint32_t rows = n_delta;
@@ -253,7 +289,7 @@ ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*
       if (it0 != c->prof_index.end()) { expand_ms_seen = c->prof[it0->second].ms; expand_launches_seen = c->prof[it0->second].launches; }
     }
     for (;;) {
-      resident_body(c, R, specs, is_max, mr, bm_quads, ch_tiles, cudaGraphConditionalHandle{}, 0);
+      resident_body(c, R, specs, H, is_max, mr, bm_quads, ch_tiles, cudaGraphConditionalHandle{}, 0);
       read_state();
       if (c->flags & XLOG_FLAG_PROFILE) {
         // per delta row and rule: key and tag read, two offsets probed, 16-byte row record and 8-byte start offset written
@@ -263,7 +299,7 @@ ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*
         // algorithmic bytes of the round's expand launches (per candidate: the looked-up columns and tag, and the slot)
         auto it = c->prof_index.find("k_res_expand");
         if (it != c->prof_index.end()) {
-          const int64_t bytes = (int64_t)(out.candidates - seen) * (4 + (specs[0].has_inner ? 4 * (specs[0].inner_free + 1) : 0));
+          const int64_t bytes = (int64_t)(out.candidates - out.small_cand - seen) * (4 + (specs[0].has_inner ? 4 * (specs[0].inner_free + 1) : 0));
           Ctx::ProfEntry& pe = c->prof[it->second];
           pe.bytes += bytes;
           if (bytes >= kProfLargeBytes) {                // this round's launches, totalled on their own like any large launch
@@ -279,7 +315,7 @@ ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*
           }
           expand_ms_seen = c->prof[it->second].ms; expand_launches_seen = c->prof[it->second].launches;
         }
-        seen = out.candidates;
+        seen = out.candidates - out.small_cand;
       }
       if (out.status != kResOk || out.n_delta == 0) break;
     }

@@ -127,7 +127,7 @@ void stratum_recursive_mirror(Ctx* c, int h, const std::vector<const RuleC*>& rs
     total_new = s.new_seen;
     dk = R->dkeys.p; dt = R->dtags.as<float>(); dn = s.n_delta;
     if (s.status == kResCap) fail(XLOG_ERR_CONVERGENCE_FAILURE, "iteration cap reached before the fixpoint");
-    if (s.status == kResOk) converged = true;             // the delta ran empty
+    if (s.status == kResOk || s.status == kResDone) converged = true;      // the delta ran empty
     // kResOverflow: a round needs more expand tiles than planned; the host redoes that round and finishes the job
   }
   for (; !converged; ++round) {

@@ -23,7 +23,7 @@
 
 namespace xlog {
 
-enum { kResOk = 0, kResCap = 1, kResOverflow = 2, kResError = 3 };
+enum { kResOk = 0, kResCap = 1, kResOverflow = 2, kResError = 3, kResDone = 4 };      // kResDone: finished inside the cluster kernel (res_cluster.cuh)
 
 struct ResState {
   uint32_t n_delta;                  // rows of the current delta
@@ -38,6 +38,9 @@ struct ResState {
   unsigned long long new_seen;       // value of the mirror's new-tuple counter at the end of the last completed round
   unsigned long long n_new;          // new tuples / improved tags of all completed rounds
   unsigned long long n_improved;
+  unsigned long long small_cand;     // candidates of rounds run by the cluster kernel (res_cluster.cuh)
+  uint32_t bodies;                   // times the loop body ran
+  uint32_t pad;
 };
 
 constexpr int kResMaxVariants = 16;
@@ -240,6 +243,7 @@ __device__ __forceinline__ void res_close_round(const bool live, ResState* __res
   __syncthreads();
   if (threadIdx.x == 0) {
     unsigned again = 0;
+    st->bodies += 1;
     if (live) {
       const unsigned long long seen = *new_counter;
       const unsigned long long fresh = seen - st->new_seen;
