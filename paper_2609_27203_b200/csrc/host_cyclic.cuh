@@ -3,6 +3,7 @@
 #pragma once
 #include "host_eval.cuh"
 #include "triangle.cuh"
+#include "tri_rank.cuh"
 #include "cycle4.cuh"
 
 namespace xlog {
@@ -41,6 +42,126 @@ void append_count_column(Ctx* c, Relation& H, KeyTags& u, const KeyLayout& cl) {
   append_counts(c, H, u, cl, counts.as<uint32_t>(), (uint32_t)c->h_ctrl[kSlotD]);
 }
 
+// ---- the triangle aggregate over the degree-ordered graph (tri_rank.cuh) ------------------------------------------------
+constexpr int kSlotTrk = 48;               // the kTrkTotals control words
+static_assert(kSlotTrk + kTrkTotals <= 64, "control words overlap the resident state block");
+
+void exclusive_scan_u32(Ctx* c, const uint32_t* in, int64_t n, uint32_t* out, uint32_t* total) {
+  const unsigned tiles = (unsigned)((n + kScanTile - 1) / kScanTile);
+  DevBuf sums(c, (size_t)tiles * 4);
+  XLOG_LAUNCH(c, (k_scan_tile_sums<uint32_t, uint32_t>), tiles, kScanBlock, 0, in, n, sums.as<uint32_t>());
+  XLOG_LAUNCH(c, (k_scan_spine<uint32_t>), 1, 1024, 0, sums.as<uint32_t>(), (int64_t)tiles, total);
+  XLOG_LAUNCH(c, (k_scan_apply<uint32_t, uint32_t>), tiles, kScanBlock, 0, in, n, (const uint32_t*)sums.as<uint32_t>(), out);
+}
+
+TriRankLists tri_rank_lists(const TriRankIndex& X, int o) {
+  return TriRankLists{X.off[o].as<uint32_t>(), X.split[o].as<uint32_t>(), X.nbr[o].as<uint32_t>(), X.num[o].as<float>(), o == 1 ? X.other.as<uint32_t>() : nullptr};
+}
+// launch 0 (by a): lower neighbours and walks in the in-lists, marks in the out-lists; launch 1 (by b): the other way round
+TriRankPass tri_rank_pass(const TriRankIndex& X, int p) {
+  TriRankPass P{};
+  P.I = tri_rank_lists(X, 1 - p); P.M = tri_rank_lists(X, p);
+  P.n_nodes = X.n_nodes; P.unit_off = X.unit_off[p].as<uint32_t>(); P.unit = X.unit[p].as<uint2>(); P.n_units = X.n_units[p];
+  return P;
+}
+
+// The ordered copy of E, made at the first call.  False: not for this relation.
+bool ensure_tri_rank(Ctx* c, Relation& E, Index& out_ix, Index& in_ix, bool lse) {
+  TriRankIndex& X = E.tri;
+  if (X.tried) return X.valid;
+  X.tried = true;
+  const int64_t nodes = std::max(out_ix.domain, in_ix.domain);
+  if (E.n < kTriRankMinEdges || nodes > kTriRankMaxNodes) return false;
+  const uint32_t N = (uint32_t)nodes, m = E.n;
+  if ((size_t)m * 64 + (size_t)N * 64 + (4u << 20) > c->arena.largest_free() / 2) return false;
+  const int32_t* src = E.cols[0].as<int32_t>(); const int32_t* dst = E.cols[1].as<int32_t>();
+  unsigned long long* tot = (unsigned long long*)(c->d_ctrl + kSlotTrk);
+  zero_ctrl(c, kSlotTrk, kTrkTotals);
+  X.rank = DevBuf(c, (size_t)N * 4);
+  {
+    DevBuf k0(c, (size_t)N * 4), v0(c, (size_t)N * 4), k1(c, (size_t)N * 4), v1(c, (size_t)N * 4);
+    XLOG_LAUNCH(c, k_trk_degrees, grid_for(N, 256), 256, 0, out_ix.off.as<uint32_t>(), out_ix.domain, in_ix.off.as<uint32_t>(), in_ix.domain, N, k0.as<uint32_t>(), v0.as<uint32_t>(), tot);
+    uint32_t* ka = k0.as<uint32_t>(); uint32_t* kb = k1.as<uint32_t>();
+    float* va = v0.as<float>(); float* vb = v1.as<float>();
+    sort_pairs<uint32_t>(c, ka, va, kb, vb, N, bit_length(2 * (int64_t)m));
+    XLOG_LAUNCH(c, k_trk_ranks, grid_for(N, 256), 256, 0, (const uint32_t*)va, N, (const unsigned long long*)tot, X.rank.as<uint32_t>());
+  }
+  const uint32_t* rank = X.rank.as<uint32_t>();
+  // the edges between corners ordered by (target, source), then by (source, target): stable sorts by one rank at a time
+  DevBuf k0(c, (size_t)m * 4), v0(c, (size_t)m * 4), k1(c, (size_t)m * 4), v1(c, (size_t)m * 4);
+  uint32_t* ka = k0.as<uint32_t>(); uint32_t* kb = k1.as<uint32_t>();
+  float* va = v0.as<float>(); float* vb = v1.as<float>();
+  XLOG_LAUNCH(c, k_trk_edges, grid_for(m, 256), 256, 0, src, dst, (const float*)E.tags(), m, rank, N, ka, reinterpret_cast<uint32_t*>(va), tot);
+  const int bits = bit_length(N);
+  sort_pairs<uint32_t>(c, ka, va, kb, vb, m, bits);
+  sync_ctrl(c);
+  float top;
+  { const uint32_t u = (uint32_t)c->h_ctrl[kSlotTrk + kTrkAbsMax]; memcpy(&top, &u, 4); }
+  X.n_edges = (uint32_t)c->h_ctrl[kSlotTrk + kTrkEdges];
+  X.n_nodes = (uint32_t)c->h_ctrl[kSlotTrk + kTrkNodes];
+  if (c->h_ctrl[kSlotTrk + kTrkLoops] || (lse && !(top <= kTriRankMaxTag)) || X.n_edges == 0) { X = TriRankIndex(); X.tried = true; return false; }
+  const uint32_t me = X.n_edges, P = X.n_nodes;
+  DevBuf place(c, (size_t)m * 4);
+  for (int o = 1; o >= 0; --o) {
+    // by target the first time (the edges come in order of the source), by source the second
+    XLOG_LAUNCH(c, k_trk_keys, grid_for(me, 256), 256, 0, reinterpret_cast<const uint32_t*>(va), me, o == 1 ? dst : src, rank, ka);
+    sort_pairs<uint32_t>(c, ka, va, kb, vb, me, bits);
+    X.off[o] = DevBuf(c, ((size_t)P + 1) * 4); X.split[o] = DevBuf(c, (size_t)P * 4); X.nbr[o] = DevBuf(c, (size_t)me * 4); X.num[o] = DevBuf(c, (size_t)me * 4);
+    XLOG_LAUNCH(c, k_build_offsets, grid_for(P + 1, 256), 256, 0, reinterpret_cast<const int32_t*>(ka), me, (int64_t)P, X.off[o].as<uint32_t>());
+    if (o == 1) {
+      // remember where every edge stands by target; the out-lists' places are filled in below
+      X.other = DevBuf(c, (size_t)me * 4);
+      XLOG_CUDA(cudaMemcpyAsync(X.other.p, va, (size_t)me * 4, cudaMemcpyDeviceToDevice, c->stream));
+    }
+#define XLOG_TRK_LISTS(EXP)                                                                                                                                                    \
+  XLOG_LAUNCH(c, (k_trk_lists<EXP>), grid_for(me, 256), 256, 0, reinterpret_cast<const uint32_t*>(va), me, o == 1 ? src : dst, (const float*)E.tags(), rank, X.nbr[o].as<uint32_t>(), \
+              X.num[o].as<float>(), o == 0 ? place.as<uint32_t>() : nullptr)
+    if (lse) XLOG_TRK_LISTS(true); else XLOG_TRK_LISTS(false);
+#undef XLOG_TRK_LISTS
+    XLOG_LAUNCH(c, k_trk_splits, grid_for(P, 256), 256, 0, (const uint32_t*)X.off[o].as<uint32_t>(), (const uint32_t*)X.nbr[o].as<uint32_t>(), P, X.split[o].as<uint32_t>());
+  }
+  XLOG_LAUNCH(c, k_trk_gather, grid_for(me, 256), 256, 0, (const uint32_t*)X.other.as<uint32_t>(), me, (const uint32_t*)place.as<uint32_t>(), X.other.as<uint32_t>());
+  DevBuf units(c, ((size_t)P + 1) * 4);
+  for (int p = 0; p < 2; ++p) {
+    X.unit_off[p] = DevBuf(c, ((size_t)P + 1) * 4);
+    XLOG_LAUNCH(c, k_trk_units, grid_for((uint64_t)P * 32, 256), 256, 0, tri_rank_lists(X, 1 - p), tri_rank_lists(X, p), P, units.as<uint32_t>(), tot + kTrkWalkA + p);
+    exclusive_scan_u32(c, units.as<uint32_t>(), (int64_t)P + 1, X.unit_off[p].as<uint32_t>(), ctrl_u32(c, kSlotTrk + kTrkUnitsA + p));
+  }
+  sync_ctrl(c);
+  X.walk = c->h_ctrl[kSlotTrk + kTrkWalkA] + c->h_ctrl[kSlotTrk + kTrkWalkB];
+  for (int p = 0; p < 2; ++p) {
+    X.n_units[p] = (uint32_t)c->h_ctrl[kSlotTrk + kTrkUnitsA + p];
+    X.unit[p] = DevBuf(c, (size_t)std::max(X.n_units[p], 1u) * 8);
+    XLOG_LAUNCH(c, k_trk_unit_fill, grid_for(P, 256), 256, 0, tri_rank_lists(X, 1 - p), tri_rank_lists(X, p), P, (const uint32_t*)X.unit_off[p].as<uint32_t>(), X.unit[p].as<uint2>());
+  }
+  ++c->r_index_builds;
+  X.valid = true;
+  return true;
+}
+
+// counts, tags and presence flags of every x
+void tri_rank_groups(Ctx* c, Relation& E, bool lse, int64_t domain, uint32_t* gcnt, float* gtag, uint32_t* flag, uint32_t* max_cnt) {
+  const TriRankIndex& X = E.tri;
+  TriRankPass Q[2] = {tri_rank_pass(X, 0), tri_rank_pass(X, 1)};
+  DevBuf usum[2], ucnt[2], esum(c, (size_t)X.n_edges * 8), ecnt(c, (size_t)X.n_edges * 4);
+  Q[0].edge_sum = esum.as<double>(); Q[0].edge_cnt = ecnt.as<uint32_t>();
+  const size_t smem = (size_t)(X.n_nodes + 31) / 32 * 8;
+  for (int p = 0; p < 2; ++p) {
+    usum[p] = DevBuf(c, ((size_t)X.n_units[p] + X.n_nodes) * 8); ucnt[p] = DevBuf(c, ((size_t)X.n_units[p] + X.n_nodes) * 4);
+    Q[p].unit_sum = usum[p].as<double>(); Q[p].unit_cnt = ucnt[p].as<uint32_t>();
+    c->note_bytes = (int64_t)X.walk / 2 * 4;
+    XLOG_CUDA(cudaFuncSetAttribute(p ? k_tri_rank<false> : k_tri_rank<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kTriRankMaxNodes / 32 * 8)));
+    if (X.n_units[p]) {
+      if (p == 0) XLOG_LAUNCH(c, (k_tri_rank<true>), X.n_units[0], kTriRankBlock, smem, Q[0]); else XLOG_LAUNCH(c, (k_tri_rank<false>), X.n_units[1], kTriRankBlock, smem, Q[1]);
+    }
+    if (p == 0) XLOG_LAUNCH(c, (k_tri_rank_small<true>), grid_for((uint64_t)X.n_nodes * 32, 256), 256, 0, Q[0]);
+    else XLOG_LAUNCH(c, (k_tri_rank_small<false>), grid_for((uint64_t)X.n_nodes * 32, 256), 256, 0, Q[1]);
+  }
+  const unsigned g = grid_for((uint64_t)domain * 32, 256);
+  if (lse) XLOG_LAUNCH(c, (k_tri_rank_groups<true>), g, 256, 0, Q[0], Q[1], X.rank.as<uint32_t>(), domain, gcnt, gtag, flag, max_cnt, ctrl_u32(c, kSlotErr));
+  else XLOG_LAUNCH(c, (k_tri_rank_groups<false>), g, 256, 0, Q[0], Q[1], X.rank.as<uint32_t>(), domain, gcnt, gtag, flag, max_cnt, ctrl_u32(c, kSlotErr));
+}
+
 // h(x[, count]) :- e(x,y), e(y,z), e(z,x): per-edge sorted-list intersection, then per-x combination.
 template <typename Op>
 void triangle_aggregate_t(Ctx* c, Relation& H, const RuleC& r) {
@@ -52,79 +173,86 @@ void triangle_aggregate_t(Ctx* c, Relation& H, const RuleC& r) {
   if (E.n == 0) { KeyTags empty; set_current(H, std::move(empty)); return; }
   Index& out_ix = ensure_index(c, E, 0);
   Index& in_ix = ensure_index(c, E, 1);
-  TriGraph G{};
-  G.n_edges = E.n;
-  G.src = E.cols[0].as<int32_t>(); G.dst = E.cols[1].as<int32_t>(); G.w = E.tags();
-  G.out_domain = out_ix.domain; G.in_domain = in_ix.domain;
-  G.out_off = out_ix.off.as<uint32_t>(); G.in_off = in_ix.off.as<uint32_t>();
-  G.in_src = in_ix.other[0]; G.in_w = in_ix.tags;
-  G.s_dst = G.dst; G.s_w = G.w;
   const int64_t domain = out_ix.domain;
-  // work items: edges cut into slices of the walked list (count -> scan -> one control read for the item total)
-  const uint32_t ne1 = E.n + 1;
-  DevBuf items(c, (size_t)ne1 * 4), item_off(c, (size_t)ne1 * 4);
-  const unsigned it_tiles = (ne1 + kScanTile - 1) / kScanTile;
-  DevBuf it_sums(c, (size_t)it_tiles * 4);
-  zero_ctrl(c, kSlotA, 4);
-  // per x: search the longer list, or mark in(x) in a shared-memory bitmap and walk every out(y) against it (triangle.cuh)
-  // the bitmap holds sources of edges into x (values of column 0) and is probed with targets (values of column 1): both ranges must fit
-  const int64_t node_domain = std::max(in_ix.domain, out_ix.domain);
-  const bool bitmap_ok = !(c->flags & XLOG_FLAG_NO_TRIANGLE_BITMAP) && node_domain <= kTriBitmapMaxDomain;
-  const int64_t sum_n = std::max<int64_t>(in_ix.domain, 1);
-  DevBuf route_sums(c, bitmap_ok ? (size_t)sum_n * 16 : 16);
-  TriRoute RT{route_sums.as<unsigned long long>(), route_sums.as<unsigned long long>() + (bitmap_ok ? sum_n : 0), bitmap_ok ? 1 : 0};
-  if (bitmap_ok) {
-    XLOG_CUDA(cudaMemsetAsync(route_sums.p, 0, (size_t)sum_n * 16, c->stream));
-    XLOG_LAUNCH(c, k_tri_route_sums, grid_for(E.n, 256), 256, 0, G, route_sums.as<unsigned long long>(), route_sums.as<unsigned long long>() + sum_n);
-  }
-  XLOG_LAUNCH(c, k_tri_plan, grid_for(ne1, 256), 256, 0, G, RT, items.as<uint32_t>(), (unsigned long long*)(c->d_ctrl + kSlotC),
-              (unsigned long long*)(c->d_ctrl + kSlotD));
-  XLOG_LAUNCH(c, (k_scan_tile_sums<uint32_t, uint32_t>), it_tiles, kScanBlock, 0, (const uint32_t*)items.as<uint32_t>(), (int64_t)ne1, it_sums.as<uint32_t>());
-  XLOG_LAUNCH(c, (k_scan_spine<uint32_t>), 1, 1024, 0, it_sums.as<uint32_t>(), (int64_t)it_tiles, ctrl_u32(c, kSlotB));
-  XLOG_LAUNCH(c, (k_scan_apply<uint32_t, uint32_t>), it_tiles, kScanBlock, 0, (const uint32_t*)items.as<uint32_t>(), (int64_t)ne1,
-              (const uint32_t*)it_sums.as<uint32_t>(), item_off.as<uint32_t>());
-  // the bitmap kernel's units: the work items of one x in slices (count -> scan; the total arrives with the same control read)
-  const int64_t nd1 = domain + 1;
-  const unsigned un_tiles = (unsigned)((nd1 + kScanTile - 1) / kScanTile);
-  DevBuf units(c, bitmap_ok ? (size_t)nd1 * 4 : 4), unit_off(c, bitmap_ok ? (size_t)nd1 * 4 : 4), un_sums(c, (size_t)un_tiles * 4);
-  if (bitmap_ok) {
-    XLOG_LAUNCH(c, k_tri_unit_count, grid_for(nd1, 256), 256, 0, G, RT, G.out_off, domain, (const uint32_t*)item_off.as<uint32_t>(), units.as<uint32_t>());
-    XLOG_LAUNCH(c, (k_scan_tile_sums<uint32_t, uint32_t>), un_tiles, kScanBlock, 0, (const uint32_t*)units.as<uint32_t>(), nd1, un_sums.as<uint32_t>());
-    XLOG_LAUNCH(c, (k_scan_spine<uint32_t>), 1, 1024, 0, un_sums.as<uint32_t>(), (int64_t)un_tiles, ctrl_u32(c, kSlotA));
-    XLOG_LAUNCH(c, (k_scan_apply<uint32_t, uint32_t>), un_tiles, kScanBlock, 0, (const uint32_t*)units.as<uint32_t>(), nd1, (const uint32_t*)un_sums.as<uint32_t>(),
-                unit_off.as<uint32_t>());
-  }
-  sync_ctrl(c);
-  const uint32_t n_items = (uint32_t)c->h_ctrl[kSlotB];
-  const uint32_t n_units = bitmap_ok ? (uint32_t)c->h_ctrl[kSlotA] : 0u;
-  const uint64_t walked = c->h_ctrl[kSlotC];               // list entries walked by the whole join (one probe each)
-  const uint64_t walked_bitmap = c->h_ctrl[kSlotD];        // those of them the bitmap kernel walks
-  items.reset(); it_sums.reset(); units.reset(); un_sums.reset();
-  DevBuf item_edge(c, (size_t)std::max(n_items, 1u) * 4), ecnt(c, (size_t)std::max(n_items, 1u) * 4), eacc(c, (size_t)std::max(n_items, 1u) * sizeof(A));
   DevBuf gcnt(c, (size_t)domain * 4), gtag(c, (size_t)domain * 4), flag(c, (size_t)domain * 4);
   const unsigned scan_tiles = (unsigned)((domain + kScanTile - 1) / kScanTile);
   DevBuf spine(c, ((size_t)scan_tiles + 1) * 4);
-  zero_ctrl(c, kSlotA, 4);
-  XLOG_LAUNCH(c, k_tri_item_edges, grid_for(E.n, 256), 256, 0, E.n, (const uint32_t*)item_off.as<uint32_t>(), item_edge.as<uint32_t>());
-  // declared work: one 4-byte entry per probe (the walked lists) plus the edge rows; the searches themselves hit L1 / L2
-  c->note_bytes = (int64_t)(walked - walked_bitmap) * 4 + (int64_t)E.n * 12;
-  c->r_candidates += (int64_t)walked;
-  XLOG_LAUNCH(c, (k_tri_edges<Op>), kSMs * 8, 256, 0, G, RT, H.sr == XLOG_SR_SUMPROD ? 1 : 0, n_items, (const uint32_t*)item_off.as<uint32_t>(),
-              (const uint32_t*)item_edge.as<uint32_t>(), ecnt.as<uint32_t>(), eacc.as<A>());
-  if (n_units) {
-    DevBuf unit(c, (size_t)n_units * 8);
-    XLOG_LAUNCH(c, k_tri_unit_fill, grid_for(domain, 256), 256, 0, G.out_off, domain, (const uint32_t*)item_off.as<uint32_t>(), (const uint32_t*)unit_off.as<uint32_t>(),
-                unit.as<uint2>());
-    const uint32_t words = (uint32_t)((node_domain + 31) / 32);
-    const size_t smem = (size_t)words * 8;
-    c->note_bytes = (int64_t)walked_bitmap * 4;
-    XLOG_CUDA(cudaFuncSetAttribute(k_tri_bitmap<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kTriBitmapMaxDomain / 32 * 8)));
-    XLOG_LAUNCH(c, (k_tri_bitmap<Op>), std::min<unsigned>(n_units, kSMs * 16), 256, smem, G, H.sr == XLOG_SR_SUMPROD ? 1 : 0, n_units, (const uint2*)unit.as<uint2>(),
-                G.out_off, (const uint32_t*)item_off.as<uint32_t>(), (const uint32_t*)item_edge.as<uint32_t>(), words, ecnt.as<uint32_t>(), eacc.as<A>());
+  const bool lse = H.sr == XLOG_SR_LOGSUMEXP;
+  if ((lse || H.sr == XLOG_SR_SUMPROD) && !(c->flags & XLOG_FLAG_NO_TRIANGLE_BITMAP) && ensure_tri_rank(c, E, out_ix, in_ix, lse)) {
+    zero_ctrl(c, kSlotA, 4);
+    c->r_candidates += (int64_t)E.tri.walk;
+    tri_rank_groups(c, E, lse, domain, gcnt.as<uint32_t>(), gtag.as<float>(), flag.as<uint32_t>(), ctrl_u32(c, kSlotD));
+  } else {
+    TriGraph G{};
+    G.n_edges = E.n;
+    G.src = E.cols[0].as<int32_t>(); G.dst = E.cols[1].as<int32_t>(); G.w = E.tags();
+    G.out_domain = out_ix.domain; G.in_domain = in_ix.domain;
+    G.out_off = out_ix.off.as<uint32_t>(); G.in_off = in_ix.off.as<uint32_t>();
+    G.in_src = in_ix.other[0]; G.in_w = in_ix.tags;
+    G.s_dst = G.dst; G.s_w = G.w;
+    // work items: edges cut into slices of the walked list (count -> scan -> one control read for the item total)
+    const uint32_t ne1 = E.n + 1;
+    DevBuf items(c, (size_t)ne1 * 4), item_off(c, (size_t)ne1 * 4);
+    const unsigned it_tiles = (ne1 + kScanTile - 1) / kScanTile;
+    DevBuf it_sums(c, (size_t)it_tiles * 4);
+    zero_ctrl(c, kSlotA, 4);
+    // per x: search the longer list, or mark in(x) in a shared-memory bitmap and walk every out(y) against it (triangle.cuh)
+    // the bitmap holds sources of edges into x (values of column 0) and is probed with targets (values of column 1): both ranges must fit
+    const int64_t node_domain = std::max(in_ix.domain, out_ix.domain);
+    const bool bitmap_ok = !(c->flags & XLOG_FLAG_NO_TRIANGLE_BITMAP) && node_domain <= kTriBitmapMaxDomain;
+    const int64_t sum_n = std::max<int64_t>(in_ix.domain, 1);
+    DevBuf route_sums(c, bitmap_ok ? (size_t)sum_n * 16 : 16);
+    TriRoute RT{route_sums.as<unsigned long long>(), route_sums.as<unsigned long long>() + (bitmap_ok ? sum_n : 0), bitmap_ok ? 1 : 0};
+    if (bitmap_ok) {
+      XLOG_CUDA(cudaMemsetAsync(route_sums.p, 0, (size_t)sum_n * 16, c->stream));
+      XLOG_LAUNCH(c, k_tri_route_sums, grid_for(E.n, 256), 256, 0, G, route_sums.as<unsigned long long>(), route_sums.as<unsigned long long>() + sum_n);
+    }
+    XLOG_LAUNCH(c, k_tri_plan, grid_for(ne1, 256), 256, 0, G, RT, items.as<uint32_t>(), (unsigned long long*)(c->d_ctrl + kSlotC),
+                (unsigned long long*)(c->d_ctrl + kSlotD));
+    XLOG_LAUNCH(c, (k_scan_tile_sums<uint32_t, uint32_t>), it_tiles, kScanBlock, 0, (const uint32_t*)items.as<uint32_t>(), (int64_t)ne1, it_sums.as<uint32_t>());
+    XLOG_LAUNCH(c, (k_scan_spine<uint32_t>), 1, 1024, 0, it_sums.as<uint32_t>(), (int64_t)it_tiles, ctrl_u32(c, kSlotB));
+    XLOG_LAUNCH(c, (k_scan_apply<uint32_t, uint32_t>), it_tiles, kScanBlock, 0, (const uint32_t*)items.as<uint32_t>(), (int64_t)ne1,
+                (const uint32_t*)it_sums.as<uint32_t>(), item_off.as<uint32_t>());
+    // the bitmap kernel's units: the work items of one x in slices (count -> scan; the total arrives with the same control read)
+    const int64_t nd1 = domain + 1;
+    const unsigned un_tiles = (unsigned)((nd1 + kScanTile - 1) / kScanTile);
+    DevBuf units(c, bitmap_ok ? (size_t)nd1 * 4 : 4), unit_off(c, bitmap_ok ? (size_t)nd1 * 4 : 4), un_sums(c, (size_t)un_tiles * 4);
+    if (bitmap_ok) {
+      XLOG_LAUNCH(c, k_tri_unit_count, grid_for(nd1, 256), 256, 0, G, RT, G.out_off, domain, (const uint32_t*)item_off.as<uint32_t>(), units.as<uint32_t>());
+      XLOG_LAUNCH(c, (k_scan_tile_sums<uint32_t, uint32_t>), un_tiles, kScanBlock, 0, (const uint32_t*)units.as<uint32_t>(), nd1, un_sums.as<uint32_t>());
+      XLOG_LAUNCH(c, (k_scan_spine<uint32_t>), 1, 1024, 0, un_sums.as<uint32_t>(), (int64_t)un_tiles, ctrl_u32(c, kSlotA));
+      XLOG_LAUNCH(c, (k_scan_apply<uint32_t, uint32_t>), un_tiles, kScanBlock, 0, (const uint32_t*)units.as<uint32_t>(), nd1, (const uint32_t*)un_sums.as<uint32_t>(),
+                  unit_off.as<uint32_t>());
+    }
+    sync_ctrl(c);
+    const uint32_t n_items = (uint32_t)c->h_ctrl[kSlotB];
+    const uint32_t n_units = bitmap_ok ? (uint32_t)c->h_ctrl[kSlotA] : 0u;
+    const uint64_t walked = c->h_ctrl[kSlotC];               // list entries walked by the whole join (one probe each)
+    const uint64_t walked_bitmap = c->h_ctrl[kSlotD];        // those of them the bitmap kernel walks
+    items.reset(); it_sums.reset(); units.reset(); un_sums.reset();
+    DevBuf item_edge(c, (size_t)std::max(n_items, 1u) * 4), ecnt(c, (size_t)std::max(n_items, 1u) * 4), eacc(c, (size_t)std::max(n_items, 1u) * sizeof(A));
+    zero_ctrl(c, kSlotA, 4);
+    XLOG_LAUNCH(c, k_tri_item_edges, grid_for(E.n, 256), 256, 0, E.n, (const uint32_t*)item_off.as<uint32_t>(), item_edge.as<uint32_t>());
+    // declared work: one 4-byte entry per probe (the walked lists) plus the edge rows; the searches themselves hit L1 / L2
+    c->note_bytes = (int64_t)(walked - walked_bitmap) * 4 + (int64_t)E.n * 12;
+    c->r_candidates += (int64_t)walked;
+    XLOG_LAUNCH(c, (k_tri_edges<Op>), kSMs * 8, 256, 0, G, RT, H.sr == XLOG_SR_SUMPROD ? 1 : 0, n_items, (const uint32_t*)item_off.as<uint32_t>(),
+                (const uint32_t*)item_edge.as<uint32_t>(), ecnt.as<uint32_t>(), eacc.as<A>());
+    if (n_units) {
+      DevBuf unit(c, (size_t)n_units * 8);
+      XLOG_LAUNCH(c, k_tri_unit_fill, grid_for(domain, 256), 256, 0, G.out_off, domain, (const uint32_t*)item_off.as<uint32_t>(), (const uint32_t*)unit_off.as<uint32_t>(),
+                  unit.as<uint2>());
+      const uint32_t words = (uint32_t)((node_domain + 31) / 32);
+      const size_t smem = (size_t)words * 8;
+      c->note_bytes = (int64_t)walked_bitmap * 4;
+      XLOG_CUDA(cudaFuncSetAttribute(k_tri_bitmap<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kTriBitmapMaxDomain / 32 * 8)));
+      XLOG_LAUNCH(c, (k_tri_bitmap<Op>), std::min<unsigned>(n_units, kSMs * 16), 256, smem, G, H.sr == XLOG_SR_SUMPROD ? 1 : 0, n_units, (const uint2*)unit.as<uint2>(),
+                  G.out_off, (const uint32_t*)item_off.as<uint32_t>(), (const uint32_t*)item_edge.as<uint32_t>(), words, ecnt.as<uint32_t>(), eacc.as<A>());
+    }
+    XLOG_LAUNCH(c, (k_tri_groups<Op>), grid_for((uint64_t)domain * 32, 256, kSMs * 8), 256, 0, G.out_off, domain, (const uint32_t*)item_off.as<uint32_t>(),
+                (const uint32_t*)ecnt.as<uint32_t>(), (const A*)eacc.as<A>(), gcnt.as<uint32_t>(), gtag.as<float>(), flag.as<uint32_t>(), ctrl_u32(c, kSlotD),
+                ctrl_u32(c, kSlotErr));
   }
-  XLOG_LAUNCH(c, (k_tri_groups<Op>), grid_for((uint64_t)domain * 32, 256, kSMs * 8), 256, 0, G.out_off, domain, (const uint32_t*)item_off.as<uint32_t>(),
-              (const uint32_t*)ecnt.as<uint32_t>(), (const A*)eacc.as<A>(), gcnt.as<uint32_t>(), gtag.as<float>(), flag.as<uint32_t>(), ctrl_u32(c, kSlotD),
-              ctrl_u32(c, kSlotErr));
   // positions of the surviving x: exclusive scan of the flags (kept in a second buffer)
   DevBuf pos(c, (size_t)domain * 4);
   XLOG_LAUNCH(c, (k_scan_tile_sums<uint32_t, uint32_t>), scan_tiles, kScanBlock, 0, (const uint32_t*)flag.as<uint32_t>(), domain, spine.as<uint32_t>());

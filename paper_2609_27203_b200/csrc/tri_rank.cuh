@@ -1,0 +1,293 @@
+// Fused triangle aggregate  h(x, count) :- e(x,y), e(y,z), e(z,x)  over a degree-ordered copy of the graph, under logsumexp and
+// sum-product.
+//
+// triangle.cuh finds every directed triangle three times, once from each of its corners, and walks 8.4e8 list entries on
+// an R-MAT 18 graph to do so.  Here the nodes are numbered by degree and a triangle v -> a -> b -> v is found from its lowest
+// corner v, whose lists are short (at most a few hundred entries whatever the hubs): 1.2e8 entries for the same graph.  Its
+// term goes to all three corners.  The tags make that cheap: the term's weight exp(w_va + w_ab + w_bv) is the product of three
+// numbers kept with the edges, and the sums are plain sums in fp64 (for sum-product the tags are such numbers already).
+// Usable while no product of three can leave the normal fp32 range (|w| <= kTriRankMaxTag under logsumexp).
+//
+// Two launches, one per group of corners, so that no sum is formed by atomics in an order that varies:
+//   by a:  mark out(a) in a shared-memory bitmap; for every lower v with v -> a walk the higher b with b -> v: a marked b closes
+//          a triangle.  S[a] is the block's sum; v's part is a sum per edge (v,a), written in v's own order.
+//   by b:  the same over the reversed graph (mark in(b), for every lower v with b -> v walk the higher a with v -> a): S[b].
+// A corner a with little to walk is handled by one warp that searches out(a) instead (k_tri_rank_small).  k_tri_rank_groups then
+// adds up each node's parts: its units' sums of both launches and its edges' sums.
+//
+// R-MAT 18 (3.9 M edges, 39 M triangles): 5.47 -> 1.29 ms per evaluation, 0.84 ms of it the two bitmap launches; the first one on a
+// new relation, which orders the graph, 5.80 -> 2.70.
+#pragma once
+#include "common.cuh"
+
+namespace xlog {
+
+constexpr int64_t kTriRankMaxNodes = (int64_t)1 << 19;       // 128 KB of bitmap and places
+constexpr uint32_t kTriRankMinEdges = 1u << 17;  // below, the plain kernels are as fast and need no second copy of the graph
+constexpr float kTriRankMaxTag = 28.f;           // exp(3 * 28) and exp(-3 * 28) are normal fp32 numbers
+constexpr int kTriRankBlock = 512;
+constexpr uint32_t kTriRankSmall = 2048;         // corners with fewer entries to walk are searched, a warp each
+constexpr int kTriRankSweeps = 4;                // sweeps of 32 list entries a warp reads before it tests them
+
+enum { kTrkEdges = 0, kTrkNodes = 1, kTrkLoops = 2, kTrkAbsMax = 3, kTrkUnitsA = 4, kTrkUnitsB = 5, kTrkWalkA = 6, kTrkWalkB = 7, kTrkTotals = 8 };
+
+// One orientation of the ordered graph: lists of neighbours in ascending rank; entries [off[v], split[v]) rank lower than v.
+struct TriRankLists {
+  const uint32_t* off;
+  const uint32_t* split;
+  const uint32_t* nbr;
+  const float* e;                    // the edge's number
+  const uint32_t* other;             // the place of the same edge in the other orientation's lists (may be null)
+};
+
+// degree of every node that can be a corner (edges in and out), else 0; loops among the edges, largest |tag|
+static __global__ void __launch_bounds__(256) k_trk_degrees(const uint32_t* __restrict__ out_off, int64_t out_domain, const uint32_t* __restrict__ in_off, int64_t in_domain,
+                                                            uint32_t n_nodes, uint32_t* __restrict__ deg, uint32_t* __restrict__ node, unsigned long long* __restrict__ totals) {
+  uint32_t corners = 0;
+  for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n_nodes; v += gridDim.x * blockDim.x) {
+    const uint32_t o = v < out_domain ? out_off[v + 1] - out_off[v] : 0u, i = v < in_domain ? in_off[v + 1] - in_off[v] : 0u;
+    const uint32_t d = o && i ? o + i : 0u;
+    deg[v] = d; node[v] = v;
+    corners += d != 0u;
+  }
+  corners = __reduce_add_sync(0xffffffffu, corners);
+  if (lane_id() == 0 && corners) atomicAdd(totals + kTrkNodes, (unsigned long long)corners);
+}
+// rank of every node among the corners, in order of degree (node: the nodes sorted by degree); the others get n_nodes
+static __global__ void __launch_bounds__(256) k_trk_ranks(const uint32_t* __restrict__ node, uint32_t n_nodes, const unsigned long long* __restrict__ totals, uint32_t* __restrict__ rank) {
+  const uint32_t skip = n_nodes - (uint32_t)totals[kTrkNodes];
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_nodes; i += gridDim.x * blockDim.x) rank[node[i]] = i >= skip ? i - skip : n_nodes;
+}
+// the edges between corners first: key = rank of the source, of the others n_nodes
+static __global__ void __launch_bounds__(256) k_trk_edges(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, const float* __restrict__ w, uint32_t n,
+                                                          const uint32_t* __restrict__ rank, uint32_t n_nodes, uint32_t* __restrict__ key, uint32_t* __restrict__ edge,
+                                                          unsigned long long* __restrict__ totals) {
+  uint32_t kept = 0, loops = 0, top = 0;
+  for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+    const uint32_t s = rank[src[e]], t = rank[dst[e]];
+    const bool in = s < n_nodes && t < n_nodes;
+    key[e] = in ? s : n_nodes;
+    edge[e] = e;
+    kept += in;
+    loops += src[e] == dst[e];
+    top = max(top, __float_as_uint(fabsf(w[e])));
+  }
+  kept = __reduce_add_sync(0xffffffffu, kept); loops = __reduce_add_sync(0xffffffffu, loops); top = __reduce_max_sync(0xffffffffu, top);
+  if (lane_id() == 0) {
+    if (kept) atomicAdd(totals + kTrkEdges, (unsigned long long)kept);
+    if (loops) atomicAdd(totals + kTrkLoops, (unsigned long long)loops);
+    atomicMax(totals + kTrkAbsMax, (unsigned long long)top);
+  }
+}
+static __global__ void __launch_bounds__(256) k_trk_keys(const uint32_t* __restrict__ edge, uint32_t n, const int32_t* __restrict__ col, const uint32_t* __restrict__ rank, uint32_t* __restrict__ key) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) key[i] = rank[col[edge[i]]];
+}
+// lists of one orientation from the edges in its order; place[e] (optional) = where edge e went
+template <bool EXP>
+__global__ void __launch_bounds__(256) k_trk_lists(const uint32_t* __restrict__ edge, uint32_t n, const int32_t* __restrict__ nbr_col, const float* __restrict__ w,
+                                                   const uint32_t* __restrict__ rank, uint32_t* __restrict__ nbr, float* __restrict__ num, uint32_t* __restrict__ place) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const uint32_t e = edge[i];
+    nbr[i] = rank[nbr_col[e]];
+    num[i] = EXP ? expf(w[e]) : w[e];
+    if (place) place[e] = i;
+  }
+}
+static __global__ void __launch_bounds__(256) k_trk_gather(const uint32_t* __restrict__ edge, uint32_t n, const uint32_t* __restrict__ place, uint32_t* __restrict__ other) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) other[i] = place[edge[i]];
+}
+static __global__ void __launch_bounds__(256) k_trk_splits(const uint32_t* __restrict__ off, const uint32_t* __restrict__ nbr, uint32_t n_nodes, uint32_t* __restrict__ split) {
+  for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n_nodes; v += gridDim.x * blockDim.x) {
+    uint32_t lo = off[v], hi = off[v + 1];
+    while (lo < hi) { const uint32_t mid = (lo + hi) >> 1; if (nbr[mid] < v) lo = mid + 1; else hi = mid; }
+    split[v] = lo;
+  }
+}
+
+// Items of a unit: enough that marking the corner's list (`marked` entries) is a small part of the unit's walk.
+__device__ __forceinline__ uint32_t trk_unit_items(uint32_t marked) { return max(256u, marked / 8u); }
+
+// A warp per corner: entries to walk in the lists of its lower neighbours in I; units of the bitmap kernel (0: searched).
+static __global__ void __launch_bounds__(256) k_trk_units(TriRankLists I, TriRankLists M, uint32_t n_nodes, uint32_t* __restrict__ units, unsigned long long* __restrict__ walk) {
+  const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+  unsigned long long sum = 0;
+  for (uint32_t a = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; a < n_nodes; a += nwarps) {
+    const uint32_t i0 = I.off[a], i1 = I.split[a];
+    uint32_t n = 0;
+    for (uint32_t i = i0 + lane_id(); i < i1; i += 32) { const uint32_t v = I.nbr[i]; n += I.off[v + 1] - I.split[v]; }
+    n = __reduce_add_sync(0xffffffffu, n);
+    if (lane_id() == 0) { const uint32_t per = trk_unit_items(M.off[a + 1] - M.off[a]); units[a] = n >= kTriRankSmall ? (i1 - i0 + per - 1) / per : 0u; }
+    sum += n;
+  }
+  if (lane_id() == 0 && sum) atomicAdd(walk, sum);
+  if (blockIdx.x == 0 && threadIdx.x == 0) units[n_nodes] = 0u;
+}
+static __global__ void __launch_bounds__(256) k_trk_unit_fill(TriRankLists I, TriRankLists M, uint32_t n_nodes, const uint32_t* __restrict__ unit_off, uint2* __restrict__ unit) {
+  for (uint32_t a = blockIdx.x * blockDim.x + threadIdx.x; a < n_nodes; a += gridDim.x * blockDim.x) {
+    const uint32_t per = trk_unit_items(M.off[a + 1] - M.off[a]);
+    for (uint32_t u = unit_off[a], i = I.off[a]; u < unit_off[a + 1]; ++u, i += per) unit[u] = make_uint2(a, i);
+  }
+}
+
+struct TriRankPass {
+  TriRankLists I;                    // the corner's neighbours (lower ones are the v), and the v's lists that are walked
+  TriRankLists M;                    // the corner's list that is marked
+  uint32_t n_nodes;
+  const uint32_t* unit_off;
+  const uint2* unit;
+  uint32_t n_units;
+  double* unit_sum;                  // per unit, then per searched corner at n_units + a
+  uint32_t* unit_cnt;
+  double* edge_sum;                  // per edge (v, corner), at its place in v's list of the other orientation (null: not wanted)
+  uint32_t* edge_cnt;
+};
+
+// One block per unit, the corners of highest degree (the longest units) first.  A warp takes an item (a lower neighbour v) and
+// walks v's higher neighbours, kTriRankSweeps sweeps of them in flight; hits multiply and add where they fall.
+template <bool EDGES>
+__global__ void __launch_bounds__(kTriRankBlock) k_tri_rank(const __grid_constant__ TriRankPass P) {
+  extern __shared__ uint32_t trk_smem[];
+  __shared__ double s_sum[kTriRankBlock / 32];
+  __shared__ uint32_t s_cnt[kTriRankBlock / 32];
+  const uint32_t words = (P.n_nodes + 31) / 32;
+  uint32_t* bits = trk_smem;
+  uint32_t* before = trk_smem + words;             // per word: place in the marked list of the first entry marked in it
+  const unsigned lane = lane_id(), wid = warp_id();
+  const uint32_t u = P.n_units - 1 - blockIdx.x;
+  const uint2 un = P.unit[u];
+  const uint32_t a = un.x, m0 = P.M.off[a], m1 = P.M.off[a + 1];
+  for (uint32_t i = threadIdx.x; i < words; i += kTriRankBlock) bits[i] = 0u;
+  __syncthreads();
+  for (uint32_t i = m0 + threadIdx.x; i < m1; i += kTriRankBlock) {
+    const uint32_t z = P.M.nbr[i];
+    atomicOr(bits + (z >> 5), 1u << (z & 31));
+    if (i == m0 || (P.M.nbr[i - 1] >> 5) != (z >> 5)) before[z >> 5] = i;
+  }
+  __syncthreads();
+  const uint32_t it0 = un.y, it1 = min(it0 + trk_unit_items(m1 - m0), P.I.split[a]);
+  double sum = 0.0;
+  uint32_t cnt = 0;
+  for (uint32_t it = it0 + wid; it < it1; it += kTriRankBlock / 32) {
+    const uint32_t v = P.I.nbr[it];
+    const float ev = P.I.e[it];
+    const uint32_t w0 = P.I.split[v], w1 = P.I.off[v + 1];
+    double isum = 0.0;
+    uint32_t icnt = 0;
+    for (uint32_t i0 = w0; i0 < w1; i0 += 32 * kTriRankSweeps) {
+      uint32_t z[kTriRankSweeps], wd[kTriRankSweeps];
+#pragma unroll
+      for (int k = 0; k < kTriRankSweeps; ++k) { const uint32_t i = i0 + k * 32 + lane; z[k] = i < w1 ? P.I.nbr[i] : 0xffffffffu; }
+#pragma unroll
+      for (int k = 0; k < kTriRankSweeps; ++k) wd[k] = z[k] != 0xffffffffu ? bits[z[k] >> 5] : 0u;
+#pragma unroll
+      for (int k = 0; k < kTriRankSweeps; ++k)
+        if ((wd[k] >> (z[k] & 31)) & 1u) {
+          const uint32_t at = before[z[k] >> 5] + __popc(wd[k] & ((1u << (z[k] & 31)) - 1u));
+          isum += (double)((ev * P.M.e[at]) * P.I.e[i0 + k * 32 + lane]);
+          ++icnt;
+        }
+    }
+    sum += isum; cnt += icnt;
+    if (EDGES) {
+      icnt = __reduce_add_sync(0xffffffffu, icnt);
+      if (icnt)
+#pragma unroll
+        for (int d = 16; d; d >>= 1) isum += __shfl_xor_sync(0xffffffffu, isum, d);
+      if (lane == 0) { const uint32_t o = P.I.other[it]; P.edge_sum[o] = isum; P.edge_cnt[o] = icnt; }
+    }
+  }
+  cnt = __reduce_add_sync(0xffffffffu, cnt);
+#pragma unroll
+  for (int d = 16; d; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+  if (lane == 0) { s_sum[wid] = sum; s_cnt[wid] = cnt; }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    uint32_t c = 0;
+    for (int w = 0; w < kTriRankBlock / 32; ++w) { t += s_sum[w]; c += s_cnt[w]; }
+    P.unit_sum[u] = t; P.unit_cnt[u] = c;
+  }
+}
+
+// The corners without units, a warp each: a lane per item, items with more than 16 entries by the whole warp; every entry is
+// searched in the corner's list.
+template <bool EDGES>
+__global__ void __launch_bounds__(256) k_tri_rank_small(const __grid_constant__ TriRankPass P) {
+  const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+  const unsigned lane = lane_id();
+  for (uint32_t a = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; a < P.n_nodes; a += nwarps) {
+    if (P.unit_off[a + 1] != P.unit_off[a]) continue;
+    const uint32_t m0 = P.M.off[a], m1 = P.M.off[a + 1], i1 = P.I.split[a];
+    double sum = 0.0;
+    uint32_t cnt = 0;
+    for (uint32_t ib = P.I.off[a]; ib < i1; ib += 32) {
+      const uint32_t it = ib + lane;
+      uint32_t w0 = 0, w1 = 0, icnt = 0;
+      float ev = 0.f;
+      double isum = 0.0;
+      if (it < i1) { const uint32_t v = P.I.nbr[it]; ev = P.I.e[it]; w0 = P.I.split[v]; w1 = P.I.off[v + 1]; }
+      auto probe = [&](uint32_t i, float e) {
+        const uint32_t z = P.I.nbr[i];
+        uint32_t lo = m0, hi = m1;
+        while (lo < hi) { const uint32_t mid = (lo + hi) >> 1; if (P.M.nbr[mid] < z) lo = mid + 1; else hi = mid; }
+        if (lo < m1 && P.M.nbr[lo] == z) { isum += (double)((e * P.M.e[lo]) * P.I.e[i]); ++icnt; }
+      };
+      if (w1 - w0 <= 16) for (uint32_t i = w0; i < w1; ++i) probe(i, ev);
+      for (unsigned big = __ballot_sync(0xffffffffu, w1 - w0 > 16); big; big &= big - 1) {
+        const int src = __ffs(big) - 1;
+        const uint32_t W0 = __shfl_sync(0xffffffffu, w0, src), W1 = __shfl_sync(0xffffffffu, w1, src);
+        const float E = __shfl_sync(0xffffffffu, ev, src);
+        const double keep = isum;
+        const uint32_t kept = icnt;
+        isum = 0.0; icnt = 0;
+        for (uint32_t i = W0 + lane; i < W1; i += 32) probe(i, E);
+        const uint32_t all = __reduce_add_sync(0xffffffffu, icnt);
+#pragma unroll
+        for (int d = 16; d; d >>= 1) isum += __shfl_xor_sync(0xffffffffu, isum, d);
+        if ((int)lane != src) { isum = keep; icnt = kept; } else icnt = all;
+        __syncwarp();
+      }
+      if (EDGES && it < i1) { const uint32_t o = P.I.other[it]; P.edge_sum[o] = isum; P.edge_cnt[o] = icnt; }
+      sum += isum; cnt += icnt;
+    }
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+#pragma unroll
+    for (int d = 16; d; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+    if (lane == 0) { P.unit_sum[P.n_units + a] = sum; P.unit_cnt[P.n_units + a] = cnt; }
+  }
+}
+
+// A warp per node of the relation: its parts from both launches and from its edges to higher corners, in a fixed order.
+template <bool LSE>
+__global__ void __launch_bounds__(256) k_tri_rank_groups(TriRankPass A, TriRankPass B, const uint32_t* __restrict__ rank, int64_t domain, uint32_t* __restrict__ grp_cnt,
+                                                         float* __restrict__ grp_tag, uint32_t* __restrict__ flag, uint32_t* __restrict__ max_cnt, uint32_t* __restrict__ err) {
+  const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+  const unsigned lane = lane_id();
+  for (int64_t x = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < domain; x += nwarps) {
+    const uint32_t v = rank[x];
+    double sum = 0.0;
+    uint64_t cnt = 0;
+    if (v < A.n_nodes) {
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        const TriRankPass& Q = p ? B : A;
+        const uint32_t u0 = Q.unit_off[v], u1 = Q.unit_off[v + 1];
+        for (uint32_t u = u0 + lane; u < u1; u += 32) { sum += Q.unit_sum[u]; cnt += Q.unit_cnt[u]; }
+        if (u0 == u1 && lane == 0) { sum += Q.unit_sum[Q.n_units + v]; cnt += Q.unit_cnt[Q.n_units + v]; }
+      }
+      const uint32_t e1 = A.M.off[v + 1];
+      for (uint32_t i = A.M.split[v] + lane; i < e1; i += 32) { sum += A.edge_sum[i]; cnt += A.edge_cnt[i]; }
+    }
+#pragma unroll
+    for (int d = 16; d; d >>= 1) { sum += __shfl_xor_sync(0xffffffffu, sum, d); cnt += __shfl_xor_sync(0xffffffffu, cnt, d); }
+    if (lane == 0) {
+      if (cnt > 0x7fffffffull) { atomicOr(err, kErrCountOverflow); cnt = 0x7fffffffull; }
+      grp_cnt[x] = (uint32_t)cnt;
+      grp_tag[x] = cnt ? (LSE ? (float)log(sum) : (float)sum) : 0.f;
+      flag[x] = cnt ? 1u : 0u;
+      if (cnt) atomicMax(max_cnt, (uint32_t)cnt);
+    }
+  }
+}
+
+}  // namespace xlog

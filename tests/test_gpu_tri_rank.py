@@ -1,0 +1,96 @@
+"""Triangle aggregate over the degree-ordered graph against the plain kernels (counts equal; tags to 1e-5 absolute in log space and
+1e-6 relative for sums: two roundings of a three-factor fp32 product against two of a three-term fp32 sum of at most 84) and
+against closed forms."""
+import numpy as np
+import pytest
+
+from paper_2609_27203_b200 import synth
+from paper_2609_27203_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def run(prog, flags=0, arena=1 << 30, again=1):
+    from paper_2609_27203_b200 import xlog
+    ctx, ids, _ = xlog.load_program(prog, arena_bytes=arena, flags=flags | xlog.FLAG_PROFILE)
+    out = []
+    for _ in range(again):
+        ctx.reset_idb()
+        ctx.fixpoint()
+        out.append(ctx.read(ids["tri_agg"]))
+    ran = "k_tri_rank_small" in ctx.profile()
+    ctx.close()
+    return out, ran
+
+
+def sum_program(s, d, w):
+    p = W.triangle_program(s, d, w)
+    p.relations = {k: (a, W.SUMPROD) for k, (a, _) in p.relations.items()}
+    return p
+
+
+@pytest.mark.parametrize("scale,ef", [(13, 30), (15, 8), (17, 4)])
+@pytest.mark.parametrize("sums", [False, True])
+def test_against_the_plain_kernels(scale, ef, sums):
+    from paper_2609_27203_b200 import xlog
+    s, d, w = synth.rmat_graph(scale, ef, scale, "n01")
+    assert len(s) >= 1 << 17
+    if scale == 13:                                           # the widest tags the products allow
+        w[::5] = np.where(w[::5] > 0, 28, -28)
+    prog = sum_program(s, d, np.exp(w * 0.1).astype(np.float32)) if sums else W.triangle_program(s, d, w)
+    (a, b), ran = run(prog, again=2)
+    (want,), plain = run(prog, xlog.FLAG_NO_TRIANGLE_BITMAP)
+    assert ran and not plain
+    assert all(np.array_equal(x, y) for x, y in zip(a[0], want[0]))
+    assert np.allclose(a[1], want[1], rtol=1e-6 if sums else 0, atol=0 if sums else 1e-5)
+    assert np.array_equal(a[1].view(np.int32), b[1].view(np.int32))            # run to run, bit for bit
+
+
+@pytest.mark.parametrize("n", [362, 363, 400, 1025])          # n (n - 1) edges: around 2^17
+def test_complete_graph(n):
+    s, d = (x.reshape(-1) for x in np.meshgrid(np.arange(n), np.arange(n), indexing="ij"))
+    s, d = s[s != d] * 5 + 3, d[s != d] * 5 + 3               # gaps between the ids
+    ((got, _), ran) = run(W.triangle_program(s, d, np.zeros(len(s), np.float32)), again=2)
+    assert ran == (n * (n - 1) >= 1 << 17)
+    cols, tags = got
+    assert cols[0].tolist() == (np.arange(n) * 5 + 3).tolist() and (cols[1] == (n - 1) * (n - 2)).all()
+    assert np.allclose(tags, np.log((n - 1) * (n - 2)), rtol=1e-6)
+
+
+def test_hub_wheels_and_lone_nodes():
+    # a hub joined both ways to every node of a long directed ring; nodes without in- or out-edges beside it
+    from paper_2609_27203_b200 import xlog
+    n = 70000
+    ring = np.arange(2, n)
+    s = np.concatenate([ring, np.zeros(n - 2, int), ring, [0, 1], np.full(500, 1), n + np.arange(300)])
+    d = np.concatenate([np.roll(ring, -1), ring, np.full(n - 2, 0), [1, 0], n + 1000 + np.arange(500), np.full(300, 1)])
+    w = np.random.default_rng(3).normal(size=len(s)).astype(np.float32)
+    prog = W.triangle_program(s, d, w)
+    (got,), ran = run(prog)
+    (want,), _ = run(prog, xlog.FLAG_NO_TRIANGLE_BITMAP)
+    assert ran and all(np.array_equal(x, y) for x, y in zip(got[0], want[0])) and np.allclose(got[1], want[1], rtol=0, atol=1e-5)
+    assert got[0][1][0] == n - 2                              # the hub closes one triangle per ring edge
+
+
+@pytest.mark.parametrize("why", ["loop", "tag", "none"])
+def test_graphs_it_leaves_to_the_plain_kernels(why):
+    from paper_2609_27203_b200 import xlog
+    s, d, w = synth.rmat_graph(13, 30, 9, "n01")
+    if why == "loop":
+        s, d, w = np.append(s, 5), np.append(d, 5), np.append(w, np.float32(1))
+    if why == "tag":
+        w[100] = 28.5
+    prog = W.triangle_program(s, d, w)
+    (got,), ran = run(prog)
+    (want,), _ = run(prog, xlog.FLAG_NO_TRIANGLE_BITMAP)
+    assert ran == (why == "none")
+    assert all(np.array_equal(x, y) for x, y in zip(got[0], want[0])) and np.allclose(got[1], want[1], rtol=0, atol=1e-5)
+    if why == "none":                                         # reloading the relation drops the ordered copy
+        ctx, ids, _ = xlog.load_program(prog, arena_bytes=1 << 30)
+        ctx.fixpoint()
+        ctx.load(ids["e"], [s[::2].copy(), d[::2].copy()], w[::2].copy())
+        ctx.fixpoint()
+        half = ctx.read(ids["tri_agg"])
+        (want,), _ = run(W.triangle_program(s[::2], d[::2], w[::2]), xlog.FLAG_NO_TRIANGLE_BITMAP)
+        assert all(np.array_equal(x, y) for x, y in zip(half[0], want[0])) and np.allclose(half[1], want[1], rtol=0, atol=1e-5)
+        ctx.close()
