@@ -15,8 +15,9 @@
 // A corner a with little to walk is handled by one warp that searches out(a) instead (k_tri_rank_small).  k_tri_rank_groups then
 // adds up each node's parts: its units' sums of both launches and its edges' sums.
 //
-// R-MAT 18 (3.9 M edges, 39 M triangles): 5.47 -> 1.29 ms per evaluation, 0.84 ms of it the two bitmap launches; the first one on a
-// new relation, which orders the graph, 5.80 -> 2.70.
+// R-MAT 18 (3.9 M edges, 39 M triangles): 5.43 -> 1.25 ms per evaluation, 0.96 ms of it the two bitmap launches (bound by instruction
+// issue: 75 % of the slots), 0.11 the searched corners; the first one on a
+// new relation, which orders the graph, 5.80 -> 2.66.
 #pragma once
 #include "common.cuh"
 
@@ -26,7 +27,9 @@ constexpr int64_t kTriRankMaxNodes = (int64_t)1 << 19;       // 128 KB of bitmap
 constexpr uint32_t kTriRankMinEdges = 1u << 17;  // below, the plain kernels are as fast and need no second copy of the graph
 constexpr float kTriRankMaxTag = 28.f;           // exp(3 * 28) and exp(-3 * 28) are normal fp32 numbers
 constexpr int kTriRankBlock = 512;
-constexpr uint32_t kTriRankSmall = 2048;         // corners with fewer entries to walk are searched, a warp each
+// corners with fewer entries to walk are searched, a warp each; a block's bitmap costs about as much as 500 searches in a row
+// (all kernels, us, at limits of 2048 / 1024 / 512: R-MAT 18 1186 / 1203 / 1212, R-MAT 16 367 / 304 / 284, R-MAT 14 271 / 200 / 173)
+constexpr uint32_t kTriRankSmall = 512;
 constexpr int kTriRankSweeps = 4;                // sweeps of 32 list entries a warp reads before it tests them
 
 enum { kTrkEdges = 0, kTrkNodes = 1, kTrkLoops = 2, kTrkAbsMax = 3, kTrkUnitsA = 4, kTrkUnitsB = 5, kTrkWalkA = 6, kTrkWalkB = 7, kTrkTotals = 8 };
@@ -209,46 +212,66 @@ __global__ void __launch_bounds__(kTriRankBlock) k_tri_rank(const __grid_constan
   }
 }
 
-// The corners without units, a warp each: a lane per item, items with more than 16 entries by the whole warp; every entry is
-// searched in the corner's list.
+// The corners without units, a warp each: 32 items at a time, their entries laid out in a line over the lanes, every entry
+// searched in the corner's list (in shared memory where it has at most kTriRankListed entries).  The values of one item are
+// neighbours in that line: a segmented scan per step brings them together in a fixed order.
+constexpr uint32_t kTriRankListed = 512;
 template <bool EDGES>
 __global__ void __launch_bounds__(256) k_tri_rank_small(const __grid_constant__ TriRankPass P) {
+  __shared__ uint32_t s_list[8][kTriRankListed];
+  __shared__ double s_item[8][32];
+  __shared__ uint32_t s_hits[8][32];
   const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-  const unsigned lane = lane_id();
+  const unsigned lane = lane_id(), wid = warp_id();
   for (uint32_t a = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; a < P.n_nodes; a += nwarps) {
     if (P.unit_off[a + 1] != P.unit_off[a]) continue;
-    const uint32_t m0 = P.M.off[a], m1 = P.M.off[a + 1], i1 = P.I.split[a];
+    const uint32_t m0 = P.M.off[a], nm = P.M.off[a + 1] - m0, i1 = P.I.split[a];
+    const bool listed = nm <= kTriRankListed;
+    __syncwarp();
+    if (listed && i1 > P.I.off[a]) for (uint32_t i = lane; i < nm; i += 32) s_list[wid][i] = P.M.nbr[m0 + i];
+    __syncwarp();
     double sum = 0.0;
     uint32_t cnt = 0;
     for (uint32_t ib = P.I.off[a]; ib < i1; ib += 32) {
       const uint32_t it = ib + lane;
-      uint32_t w0 = 0, w1 = 0, icnt = 0;
+      uint32_t w0 = 0, n = 0;
       float ev = 0.f;
-      double isum = 0.0;
-      if (it < i1) { const uint32_t v = P.I.nbr[it]; ev = P.I.e[it]; w0 = P.I.split[v]; w1 = P.I.off[v + 1]; }
-      auto probe = [&](uint32_t i, float e) {
-        const uint32_t z = P.I.nbr[i];
-        uint32_t lo = m0, hi = m1;
-        while (lo < hi) { const uint32_t mid = (lo + hi) >> 1; if (P.M.nbr[mid] < z) lo = mid + 1; else hi = mid; }
-        if (lo < m1 && P.M.nbr[lo] == z) { isum += (double)((e * P.M.e[lo]) * P.I.e[i]); ++icnt; }
-      };
-      if (w1 - w0 <= 16) for (uint32_t i = w0; i < w1; ++i) probe(i, ev);
-      for (unsigned big = __ballot_sync(0xffffffffu, w1 - w0 > 16); big; big &= big - 1) {
-        const int src = __ffs(big) - 1;
-        const uint32_t W0 = __shfl_sync(0xffffffffu, w0, src), W1 = __shfl_sync(0xffffffffu, w1, src);
-        const float E = __shfl_sync(0xffffffffu, ev, src);
-        const double keep = isum;
-        const uint32_t kept = icnt;
-        isum = 0.0; icnt = 0;
-        for (uint32_t i = W0 + lane; i < W1; i += 32) probe(i, E);
-        const uint32_t all = __reduce_add_sync(0xffffffffu, icnt);
+      if (it < i1) { const uint32_t v = P.I.nbr[it]; ev = P.I.e[it]; w0 = P.I.split[v]; n = P.I.off[v + 1] - w0; }
+      if (EDGES) { s_item[wid][lane] = 0.0; s_hits[wid][lane] = 0u; }
+      const uint32_t incl = warp_scan_incl(n), total = __shfl_sync(0xffffffffu, incl, 31);
+      const uint32_t from = w0 + n - incl;             // entry p of the line is entry from + p of its item's list
+      __syncwarp();
+      for (uint32_t p0 = 0; p0 < total; p0 += 32) {
+        const uint32_t p = p0 + lane;
+        uint32_t owner = 0;                            // first item whose inclusive prefix exceeds p
 #pragma unroll
-        for (int d = 16; d; d >>= 1) isum += __shfl_xor_sync(0xffffffffu, isum, d);
-        if ((int)lane != src) { isum = keep; icnt = kept; } else icnt = all;
-        __syncwarp();
+        for (int d = 16; d; d >>= 1) { const uint32_t x = __shfl_sync(0xffffffffu, incl, owner + d - 1); if (x <= p) owner += d; }
+        const uint32_t i = __shfl_sync(0xffffffffu, from, owner) + p;
+        const float e = __shfl_sync(0xffffffffu, ev, owner);
+        double val = 0.0;
+        uint32_t hit = 0;
+        if (p < total) {
+          const uint32_t z = P.I.nbr[i];
+          uint32_t lo = 0, hi = nm;
+          if (listed) while (lo < hi) { const uint32_t mid = (lo + hi) >> 1; if (s_list[wid][mid] < z) lo = mid + 1; else hi = mid; }
+          else while (lo < hi) { const uint32_t mid = (lo + hi) >> 1; if (P.M.nbr[m0 + mid] < z) lo = mid + 1; else hi = mid; }
+          if (lo < nm && (listed ? s_list[wid][lo] : P.M.nbr[m0 + lo]) == z) { hit = 1u; val = (double)((e * P.M.e[m0 + lo]) * P.I.e[i]); }
+        }
+        sum += val; cnt += hit;
+        if (EDGES && __any_sync(0xffffffffu, hit)) {
+#pragma unroll
+          for (int d = 1; d < 32; d <<= 1) {
+            const double ov = __shfl_up_sync(0xffffffffu, val, d);
+            const uint32_t oh = __shfl_up_sync(0xffffffffu, hit, d), oo = __shfl_up_sync(0xffffffffu, owner, d);
+            if ((int)lane >= d && oo == owner) { val += ov; hit += oh; }
+          }
+          const uint32_t next = __shfl_down_sync(0xffffffffu, owner, 1);
+          if (hit && (lane == 31 || next != owner)) { s_item[wid][owner] += val; s_hits[wid][owner] += hit; }
+          __syncwarp();
+        }
       }
-      if (EDGES && it < i1) { const uint32_t o = P.I.other[it]; P.edge_sum[o] = isum; P.edge_cnt[o] = icnt; }
-      sum += isum; cnt += icnt;
+      if (EDGES && it < i1) { const uint32_t o = P.I.other[it]; P.edge_sum[o] = s_item[wid][lane]; P.edge_cnt[o] = s_hits[wid][lane]; }
+      __syncwarp();
     }
     cnt = __reduce_add_sync(0xffffffffu, cnt);
 #pragma unroll
