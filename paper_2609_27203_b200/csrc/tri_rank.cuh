@@ -15,9 +15,9 @@
 // A corner a with little to walk is handled by one warp that searches out(a) instead (k_tri_rank_small).  k_tri_rank_groups then
 // adds up each node's parts: its units' sums of both launches and its edges' sums.
 //
-// R-MAT 18 (3.9 M edges, 39 M triangles): 5.43 -> 1.25 ms per evaluation, 0.96 ms of it the two bitmap launches (bound by instruction
+// R-MAT 18 (3.9 M edges, 39 M triangles): 5.51 -> 1.17 ms per evaluation, 0.88 ms of it the two bitmap launches (bound by instruction
 // issue: 75 % of the slots), 0.11 the searched corners; the first one on a
-// new relation, which orders the graph, 5.80 -> 2.66.
+// new relation, which orders the graph, 5.84 -> 2.59.
 #pragma once
 #include "common.cuh"
 
@@ -30,7 +30,7 @@ constexpr int kTriRankBlock = 512;
 // corners with fewer entries to walk are searched, a warp each; a block's bitmap costs about as much as 500 searches in a row
 // (all kernels, us, at limits of 2048 / 1024 / 512: R-MAT 18 1186 / 1203 / 1212, R-MAT 16 367 / 304 / 284, R-MAT 14 271 / 200 / 173)
 constexpr uint32_t kTriRankSmall = 512;
-constexpr int kTriRankSweeps = 4;                // sweeps of 32 list entries a warp reads before it tests them
+constexpr int kTriRankSweeps = 2;                // sweeps of 32 list entries a warp reads before it tests them (both launches, us: 1 907, 2 878, 3 909, 4 962)
 
 enum { kTrkEdges = 0, kTrkNodes = 1, kTrkLoops = 2, kTrkAbsMax = 3, kTrkUnitsA = 4, kTrkUnitsB = 5, kTrkWalkA = 6, kTrkWalkB = 7, kTrkTotals = 8 };
 
