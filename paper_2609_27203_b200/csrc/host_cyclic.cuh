@@ -5,6 +5,7 @@
 #include "triangle.cuh"
 #include "tri_rank.cuh"
 #include "cycle4.cuh"
+#include "bits_join.cuh"
 
 namespace xlog {
 namespace {
@@ -274,6 +275,69 @@ void triangle_aggregate_t(Ctx* c, Relation& H, const RuleC& r) {
   else set_current(H, std::move(kt));
 }
 
+// ---- closing a cycle over dense lists (bits_join.cuh) ----------------------------------------------------------------------
+// Both lists' entries number at least one per kBitsSparsest values of w on average, over the lists that can be looked up, and
+// the bitmaps are small.  Four-cycles of relations of 65,536 rows, bitmaps / list kernels (us per fixpoint) at one entry per
+// 16: 630 / 2407, 100: 396 / 800, 324: 308 / 571, 900: 288 / 654; of 4,096 rows at 324 and below 149 / 142, all launches.
+constexpr uint64_t kBitsSparsest = 1024;
+constexpr size_t kBitsMaxBytes = (size_t)64 << 20;
+
+uint32_t bits_words(const Relation& A, int a_col, const Relation& B, int b_col) {      // columns that hold w
+  return bits_padded((uint32_t)(std::max(A.val_max[a_col], B.val_max[b_col]) / 32 + 1));
+}
+bool bits_join_applies(Ctx* c, const Relation& A, const Index& aix, const Relation& B, const Index& bix, uint32_t words) {
+  if (words > kBitsMaxWords) return false;
+  if ((uint64_t)A.n * kBitsSparsest < (uint64_t)aix.domain * words * 32 || (uint64_t)B.n * kBitsSparsest < (uint64_t)bix.domain * words * 32) return false;
+  const size_t bytes = (size_t)(aix.domain + bix.domain) * words * 6;
+  return bytes <= kBitsMaxBytes && bytes <= c->arena.largest_free() / 4;
+}
+BitsLists ensure_bits(Ctx* c, Index& ix, uint32_t words) {
+  if (ix.bit_words != words) {
+    ix.bits = DevBuf(c, (size_t)ix.domain * words * 4); ix.bit_rank = DevBuf(c, (size_t)ix.domain * words * 2);
+    XLOG_CUDA(cudaMemsetAsync(ix.bits.p, 0, (size_t)ix.domain * words * 4, c->stream));
+    const unsigned g = grid_for((uint64_t)ix.domain * 32, 256);
+    XLOG_LAUNCH(c, k_bits_rows, g, 256, 0, (const uint32_t*)ix.off.as<uint32_t>(), ix.domain, ix.other[0], words, ix.bits.as<uint32_t>());
+    XLOG_LAUNCH(c, k_bits_ranks, g, 256, 0, (const uint32_t*)ix.bits.as<uint32_t>(), ix.domain, words, ix.bit_rank.as<uint16_t>());
+    ix.bit_words = words;
+  }
+  return BitsLists{ix.bits.as<uint32_t>(), ix.bit_rank.as<uint16_t>(), ix.off.as<uint32_t>(), ix.tags, (uint32_t)ix.domain};
+}
+template <typename K2, typename K>
+void bits_emit(Ctx* c, const BitsJoin& P, const void* keys, const float* tags, uint64_t n, const uint64_t* off, void* ok, float* ot) {
+  const unsigned g = grid_for(n, 256);
+  if (P.words > 16) XLOG_LAUNCH(c, (k_bits_emit<K2, K, 8>), g, 256, 0, P, (const K2*)keys, tags, n, off, (K*)ok, ot);
+  else XLOG_LAUNCH(c, (k_bits_emit<K2, K, 4>), g, 256, 0, P, (const K2*)keys, tags, n, off, (K*)ok, ot);
+}
+// All rows of the join of n paths: count -> scan -> one control read -> write.
+KeyTags bits_join(Ctx* c, const BitsJoin& P, const void* keys, int key_bytes, const float* tags, uint64_t n, int head_bytes, const char* what) {
+  DevBuf cnt(c, n * 4), off(c, n * 8);
+  const unsigned tiles = (unsigned)((n + kScanTile - 1) / kScanTile);
+  DevBuf sums(c, (size_t)tiles * 8);
+  c->note_bytes = (int64_t)n * (key_bytes + 4);
+  DISPATCH_K(key_bytes, {
+    if (P.words > 16) XLOG_LAUNCH(c, (k_bits_count<K, 8>), grid_for(n, 256), 256, 0, P, (const K*)keys, n, cnt.as<uint32_t>());
+    else XLOG_LAUNCH(c, (k_bits_count<K, 4>), grid_for(n, 256), 256, 0, P, (const K*)keys, n, cnt.as<uint32_t>());
+  });
+  XLOG_LAUNCH(c, (k_scan_tile_sums<uint32_t, uint64_t>), tiles, kScanBlock, 0, (const uint32_t*)cnt.as<uint32_t>(), (int64_t)n, sums.as<uint64_t>());
+  XLOG_LAUNCH(c, (k_scan_spine<uint64_t>), 1, 1024, 0, sums.as<uint64_t>(), (int64_t)tiles, (uint64_t*)(c->d_ctrl + kSlotTotals));
+  XLOG_LAUNCH(c, (k_scan_apply<uint32_t, uint64_t>), tiles, kScanBlock, 0, (const uint32_t*)cnt.as<uint32_t>(), (int64_t)n, (const uint64_t*)sums.as<uint64_t>(), off.as<uint64_t>());
+  sync_ctrl(c);                                            // the one small metadata read that sizes the output
+  const uint64_t total = c->h_ctrl[kSlotTotals];
+  if (total > kSortMaxN) fail(XLOG_ERR_CAPACITY_EXCEEDED, std::string("materialised ") + what + " relation exceeds 2^30 - 1 rows");
+  KeyTags kt;
+  kt.n = (uint32_t)total;
+  kt.keys = DevBuf(c, (size_t)std::max<uint64_t>(total, 1) * head_bytes);
+  kt.tags = DevBuf(c, (size_t)std::max<uint64_t>(total, 1) * 4);
+  c->note_bytes = (int64_t)n * (key_bytes + 12) + (int64_t)total * (head_bytes + 4);
+  if (total) {
+    if (key_bytes == 4 && head_bytes == 4) bits_emit<uint32_t, uint32_t>(c, P, keys, tags, n, off.as<uint64_t>(), kt.keys.p, kt.tags.as<float>());
+    else if (key_bytes == 4) bits_emit<uint32_t, uint64_t>(c, P, keys, tags, n, off.as<uint64_t>(), kt.keys.p, kt.tags.as<float>());
+    else if (head_bytes == 4) bits_emit<uint64_t, uint32_t>(c, P, keys, tags, n, off.as<uint64_t>(), kt.keys.p, kt.tags.as<float>());
+    else bits_emit<uint64_t, uint64_t>(c, P, keys, tags, n, off.as<uint64_t>(), kt.keys.p, kt.tags.as<float>());
+  }
+  return kt;
+}
+
 // tri(x,y,z) :- e(x,y), e(y,z), e(z,x): count per edge -> scan -> materialise; the result is born sorted.
 // tri(x,y,z) :- r(x,y), s(y,z), t(z,x), materialised.  Two plans (paper: "Worst-case-optimal joins"):
 //  - multiway: for every r row intersect s's out-list of y with t's in-list of x (count -> scan -> write);
@@ -374,6 +438,14 @@ void triangle_materialise(Ctx* c, Relation& H, const RuleC& r) {
   c->last_triangle_plan = XLOG_PLAN_WCOJ;
   Index& out_ix = ensure_index(c, S, 0);
   Index& in_ix = ensure_index(c, T, 1);
+  const uint32_t words = bits_words(S, 1, T, 0);
+  if (!R.dict_n[0] && !R.dict_n[1] && bits_join_applies(c, S, out_ix, T, in_ix, words)) {
+    BitsJoin P{R.layout, H.layout, ensure_bits(c, out_ix, words), ensure_bits(c, in_ix, words), words, times};
+    KeyTags kt = bits_join(c, P, R.keys(), R.key_bytes, R.tags(), R.n, H.key_bytes, "triangle");
+    c->r_candidates += kt.n; c->r_unique += kt.n;
+    set_current(H, std::move(kt));
+    return;
+  }
   ensure_soa(c, R);
   ensure_soa(c, S);
   TriGraph G{};
@@ -474,8 +546,6 @@ void cycle4_materialise(Ctx* c, Relation& H, const RuleC& r) {
     DISPATCH_K(ckb, XLOG_LAUNCH(c, (k_c4_chain_count<K>), grid, 256, 0, P3, (const K*)k0.p, n2, cnt.as<uint32_t>()));
     XLOG_LAUNCH(c, (k_scan_tile_sums<uint32_t, uint64_t>), tiles, kScanBlock, 0, (const uint32_t*)cnt.as<uint32_t>(), (int64_t)n2, sums.as<uint64_t>());
     XLOG_LAUNCH(c, (k_scan_spine<uint64_t>), 1, 1024, 0, sums.as<uint64_t>(), (int64_t)tiles, (uint64_t*)(c->d_ctrl + kSlotTotals));
-    XLOG_LAUNCH(c, (k_scan_apply<uint32_t, uint64_t>), tiles, kScanBlock, 0, (const uint32_t*)cnt.as<uint32_t>(), (int64_t)n2,
-                (const uint64_t*)sums.as<uint64_t>(), off.as<uint64_t>());
     sync_ctrl(c);
     const uint64_t n3 = c->h_ctrl[kSlotTotals];
     const uint64_t biggest = std::max<uint64_t>(std::max<uint64_t>(R.n, S.n), std::max<uint64_t>(T.n, U.n));
@@ -490,6 +560,8 @@ void cycle4_materialise(Ctx* c, Relation& H, const RuleC& r) {
       c->last_triangle_plan = XLOG_PLAN_CHAIN;
       c->r_candidates += (int64_t)n3;
       if (n3 == 0) { KeyTags empty; set_current(H, std::move(empty)); return; }
+      XLOG_LAUNCH(c, (k_scan_apply<uint32_t, uint64_t>), tiles, kScanBlock, 0, (const uint32_t*)cnt.as<uint32_t>(), (int64_t)n2,
+                  (const uint64_t*)sums.as<uint64_t>(), off.as<uint64_t>());
       DevBuf k3(c, n3 * kb3), t3(c, n3 * 4);
       c->note_bytes = (int64_t)n2 * (ckb + 4 + 8) + (int64_t)n3 * (kb3 + 4 + 8);
 #define XLOG_C4_CHAIN(K2, K3) \
@@ -536,6 +608,15 @@ void cycle4_materialise(Ctx* c, Relation& H, const RuleC& r) {
       return;
     }
     zero_ctrl(c, kSlotTotals);
+  }
+  const uint32_t words = bits_words(T, 1, U, 0);
+  if (bits_join_applies(c, T, tix, U, uix, words)) {
+    cnt.reset(); off.reset(); sums.reset();
+    BitsJoin Q{H2.layout, H.layout, ensure_bits(c, tix, words), ensure_bits(c, uix, words), words, P.times};
+    kt = bits_join(c, Q, k0.p, ckb, t0.as<float>(), n2, H.key_bytes, "four-cycle");
+    c->r_unique += kt.n;
+    set_current(H, std::move(kt));
+    return;
   }
   // long runs of equal x and small w values: the bitmap kernel (see cycle4.cuh)
   const uint64_t w_max = (uint64_t)(U.val_max[0] ? U.val_max[0] : U.col_max[0]);

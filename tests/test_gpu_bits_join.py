@@ -1,0 +1,78 @@
+"""Cyclic joins over dense lists through bitmaps: rows and tags bit for bit those of the binary-join chain, at domains around a word,
+a group of lanes and a warp of words; lists that are empty, full and out of the other relation's range."""
+import numpy as np
+import pytest
+
+from paper_2609_27203_b200 import workloads as W
+from tests import helpers as H
+
+pytestmark = pytest.mark.gpu
+
+
+def pairs(r, da, db, density):
+    m = r.random((da, db)) < density
+    m[: max(da // 8, 1)] = False                              # values without a list
+    m[-1] = True                                              # and one with every value
+    a, b = np.nonzero(m)
+    o = r.permutation(len(a))
+    return a[o].astype(np.int32), b[o].astype(np.int32), (-r.random(len(a))).astype(np.float32)
+
+
+def both(prog, out, kernel):
+    from paper_2609_27203_b200 import xlog
+    got = []
+    for f in (xlog.FLAG_FORCE_WCOJ, xlog.FLAG_FORCE_CHAIN):
+        ctx, ids, _ = xlog.load_program(prog, arena_bytes=4 << 30, flags=f | xlog.FLAG_CHECK_INVARIANTS | xlog.FLAG_PROFILE)
+        ctx.fixpoint()
+        first = ctx.read(ids[out])
+        ctx.reset_idb()
+        ctx.fixpoint()                                        # the bitmaps are there already
+        got.append(ctx.read(ids[out]))
+        assert H.compare_relations(first, got[-1])["bit_unequal"] == 0
+        ran = kernel in ctx.profile()
+        assert ran == (f == xlog.FLAG_FORCE_WCOJ)
+        ctx.close()
+    assert len(got[0][1]) > 0 and H.compare_relations(got[0], got[1], what="bitmaps vs chain")["bit_unequal"] == 0
+
+
+@pytest.mark.parametrize("sr", [W.MAXPLUS, W.SUMPROD])
+@pytest.mark.parametrize("w_dom", [5, 32, 33, 256, 257, 512, 513, 1025, 2111])
+def test_triangle_join(sr, w_dom):
+    r = np.random.default_rng(w_dom)
+    x, y, full = 70, 130, max(0.1, 8 / w_dom)
+    prog = W.triangle_join_program(pairs(r, x, y, 0.5), pairs(r, y, w_dom, full), _turn(pairs(r, x, w_dom, full)), semiring=sr)
+    both(prog, "tri", "k_bits_emit")
+
+
+@pytest.mark.parametrize("sr", [W.MINPLUS, W.SUMPROD])
+@pytest.mark.parametrize("w_dom", [9, 33, 400, 1024, 1025])
+def test_four_cycle(sr, w_dom):
+    r = np.random.default_rng(w_dom)
+    full = max(0.08, 5 / w_dom)
+    prog = W.four_cycle_program(pairs(r, 40, 50, 0.4), pairs(r, 50, 60, 0.4), pairs(r, 60, w_dom, full), _turn(pairs(r, 48, w_dom, full)), semiring=sr)
+    both(prog, "c4", "k_bits_emit")
+
+
+def _turn(p):
+    return p[1], p[0], p[2]
+
+
+@pytest.mark.parametrize("dom", [13312, 16384, 16385])
+def test_sparse_lists_and_wide_values_keep_the_list_kernels(dom):
+    from paper_2609_27203_b200 import xlog
+    r = np.random.default_rng(1)
+    rel = [(r.integers(0, 60, 400).astype(np.int32), r.integers(0, 60, 400).astype(np.int32), -r.random(400).astype(np.float32)) for _ in range(2)]
+    n = 700 if dom == 13312 else 90000
+    t = (r.integers(0, 60, n).astype(np.int32), r.integers(0, dom, n).astype(np.int32), -r.random(n).astype(np.float32))
+    t[1][0] = dom - 1
+    u = (np.minimum(r.integers(0, dom, n), dom - 1).astype(np.int32), r.integers(0, 60, n).astype(np.int32), -r.random(n).astype(np.float32))
+    prog = W.four_cycle_program(*rel, t, u)
+    ctx, ids, _ = xlog.load_program(prog, arena_bytes=4 << 30, flags=xlog.FLAG_FORCE_WCOJ | xlog.FLAG_PROFILE)
+    ctx.fixpoint()
+    got, ran = ctx.read(ids["c4"]), "k_bits_emit" in ctx.profile()
+    ctx.close()
+    ctx, ids, _ = xlog.load_program(prog, arena_bytes=4 << 30, flags=xlog.FLAG_FORCE_CHAIN)
+    ctx.fixpoint()
+    assert H.compare_relations(got, ctx.read(ids["c4"]))["bit_unequal"] == 0
+    ctx.close()
+    assert ran == (dom == 16384)
