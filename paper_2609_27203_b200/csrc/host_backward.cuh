@@ -28,12 +28,6 @@ void rule_backward(Ctx* c, const RuleC& r, const float* g, float* const* grads) 
   Relation& RA = *c->rels[r.plan.atoms[outer].rel];
   if (RA.n == 0 || H.n == 0) { XLOG_CUDA(cudaStreamSynchronize(c->stream)); return; }
   Variant v{&r, outer, full_source(RA)};
-  Counted q;
-  count_variant(c, v, H, q, kSlotTotals);
-  sync_ctrl(c);
-  q.total = c->h_ctrl[q.slot];
-  const int ckb = q.spec.head.total_bits <= 32 ? 4 : 8;
-  if (ckb != H.key_bytes) fail(XLOG_ERR_UNSUPPORTED, "backward: head key width differs from the declared-column key width");
   BwdArgs bw{};
   bw.head_keys = H.keys(); bw.head_tags = H.tags(); bw.n_head = H.n;
   bw.count_bits = r.plan.emit_count_column ? H.layout.shift[r.plan.n_head_cols - 1] : 0;
@@ -41,6 +35,30 @@ void rule_backward(Ctx* c, const RuleC& r, const float* g, float* const* grads) 
   bw.grad_outer = grads[outer];
   bw.grad_inner = r.kind == 2 ? grads[1 - outer] : nullptr;     // a negated atom (kind 5) carries no tag: its buffer stays zero
   bw.lse = H.sr == XLOG_SR_LOGSUMEXP ? 1 : 0;
+  GroupRule gs;
+  if (group_rule_applies(c, v, H, gs)) {
+    // groups that are products of two runs: no candidates laid out over the whole rule
+    const unsigned grid = group_rule_grid(gs);
+    c->note_bytes = (int64_t)v.outer.n * (v.outer.key_bytes + 16) + (int64_t)H.n * (H.key_bytes + 8);
+#define XLOG_GROUP_BWD(KO, KH) \
+  do { \
+    if (bw.lse) XLOG_LAUNCH(c, (k_group_backward<KO, KH, true>), grid, kGroupBlock, 0, gs, (const KO*)v.outer.keys, bw); \
+    else XLOG_LAUNCH(c, (k_group_backward<KO, KH, false>), grid, kGroupBlock, 0, gs, (const KO*)v.outer.keys, bw); \
+  } while (0)
+    if (v.outer.key_bytes == 4 && H.key_bytes == 4) XLOG_GROUP_BWD(uint32_t, uint32_t);
+    else if (v.outer.key_bytes == 4) XLOG_GROUP_BWD(uint32_t, uint64_t);
+    else if (H.key_bytes == 4) XLOG_GROUP_BWD(uint64_t, uint32_t);
+    else XLOG_GROUP_BWD(uint64_t, uint64_t);
+#undef XLOG_GROUP_BWD
+    sync_ctrl(c);
+    return;
+  }
+  Counted q;
+  count_variant(c, v, H, q, kSlotTotals);
+  sync_ctrl(c);
+  q.total = c->h_ctrl[q.slot];
+  const int ckb = q.spec.head.total_bits <= 32 ? 4 : 8;
+  if (ckb != H.key_bytes) fail(XLOG_ERR_UNSUPPORTED, "backward: head key width differs from the declared-column key width");
   if (q.total) launch_expand<true>(c, q, 0, q.total, ckb, nullptr, nullptr, bw);
   sync_ctrl(c);
 }

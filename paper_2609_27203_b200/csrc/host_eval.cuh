@@ -2,6 +2,7 @@
 // Host-side driver code of the engine; included by xlog_api.cu only (one translation unit).
 #pragma once
 #include "host_plan.cuh"
+#include "group_rule.cuh"
 
 namespace xlog {
 namespace {
@@ -160,30 +161,34 @@ JoinSpec make_spec(Ctx* c, const Variant& v, const Relation& H, const KeyLayout*
   return S;
 }
 
+// Leading head columns that follow the leading columns of the scanned atom, in the same order, through strictly
+// increasing maps (column = mul * v + add with mul >= 1 in the atom, c0 + coef * v with coef >= 1 in the head, v in no
+// earlier column): the scanned relation is sorted by those columns (dictionary codes keep the order of the values),
+// equal column values give equal head values and the other way round, so the candidate stream is already ordered by
+// those key bits.  sum(p, a + b) :- digit(2p, a), digit(2p + 1, b) has its first head column of this kind.
+int leading_head_columns(Ctx* c, const xlog_plan& p, int outer_atom) {
+  const xlog_atom& A = p.atoms[outer_atom];
+  const int ka = c->rels[A.rel]->arity;
+  int k = 0;
+  for (; k < p.n_head_cols && k < ka; ++k) {
+    if (A.args[k].kind != XLOG_ARG_VAR || A.args[k].mul < 1) break;
+    const int var = A.args[k].var;
+    bool fresh = true;
+    for (int j = 0; j < k; ++j) fresh = fresh && A.args[j].var != var;
+    bool mono = fresh && p.head[k].coef[var] >= 1;
+    for (int w = 0; w < kMaxVars; ++w) mono = mono && (w == var || p.head[k].coef[w] == 0);
+    if (!mono) break;
+  }
+  return k;
+}
+
 // count -> scan for one variant; the grand total lands in control slot `slot` (read after sync_ctrl)
 void count_variant(Ctx* c, const Variant& v, const Relation& H, Counted& q, int slot, const KeyLayout* head_layout = nullptr) {
   q.spec = make_spec(c, v, H, head_layout);
   q.outer = v.outer;
   q.slot = slot;
   {
-    // Leading head columns that follow the leading columns of the scanned atom, in the same order, through strictly
-    // increasing maps (column = mul * v + add with mul >= 1 in the atom, c0 + coef * v with coef >= 1 in the head, v in no
-    // earlier column): the scanned relation is sorted by those columns (dictionary codes keep the order of the values),
-    // equal column values give equal head values and the other way round, so the candidate stream is already ordered by
-    // those key bits.  sum(p, a + b) :- digit(2p, a), digit(2p + 1, b) has its first head column of this kind.
-    const xlog_plan& p = v.rule->plan;
-    const xlog_atom& A = p.atoms[v.outer_atom];
-    const int ka = c->rels[A.rel]->arity;
-    int k = 0;
-    for (; k < p.n_head_cols && k < ka; ++k) {
-      if (A.args[k].kind != XLOG_ARG_VAR || A.args[k].mul < 1) break;
-      const int var = A.args[k].var;
-      bool fresh = true;
-      for (int j = 0; j < k; ++j) fresh = fresh && A.args[j].var != var;
-      bool mono = fresh && p.head[k].coef[var] >= 1;
-      for (int w = 0; w < kMaxVars; ++w) mono = mono && (w == var || p.head[k].coef[w] == 0);
-      if (!mono) break;
-    }
+    const int k = leading_head_columns(c, v.rule->plan, v.outer_atom);
     q.presorted_top = k ? q.spec.head.total_bits - q.spec.head.shift[k - 1] : 0;
   }
   const uint32_t n = v.outer.n;
@@ -337,6 +342,99 @@ KeyTags evaluate(Ctx* c, Relation& H, std::vector<Variant>& variants, const Sour
   }
   if (result.n_slot < 0) c->r_unique += result.n;     // a deferred count is added by the caller once it is known
   return result;
+}
+
+// ---- rules whose head groups are products of two runs (group_rule.cuh) --------------------------------------------------------
+constexpr int kSlotGroup = 60;             // rows, candidates
+
+// Is the variant's rule of that form, without dictionaries, over binary relations, and do the head's values and the groups
+// fit: at most kGroupSlots values of the second column, at most two groups per scanned row (an aggregate array of up to 256
+// bytes per row), with room for all of it.  Fills the compiled rule, without its outputs.
+bool group_rule_applies(Ctx* c, const Variant& v, const Relation& H, GroupRule& P) {
+  const xlog_plan& p = v.rule->plan;
+  if (v.rule->kind != 2 || p.emit_count_column || p.n_head_cols != 2 || H.arity != 2) return false;
+  const JoinShape& sh = v.rule->shape[v.outer_atom];
+  if (!sh.ok || sh.probe_col != 0) return false;
+  const xlog_atom& A = p.atoms[v.outer_atom];
+  const xlog_atom& B = p.atoms[sh.inner];
+  Relation& RA = *c->rels[A.rel];
+  Relation& RB = *c->rels[B.rel];
+  if (RA.arity != 2 || RB.arity != 2 || RA.dict_n[0] || RA.dict_n[1] || RB.dict_n[0] || RB.dict_n[1] || H.dict_n[0] || H.dict_n[1]) return false;
+  if (H.col_max[1] >= kGroupSlots || v.outer.keys != RA.keys() || v.outer.n == 0 || RB.n == 0) return false;
+  const auto& a0 = A.args[0];
+  const auto& a1 = A.args[1];
+  const auto& b1 = B.args[1];
+  // d(m p + s, a): both atoms are met on p, a and b are further variables
+  if (a0.kind != XLOG_ARG_VAR || a0.mul < 1 || a0.add > 0 || sh.probe_var != a0.var || sh.probe_mul < 1) return false;
+  if (!is_plain_var(a1) || !is_plain_var(b1) || a1.var == a0.var || b1.var == a0.var || b1.var == a1.var) return false;
+  const auto &h0 = p.head[0], &h1 = p.head[1];
+  for (int k = 0; k < kMaxVars; ++k) {
+    if (k != a0.var && h0.coef[k] != 0) return false;
+    if (k != a0.var && k != a1.var && k != b1.var && h1.coef[k] != 0) return false;
+  }
+  if (h0.coef[a0.var] < 1 || h1.coef[b1.var] < 1) return false;
+  const int64_t groups = ((int64_t)RA.val_max[0] - a0.add) / a0.mul + 1;
+  if (groups > 2 * (int64_t)v.outer.n + 1024) return false;
+  const uint32_t slots = (uint32_t)H.col_max[1] + 1;
+  if (c->arena.largest_free() < (size_t)groups * (slots * 12 + 4) * 2 + ((size_t)1 << 20)) return false;
+  Index& ia = ensure_index(c, RA, 0);
+  Index& ib = ensure_index(c, RB, 0);
+  P = GroupRule{};
+  P.n_groups = (uint32_t)groups;
+  P.mul0 = a0.mul; P.add0 = a0.add; P.mul1 = sh.probe_mul; P.add1 = sh.probe_add;
+  P.off0 = ia.off.as<uint32_t>(); P.off1 = ib.off.as<uint32_t>();
+  P.domain0 = ia.domain; P.domain1 = ib.domain;
+  P.mask0 = RA.layout.mask[1]; P.tag0 = v.outer.tags;
+  P.col1 = ib.other[0]; P.tag1 = ib.tags;
+  P.top_c0 = h0.c0; P.top_mul = h0.coef[a0.var];
+  P.c0 = h1.c0; P.mulp = h1.coef[a0.var]; P.k0 = h1.coef[a1.var]; P.k1 = (uint32_t)h1.coef[b1.var];
+  P.shift = H.layout.shift[0];
+  P.top_mask = H.layout.mask[0];
+  P.slots = slots;
+  P.per_warp = std::max<uint32_t>(1, (P.n_groups + kSMs * 64 - 1) / (kSMs * 64));       // 64 warps fit an SM
+  P.err = ctrl_u32(c, kSlotErr);
+  return true;
+}
+
+unsigned group_rule_grid(const GroupRule& P) {
+  const uint64_t per_block = (uint64_t)P.per_warp * (kGroupBlock / 32);
+  return (unsigned)((P.n_groups + per_block - 1) / per_block);
+}
+
+KeyTags group_rule(Ctx* c, Relation& H, const Variant& v, GroupRule& P) {
+  const uint32_t ng = P.n_groups;
+  const unsigned grid = group_rule_grid(P);
+  const size_t room = (size_t)ng * P.slots;
+  DevBuf mask(c, (size_t)ng * 4), agg(c, room * 4), sums(c, (size_t)grid * sizeof(ulonglong2));
+  P.mask = mask.as<uint32_t>(); P.agg = agg.as<float>(); P.sums = sums.as<ulonglong2>();
+  KeyTags out;
+  out.keys = DevBuf(c, room * H.key_bytes);
+  out.tags = DevBuf(c, room * 4);
+  c->note_bytes = (int64_t)v.outer.n * (v.outer.key_bytes + 12) + (int64_t)ng * (16 + 4 * P.slots);
+#define XLOG_GROUP_RULE(OP, TIMES) DISPATCH_K(v.outer.key_bytes, XLOG_LAUNCH(c, (k_group_rule<K, OP, TIMES>), grid, kGroupBlock, 0, P, (const K*)v.outer.keys))
+  switch (H.sr) {
+    case XLOG_SR_MAXPLUS: XLOG_GROUP_RULE(OpMax, false); break;
+    case XLOG_SR_MINPLUS: XLOG_GROUP_RULE(OpMin, false); break;
+    case XLOG_SR_LOGSUMEXP: XLOG_GROUP_RULE(OpLse, false); break;
+    default: XLOG_GROUP_RULE(OpSum, true); break;
+  }
+#undef XLOG_GROUP_RULE
+  c->note_bytes = (int64_t)ng * (4 + 4 * P.slots) + (int64_t)room * (H.key_bytes + 4);
+  DISPATCH_K(H.key_bytes, XLOG_LAUNCH(c, (k_group_emit<K>), grid, kGroupBlock, 0, P, out.keys.as<K>(), out.tags.as<float>(), (unsigned long long*)(c->d_ctrl + kSlotGroup)));
+  sync_ctrl(c);
+  out.n = (uint32_t)c->h_ctrl[kSlotGroup];
+  c->r_candidates += (int64_t)c->h_ctrl[kSlotGroup + 1];
+  c->r_unique += out.n;
+  if ((size_t)out.n * 2 < room) {                      // mostly empty slots: the relation keeps arrays of its own size
+    KeyTags fit;
+    fit.n = out.n;
+    fit.keys = DevBuf(c, (size_t)std::max(out.n, 1u) * H.key_bytes);
+    fit.tags = DevBuf(c, (size_t)std::max(out.n, 1u) * 4);
+    XLOG_CUDA(cudaMemcpyAsync(fit.keys.p, out.keys.p, (size_t)out.n * H.key_bytes, cudaMemcpyDeviceToDevice, c->stream));
+    XLOG_CUDA(cudaMemcpyAsync(fit.tags.p, out.tags.p, (size_t)out.n * 4, cudaMemcpyDeviceToDevice, c->stream));
+    return fit;
+  }
+  return out;
 }
 
 // Which atom a rule scans in the seed round (every atom reads its full relation): the recursive side if exactly one atom

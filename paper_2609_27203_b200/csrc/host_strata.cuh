@@ -26,6 +26,12 @@ void stratum_once(Ctx* c, int head, const std::vector<const RuleC*>& rs) {
     if (r->kind == 2 && !r->shape[0].ok) outer = 1;
     vs.push_back(Variant{r, outer, full_source(*c->rels[r->plan.atoms[outer].rel])});
   }
+  GroupRule gs;
+  if (vs.size() == 1 && H.n_facts == 0 && group_rule_applies(c, vs[0], H, gs)) {
+    set_current(H, group_rule(c, H, vs[0], gs));
+    c->r_new += H.n;
+    return;
+  }
   KeyLayout cl = H.layout;
   if (counted) { int32_t mx[kMaxArity] = {0, 0, 0, 0}; for (int i = 0; i < rs[0]->plan.n_head_cols; ++i) mx[i] = H.col_max[i]; cl = make_layout(rs[0]->plan.n_head_cols, mx); }
   Source facts{H.fact_keys.p, H.fact_tags.as<float>(), H.n_facts, H.layout, H.key_bytes};

@@ -1,0 +1,85 @@
+"""Rules whose groups are products of two runs, against the oracle: forward, receipt and gradient.
+Max / min are exact.  Logsumexp 1e-4 absolute, as everywhere.  Sums: fp64 inside a group, one rounding to fp32 per product and
+one at the end (1e-6 relative, over ten ulps).  Gradients are fp32 sums of up to a few hundred terms: 1e-4 relative, 1e-5 absolute."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2609_27203_b200 import workloads as W
+from tests import helpers as H
+
+pytestmark = pytest.mark.gpu
+
+
+def pairs(rng, n, top, fill):
+    """Distinct (x, y), x < n, y <= top, about `fill` of all; some x without any."""
+    at = rng.random((n, top + 1)) < fill
+    at[rng.random(n) < 0.15] = False
+    at[0, 0] = at[n - 1, top] = True
+    x, y = np.nonzero(at)
+    return x.astype(np.int32), y.astype(np.int32)
+
+
+def program(sr, groups, a_top, b_top, c0, k0, k1, mul, more, seed):
+    rng = np.random.default_rng(seed)
+    d, e = pairs(rng, groups * mul, a_top, 0.8), pairs(rng, groups * mul + 1, b_top, 0.8)
+    tags = lambda n: (0.25 + rng.random(n)).astype(np.float32) if sr == W.SUMPROD else (-4.0 * rng.random(n)).astype(np.float32)
+    relations = {"d": (2, sr), "e": (2, sr), "h": (2, sr)}
+    terms = (((1, k0),) if k0 else ()) + ((2, k1),)
+    rules = [W.Rule("h", (W.Affine(3, ((0, 2),)), W.Affine(c0, terms)), (W.Atom("d", (W.Var(0, mul, 0), W.Var(1))), W.Atom("e", (W.Var(0, mul, 1), W.Var(2)))))]
+    facts = {"d": (list(d), tags(len(d[0]))), "e": (list(e), tags(len(e[0])))}
+    if more:                                                  # rows of the head that another rule makes, between and inside the groups
+        f = pairs(rng, 2 * groups + 5, c0 + k0 * a_top + k1 * b_top, 0.3)
+        relations["f"] = (2, sr)
+        rules.append(W.Rule("h", (W.V(0), W.V(1)), (W.Atom("f", (W.Var(0), W.Var(1))),)))
+        facts["f"] = (list(f), tags(len(f[0])))
+    return W.Program("groups", relations, rules, facts, ("h",))
+
+
+@pytest.mark.parametrize("sr", [W.SUMPROD, W.LOGSUMEXP, W.MAXPLUS, W.MINPLUS])
+@pytest.mark.parametrize("groups,a_top,b_top,c0,k0,k1,mul,more", [
+    (1, 0, 0, 0, 1, 1, 1, False),                             # one candidate
+    (9, 9, 9, 0, 1, 1, 2, False),                             # digit pairs, one block and a group
+    (300, 9, 9, 0, 1, 1, 2, True),
+    (40, 14, 16, 1, 1, 1, 1, False),                          # 32 slots, runs of up to 17: a whole warp per row
+    (40, 15, 15, 0, 1, 1, 3, True),                           # runs of up to 16: half a warp per row
+    (33, 80, 31, 0, 0, 1, 1, False),                          # d's column does not reach the head: runs of over 32 rows
+    (33, 4, 9, 0, 1, 3, 1, True),                             # slots that only some rows reach
+    (33, 10, 11, 10, 1, 1, 1, False),                         # 32 slots with a constant
+    (33, 11, 11, 10, 1, 1, 1, False),                         # 33: the sorting route
+    (9480, 3, 3, 0, 1, 1, 2, False), (30000, 2, 3, 0, 1, 1, 1, True)])     # one group and more per warp of the whole device
+def test_groups(sr, groups, a_top, b_top, c0, k0, k1, mul, more):
+    import torch
+    from paper_2609_27203_b200 import xlog
+    prog = program(sr, groups, a_top, b_top, c0, k0, k1, mul, more, groups + a_top)
+    ctx, ids, rules = xlog.load_program(prog, arena_bytes=1 << 28, flags=xlog.FLAG_CHECK_INVARIANTS)
+    o, oids, orules = oracle.load_program(prog)
+    o.run("seminaive")
+    tol = {W.SUMPROD: dict(rel_tol=1e-6), W.LOGSUMEXP: dict(abs_tol=1e-4)}.get(sr, {})
+    for _ in range(2):
+        receipt = ctx.fixpoint()
+        rep = H.compare_relations(ctx.read(ids["h"]), o.read(oids["h"]), what="groups", **tol)
+        (d0, _), (e0, _) = prog.facts["d"][0], prog.facts["e"][0]
+        nd, ne = (np.bincount(x, minlength=groups * mul + 2) for x in (d0, e0))
+        cand = sum(int(nd[p * mul] * ne[p * mul + 1]) for p in range(groups))
+        cand += len(prog.facts["f"][1]) if more else 0
+        assert receipt["candidates"] == cand and receipt["derived_tuples"] == rep["rows"] and receipt["new_tuples"] == rep["rows"]
+    if sr in (W.SUMPROD, W.LOGSUMEXP):
+        g = np.random.default_rng(7).standard_normal(rep["rows"]).astype(np.float32)
+        parts = ctx.backward(rules[0], torch.from_numpy(g).cuda(), same_buffer_for_same_relation=False)
+        for got, want in zip(parts, o.backward(orules[0], g)):
+            want = want.astype(np.float64)
+            assert np.all(np.abs(got.cpu().numpy() - want) <= 1e-5 + 1e-4 * np.abs(want))
+    ctx.close()
+
+
+def test_a_small_arena_takes_the_sorting_route_or_the_groups_alike():
+    from paper_2609_27203_b200 import xlog
+    prog = program(W.LOGSUMEXP, 2000, 1, 1, 0, 1, 29, 1, False, 3)          # 31 slots of which four a group are taken
+    o, oids, _ = oracle.load_program(prog)
+    o.run("seminaive")
+    for mb in (4, 64):
+        ctx, ids, _ = xlog.load_program(prog, arena_bytes=mb << 20)
+        ctx.fixpoint()
+        H.compare_relations(ctx.read(ids["h"]), o.read(oids["h"]), abs_tol=1e-4, what="small arena")
+        ctx.close()
