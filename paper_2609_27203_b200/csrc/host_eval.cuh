@@ -421,7 +421,7 @@ KeyTags group_rule(Ctx* c, Relation& H, const Variant& v, GroupRule& P) {
 #undef XLOG_GROUP_RULE
   c->note_bytes = (int64_t)ng * (4 + 4 * P.slots) + (int64_t)room * (H.key_bytes + 4);
   DISPATCH_K(H.key_bytes, XLOG_LAUNCH(c, (k_group_emit<K>), grid, kGroupBlock, 0, P, out.keys.as<K>(), out.tags.as<float>(), (unsigned long long*)(c->d_ctrl + kSlotGroup)));
-  sync_ctrl(c);
+  sync_ctrl_end(c);
   out.n = (uint32_t)c->h_ctrl[kSlotGroup];
   c->r_candidates += (int64_t)c->h_ctrl[kSlotGroup + 1];
   c->r_unique += out.n;
@@ -432,6 +432,7 @@ KeyTags group_rule(Ctx* c, Relation& H, const Variant& v, GroupRule& P) {
     fit.tags = DevBuf(c, (size_t)std::max(out.n, 1u) * 4);
     XLOG_CUDA(cudaMemcpyAsync(fit.keys.p, out.keys.p, (size_t)out.n * H.key_bytes, cudaMemcpyDeviceToDevice, c->stream));
     XLOG_CUDA(cudaMemcpyAsync(fit.tags.p, out.tags.p, (size_t)out.n * 4, cudaMemcpyDeviceToDevice, c->stream));
+    c->ended_at = -1;
     return fit;
   }
   return out;

@@ -235,6 +235,7 @@ void run_fixpoint(Ctx* c) {
   c->stratum_done.assign(c->rels.size(), 0);
   if (c->poisoned) fail(XLOG_ERR_INVALID_STATE, "derived relations are poisoned by an earlier failure; call xlog_ctx_reset_idb");
   c->poisoned = true;                      // cleared on success
+  c->ended_at = -1;
   zero_ctrl(c, kSlotErr);
   propagate_bounds(c);
   for (const std::vector<int>& comp : components(c)) {
@@ -249,7 +250,7 @@ void run_fixpoint(Ctx* c) {
     if (!recursive) stratum_once(c, comp[0], rs); else stratum_recursive(c, comp, rs);
     for (int p : comp) c->stratum_done[p] = 1;
   }
-  sync_ctrl(c);
+  if (c->ended_at != c->launches) sync_ctrl_end(c);
   c->poisoned = false;
   c->evaluated = true;
 }

@@ -171,9 +171,8 @@ xlog_status xlog_fixpoint(xlog_ctx* c, xlog_receipt* receipt) {
   cudaSetDevice(c->device);
   cudaEventRecord(c->ev0, c->stream);
   xlog_status st = guarded(c, [&] { run_fixpoint(c); });
-  cudaEventRecord(c->ev1, c->stream);
-  cudaEventSynchronize(c->ev1);
   if (st != XLOG_OK) {
+    cudaEventRecord(c->ev1, c->stream);
     // leave no work in flight and no error flag behind; the derived relations stay poisoned
     cudaStreamSynchronize(c->stream);
     cudaMemsetAsync(c->d_ctrl, 0, kCtrlSlots * sizeof(uint64_t), c->stream);
