@@ -124,10 +124,17 @@ void load_relation(Ctx* c, Relation& R, const int32_t* const* cols, const float*
   }
 
   // validate, find the column maxima (they fix the key layout)
-  zero_ctrl(c, kSlotErr);
-  zero_ctrl(c, kSlotA, 4);
-  XLOG_LAUNCH(c, k_col_stats, grid_for(n, 256, kSMs * 8), 256, 0, in, dtags, n, R.arity, R.sr,
-              reinterpret_cast<int32_t*>(c->d_ctrl + kSlotA), ctrl_u32(c, kSlotErr), ctrl_u32(c, kSlotC));
+  const bool small = n <= kLoadSmall;
+  if (small) {
+    R.fact_keys = DevBuf(c, (size_t)n * 8);
+    R.fact_tags = DevBuf(c, (size_t)n * 4);
+    XLOG_LAUNCH(c, k_load_small, 1, 1024, 0, in, dtags, n, R.arity, R.sr, one_of(R.sr), R.fact_keys.p, R.fact_tags.as<float>(),
+                reinterpret_cast<int32_t*>(c->d_ctrl + kSlotA), ctrl_u32(c, kSlotErr), ctrl_u32(c, kSlotC));
+  } else {
+    zero_ctrl(c, kSlotErr, kSlotD + 1);                       // the words between the two are not used
+    XLOG_LAUNCH(c, k_col_stats, grid_for(n, 256, kSMs * 8), 256, 0, in, dtags, n, R.arity, R.sr,
+                reinterpret_cast<int32_t*>(c->d_ctrl + kSlotA), ctrl_u32(c, kSlotErr), ctrl_u32(c, kSlotC));
+  }
   sync_ctrl(c);
   const bool in_order = (uint32_t)c->h_ctrl[kSlotC] == 0;     // rows arrived strictly increasing: nothing to sort or combine
   const int32_t* mx = reinterpret_cast<const int32_t*>(c->h_ctrl + kSlotA);
@@ -138,7 +145,8 @@ void load_relation(Ctx* c, Relation& R, const int32_t* const* cols, const float*
   R.key_bytes = R.layout.total_bits <= 32 ? 4 : 8;
 
   // pack -> sort -> combine duplicates
-  if (in_order) {
+  if (in_order && small) R.n_facts = R.n = (uint32_t)n;       // packed already
+  else if (in_order) {
     DISPATCH_K(R.key_bytes, {
       R.fact_keys = DevBuf(c, (size_t)n * sizeof(K));
       R.fact_tags = DevBuf(c, (size_t)n * 4);
@@ -148,6 +156,7 @@ void load_relation(Ctx* c, Relation& R, const int32_t* const* cols, const float*
     // the pack kernel reads the caller's columns: the load has copied them only once it has run
     XLOG_CUDA(cudaStreamSynchronize(c->stream));
   } else DISPATCH_K(R.key_bytes, {
+    R.fact_keys.reset(); R.fact_tags.reset();
     DevBuf k0(c, (size_t)n * sizeof(K)), t0(c, (size_t)n * 4), k1(c, (size_t)n * sizeof(K)), t1(c, (size_t)n * 4);
     XLOG_LAUNCH(c, (k_pack<K>), grid_for(n, 256), 256, 0, in, dtags, n, R.layout, DictSet{}, one_of(R.sr), k0.as<K>(), t0.as<float>());
     for (int i = 0; i < kMaxArity; ++i) stage[i].reset();

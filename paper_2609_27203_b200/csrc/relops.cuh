@@ -15,43 +15,51 @@ namespace xlog {
 struct ColPtrs { const int32_t* c[kMaxArity]; };
 struct ColPtrsMut { int32_t* c[kMaxArity]; };
 
+// One row's part of the validation, the maxima and the order test: is it lexicographically greater than the row before it?
+__device__ __forceinline__ bool load_row_rises(const ColPtrs& cols, const float* __restrict__ tags, int64_t i, int arity, int sr, int32_t* mx, uint32_t& e) {
+  int cmp = 0;                                          // sign of (row i - row i-1), decided by the first differing column
+#pragma unroll
+  for (int c = 0; c < kMaxArity; ++c)
+    if (c < arity) {
+      const int32_t v = cols.c[c][i];
+      if (v < 0) e |= kErrNegativeKey;
+      mx[c] = max(mx[c], v);
+      if (i > 0 && cmp == 0) { const int32_t p = cols.c[c][i - 1]; cmp = v > p ? 1 : v < p ? -1 : 0; }
+    }
+  if (tags) {
+    const float t = tags[i];
+    const bool zero = sr == 0 || sr == 2 ? t == -INFINITY : sr == 1 ? t == INFINITY : false;
+    if (isnan(t) || zero) e |= kErrBadTag;
+  }
+  return i == 0 || cmp > 0;
+}
+
 // Validation, column maxima and an order test in one read of the input: *unordered is raised when some row is not
 // lexicographically greater than the row before it (rows that arrive strictly increasing need no sort and hold no duplicates).
+// One atomic per block and column: with one per warp the ten thousand updates of one word took longer than reading the rows
+// (1.3 million rows of two columns: 22 -> 14 us).
 static __global__ void __launch_bounds__(256) k_col_stats(ColPtrs cols, const float* __restrict__ tags, int64_t n, int arity, int sr,
                                                    int32_t* __restrict__ col_max /*[arity]*/, uint32_t* __restrict__ err,
                                                    uint32_t* __restrict__ unordered) {
+  __shared__ int32_t s_max[8][kMaxArity];
   int32_t mx[kMaxArity] = {0, 0, 0, 0};
   uint32_t e = 0;
   bool out_of_order = false;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    int cmp = 0;                                        // sign of (row i - row i-1), decided by the first differing column
-#pragma unroll
-    for (int c = 0; c < kMaxArity; ++c)
-      if (c < arity) {
-        const int32_t v = cols.c[c][i];
-        if (v < 0) e |= kErrNegativeKey;
-        mx[c] = max(mx[c], v);
-        if (i > 0 && cmp == 0) { const int32_t p = cols.c[c][i - 1]; cmp = v > p ? 1 : v < p ? -1 : 0; }
-      }
-    if (i > 0 && cmp <= 0) out_of_order = true;
-    if (tags) {
-      const float t = tags[i];
-      const bool zero = sr == 0 || sr == 2 ? t == -INFINITY : sr == 1 ? t == INFINITY : false;
-      if (isnan(t) || zero) e |= kErrBadTag;
-    }
-  }
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    out_of_order |= !load_row_rises(cols, tags, i, arity, sr, mx, e);
 #pragma unroll
   for (int c = 0; c < kMaxArity; ++c) {
-#pragma unroll
-    for (int d = 16; d; d >>= 1) mx[c] = max(mx[c], __shfl_xor_sync(0xffffffffu, mx[c], d));
+    mx[c] = __reduce_max_sync(0xffffffffu, mx[c]);
+    if (lane_id() == 0) s_max[warp_id()][c] = mx[c];
   }
-#pragma unroll
-  for (int d = 16; d; d >>= 1) e |= __shfl_xor_sync(0xffffffffu, e, d);
-  if (lane_id() == 0) {
-    for (int c = 0; c < arity; ++c) atomicMax(&col_max[c], mx[c]);
-    if (e) atomicOr(err, e);
+  e = __reduce_or_sync(0xffffffffu, e);
+  if (lane_id() == 0 && e) atomicOr(err, e);
+  if (__syncthreads_or(out_of_order) && threadIdx.x == 0) atomicOr(unordered, 1u);
+  if ((int)threadIdx.x < arity) {
+    int32_t m = 0;
+    for (int w = 0; w < 8; ++w) m = max(m, s_max[w][threadIdx.x]);
+    atomicMax(&col_max[threadIdx.x], m);
   }
-  if (__any_sync(0xffffffffu, out_of_order) && lane_id() == 0) atomicOr(unordered, 1u);
 }
 
 template <typename K>
@@ -65,6 +73,57 @@ __global__ void __launch_bounds__(256) k_pack(ColPtrs cols, const float* __restr
       if (c < L.arity && D.n[c]) v[c] = (int32_t)dict_rank(D.v[c], D.n[c], v[c]);
     }
     keys[i] = pack_key<K>(L, v);
+    float t = tags ? tags[i] : one;
+    if (t == 0.f) t = 0.f;                         // -0.0 -> +0.0
+    tag_out[i] = t;
+  }
+}
+
+// A small load in one launch of one block: the test above, then, if the rows are sound and rise, the packed keys (in 4 bytes if
+// they fit) under the layout that the maxima give.  It saves a launch and a wait.  A load of
+// 320 rows of two columns 47 -> 34 us, of 4,000 48 -> 38 us, of 8,000 46 -> 40 us, of 16,380 43 -> 48 us: the line lies between.
+constexpr int64_t kLoadSmall = 8192;
+static __global__ void __launch_bounds__(1024) k_load_small(ColPtrs cols, const float* __restrict__ tags, int64_t n, int arity, int sr, float one, void* __restrict__ keys,
+                                                     float* __restrict__ tag_out, int32_t* __restrict__ col_max, uint32_t* __restrict__ err, uint32_t* __restrict__ unordered) {
+  __shared__ int32_t s_max[32][kMaxArity];
+  __shared__ KeyLayout s_layout;
+  int32_t mx[kMaxArity] = {0, 0, 0, 0};
+  uint32_t e = 0;
+  bool out_of_order = false;
+  for (int64_t i = threadIdx.x; i < n; i += 1024) out_of_order |= !load_row_rises(cols, tags, i, arity, sr, mx, e);
+#pragma unroll
+  for (int c = 0; c < kMaxArity; ++c) {
+    mx[c] = __reduce_max_sync(0xffffffffu, mx[c]);
+    if (lane_id() == 0) s_max[warp_id()][c] = mx[c];
+  }
+  e = __reduce_or_sync(0xffffffffu, e);
+  if (threadIdx.x == 0) { *err = 0; s_layout = KeyLayout{}; }
+  const bool down = __syncthreads_or(out_of_order), bad = __syncthreads_or(e != 0);
+  if (lane_id() == 0 && e) atomicOr(err, e);
+  if (warp_id() == 0) {
+    int32_t top[kMaxArity];
+    int total = 0;
+#pragma unroll
+    for (int c = 0; c < kMaxArity; ++c) { top[c] = __reduce_max_sync(0xffffffffu, s_max[lane_id()][c]); if (c < arity) total += max(32 - __clz(top[c]), 1); }
+    if (lane_id() == 0) {
+      int sh = total;
+      s_layout.arity = arity;
+      s_layout.total_bits = total;
+#pragma unroll
+      for (int c = 0; c < kMaxArity; ++c)
+        if (c < arity) { const int bits = max(32 - __clz(top[c]), 1); sh -= bits; s_layout.shift[c] = sh; s_layout.mask[c] = (uint32_t)((1ull << bits) - 1); col_max[c] = top[c]; }
+      *unordered = down ? 1u : 0u;
+    }
+  }
+  __syncthreads();
+  if (down || bad || s_layout.total_bits > 64) return;
+  const KeyLayout L = s_layout;
+  for (int64_t i = threadIdx.x; i < n; i += 1024) {
+    int32_t v[kMaxArity];
+#pragma unroll
+    for (int c = 0; c < kMaxArity; ++c) v[c] = c < arity ? cols.c[c][i] : 0;
+    if (L.total_bits <= 32) reinterpret_cast<uint32_t*>(keys)[i] = pack_key<uint32_t>(L, v);
+    else reinterpret_cast<uint64_t*>(keys)[i] = pack_key<uint64_t>(L, v);
     float t = tags ? tags[i] : one;
     if (t == 0.f) t = 0.f;                         // -0.0 -> +0.0
     tag_out[i] = t;
