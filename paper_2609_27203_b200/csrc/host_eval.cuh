@@ -208,11 +208,21 @@ void count_variant(Ctx* c, const Variant& v, const Relation& H, Counted& q, int 
               (const uint64_t*)q.sums.as<uint64_t>(), q.start.as<uint64_t>());
 }
 
+// Candidates per block of a launch over `take` of a variant's `total` candidates from n rows: the most a block can hold, unless
+// that leaves SMs idle, or unless a tile would usually span more rows than a block can stage (rules with about one match a
+// row), when every candidate would search for its row.  Seeds of 4,000 rows 17 to 23 -> 8 us, of 300,000 25 -> 11 us.
+template <int SINK>
+uint32_t expand_tile_for(uint64_t take, uint64_t total, uint32_t n) {
+  typedef ExpShapeT<SINK != kSinkWrite> SH;
+  const uint64_t spread = take / (kSMs * 8), staged = (uint64_t)SH::rows * 3 / 4 * total / std::max(n, 1u);
+  return (uint32_t)std::min<uint64_t>(SH::tile, std::max<uint64_t>(kExpBlock, std::min(spread, staged) / kExpBlock * kExpBlock));
+}
+
 // materialise candidates [lo, hi) of a counted variant into (ckeys, ctags), or (MODE == kExpBackward) run the backward
 // scatter, or (SINK != kSinkWrite) apply them to the head relation's tag mirror
 template <int MODE, int SINK>
 void launch_expand_mode(Ctx* c, Counted& q, uint64_t lo, uint64_t hi, int ckb, void* ckeys, float* ctags, const BwdArgs& bw, const MirrorArgs& mr) {
-  constexpr uint32_t tile = SINK == kSinkWrite ? kExpTileWrite : kExpTileMirror;
+  const uint32_t tile = expand_tile_for<SINK>(hi - lo, q.total, q.outer.n);
   const unsigned blocks = (unsigned)((hi - lo + tile - 1) / tile);
   if (blocks == 0) return;                               // no candidates in the range
   const uint64_t* st = q.start.as<uint64_t>();
@@ -220,22 +230,28 @@ void launch_expand_mode(Ctx* c, Counted& q, uint64_t lo, uint64_t hi, int ckb, v
   uint32_t* err = ctrl_u32(c, kSlotErr);
   // all work is issued on one stream, so a scratch block may be released as soon as its last kernel is queued:
   // whatever reuses the memory runs later in stream order
-  DevBuf tile_rows(c, (size_t)blocks * 8);
-  const int64_t bytes = c->note_bytes;
-  c->note_bytes = 0;
-  XLOG_LAUNCH(c, k_expand_partition, (blocks + 255) / 256, 256, 0, st, q.outer.n, lo, hi, blocks, tile, tile_rows.as<uint2>());
-  const uint2* tr = tile_rows.as<uint2>();
-  c->note_bytes = bytes;
+  DevBuf tile_rows;
+  const uint2* tr = nullptr;
+  // more than one wave: the lookups of all tiles in a launch of their own; up to one, a launch of 7 to 14 us costs more than the
+  // 1 to 2 us that it takes the blocks to look their rows up
+  if (blocks > kSMs * 8) {
+    tile_rows = DevBuf(c, (size_t)blocks * 8);
+    const int64_t bytes = c->note_bytes;
+    c->note_bytes = 0;
+    XLOG_LAUNCH(c, k_expand_partition, (blocks + 255) / 256, 256, 0, st, q.outer.n, lo, hi, blocks, tile, tile_rows.as<uint2>());
+    tr = tile_rows.as<uint2>();
+    c->note_bytes = bytes;
+  }
   if (q.outer.key_bytes == 4 && ckb == 4)
-    XLOG_LAUNCH(c, (k_join_expand<uint32_t, uint32_t, MODE, SINK>), blocks, kExpBlock, 0, q.spec, (const uint32_t*)q.outer.keys, q.outer.n, st, ri, tr, lo, hi, (uint32_t*)ckeys, ctags, err, bw, mr);
+    XLOG_LAUNCH(c, (k_join_expand<uint32_t, uint32_t, MODE, SINK>), blocks, kExpBlock, 0, q.spec, (const uint32_t*)q.outer.keys, q.outer.n, st, ri, tr, tile, lo, hi, (uint32_t*)ckeys, ctags, err, bw, mr);
   else if (ckb == 4)
-    XLOG_LAUNCH(c, (k_join_expand<uint64_t, uint32_t, MODE, SINK>), blocks, kExpBlock, 0, q.spec, (const uint64_t*)q.outer.keys, q.outer.n, st, ri, tr, lo, hi, (uint32_t*)ckeys, ctags, err, bw, mr);
+    XLOG_LAUNCH(c, (k_join_expand<uint64_t, uint32_t, MODE, SINK>), blocks, kExpBlock, 0, q.spec, (const uint64_t*)q.outer.keys, q.outer.n, st, ri, tr, tile, lo, hi, (uint32_t*)ckeys, ctags, err, bw, mr);
   else if (SINK != kSinkWrite)
     fail(XLOG_ERR_INTERNAL, "tag mirror with wide keys");
   else if (q.outer.key_bytes == 4)
-    XLOG_LAUNCH(c, (k_join_expand<uint32_t, uint64_t, MODE, kSinkWrite>), blocks, kExpBlock, 0, q.spec, (const uint32_t*)q.outer.keys, q.outer.n, st, ri, tr, lo, hi, (uint64_t*)ckeys, ctags, err, bw, mr);
+    XLOG_LAUNCH(c, (k_join_expand<uint32_t, uint64_t, MODE, kSinkWrite>), blocks, kExpBlock, 0, q.spec, (const uint32_t*)q.outer.keys, q.outer.n, st, ri, tr, tile, lo, hi, (uint64_t*)ckeys, ctags, err, bw, mr);
   else
-    XLOG_LAUNCH(c, (k_join_expand<uint64_t, uint64_t, MODE, kSinkWrite>), blocks, kExpBlock, 0, q.spec, (const uint64_t*)q.outer.keys, q.outer.n, st, ri, tr, lo, hi, (uint64_t*)ckeys, ctags, err, bw, mr);
+    XLOG_LAUNCH(c, (k_join_expand<uint64_t, uint64_t, MODE, kSinkWrite>), blocks, kExpBlock, 0, q.spec, (const uint64_t*)q.outer.keys, q.outer.n, st, ri, tr, tile, lo, hi, (uint64_t*)ckeys, ctags, err, bw, mr);
 }
 template <bool BWD>
 void launch_expand(Ctx* c, Counted& q, uint64_t lo, uint64_t hi, int ckb, void* ckeys, float* ctags, const BwdArgs& bw) {

@@ -295,6 +295,25 @@ static __global__ void __launch_bounds__(256) k_expand_partition(const uint64_t*
   tile_rows[t] = make_uint2(r[0], r[1]);
 }
 
+// The same for one block's own tile: warps 0 and 1 look up its two ends, 32 probes a step.  Called by all threads.
+__device__ __forceinline__ uint2 expand_rows_of_tile(const uint64_t* __restrict__ start, uint32_t n_outer, uint64_t t_lo, uint64_t t_hi) {
+  __shared__ uint32_t s_row[2];
+  if (warp_id() < 2) {
+    const uint64_t target = warp_id() == 0 ? t_lo : t_hi - 1;
+    uint32_t lo = 0, hi = n_outer;                    // the first start > target lies in [lo, hi]
+    while (hi - lo > 32) {
+      const uint32_t step = (hi - lo) / 32;
+      const int k = __popc(__ballot_sync(0xffffffffu, start[lo + (lane_id() + 1) * step - 1] <= target));
+      if (k < 32) hi = lo + (k + 1) * step - 1;
+      lo += k * step;
+    }
+    const uint32_t up = lo + __popc(__ballot_sync(0xffffffffu, lo + lane_id() < hi && start[lo + lane_id()] <= target));
+    if (lane_id() == 0) s_row[warp_id()] = up - 1;
+  }
+  __syncthreads();
+  return make_uint2(s_row[0], s_row[1]);
+}
+
 template <typename SH> struct ExpSmem {
   uint32_t sstart[SH::rows];
   uint4 sinfo[SH::rows];
@@ -513,23 +532,24 @@ __device__ __forceinline__ void expand_tile(ExpSmem<ExpShapeT<SINK != kSinkWrite
   }
 }
 
-// Block b produces candidates [out_lo + b*tile, ...).  `start` is the exclusive scan of `deg`
+// Block b produces candidates [out_lo + b*tile, ...), tile <= ExpShapeT::tile; without tile_rows it looks its rows up itself.  `start` is the exclusive scan of `deg`
 // (global candidate index of each outer row's first match).  The outer rows covering the tile are
 // staged in shared memory (their starts relative to the tile and their row records), so the per-
 // candidate work is a short binary search in shared memory plus the coalesced inner reads.
 template <typename KO, typename KH, int MODE, int SINK = kSinkWrite>
 __global__ void __launch_bounds__(kExpBlock, SINK == kSinkWrite ? kExpWriteBlocksPerSM : kExpMirrorBlocksPerSM) k_join_expand(JoinSpec S, const KO* __restrict__ okeys, uint32_t n_outer,
                                                            const uint64_t* __restrict__ start, const uint4* __restrict__ rowinfo,
-                                                           const uint2* __restrict__ tile_rows, uint64_t out_lo, uint64_t out_hi,
+                                                           const uint2* __restrict__ tile_rows, uint32_t tile, uint64_t out_lo, uint64_t out_hi,
                                                            KH* __restrict__ ckeys,
                                                            float* __restrict__ ctags, uint32_t* __restrict__ err, BwdArgs bw, MirrorArgs mr) {
   typedef ExpShapeT<SINK != kSinkWrite> SH;
   __shared__ ExpSmem<SH> sm;
-  const uint64_t t_lo = out_lo + (uint64_t)blockIdx.x * SH::tile;
-  const uint64_t t_hi = min(t_lo + SH::tile, out_hi);
+  const uint64_t t_lo = out_lo + (uint64_t)blockIdx.x * tile;
+  const uint64_t t_hi = min(t_lo + tile, out_hi);
   if (t_lo >= t_hi) return;
   uint32_t e = 0;
-  expand_tile<KO, KH, MODE, SINK>(sm, S, okeys, n_outer, start, rowinfo, tile_rows[blockIdx.x], t_lo, t_hi, out_lo, ckeys, ctags, bw, mr, e);
+  const uint2 tr = tile_rows ? tile_rows[blockIdx.x] : expand_rows_of_tile(start, n_outer, t_lo, t_hi);
+  expand_tile<KO, KH, MODE, SINK>(sm, S, okeys, n_outer, start, rowinfo, tr, t_lo, t_hi, out_lo, ckeys, ctags, bw, mr, e);
   if (e) atomicOr(err, e);
 }
 
