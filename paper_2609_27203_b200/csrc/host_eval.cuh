@@ -389,6 +389,9 @@ bool group_rule_applies(Ctx* c, const Variant& v, const Relation& H, GroupRule& 
     if (k != a0.var && k != a1.var && k != b1.var && h1.coef[k] != 0) return false;
   }
   if (h0.coef[a0.var] < 1 || h1.coef[b1.var] < 1) return false;
+  // the kernels test the part of the second column that d's row gives and e's part each on its own, but only their sum has to
+  // be a value: neither may be negative
+  if (h1.c0 < 0 || h1.coef[a0.var] < 0 || h1.coef[a1.var] < 0) return false;
   const int64_t groups = ((int64_t)RA.val_max[0] - a0.add) / a0.mul + 1;
   if (groups > 2 * (int64_t)v.outer.n + 1024) return false;
   const uint32_t slots = (uint32_t)H.col_max[1] + 1;

@@ -83,3 +83,56 @@ def test_a_small_arena_takes_the_sorting_route_or_the_groups_alike():
         ctx.fixpoint()
         H.compare_relations(ctx.read(ids["h"]), o.read(oids["h"]), abs_tol=1e-4, what="small arena")
         ctx.close()
+
+
+def whole_values(which, groups, sr, seed):
+    """Programs of the same form whose second head column is a sum with negative parts, its value in range for every pair of rows."""
+    rng = np.random.default_rng(seed)
+    lo, hi, expr = {
+        "two dice": (range(1, 7), range(1, 7), (-2, ((1, 1), (2, 1)))),                 # a + b - 2
+        "difference": (range(0, 9), range(8, 32), (0, ((1, -1), (2, 1)))),              # b - a
+        "twice the difference": (range(3, 7), range(6, 16), (1, ((1, -2), (2, 2)))),
+        "by group": (range(0, 3), range(0, 5), (8, ((0, -1), (1, 1), (2, 1)))),         # 8 - p + a + b over p < 9
+        "all of them": (range(0, 4), range(5, 9), (10, ((0, -1), (1, -2), (2, 1)))),    # 10 - p - 2 a + b over p < 9
+    }[which]
+    if which in ("by group", "all of them"):
+        groups = min(groups, 9)
+    d = np.array([(p, a) for p in range(groups) for a in lo if rng.random() < 0.85 or p == 0], np.int32).T
+    e = np.array([(p, b) for p in range(groups) for b in hi if rng.random() < 0.85 or p == 0], np.int32).T
+    tags = lambda n: (0.25 + rng.random(n)).astype(np.float32) if sr == W.SUMPROD else (-4.0 * rng.random(n)).astype(np.float32)
+    rule = W.Rule("h", (W.V(0), W.Affine(*expr)), (W.Atom("d", (W.Var(0), W.Var(1))), W.Atom("e", (W.Var(0), W.Var(2)))))
+    return W.Program("whole values", {k: (2, sr) for k in "deh"}, [rule], {"d": (list(d), tags(d.shape[1])), "e": (list(e), tags(e.shape[1]))}, ("h",))
+
+
+@pytest.mark.parametrize("sr", [W.SUMPROD, W.LOGSUMEXP, W.MAXPLUS])
+@pytest.mark.parametrize("which", ["two dice", "difference", "twice the difference", "by group", "all of them"])
+def test_only_the_whole_value_has_to_be_in_range(sr, which):
+    import torch
+    from paper_2609_27203_b200 import xlog
+    prog = whole_values(which, 50, sr, 11)
+    ctx, ids, rules = xlog.load_program(prog, arena_bytes=1 << 28, flags=xlog.FLAG_CHECK_INVARIANTS)
+    o, oids, orules = oracle.load_program(prog)
+    o.run("seminaive")
+    ctx.fixpoint()
+    tol = {W.SUMPROD: dict(rel_tol=1e-6), W.LOGSUMEXP: dict(abs_tol=1e-4)}.get(sr, {})
+    rep = H.compare_relations(ctx.read(ids["h"]), o.read(oids["h"]), what=which, **tol)
+    if sr != W.MAXPLUS:
+        g = np.random.default_rng(7).standard_normal(rep["rows"]).astype(np.float32)
+        parts = ctx.backward(rules[0], torch.from_numpy(g).cuda(), same_buffer_for_same_relation=False)
+        for got, want in zip(parts, o.backward(orules[0], g)):
+            want = want.astype(np.float64)
+            assert np.all(np.abs(got.cpu().numpy() - want) <= 1e-5 + 1e-4 * np.abs(want))
+    ctx.close()
+
+
+@pytest.mark.parametrize("c0,k0", [(-1, 1), (5, -1)])
+def test_a_value_out_of_range_is_still_refused(c0, k0):
+    from paper_2609_27203_b200 import xlog
+    a = np.arange(7, dtype=np.int32)                          # -1 + 0 + 0, and 5 - 6 + 0
+    rule = W.Rule("h", (W.V(0), W.Affine(c0, ((1, k0), (2, 1)))), (W.Atom("d", (W.Var(0), W.Var(1))), W.Atom("e", (W.Var(0), W.Var(2)))))
+    prog = W.Program("out", {k: (2, W.SUMPROD) for k in "deh"}, [rule], {k: ([0 * a, a], None) for k in "de"}, ("h",))
+    ctx, _, _ = xlog.load_program(prog, arena_bytes=1 << 26)
+    with pytest.raises(xlog.XlogError) as err:
+        ctx.fixpoint()
+    assert err.value.status == "CAPACITY_EXCEEDED"
+    ctx.close()
