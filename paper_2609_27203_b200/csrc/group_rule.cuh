@@ -2,9 +2,9 @@
 // (the digit sum is  sum(p, a + b) :- digit(2p, a), digit(2p + 1, b)).
 //
 // Both atoms are met on p, so the group of p is the product of one run of d and one run of e, and when the head's second column
-// takes at most 32 values ("slots") a warp needs no candidate in memory: a lane holds the tag of the e row that would land in
-// its slot from row part 0, each row of d moves those tags along by its own part (one shuffle), and each lane folds what comes
-// by.  The sorting route writes every candidate, sorts, and reduces by key.
+// takes at most 32 values ("slots") and so does d's, a run is at most a row a lane and a warp needs no candidate in memory: a
+// lane holds the tag of the e row that would land in its slot from row part 0, each row of d moves those tags along by its own
+// part (one read of shared memory), and each lane folds what comes by.  The sorting route writes every candidate, sorts, and reduces by key.
 //
 //   k_group_rule      a warp per p: aggregates and the mask of slots that have any; counts of rows and candidates per block
 //   k_group_emit      the same blocks: the counts of the blocks before are the offset, rows go out in key order.  The host
@@ -124,31 +124,28 @@ __global__ void __launch_bounds__(kGroupBlock) k_group_rule(const __grid_constan
       sm.tab[32 + lane] = kGroupEmpty;
       __syncwarp();
       uint32_t at_b = 0;
-      for (uint32_t j = r.z + lane; j < r.w; j += 32) {
-        const uint32_t z = group_slot(P, (uint32_t)P.col1[j], e);
-        sm.tab[32 + z] = __float_as_uint(P.tag1[j]);
-        at_b |= 1u << z;
+      if (r.z + lane < r.w) {
+        const uint32_t z = group_slot(P, (uint32_t)P.col1[r.z + lane], e);
+        sm.tab[32 + z] = __float_as_uint(P.tag1[r.z + lane]);
+        at_b = 1u << z;
       }
       at_b = __reduce_or_sync(0xffffffffu, at_b);
       GroupFold<Op> f;
       uint32_t mask = 0;
-      for (uint32_t i0 = r.x; i0 < r.y; i0 += 32) {
-        const uint32_t nr = min(32u, r.y - i0);
-        if (i0 != r.x && lane < nr) { ka = (uint32_t)key0[i0 + lane] & P.mask0; ta = P.tag0[i0 + lane]; }
-        if (lane < nr) {
-          const uint32_t off = group_row_part(P, p, ka, e);
-          sm.row[lane] = make_float2(__uint_as_float(off), ta);
-          mask |= at_b << off;
-          if (off + (31 - __clz(at_b)) >= P.slots) e |= kErrHeadRange;
-        }
-        __syncwarp();
-        for (uint32_t i = 0; i < nr; ++i) {
-          const float2 row = sm.row[i];
-          const uint32_t bt = sm.tab[32 + lane - __float_as_uint(row.x)];
-          f.take(TIMES ? row.y * __uint_as_float(bt) : row.y + __uint_as_float(bt), bt != kGroupEmpty);
-        }
-        __syncwarp();
+      const uint32_t nr = min(32u, r.y - r.x);
+      if (lane < nr) {
+        const uint32_t off = group_row_part(P, p, ka, e);
+        sm.row[lane] = make_float2(__uint_as_float(off), ta);
+        mask = at_b << off;
+        if (off + (31 - __clz(at_b)) >= P.slots) e |= kErrHeadRange;
       }
+      __syncwarp();
+      for (uint32_t i = 0; i < nr; ++i) {
+        const float2 row = sm.row[i];
+        const uint32_t bt = sm.tab[32 + lane - __float_as_uint(row.x)];
+        f.take(TIMES ? row.y * __uint_as_float(bt) : row.y + __uint_as_float(bt), bt != kGroupEmpty);
+      }
+      __syncwarp();
       mask = __reduce_or_sync(0xffffffffu, mask);
       if ((mask >> lane) & 1u && lane < P.slots) P.agg[(size_t)p * P.slots + lane] = f.lower();
       if ((int)lane == g) my_mask = mask;
@@ -226,11 +223,11 @@ __global__ void __launch_bounds__(kGroupBlock) k_group_backward(const __grid_con
       const int gi = __ffs(todo) - 1;
       const uint32_t p = p0 + gi;
       const uint4 r = group_runs_of(runs, gi);
-      const uint32_t nb0 = min(32u, r.w - r.z), wide = nb0 > 16 ? 32u : 16u, sub = lane & (wide - 1);
+      const uint32_t nb = min(32u, r.w - r.z), wide = nb > 16 ? 32u : 16u, sub = lane & (wide - 1);
       uint32_t ka = 0, zb = 0;
       float ta = 0.f, tb = 0.f;
       if (r.x + lane < r.y) { ka = (uint32_t)key0[r.x + lane] & P.mask0; ta = P.tag0[r.x + lane]; }
-      if (sub < nb0) { zb = (uint32_t)P.col1[r.z + sub]; tb = P.tag1[r.z + sub]; }
+      if (sub < nb) { zb = (uint32_t)P.col1[r.z + sub]; tb = P.tag1[r.z + sub]; }
       // the group's head rows, a lane per row, then a place per slot
       const KH top = (KH)(P.top_c0 + P.top_mul * p), want = top << P.shift;
       KH k = 0;
@@ -255,41 +252,34 @@ __global__ void __launch_bounds__(kGroupBlock) k_group_backward(const __grid_con
       h += __popc(__ballot_sync(0xffffffffu, at));
       const uint32_t present = __reduce_or_sync(0xffffffffu, at ? 1u << mine : 0u);
 
-      for (uint32_t i0 = r.x; i0 < r.y; i0 += 32) {
-        const uint32_t nr = min(32u, r.y - i0);
-        if (i0 != r.x && lane < nr) { ka = (uint32_t)key0[i0 + lane] & P.mask0; ta = P.tag0[i0 + lane]; }
-        if (lane < nr) sm.row[lane] = make_float2(__uint_as_float(group_row_part(P, p, ka, e)), ta);
-        sm.row_sum[lane] = 0.f;
-        for (uint32_t j0 = r.z; j0 < r.w; j0 += 32) {
-          const uint32_t nb = min(32u, r.w - j0);
-          if (r.w - r.z > 32 && lane < nb) { zb = (uint32_t)P.col1[j0 + lane]; tb = P.tag1[j0 + lane]; }
-          const uint32_t z = sub < nb ? group_slot(P, zb, e) : 0u;
-          float inner = 0.f;
-          __syncwarp();
-          for (uint32_t i = lane / wide; i < nr + lane / wide; i += 32 / wide) {       // the same number of turns for every lane
-            float to_a = 0.f;
-            if (i < nr && sub < nb) {
-              const float2 row = sm.row[i];
-              const uint32_t slot = __float_as_uint(row.x) + z;
-              if (slot > 31 || !((present >> slot) & 1u)) e |= kErrInternal;
-              else {
-                const float2 head = sm.head[slot];
-                if (LSE) { to_a = head.x * expf(row.y + tb - head.y); inner += to_a; }
-                else { to_a = head.x * tb; inner += head.x * row.y; }
-              }
-            }
-#pragma unroll
-            for (int d = 8; d; d >>= 1) to_a += __shfl_xor_sync(0xffffffffu, to_a, d);
-            if (wide == 32) to_a += __shfl_xor_sync(0xffffffffu, to_a, 16);
-            if (sub == 0 && i < nr) sm.row_sum[i] += to_a;
+      const uint32_t nr = min(32u, r.y - r.x);
+      if (lane < nr) sm.row[lane] = make_float2(__uint_as_float(group_row_part(P, p, ka, e)), ta);
+      sm.row_sum[lane] = 0.f;
+      const uint32_t z = sub < nb ? group_slot(P, zb, e) : 0u;
+      float inner = 0.f;
+      __syncwarp();
+      for (uint32_t i = lane / wide; i < nr + lane / wide; i += 32 / wide) {       // the same number of turns for every lane
+        float to_a = 0.f;
+        if (i < nr && sub < nb) {
+          const float2 row = sm.row[i];
+          const uint32_t slot = __float_as_uint(row.x) + z;
+          if (slot > 31 || !((present >> slot) & 1u)) e |= kErrInternal;
+          else {
+            const float2 head = sm.head[slot];
+            if (LSE) { to_a = head.x * expf(row.y + tb - head.y); inner += to_a; }
+            else { to_a = head.x * tb; inner += head.x * row.y; }
           }
-          if (wide == 16) inner += __shfl_xor_sync(0xffffffffu, inner, 16);
-          if (bw.grad_inner && lane < nb) atomicAdd(bw.grad_inner + j0 + lane, inner);
         }
-        __syncwarp();
-        if (lane < nr) atomicAdd(bw.grad_outer + i0 + lane, sm.row_sum[lane]);
-        __syncwarp();
+#pragma unroll
+        for (int d = 8; d; d >>= 1) to_a += __shfl_xor_sync(0xffffffffu, to_a, d);
+        if (wide == 32) to_a += __shfl_xor_sync(0xffffffffu, to_a, 16);
+        if (sub == 0 && i < nr) sm.row_sum[i] = to_a;
       }
+      if (wide == 16) inner += __shfl_xor_sync(0xffffffffu, inner, 16);
+      if (bw.grad_inner && lane < nb) atomicAdd(bw.grad_inner + r.z + lane, inner);
+      __syncwarp();
+      if (lane < nr) atomicAdd(bw.grad_outer + r.x + lane, sm.row_sum[lane]);
+      __syncwarp();
     }
   }
   if (e) atomicOr(P.err, e);

@@ -364,8 +364,8 @@ KeyTags evaluate(Ctx* c, Relation& H, std::vector<Variant>& variants, const Sour
 constexpr int kSlotGroup = 60;             // rows, candidates
 
 // Is the variant's rule of that form, without dictionaries, over binary relations, and do the head's values and the groups
-// fit: at most kGroupSlots values of the second column, at most two groups per scanned row (an aggregate array of up to 256
-// bytes per row), with room for all of it.  Fills the compiled rule, without its outputs.
+// fit: at most kGroupSlots values of the head's and of d's second column, at most two groups per scanned row (an aggregate array
+// of up to 256 bytes per row), with room for all of it.  Fills the compiled rule, without its outputs.
 bool group_rule_applies(Ctx* c, const Variant& v, const Relation& H, GroupRule& P) {
   const xlog_plan& p = v.rule->plan;
   if (v.rule->kind != 2 || p.emit_count_column || p.n_head_cols != 2 || H.arity != 2) return false;
@@ -377,6 +377,10 @@ bool group_rule_applies(Ctx* c, const Variant& v, const Relation& H, GroupRule& 
   Relation& RB = *c->rels[B.rel];
   if (RA.arity != 2 || RB.arity != 2 || RA.dict_n[0] || RA.dict_n[1] || RB.dict_n[0] || RB.dict_n[1] || H.dict_n[0] || H.dict_n[1]) return false;
   if (H.col_max[1] >= kGroupSlots || v.outer.keys != RA.keys() || v.outer.n == 0 || RB.n == 0) return false;
+  // A warp goes through d's run of a group one row after the other: at most a row a lane.  e's run is that short because its
+  // values reach the head; d's need not be.  Ten groups, eight rows of e, rows of d in each (us, evaluation / gradient, here and
+  // over the join): 64 34 / 42 and 144 / 89, 1,024 85 / 164 and 157 / 102, 65,536 3430 / 8060 and 288 / 621.
+  if (RA.val_max[1] >= kGroupSlots) return false;
   const auto& a0 = A.args[0];
   const auto& a1 = A.args[1];
   const auto& b1 = B.args[1];

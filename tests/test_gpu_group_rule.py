@@ -136,3 +136,44 @@ def test_a_value_out_of_range_is_still_refused(c0, k0):
         ctx.fixpoint()
     assert err.value.status == "CAPACITY_EXCEEDED"
     ctx.close()
+
+
+@pytest.mark.parametrize("sr", [W.SUMPROD, W.LOGSUMEXP, W.MINPLUS])
+@pytest.mark.parametrize("run", [1, 31, 32, 33, 200, 30000])
+def test_long_runs_are_spread_over_the_device(sr, run):
+    """h(p, b) :- d(p, a), e(p, b): d's column does not reach the head, so nothing but d bounds a group's rows; the group kernels
+    take at most 32.  One value in eight of d is missing but the last."""
+    import torch
+    from paper_2609_27203_b200 import xlog
+    r = np.random.default_rng(run)
+    there = r.random((3, run)) < 0.875
+    there[:, -1] = True
+    d, e = [x.astype(np.int32) for x in np.nonzero(there)], [x.astype(np.int32) for x in np.nonzero(np.ones((3, 5)))]
+    tags = lambda n: (0.25 + r.random(n)).astype(np.float32) if sr == W.SUMPROD else (-4.0 * r.random(n)).astype(np.float32)
+    rule = W.Rule("h", (W.V(0), W.V(2)), (W.Atom("d", (W.Var(0), W.Var(1))), W.Atom("e", (W.Var(0), W.Var(2)))))
+    prog = W.Program("runs", {k: (2, sr) for k in "deh"}, [rule], {"d": (d, tags(len(d[0]))), "e": (e, tags(15))}, ("h",))
+    ctx, ids, rules = xlog.load_program(prog, arena_bytes=1 << 28, flags=xlog.FLAG_PROFILE)
+    o, oids, orules = oracle.load_program(prog)
+    o.run("seminaive")
+    ctx.fixpoint()
+    tol = {W.SUMPROD: dict(rel_tol=1e-6), W.LOGSUMEXP: dict(abs_tol=1e-4)}.get(sr, {})
+    rep = H.compare_relations(ctx.read(ids["h"]), o.read(oids["h"]), what=f"runs of {run}", **tol)
+    assert rep["rows"] == 15 and ("k_group_rule" in ctx.profile()) == (run <= 32)
+    if sr != W.MINPLUS:
+        g = r.standard_normal(15).astype(np.float32)
+        parts = ctx.backward(rules[0], torch.from_numpy(g).cuda(), same_buffer_for_same_relation=False)
+        assert ("k_group_backward" in ctx.profile()) == (run <= 32)
+        # against 64 bits: every term is rounded a few times and the sums have up to 26,250 of them, added in fp32 in any order
+        want = [np.zeros(len(d[0])), np.zeros(15)]
+        head, td, te = ctx.read(ids["h"])[1].astype(np.float64).reshape(3, 5), prog.facts["d"][1].astype(np.float64), prog.facts["e"][1].astype(np.float64).reshape(3, 5)
+        size = np.zeros(15)
+        for p in range(3):
+            at = d[0] == p
+            gp = g.reshape(3, 5)[p].astype(np.float64)
+            share = np.exp(td[at][:, None] + te[p] - head[p]) if sr == W.LOGSUMEXP else None
+            want[0][at] = (share * gp).sum(1) if share is not None else (te[p] * gp).sum()
+            want[1].reshape(3, 5)[p] = (share * gp).sum(0) if share is not None else gp * td[at].sum()
+            size.reshape(3, 5)[p] = np.abs(share * gp).sum(0) if share is not None else np.abs(gp) * td[at].sum()
+        assert np.allclose(parts[0].cpu().numpy(), want[0], rtol=1e-4, atol=1e-5)
+        assert np.all(np.abs(parts[1].cpu().numpy() - want[1]) <= 1e-5 + 1e-4 * size)
+    ctx.close()
