@@ -96,11 +96,12 @@ bool ensure_tri_rank(Ctx* c, Relation& E, Index& out_ix, Index& in_ix, bool lse)
   const int bits = bit_length(N);
   sort_pairs<uint32_t>(c, ka, va, kb, vb, m, bits);
   sync_ctrl(c);
-  float top;
-  { const uint32_t u = (uint32_t)c->h_ctrl[kSlotTrk + kTrkAbsMax]; memcpy(&top, &u, 4); }
+  float top, low;
+  { const uint32_t u = (uint32_t)c->h_ctrl[kSlotTrk + kTrkAbsMax], v = ~(uint32_t)c->h_ctrl[kSlotTrk + kTrkAbsMin]; memcpy(&top, &u, 4); memcpy(&low, &v, 4); }
+  const bool in_range = lse ? top <= kTriRankMaxTag : top <= kTriRankMaxNum && (top == 0.f || low >= kTriRankMinNum);      // false for NaN
   X.n_edges = (uint32_t)c->h_ctrl[kSlotTrk + kTrkEdges];
   X.n_nodes = (uint32_t)c->h_ctrl[kSlotTrk + kTrkNodes];
-  if (c->h_ctrl[kSlotTrk + kTrkLoops] || (lse && !(top <= kTriRankMaxTag)) || X.n_edges == 0) { X = TriRankIndex(); X.tried = true; return false; }
+  if (c->h_ctrl[kSlotTrk + kTrkLoops] || !in_range || X.n_edges == 0) { X = TriRankIndex(); X.tried = true; return false; }
   const uint32_t me = X.n_edges, P = X.n_nodes;
   DevBuf place(c, (size_t)m * 4);
   for (int o = 1; o >= 0; --o) {

@@ -6,7 +6,8 @@
 // corner v, whose lists are short (at most a few hundred entries whatever the hubs): 1.2e8 entries for the same graph.  Its
 // term goes to all three corners.  The tags make that cheap: the term's weight exp(w_va + w_ab + w_bv) is the product of three
 // numbers kept with the edges, and the sums are plain sums in fp64 (for sum-product the tags are such numbers already).
-// Usable while no product of three can leave the normal fp32 range (|w| <= kTriRankMaxTag under logsumexp).
+// Usable while no product of two or three can leave the normal fp32 range, in whatever order a corner sees its factors: |w| <=
+// kTriRankMaxTag under logsumexp, w = 0 or kTriRankMinNum <= |w| <= kTriRankMaxNum under sum-product.
 //
 // Two launches, one per group of corners, so that no sum is formed by atomics in an order that varies:
 //   by a:  mark out(a) in a shared-memory bitmap; for every lower v with v -> a walk the higher b with b -> v: a marked b closes
@@ -26,13 +27,15 @@ namespace xlog {
 constexpr int64_t kTriRankMaxNodes = (int64_t)1 << 19;       // 128 KB of bitmap and places
 constexpr uint32_t kTriRankMinEdges = 1u << 17;  // below, the plain kernels are as fast and need no second copy of the graph
 constexpr float kTriRankMaxTag = 28.f;           // exp(3 * 28) and exp(-3 * 28) are normal fp32 numbers
+constexpr float kTriRankMaxNum = 0x1p42f, kTriRankMinNum = 0x1p-42f;      // as are 2^126 and 2^-126
 constexpr int kTriRankBlock = 512;
 // corners with fewer entries to walk are searched, a warp each; a block's bitmap costs about as much as 500 searches in a row
 // (all kernels, us, at limits of 2048 / 1024 / 512: R-MAT 18 1186 / 1203 / 1212, R-MAT 16 367 / 304 / 284, R-MAT 14 271 / 200 / 173)
 constexpr uint32_t kTriRankSmall = 512;
 constexpr int kTriRankSweeps = 2;                // sweeps of 32 list entries a warp reads before it tests them (both launches, us: 1 907, 2 878, 3 909, 4 962)
 
-enum { kTrkEdges = 0, kTrkNodes = 1, kTrkLoops = 2, kTrkAbsMax = 3, kTrkUnitsA = 4, kTrkUnitsB = 5, kTrkWalkA = 6, kTrkWalkB = 7, kTrkTotals = 8 };
+enum { kTrkEdges = 0, kTrkNodes = 1, kTrkLoops = 2, kTrkAbsMax = 3, kTrkUnitsA = 4, kTrkUnitsB = 5, kTrkWalkA = 6, kTrkWalkB = 7,
+       kTrkAbsMin = 8, kTrkTotals = 9 };        // kTrkAbsMin: complement of the smallest |tag| that is not zero (0: none)
 
 // One orientation of the ordered graph: lists of neighbours in ascending rank; entries [off[v], split[v]) rank lower than v.
 struct TriRankLists {
@@ -65,21 +68,24 @@ static __global__ void __launch_bounds__(256) k_trk_ranks(const uint32_t* __rest
 static __global__ void __launch_bounds__(256) k_trk_edges(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, const float* __restrict__ w, uint32_t n,
                                                           const uint32_t* __restrict__ rank, uint32_t n_nodes, uint32_t* __restrict__ key, uint32_t* __restrict__ edge,
                                                           unsigned long long* __restrict__ totals) {
-  uint32_t kept = 0, loops = 0, top = 0;
+  uint32_t kept = 0, loops = 0, top = 0, low = 0;
   for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
-    const uint32_t s = rank[src[e]], t = rank[dst[e]];
-    const bool in = s < n_nodes && t < n_nodes;
+    const uint32_t s = rank[src[e]];
+    const bool in = s < n_nodes && rank[dst[e]] < n_nodes;
     key[e] = in ? s : n_nodes;
     edge[e] = e;
     kept += in;
     loops += src[e] == dst[e];
-    top = max(top, __float_as_uint(fabsf(w[e])));
+    const uint32_t t = __float_as_uint(fabsf(w[e]));
+    top = max(top, t);
+    if (t) low = max(low, ~t);
   }
-  kept = __reduce_add_sync(0xffffffffu, kept); loops = __reduce_add_sync(0xffffffffu, loops); top = __reduce_max_sync(0xffffffffu, top);
+  kept = __reduce_add_sync(0xffffffffu, kept); loops = __reduce_add_sync(0xffffffffu, loops); top = __reduce_max_sync(0xffffffffu, top); low = __reduce_max_sync(0xffffffffu, low);
   if (lane_id() == 0) {
     if (kept) atomicAdd(totals + kTrkEdges, (unsigned long long)kept);
     if (loops) atomicAdd(totals + kTrkLoops, (unsigned long long)loops);
     atomicMax(totals + kTrkAbsMax, (unsigned long long)top);
+    atomicMax(totals + kTrkAbsMin, (unsigned long long)low);
   }
 }
 static __global__ void __launch_bounds__(256) k_trk_keys(const uint32_t* __restrict__ edge, uint32_t n, const int32_t* __restrict__ col, const uint32_t* __restrict__ rank, uint32_t* __restrict__ key) {

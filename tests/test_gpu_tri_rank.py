@@ -94,3 +94,36 @@ def test_graphs_it_leaves_to_the_plain_kernels(why):
         (want,), _ = run(W.triangle_program(s[::2], d[::2], w[::2]), xlog.FLAG_NO_TRIANGLE_BITMAP)
         assert all(np.array_equal(x, y) for x, y in zip(half[0], want[0])) and np.allclose(half[1], want[1], rtol=0, atol=1e-5)
         ctx.close()
+
+
+@pytest.mark.parametrize("why", ["large", "small", "zeros", "edges of the range"])
+def test_sums_whose_products_could_leave_the_range(why):
+    """Sum-product tags of very different sizes: each corner meets its three factors in another order, and a partial product must not
+    overflow or lose bits below the smallest normal number.  The weights have one size per edge class of a tripartite graph, so
+    that a whole product is near 1 and every pair of factors is not; against 64 bits."""
+    from paper_2609_27203_b200 import xlog
+    k, r = 300, np.random.default_rng(4)
+    big = {"large": 2.5e19, "small": 6e-20, "zeros": 1e12, "edges of the range": 2.0 ** 41}[why]
+    size = [big, big, 1 / big / big] if why in ("large", "small") else [big, 1 / big, 1.0]
+    s, d, w = [], [], []
+    for part in range(3):                                     # part -> the next part, about half of the pairs
+        a, b = np.nonzero(r.random((k, k)) < 0.55)
+        s.append(a + part * k)
+        d.append(b + (part + 1) % 3 * k)
+        w.append((size[part] * r.uniform(0.5, 0.999, len(a))).astype(np.float32))
+    s, d, w = np.concatenate(s), np.concatenate(d), np.concatenate(w)
+    if why == "zeros":
+        w[::7] = 0.0
+    assert len(s) >= 1 << 17
+    (got,), ran = run(sum_program(s.astype(np.int32), d.astype(np.int32), w))
+    assert ran == (why in ("zeros", "edges of the range"))
+    m = np.zeros((3 * k, 3 * k))
+    there = np.zeros((3 * k, 3 * k))
+    m[s, d], there[s, d] = w, 1
+    want, cnt = ((m @ m) * m.T).sum(1), ((there @ there) * there.T).sum(1)
+    assert np.array_equal(got[0][0], np.arange(3 * k)) and np.array_equal(got[0][1], cnt.astype(np.int32))
+    if ran:
+        assert np.allclose(got[1], want, rtol=1e-6, atol=0)
+    else:                                                     # the plain kernels: the order of an edge list's own corner
+        plain, _ = run(sum_program(s.astype(np.int32), d.astype(np.int32), w), xlog.FLAG_NO_TRIANGLE_BITMAP)
+        assert np.array_equal(got[1].view(np.int32), plain[0][1].view(np.int32))
