@@ -80,9 +80,9 @@ struct Index {                          // sorted access path on one column of a
 };
 
 // Degree-ordered copy of a binary relation for the triangle aggregate (tri_rank.cuh): rank of every node, lists of both
-// orientations, work units of both launches.  Made when first wanted, dropped with the join indices.
+// orientations, work units of both launches.  Made when it pays, dropped with the join indices.
 struct TriRankIndex {
-  bool tried = false, valid = false;      // tried and not valid: the relation does not lend itself to it
+  bool checked = false, fit = false, valid = false;      // fit: the relation lends itself to it
   uint32_t n_nodes = 0, n_edges = 0, n_units[2] = {0, 0};
   uint64_t walk = 0;
   DevBuf rank, off[2], split[2], nbr[2], num[2], other, unit_off[2], unit[2];      // [0] out-lists, [1] in-lists; units of the launch by a, by b

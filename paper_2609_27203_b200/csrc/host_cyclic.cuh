@@ -66,14 +66,37 @@ TriRankPass tri_rank_pass(const TriRankIndex& X, int p) {
   return P;
 }
 
+// Does E lend itself to the order, and does making it pay (tri_rank.cuh)?  One read of the edges and of the offsets and one
+// control read, before anything is sorted: a graph that is turned away has not paid for half of the order.
+void check_tri_rank(Ctx* c, Relation& E, Index& out_ix, Index& in_ix, bool lse) {
+  TriRankIndex& X = E.tri;
+  X.checked = true;
+  const int64_t nodes = std::max(out_ix.domain, in_ix.domain);
+  if (E.n < kTriRankMinEdges || nodes > kTriRankMaxNodes) return;
+  unsigned long long* tot = (unsigned long long*)(c->d_ctrl + kSlotTrk);
+  zero_ctrl(c, kSlotTrk, kTrkTotals);
+  XLOG_LAUNCH(c, k_trk_corners, grid_for(nodes, 256), 256, 0, out_ix.off.as<uint32_t>(), out_ix.domain, in_ix.off.as<uint32_t>(), in_ix.domain, (uint32_t)nodes, tot);
+  XLOG_LAUNCH(c, k_trk_check, grid_for(E.n, 256), 256, 0, E.cols[0].as<int32_t>(), E.cols[1].as<int32_t>(), (const float*)E.tags(), E.n, out_ix.off.as<uint32_t>(), out_ix.domain,
+              in_ix.off.as<uint32_t>(), in_ix.domain, tot);
+  sync_ctrl(c);
+  const uint64_t* t = c->h_ctrl + kSlotTrk;
+  float top, low;
+  { const uint32_t u = (uint32_t)t[kTrkAbsMax], v = ~(uint32_t)t[kTrkAbsMin]; memcpy(&top, &u, 4); memcpy(&low, &v, 4); }
+  const bool in_range = lse ? top <= kTriRankMaxTag : top <= kTriRankMaxNum && (top == 0.f || low >= kTriRankMinNum);      // false for NaN
+  X.n_edges = (uint32_t)t[kTrkEdges];
+  X.n_nodes = (uint32_t)t[kTrkNodes];
+  const uint64_t walk = t[kTrkPlain], m = E.n;
+  const bool pays = walk >= kTriRankPerEdge * m || walk + 5 * m >= kTriRankEntries || t[kTrkLongest] >= kTriRankHub;
+  X.fit = !t[kTrkLoops] && in_range && X.n_edges && pays;
+}
+
 // The ordered copy of E, made at the first call.  False: not for this relation.
 bool ensure_tri_rank(Ctx* c, Relation& E, Index& out_ix, Index& in_ix, bool lse) {
   TriRankIndex& X = E.tri;
-  if (X.tried) return X.valid;
-  X.tried = true;
-  const int64_t nodes = std::max(out_ix.domain, in_ix.domain);
-  if (E.n < kTriRankMinEdges || nodes > kTriRankMaxNodes) return false;
-  const uint32_t N = (uint32_t)nodes, m = E.n;
+  if (X.valid) return true;
+  if (!X.checked) check_tri_rank(c, E, out_ix, in_ix, lse);
+  if (!X.fit) return false;
+  const uint32_t N = (uint32_t)std::max(out_ix.domain, in_ix.domain), m = E.n;
   if ((size_t)m * 64 + (size_t)N * 64 + (4u << 20) > c->arena.largest_free() / 2) return false;
   const int32_t* src = E.cols[0].as<int32_t>(); const int32_t* dst = E.cols[1].as<int32_t>();
   unsigned long long* tot = (unsigned long long*)(c->d_ctrl + kSlotTrk);
@@ -81,27 +104,20 @@ bool ensure_tri_rank(Ctx* c, Relation& E, Index& out_ix, Index& in_ix, bool lse)
   X.rank = DevBuf(c, (size_t)N * 4);
   {
     DevBuf k0(c, (size_t)N * 4), v0(c, (size_t)N * 4), k1(c, (size_t)N * 4), v1(c, (size_t)N * 4);
-    XLOG_LAUNCH(c, k_trk_degrees, grid_for(N, 256), 256, 0, out_ix.off.as<uint32_t>(), out_ix.domain, in_ix.off.as<uint32_t>(), in_ix.domain, N, k0.as<uint32_t>(), v0.as<uint32_t>(), tot);
+    XLOG_LAUNCH(c, k_trk_degrees, grid_for(N, 256), 256, 0, out_ix.off.as<uint32_t>(), out_ix.domain, in_ix.off.as<uint32_t>(), in_ix.domain, N, k0.as<uint32_t>(), v0.as<uint32_t>());
     uint32_t* ka = k0.as<uint32_t>(); uint32_t* kb = k1.as<uint32_t>();
     float* va = v0.as<float>(); float* vb = v1.as<float>();
     sort_pairs<uint32_t>(c, ka, va, kb, vb, N, bit_length(2 * (int64_t)m));
-    XLOG_LAUNCH(c, k_trk_ranks, grid_for(N, 256), 256, 0, (const uint32_t*)va, N, (const unsigned long long*)tot, X.rank.as<uint32_t>());
+    XLOG_LAUNCH(c, k_trk_ranks, grid_for(N, 256), 256, 0, (const uint32_t*)va, N, X.n_nodes, X.rank.as<uint32_t>());
   }
   const uint32_t* rank = X.rank.as<uint32_t>();
   // the edges between corners ordered by (target, source), then by (source, target): stable sorts by one rank at a time
   DevBuf k0(c, (size_t)m * 4), v0(c, (size_t)m * 4), k1(c, (size_t)m * 4), v1(c, (size_t)m * 4);
   uint32_t* ka = k0.as<uint32_t>(); uint32_t* kb = k1.as<uint32_t>();
   float* va = v0.as<float>(); float* vb = v1.as<float>();
-  XLOG_LAUNCH(c, k_trk_edges, grid_for(m, 256), 256, 0, src, dst, (const float*)E.tags(), m, rank, N, ka, reinterpret_cast<uint32_t*>(va), tot);
+  XLOG_LAUNCH(c, k_trk_edges, grid_for(m, 256), 256, 0, src, dst, m, rank, N, ka, reinterpret_cast<uint32_t*>(va));
   const int bits = bit_length(N);
   sort_pairs<uint32_t>(c, ka, va, kb, vb, m, bits);
-  sync_ctrl(c);
-  float top, low;
-  { const uint32_t u = (uint32_t)c->h_ctrl[kSlotTrk + kTrkAbsMax], v = ~(uint32_t)c->h_ctrl[kSlotTrk + kTrkAbsMin]; memcpy(&top, &u, 4); memcpy(&low, &v, 4); }
-  const bool in_range = lse ? top <= kTriRankMaxTag : top <= kTriRankMaxNum && (top == 0.f || low >= kTriRankMinNum);      // false for NaN
-  X.n_edges = (uint32_t)c->h_ctrl[kSlotTrk + kTrkEdges];
-  X.n_nodes = (uint32_t)c->h_ctrl[kSlotTrk + kTrkNodes];
-  if (c->h_ctrl[kSlotTrk + kTrkLoops] || !in_range || X.n_edges == 0) { X = TriRankIndex(); X.tried = true; return false; }
   const uint32_t me = X.n_edges, P = X.n_nodes;
   DevBuf place(c, (size_t)m * 4);
   for (int o = 1; o >= 0; --o) {

@@ -26,6 +26,14 @@ namespace xlog {
 
 constexpr int64_t kTriRankMaxNodes = (int64_t)1 << 19;       // 128 KB of bitmap and places
 constexpr uint32_t kTriRankMinEdges = 1u << 17;  // below, the plain kernels are as fast and need no second copy of the graph
+// Ordering a graph costs 0.25 ms and 0.16 ms per million edges once; it is ordered where that is back by the second evaluation.
+// Which way a graph goes depends on the graph alone, so that its results repeat bit for bit.  Entries to walk: per edge the
+// shorter of the two lists that the plain kernels meet.  First / later evaluation, ms, plain and ordered:
+//   R-MAT 15, 0.16 M edges, 33 entries an edge   0.46 / 0.37 and 0.53 / 0.16     16, 0.96 M, 106   1.50 / 1.38 and 0.89 / 0.32
+//   even, 2,000 nodes, 0.20 M edges, 92 an edge  0.40 / 0.32 and 0.49 / 0.15     60,000 nodes, 1.0 M, 14   0.54 / 0.42 and 0.68 / 0.16
+// and, below the line, even, 100,000 nodes, 0.14 M, 0.8   0.28 / 0.18 and 0.53 / 0.11     250,000 nodes, 1.0 M, 3   0.56 / 0.41 and 0.87 / 0.26
+constexpr uint64_t kTriRankPerEdge = 32, kTriRankEntries = 10000000;      // entries per edge; entries and five times the edges
+constexpr uint32_t kTriRankHub = 1u << 15;       // a list so long that few of the corners it belongs to are lower
 constexpr float kTriRankMaxTag = 28.f;           // exp(3 * 28) and exp(-3 * 28) are normal fp32 numbers
 constexpr float kTriRankMaxNum = 0x1p42f, kTriRankMinNum = 0x1p-42f;      // as are 2^126 and 2^-126
 constexpr int kTriRankBlock = 512;
@@ -35,7 +43,7 @@ constexpr uint32_t kTriRankSmall = 512;
 constexpr int kTriRankSweeps = 2;                // sweeps of 32 list entries a warp reads before it tests them (both launches, us: 1 907, 2 878, 3 909, 4 962)
 
 enum { kTrkEdges = 0, kTrkNodes = 1, kTrkLoops = 2, kTrkAbsMax = 3, kTrkUnitsA = 4, kTrkUnitsB = 5, kTrkWalkA = 6, kTrkWalkB = 7,
-       kTrkAbsMin = 8, kTrkTotals = 9 };        // kTrkAbsMin: complement of the smallest |tag| that is not zero (0: none)
+       kTrkAbsMin = 8, kTrkPlain = 9, kTrkLongest = 10, kTrkTotals = 11 };      // kTrkAbsMin: complement of the smallest |tag| that is not zero (0: none)
 
 // One orientation of the ordered graph: lists of neighbours in ascending rank; entries [off[v], split[v]) rank lower than v.
 struct TriRankLists {
@@ -46,46 +54,73 @@ struct TriRankLists {
   const uint32_t* other;             // the place of the same edge in the other orientation's lists (may be null)
 };
 
-// degree of every node that can be a corner (edges in and out), else 0; loops among the edges, largest |tag|
-static __global__ void __launch_bounds__(256) k_trk_degrees(const uint32_t* __restrict__ out_off, int64_t out_domain, const uint32_t* __restrict__ in_off, int64_t in_domain,
-                                                            uint32_t n_nodes, uint32_t* __restrict__ deg, uint32_t* __restrict__ node, unsigned long long* __restrict__ totals) {
-  uint32_t corners = 0;
+// number of corners (nodes with edges in and out), longest list
+static __global__ void __launch_bounds__(256) k_trk_corners(const uint32_t* __restrict__ out_off, int64_t out_domain, const uint32_t* __restrict__ in_off, int64_t in_domain,
+                                                            uint32_t n_nodes, unsigned long long* __restrict__ totals) {
+  uint32_t corners = 0, longest = 0;
   for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n_nodes; v += gridDim.x * blockDim.x) {
     const uint32_t o = v < out_domain ? out_off[v + 1] - out_off[v] : 0u, i = v < in_domain ? in_off[v + 1] - in_off[v] : 0u;
-    const uint32_t d = o && i ? o + i : 0u;
-    deg[v] = d; node[v] = v;
-    corners += d != 0u;
+    corners += o && i;
+    longest = max(longest, max(o, i));
   }
-  corners = __reduce_add_sync(0xffffffffu, corners);
-  if (lane_id() == 0 && corners) atomicAdd(totals + kTrkNodes, (unsigned long long)corners);
+  corners = __reduce_add_sync(0xffffffffu, corners); longest = __reduce_max_sync(0xffffffffu, longest);
+  if (lane_id() == 0) { if (corners) atomicAdd(totals + kTrkNodes, (unsigned long long)corners); atomicMax(totals + kTrkLongest, (unsigned long long)longest); }
+}
+// degree of every corner, of the other nodes 0
+static __global__ void __launch_bounds__(256) k_trk_degrees(const uint32_t* __restrict__ out_off, int64_t out_domain, const uint32_t* __restrict__ in_off, int64_t in_domain,
+                                                            uint32_t n_nodes, uint32_t* __restrict__ deg, uint32_t* __restrict__ node) {
+  for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n_nodes; v += gridDim.x * blockDim.x) {
+    const uint32_t o = v < out_domain ? out_off[v + 1] - out_off[v] : 0u, i = v < in_domain ? in_off[v + 1] - in_off[v] : 0u;
+    deg[v] = o && i ? o + i : 0u;
+    node[v] = v;
+  }
 }
 // rank of every node among the corners, in order of degree (node: the nodes sorted by degree); the others get n_nodes
-static __global__ void __launch_bounds__(256) k_trk_ranks(const uint32_t* __restrict__ node, uint32_t n_nodes, const unsigned long long* __restrict__ totals, uint32_t* __restrict__ rank) {
-  const uint32_t skip = n_nodes - (uint32_t)totals[kTrkNodes];
+static __global__ void __launch_bounds__(256) k_trk_ranks(const uint32_t* __restrict__ node, uint32_t n_nodes, uint32_t corners, uint32_t* __restrict__ rank) {
+  const uint32_t skip = n_nodes - corners;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_nodes; i += gridDim.x * blockDim.x) rank[node[i]] = i >= skip ? i - skip : n_nodes;
 }
-// the edges between corners first: key = rank of the source, of the others n_nodes
-static __global__ void __launch_bounds__(256) k_trk_edges(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, const float* __restrict__ w, uint32_t n,
-                                                          const uint32_t* __restrict__ rank, uint32_t n_nodes, uint32_t* __restrict__ key, uint32_t* __restrict__ edge,
+// What decides whether the graph is ordered, in one read of its edges: edges between corners, loops, the range of |tag|, and the
+// entries that the plain kernels would walk (per edge the shorter of the two lists that are met).
+static __global__ void __launch_bounds__(256) k_trk_check(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, const float* __restrict__ w, uint32_t n,
+                                                          const uint32_t* __restrict__ out_off, int64_t out_domain, const uint32_t* __restrict__ in_off, int64_t in_domain,
                                                           unsigned long long* __restrict__ totals) {
+  __shared__ unsigned long long s_walk;
+  __shared__ uint32_t s_kept, s_loops, s_top, s_low;
+  if (threadIdx.x == 0) { s_walk = 0; s_kept = s_loops = s_top = s_low = 0; }
+  __syncthreads();
   uint32_t kept = 0, loops = 0, top = 0, low = 0;
+  unsigned long long walk = 0;
   for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
-    const uint32_t s = rank[src[e]];
-    const bool in = s < n_nodes && rank[dst[e]] < n_nodes;
-    key[e] = in ? s : n_nodes;
-    edge[e] = e;
-    kept += in;
-    loops += src[e] == dst[e];
+    const int32_t s = src[e], d = dst[e];
+    const uint32_t si = s < in_domain ? in_off[s + 1] - in_off[s] : 0u, dn = d < out_domain ? out_off[d + 1] - out_off[d] : 0u;
+    kept += si && dn;                               // the source has edges out, the target has edges in: this one
+    walk += min(si, dn);
+    loops += s == d;
     const uint32_t t = __float_as_uint(fabsf(w[e]));
     top = max(top, t);
     if (t) low = max(low, ~t);
   }
   kept = __reduce_add_sync(0xffffffffu, kept); loops = __reduce_add_sync(0xffffffffu, loops); top = __reduce_max_sync(0xffffffffu, top); low = __reduce_max_sync(0xffffffffu, low);
-  if (lane_id() == 0) {
-    if (kept) atomicAdd(totals + kTrkEdges, (unsigned long long)kept);
-    if (loops) atomicAdd(totals + kTrkLoops, (unsigned long long)loops);
-    atomicMax(totals + kTrkAbsMax, (unsigned long long)top);
-    atomicMax(totals + kTrkAbsMin, (unsigned long long)low);
+#pragma unroll
+  for (int d = 16; d; d >>= 1) walk += __shfl_xor_sync(0xffffffffu, walk, d);
+  if (lane_id() == 0) { atomicAdd(&s_walk, walk); atomicAdd(&s_kept, kept); atomicAdd(&s_loops, loops); atomicMax(&s_top, top); atomicMax(&s_low, low); }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    atomicAdd(totals + kTrkEdges, (unsigned long long)s_kept);
+    if (s_loops) atomicAdd(totals + kTrkLoops, (unsigned long long)s_loops);
+    atomicAdd(totals + kTrkPlain, s_walk);
+    atomicMax(totals + kTrkAbsMax, (unsigned long long)s_top);
+    atomicMax(totals + kTrkAbsMin, (unsigned long long)s_low);
+  }
+}
+// the edges between corners first: key = rank of the source, of the others n_nodes
+static __global__ void __launch_bounds__(256) k_trk_edges(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, uint32_t n,
+                                                          const uint32_t* __restrict__ rank, uint32_t n_nodes, uint32_t* __restrict__ key, uint32_t* __restrict__ edge) {
+  for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+    const uint32_t s = rank[src[e]];
+    key[e] = s < n_nodes && rank[dst[e]] < n_nodes ? s : n_nodes;
+    edge[e] = e;
   }
 }
 static __global__ void __launch_bounds__(256) k_trk_keys(const uint32_t* __restrict__ edge, uint32_t n, const int32_t* __restrict__ col, const uint32_t* __restrict__ rank, uint32_t* __restrict__ key) {

@@ -127,3 +127,46 @@ def test_sums_whose_products_could_leave_the_range(why):
     else:                                                     # the plain kernels: the order of an edge list's own corner
         plain, _ = run(sum_program(s.astype(np.int32), d.astype(np.int32), w), xlog.FLAG_NO_TRIANGLE_BITMAP)
         assert np.array_equal(got[1].view(np.int32), plain[0][1].view(np.int32))
+
+
+def launches(prog, evaluations, reload=False):
+    """Kernel names of every evaluation of one context, the graph loaded again before each if `reload`."""
+    from paper_2609_27203_b200 import xlog
+    ctx, ids, _ = xlog.load_program(prog, arena_bytes=1 << 30, flags=xlog.FLAG_PROFILE)
+    out = []
+    for _ in range(evaluations):
+        if reload:
+            ctx.load(ids["e"], *prog.facts["e"])
+        ctx.reset_idb()
+        ctx.profile_reset()
+        ctx.fixpoint()
+        out.append((set(ctx.profile()), ctx.read(ids["tri_agg"])))
+    ctx.close()
+    return out
+
+
+@pytest.mark.parametrize("why", ["loop", "tag"])
+def test_a_graph_that_is_turned_away_pays_for_no_part_of_the_order(why):
+    s, d, w = synth.rmat_graph(13, 30, 9, "n01")
+    if why == "loop":
+        s, d, w = np.append(s, 5).astype(np.int32), np.append(d, 5).astype(np.int32), np.append(w, np.float32(1))
+    else:
+        w[100] = -28.5
+    for ran, _ in launches(W.triangle_program(s, d, w), 3, reload=True):
+        assert "k_trk_check" in ran and not ran & {"k_trk_degrees", "k_trk_edges", "k_tri_rank", "k_tri_rank_small"}
+
+
+@pytest.mark.parametrize("n,m,ordered", [(100000, 140000, False), (4000, 180000, True), (60000, 1000000, True), (250000, 1000000, False), (250000, 1700000, True)])
+def test_graphs_on_both_sides_of_the_line(n, m, ordered):
+    """Edges spread evenly: few entries to walk, more than 32 an edge, many in all, and many edges; every evaluation of a graph goes
+    the same way and gives the same bits."""
+    r = np.random.default_rng(n)
+    key = np.unique(r.integers(0, n * n, m))
+    s, d = (key // n).astype(np.int32), (key % n).astype(np.int32)
+    s, d = s[s != d], d[s != d]
+    prog = W.triangle_program(s, d, r.standard_normal(len(s)).astype(np.float32))
+    got = launches(prog, 3) + launches(prog, 2, reload=True)
+    assert ["k_tri_rank_small" in ran for ran, _ in got] == [ordered] * 5
+    assert ["k_trk_check" in ran for ran, _ in got] == [True, False, False, True, True]
+    for _, (cols, tags) in got[1:]:
+        assert all(np.array_equal(x, y) for x, y in zip(cols, got[0][1][0])) and np.array_equal(tags.view(np.int32), got[0][1][1].view(np.int32))
