@@ -75,9 +75,8 @@ void check_tri_rank(Ctx* c, Relation& E, Index& out_ix, Index& in_ix, bool lse) 
   if (E.n < kTriRankMinEdges || nodes > kTriRankMaxNodes) return;
   unsigned long long* tot = (unsigned long long*)(c->d_ctrl + kSlotTrk);
   zero_ctrl(c, kSlotTrk, kTrkTotals);
-  XLOG_LAUNCH(c, k_trk_corners, grid_for(nodes, 256), 256, 0, out_ix.off.as<uint32_t>(), out_ix.domain, in_ix.off.as<uint32_t>(), in_ix.domain, (uint32_t)nodes, tot);
   XLOG_LAUNCH(c, k_trk_check, grid_for(E.n, 256), 256, 0, E.cols[0].as<int32_t>(), E.cols[1].as<int32_t>(), (const float*)E.tags(), E.n, out_ix.off.as<uint32_t>(), out_ix.domain,
-              in_ix.off.as<uint32_t>(), in_ix.domain, tot);
+              in_ix.off.as<uint32_t>(), in_ix.domain, (uint32_t)nodes, tot);
   sync_ctrl(c);
   const uint64_t* t = c->h_ctrl + kSlotTrk;
   float top, low;
@@ -136,13 +135,17 @@ bool ensure_tri_rank(Ctx* c, Relation& E, Index& out_ix, Index& in_ix, bool lse)
               X.num[o].as<float>(), o == 0 ? place.as<uint32_t>() : nullptr)
     if (lse) XLOG_TRK_LISTS(true); else XLOG_TRK_LISTS(false);
 #undef XLOG_TRK_LISTS
-    XLOG_LAUNCH(c, k_trk_splits, grid_for(P, 256), 256, 0, (const uint32_t*)X.off[o].as<uint32_t>(), (const uint32_t*)X.nbr[o].as<uint32_t>(), P, X.split[o].as<uint32_t>());
   }
   XLOG_LAUNCH(c, k_trk_gather, grid_for(me, 256), 256, 0, (const uint32_t*)X.other.as<uint32_t>(), me, (const uint32_t*)place.as<uint32_t>(), X.other.as<uint32_t>());
-  DevBuf units(c, ((size_t)P + 1) * 4);
+  XLOG_LAUNCH(c, k_trk_splits, grid_for((uint64_t)P * 2, 256), 256, 0, (const uint32_t*)X.off[0].as<uint32_t>(), (const uint32_t*)X.nbr[0].as<uint32_t>(), X.split[0].as<uint32_t>(),
+              (const uint32_t*)X.off[1].as<uint32_t>(), (const uint32_t*)X.nbr[1].as<uint32_t>(), X.split[1].as<uint32_t>(), P);
+  DevBuf units(c, ((size_t)P + 1) * 4), work(c, (size_t)P * 8);
+  XLOG_CUDA(cudaMemsetAsync(work.p, 0, (size_t)P * 8, c->stream));
   for (int p = 0; p < 2; ++p) {
     X.unit_off[p] = DevBuf(c, ((size_t)P + 1) * 4);
-    XLOG_LAUNCH(c, k_trk_units, grid_for((uint64_t)P * 32, 256), 256, 0, tri_rank_lists(X, 1 - p), tri_rank_lists(X, p), P, units.as<uint32_t>(), tot + kTrkWalkA + p);
+    uint32_t* const w = work.as<uint32_t>() + (size_t)p * P;
+    XLOG_LAUNCH(c, k_trk_work, grid_for((uint64_t)P * 8, 256), 256, 0, tri_rank_lists(X, 1 - p), tri_rank_lists(X, p), P, w);
+    XLOG_LAUNCH(c, k_trk_units, grid_for((uint64_t)P + 1, 256), 256, 0, tri_rank_lists(X, 1 - p), tri_rank_lists(X, p), P, (const uint32_t*)w, units.as<uint32_t>(), tot + kTrkWalkA + p);
     exclusive_scan_u32(c, units.as<uint32_t>(), (int64_t)P + 1, X.unit_off[p].as<uint32_t>(), ctrl_u32(c, kSlotTrk + kTrkUnitsA + p));
   }
   sync_ctrl(c);

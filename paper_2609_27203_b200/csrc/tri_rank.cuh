@@ -33,7 +33,7 @@ constexpr uint32_t kTriRankMinEdges = 1u << 17;  // below, the plain kernels are
 //   even, 2,000 nodes, 0.20 M edges, 92 an edge  0.40 / 0.32 and 0.49 / 0.15     60,000 nodes, 1.0 M, 14   0.54 / 0.42 and 0.68 / 0.16
 // and, below the line, even, 100,000 nodes, 0.14 M, 0.8   0.28 / 0.18 and 0.53 / 0.11     250,000 nodes, 1.0 M, 3   0.56 / 0.41 and 0.87 / 0.26
 constexpr uint64_t kTriRankPerEdge = 32, kTriRankEntries = 10000000;      // entries per edge; entries and five times the edges
-constexpr uint32_t kTriRankHub = 1u << 15;       // a list so long that few of the corners it belongs to are lower
+constexpr uint32_t kTriRankHub = 1u << 15;       // a list that the plain kernels are slow with: wheel of 70,000 nodes 1.17 / 1.08 and 0.89 / 0.34
 constexpr float kTriRankMaxTag = 28.f;           // exp(3 * 28) and exp(-3 * 28) are normal fp32 numbers
 constexpr float kTriRankMaxNum = 0x1p42f, kTriRankMinNum = 0x1p-42f;      // as are 2^126 and 2^-126
 constexpr int kTriRankBlock = 512;
@@ -54,18 +54,6 @@ struct TriRankLists {
   const uint32_t* other;             // the place of the same edge in the other orientation's lists (may be null)
 };
 
-// number of corners (nodes with edges in and out), longest list
-static __global__ void __launch_bounds__(256) k_trk_corners(const uint32_t* __restrict__ out_off, int64_t out_domain, const uint32_t* __restrict__ in_off, int64_t in_domain,
-                                                            uint32_t n_nodes, unsigned long long* __restrict__ totals) {
-  uint32_t corners = 0, longest = 0;
-  for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n_nodes; v += gridDim.x * blockDim.x) {
-    const uint32_t o = v < out_domain ? out_off[v + 1] - out_off[v] : 0u, i = v < in_domain ? in_off[v + 1] - in_off[v] : 0u;
-    corners += o && i;
-    longest = max(longest, max(o, i));
-  }
-  corners = __reduce_add_sync(0xffffffffu, corners); longest = __reduce_max_sync(0xffffffffu, longest);
-  if (lane_id() == 0) { if (corners) atomicAdd(totals + kTrkNodes, (unsigned long long)corners); atomicMax(totals + kTrkLongest, (unsigned long long)longest); }
-}
 // degree of every corner, of the other nodes 0
 static __global__ void __launch_bounds__(256) k_trk_degrees(const uint32_t* __restrict__ out_off, int64_t out_domain, const uint32_t* __restrict__ in_off, int64_t in_domain,
                                                             uint32_t n_nodes, uint32_t* __restrict__ deg, uint32_t* __restrict__ node) {
@@ -80,16 +68,22 @@ static __global__ void __launch_bounds__(256) k_trk_ranks(const uint32_t* __rest
   const uint32_t skip = n_nodes - corners;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_nodes; i += gridDim.x * blockDim.x) rank[node[i]] = i >= skip ? i - skip : n_nodes;
 }
-// What decides whether the graph is ordered, in one read of its edges: edges between corners, loops, the range of |tag|, and the
-// entries that the plain kernels would walk (per edge the shorter of the two lists that are met).
+// What decides whether the graph is ordered, in one read of its nodes and edges: corners (nodes with edges in and out), longest
+// list, edges between corners, loops, the range of |tag|, and the entries that the plain kernels would walk (per edge the shorter
+// of the two lists that are met).
 static __global__ void __launch_bounds__(256) k_trk_check(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, const float* __restrict__ w, uint32_t n,
                                                           const uint32_t* __restrict__ out_off, int64_t out_domain, const uint32_t* __restrict__ in_off, int64_t in_domain,
-                                                          unsigned long long* __restrict__ totals) {
+                                                          uint32_t n_nodes, unsigned long long* __restrict__ totals) {
   __shared__ unsigned long long s_walk;
-  __shared__ uint32_t s_kept, s_loops, s_top, s_low;
-  if (threadIdx.x == 0) { s_walk = 0; s_kept = s_loops = s_top = s_low = 0; }
+  __shared__ uint32_t s_kept, s_loops, s_top, s_low, s_corners, s_longest;
+  if (threadIdx.x == 0) { s_walk = 0; s_kept = s_loops = s_top = s_low = s_corners = s_longest = 0; }
   __syncthreads();
-  uint32_t kept = 0, loops = 0, top = 0, low = 0;
+  uint32_t kept = 0, loops = 0, top = 0, low = 0, corners = 0, longest = 0;
+  for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n_nodes; v += gridDim.x * blockDim.x) {
+    const uint32_t o = v < out_domain ? out_off[v + 1] - out_off[v] : 0u, i = v < in_domain ? in_off[v + 1] - in_off[v] : 0u;
+    corners += o && i;
+    longest = max(longest, max(o, i));
+  }
   unsigned long long walk = 0;
   for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
     const int32_t s = src[e], d = dst[e];
@@ -102,9 +96,10 @@ static __global__ void __launch_bounds__(256) k_trk_check(const int32_t* __restr
     if (t) low = max(low, ~t);
   }
   kept = __reduce_add_sync(0xffffffffu, kept); loops = __reduce_add_sync(0xffffffffu, loops); top = __reduce_max_sync(0xffffffffu, top); low = __reduce_max_sync(0xffffffffu, low);
+  corners = __reduce_add_sync(0xffffffffu, corners); longest = __reduce_max_sync(0xffffffffu, longest);
 #pragma unroll
   for (int d = 16; d; d >>= 1) walk += __shfl_xor_sync(0xffffffffu, walk, d);
-  if (lane_id() == 0) { atomicAdd(&s_walk, walk); atomicAdd(&s_kept, kept); atomicAdd(&s_loops, loops); atomicMax(&s_top, top); atomicMax(&s_low, low); }
+  if (lane_id() == 0) { atomicAdd(&s_walk, walk); atomicAdd(&s_kept, kept); atomicAdd(&s_loops, loops); atomicMax(&s_top, top); atomicMax(&s_low, low); atomicAdd(&s_corners, corners); atomicMax(&s_longest, longest); }
   __syncthreads();
   if (threadIdx.x == 0) {
     atomicAdd(totals + kTrkEdges, (unsigned long long)s_kept);
@@ -112,6 +107,8 @@ static __global__ void __launch_bounds__(256) k_trk_check(const int32_t* __restr
     atomicAdd(totals + kTrkPlain, s_walk);
     atomicMax(totals + kTrkAbsMax, (unsigned long long)s_top);
     atomicMax(totals + kTrkAbsMin, (unsigned long long)s_low);
+    if (s_corners) atomicAdd(totals + kTrkNodes, (unsigned long long)s_corners);
+    atomicMax(totals + kTrkLongest, (unsigned long long)s_longest);
   }
 }
 // the edges between corners first: key = rank of the source, of the others n_nodes
@@ -140,31 +137,55 @@ __global__ void __launch_bounds__(256) k_trk_lists(const uint32_t* __restrict__ 
 static __global__ void __launch_bounds__(256) k_trk_gather(const uint32_t* __restrict__ edge, uint32_t n, const uint32_t* __restrict__ place, uint32_t* __restrict__ other) {
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) other[i] = place[edge[i]];
 }
-static __global__ void __launch_bounds__(256) k_trk_splits(const uint32_t* __restrict__ off, const uint32_t* __restrict__ nbr, uint32_t n_nodes, uint32_t* __restrict__ split) {
-  for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n_nodes; v += gridDim.x * blockDim.x) {
+// first entry that ranks higher than v in each of v's two lists
+static __global__ void __launch_bounds__(256) k_trk_splits(const uint32_t* __restrict__ off0, const uint32_t* __restrict__ nbr0, uint32_t* __restrict__ split0,
+                                                           const uint32_t* __restrict__ off1, const uint32_t* __restrict__ nbr1, uint32_t* __restrict__ split1, uint32_t n_nodes) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < 2 * n_nodes; i += gridDim.x * blockDim.x) {
+    const uint32_t v = i < n_nodes ? i : i - n_nodes;
+    const uint32_t* __restrict__ off = i < n_nodes ? off0 : off1;
+    const uint32_t* __restrict__ nbr = i < n_nodes ? nbr0 : nbr1;
     uint32_t lo = off[v], hi = off[v + 1];
     while (lo < hi) { const uint32_t mid = (lo + hi) >> 1; if (nbr[mid] < v) lo = mid + 1; else hi = mid; }
-    split[v] = lo;
+    (i < n_nodes ? split0 : split1)[v] = lo;
   }
 }
 
-// Items of a unit: enough that marking the corner's list (`marked` entries) is a small part of the unit's walk.
-__device__ __forceinline__ uint32_t trk_unit_items(uint32_t marked) { return max(256u, marked / 8u); }
+// Items of a unit: enough that marking the corner's list (`marked` entries) is a small part of the unit's walk; for a hub, whose
+// items are many and walk an entry or two each, enough units that the blocks of one corner fill the device (wheels of 70,000 and
+// 400,000 nodes, ms per evaluation, an eighth / a 64th of the list: 0.94 / 0.34 and 5.37 / 1.63; the plain kernels 1.08 and 5.48).
+__device__ __forceinline__ uint32_t trk_unit_items(uint32_t marked) { return marked >= kTriRankHub ? marked / 64u : max(256u, marked / 8u); }
 
-// A warp per corner: entries to walk in the lists of its lower neighbours in I; units of the bitmap kernel (0: searched).
-static __global__ void __launch_bounds__(256) k_trk_units(TriRankLists I, TriRankLists M, uint32_t n_nodes, uint32_t* __restrict__ units, unsigned long long* __restrict__ walk) {
-  const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-  unsigned long long sum = 0;
-  for (uint32_t a = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; a < n_nodes; a += nwarps) {
-    const uint32_t i0 = I.off[a], i1 = I.split[a];
-    uint32_t n = 0;
-    for (uint32_t i = i0 + lane_id(); i < i1; i += 32) { const uint32_t v = I.nbr[i]; n += I.off[v + 1] - I.split[v]; }
-    n = __reduce_add_sync(0xffffffffu, n);
-    if (lane_id() == 0) { const uint32_t per = trk_unit_items(M.off[a + 1] - M.off[a]); units[a] = n >= kTriRankSmall ? (i1 - i0 + per - 1) / per : 0u; }
-    sum += n;
+// Entries that every corner a walks in the lists of its lower neighbours, work[a] (zero on entry): each v adds the length of its
+// higher list in I to its higher neighbours in M, which are the corners that it is a lower neighbour of.  Eight lanes a v, whose
+// higher lists are short whatever the hubs; a warp a corner took 5 ms to go through the 400,000 neighbours of a wheel's hub.
+static __global__ void __launch_bounds__(256) k_trk_work(TriRankLists I, TriRankLists M, uint32_t n_nodes, uint32_t* __restrict__ work) {
+  const uint32_t sub = threadIdx.x % 8;
+  for (uint32_t v = (blockIdx.x * blockDim.x + threadIdx.x) / 8; v < n_nodes; v += gridDim.x * blockDim.x / 8) {
+    const uint32_t n = I.off[v + 1] - I.split[v], e1 = M.off[v + 1];
+    if (n) for (uint32_t i = M.split[v] + sub; i < e1; i += 8) atomicAdd(work + M.nbr[i], n);
   }
-  if (lane_id() == 0 && sum) atomicAdd(walk, sum);
-  if (blockIdx.x == 0 && threadIdx.x == 0) units[n_nodes] = 0u;
+}
+// units of the bitmap kernel (0: the corner is searched); *walk += all of work
+static __global__ void __launch_bounds__(256) k_trk_units(TriRankLists I, TriRankLists M, uint32_t n_nodes, const uint32_t* __restrict__ work, uint32_t* __restrict__ units,
+                                                          unsigned long long* __restrict__ walk) {
+  __shared__ unsigned long long s_sum;
+  if (threadIdx.x == 0) s_sum = 0;
+  __syncthreads();
+  unsigned long long sum = 0;
+  for (uint32_t a = blockIdx.x * blockDim.x + threadIdx.x; a <= n_nodes; a += gridDim.x * blockDim.x) {
+    uint32_t u = 0;
+    if (a < n_nodes) {
+      const uint32_t n = work[a], per = trk_unit_items(M.off[a + 1] - M.off[a]);
+      if (n >= kTriRankSmall) u = (I.split[a] - I.off[a] + per - 1) / per;
+      sum += n;
+    }
+    units[a] = u;
+  }
+#pragma unroll
+  for (int d = 16; d; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+  if (lane_id() == 0 && sum) atomicAdd(&s_sum, sum);
+  __syncthreads();
+  if (threadIdx.x == 0 && s_sum) atomicAdd(walk, s_sum);
 }
 static __global__ void __launch_bounds__(256) k_trk_unit_fill(TriRankLists I, TriRankLists M, uint32_t n_nodes, const uint32_t* __restrict__ unit_off, uint2* __restrict__ unit) {
   for (uint32_t a = blockIdx.x * blockDim.x + threadIdx.x; a < n_nodes; a += gridDim.x * blockDim.x) {

@@ -170,3 +170,20 @@ def test_graphs_on_both_sides_of_the_line(n, m, ordered):
     assert ["k_trk_check" in ran for ran, _ in got] == [True, False, False, True, True]
     for _, (cols, tags) in got[1:]:
         assert all(np.array_equal(x, y) for x, y in zip(cols, got[0][1][0])) and np.array_equal(tags.view(np.int32), got[0][1][1].view(np.int32))
+
+
+@pytest.mark.parametrize("n", [32767, 32768, 32770, 100003])
+@pytest.mark.parametrize("sums", [False, True])
+def test_hubs_in_many_units(n, sums):
+    """Two hubs joined both ways to the same ring: lists on both sides of the length from which a corner's units are cut finer."""
+    from paper_2609_27203_b200 import xlog
+    ring = np.arange(2, n + 2)
+    pairs = [(ring, np.roll(ring, -1)), (ring[::2], np.roll(ring, 3)[::2])] + [e for h in (0, 1) for e in ((0 * ring + h, ring), (ring, 0 * ring + h))]
+    s, d = (np.concatenate([p[i] for p in pairs]).astype(np.int32) for i in (0, 1))
+    w = np.random.default_rng(n).normal(size=len(s)).astype(np.float32)
+    prog = sum_program(s, d, np.exp(w * 0.1).astype(np.float32)) if sums else W.triangle_program(s, d, w)
+    (got, twice), ran = run(prog, again=2)
+    (want,), _ = run(prog, xlog.FLAG_NO_TRIANGLE_BITMAP)
+    assert ran == (n >= 32768)
+    assert all(np.array_equal(x, y) for x, y in zip(got[0], want[0])) and np.allclose(got[1], want[1], rtol=1e-6 if sums else 0, atol=0 if sums else 1e-5)
+    assert np.array_equal(got[1].view(np.int32), twice[1].view(np.int32))
