@@ -75,6 +75,7 @@ struct Index {                          // sorted access path on one column of a
   const float* tags = nullptr;
   DevBuf own_cols[kMaxArity - 1];       // owned storage when the index is a permuted copy
   DevBuf own_tags;
+  int64_t longest = -1;                 // rows of the longest run, when it has been looked for
   uint32_t bit_words = 0;               // > 0: the lists as bitmaps of that many words, with running counts (bits_join.cuh)
   DevBuf bits, bit_rank;
 };

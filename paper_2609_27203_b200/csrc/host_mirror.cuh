@@ -138,9 +138,27 @@ void resident_count(Ctx* c, Resident& R, const JoinSpec& S, size_t v) {
 }
 
 // Small rounds inside a thread-block cluster (res_cluster.cuh): one rule, in the linear-key form with one looked-up column, over
-// a key space whose mirror fits the shared memory of the cluster.
-bool res_cluster_applies(const std::vector<JoinSpec>& specs, int bits) {
-  return specs.size() == 1 && specs[0].fast && specs[0].has_inner && specs[0].inner_free == 1 && !specs[0].times && bits >= kRcMinBits && bits <= kRcMaxBits;
+// a key space whose mirror fits the shared memory of the cluster; and a looked-up relation whose runs are short, or that is so
+// small that no round is long.  Returns its longest run, 0: grid-wide rounds.
+// Shortest paths, us per query, grid-wide / in the cluster: a star of 131,000 leaves 124 / 292, R-MAT 15 with 0.4 M edges 181 / 392, a
+// complete graph of 2,000 nodes 202 / 429; random edges over 100,000 nodes, 8 a node 407 / 325, a grid of 90,601 nodes 9,575 /
+// 2,200.  Past kRcMaxBits a grid costs 16 us a round: 131,769 nodes 11,570, where 130,321 take 2,940.
+uint32_t res_cluster_longest(Ctx* c, int h, const std::vector<const RuleC*>& rs, const std::vector<JoinSpec>& specs, int bits) {
+  if (specs.size() != 1 || !specs[0].fast || !specs[0].has_inner || specs[0].inner_free != 1 || specs[0].times || bits < kRcMinBits || bits > kRcMaxBits) return 0;
+  for (const RuleC* r : rs)
+    for (int j = 0; j < r->plan.n_atoms; ++j) {
+      if (r->plan.atoms[j].rel != h) continue;
+      Relation& RB = *c->rels[r->plan.atoms[r->shape[j].inner].rel];
+      Index& ix = ensure_index(c, RB, r->shape[j].probe_col);
+      if (ix.longest < 0) {
+        zero_ctrl(c, kSlotA);
+        XLOG_LAUNCH(c, k_longest_run, grid_for(ix.domain, 256, kSMs * 4), 256, 0, (const uint32_t*)ix.off.as<uint32_t>(), ix.domain, ctrl_u32(c, kSlotA));
+        sync_ctrl(c);
+        ix.longest = (int64_t)(uint32_t)c->h_ctrl[kSlotA];
+      }
+      return ix.longest <= (int64_t)kRcMaxRun || RB.n <= kRcFewRows ? (uint32_t)std::max<int64_t>(ix.longest, 1) : 0u;
+    }
+  return 0;
 }
 // The largest key the columns' bounds allow ends the key space; whole bitmap words for every CTA.
 uint32_t res_cluster_slots(const Relation& H) {
@@ -167,16 +185,15 @@ void launch_res_cluster(Ctx* c, const JoinSpec& S, const ResCluster& P) {
 // One round's launches.  Nothing here allocates, copies or waits: the same calls are either captured into the WHILE
 // body or issued directly (host-driven rounds, used when launches are being timed one by one).
 void resident_body(Ctx* c, Resident& R, const std::vector<JoinSpec>& specs, const Relation& H, bool is_max, const MirrorArgs& mr, uint32_t bm_quads, unsigned ch_tiles,
-                   cudaGraphConditionalHandle handle, int use_handle) {
+                   uint32_t longest, cudaGraphConditionalHandle handle, int use_handle) {
   ResState* st = res_state(c);
   uint32_t* err = ctrl_u32(c, kSlotErr);
   const uint32_t* dk = R.dkeys.as<uint32_t>();
   const ResScratch sc{R.scan_status.as<unsigned long long>(), R.scan_tiles_cap, R.tickets.as<uint32_t>()};
   const bool fused = specs.size() == 1;                  // the count of the next round rides on the emit kernel; the first round's is launched before the loop
-  const int bits = H.layout.total_bits;
-  if (res_cluster_applies(specs, bits)) {
+  if (longest) {
     const uint32_t slots = res_cluster_slots(H);
-    const ResCluster P{slots, R.table.as<int32_t>(), R.bitmap.as<uint32_t>(), R.present.as<uint32_t>(), dk, R.dtags.as<float>(), st, mr.n_new, std::min(mr.key_max, slots - 1), err};
+    const ResCluster P{slots, R.table.as<int32_t>(), R.bitmap.as<uint32_t>(), R.present.as<uint32_t>(), dk, R.dtags.as<float>(), st, mr.n_new, std::min(mr.key_max, slots - 1), longest, err};
     if (is_max) launch_res_cluster<kSinkMax>(c, specs[0], P); else launch_res_cluster<kSinkMin>(c, specs[0], P);
   }
   for (size_t v = 0; v < specs.size(); ++v) {
@@ -223,10 +240,12 @@ ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*
   if (specs.size() > 16) fail(XLOG_ERR_UNSUPPORTED, "too many rule variants for one head");
   const uint32_t budget = (uint32_t)std::min<int64_t>(rounds_left, 0x7fffffff);
   const ResScratch sc{R.scan_status.as<unsigned long long>(), R.scan_tiles_cap, R.tickets.as<uint32_t>()};
+  const uint32_t longest = res_cluster_longest(c, h, rs, specs, H.layout.total_bits);
   XLOG_LAUNCH(c, k_res_init, 1, 1024, 0, res_state(c), sc, (uint32_t)specs.size(), n_delta, budget, R.max_tiles, (unsigned long long)new_seen);
   const MirrorArgs& mr = mr_host;
   const bool fused = specs.size() == 1;
-  const bool in_cluster = res_cluster_applies(specs, H.layout.total_bits) && n_delta > 0 && n_delta <= kRcMaxRows;      // the cluster kernel takes the first round and counts it itself
+  // where the rows alone bound the first round's candidates, the cluster kernel takes it and counts it itself
+  const bool in_cluster = longest && n_delta > 0 && n_delta <= kRcMaxRows && n_delta * (uint64_t)longest <= kRcMaxCand;
   if (fused && !in_cluster) resident_count(c, R, specs[0], 0);          // the first round's count; every later one rides on the emit kernel
   const int64_t l0 = c->launches;
   const bool use_graph = !(c->flags & (XLOG_FLAG_PROFILE | XLOG_FLAG_NO_GRAPH));
@@ -239,7 +258,8 @@ ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*
     std::vector<char> sig;
     for (const JoinSpec& S : specs) sig_add(sig, S);
     sig_add(sig, mr.table); sig_add(sig, mr.changed); sig_add(sig, mr.n_new); sig_add(sig, mr.key_max); sig_add(sig, mr.err); sig_add(sig, R.present.p);
-    if (res_cluster_applies(specs, H.layout.total_bits)) sig_add(sig, res_cluster_slots(H));
+    sig_add(sig, longest);
+    if (longest) sig_add(sig, res_cluster_slots(H));
     sig_add(sig, is_max); sig_add(sig, bm_quads); sig_add(sig, ch_tiles); sig_add(sig, c->d_ctrl); sig_add(sig, c->spin_limit);
     if (!R.exec || sig != R.sig) {
       if (R.exec) { cudaGraphExecDestroy(R.exec); R.exec = nullptr; }
@@ -263,7 +283,7 @@ ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*
       c->stream = c->capture_stream;
       const int64_t b0 = c->launches;
       try {
-        resident_body(c, R, specs, H, is_max, mr, bm_quads, ch_tiles, handle, 1);
+        resident_body(c, R, specs, H, is_max, mr, bm_quads, ch_tiles, longest, handle, 1);
       } catch (...) {
         c->stream = caller;
         cudaGraph_t dummy = nullptr;
@@ -289,7 +309,7 @@ ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*
       if (it0 != c->prof_index.end()) { expand_ms_seen = c->prof[it0->second].ms; expand_launches_seen = c->prof[it0->second].launches; }
     }
     for (;;) {
-      resident_body(c, R, specs, H, is_max, mr, bm_quads, ch_tiles, cudaGraphConditionalHandle{}, 0);
+      resident_body(c, R, specs, H, is_max, mr, bm_quads, ch_tiles, longest, cudaGraphConditionalHandle{}, 0);
       read_state();
       if (c->flags & XLOG_FLAG_PROFILE) {
         // per delta row and rule: key and tag read, two offsets probed, 16-byte row record and 8-byte start offset written

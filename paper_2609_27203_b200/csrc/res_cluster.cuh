@@ -7,13 +7,16 @@
 // it a CTA turns its changed bits into its part of the next delta, in its own shared memory.  Round r here is round r of the
 // resident loop; the books kept in the state block are the same.
 //
-// The kernel is the first node of the loop body: it takes over when the delta (at most kRcMaxRows rows, kRcMaxCand candidates)
-// is small and runs rounds until the relation is finished or a round changes more slots than that; it then writes the mirror and
-// the changed bits back, and the body's join (nothing to do) and emit kernels close that round and go on grid-wide.
+// The kernel is the first node of the loop body: it takes over when the delta is small (at most kRcMaxRows rows and kRcMaxCand
+// candidates) and runs rounds until the relation is finished or the next round would not be; it then writes the mirror and the
+// changed bits back, and the body's join (nothing to do) and emit kernels close that round and go on grid-wide.  Eight SMs have a
+// twentieth of the device's lanes, so candidates are what counts: a CTA may have kRcMaxCta of them in a round.  With rows of at
+// most kRcMaxRun matches (the host looks, see host_mirror.cuh) the rows bound them well enough while they are few; above, the
+// degrees of the changed keys are added up before their round is begun, at the price of one more barrier.
 //
 // What bounds it: a chain per round of two L2 reads (offsets, then columns; the barrier's acquire empties L1), one
-// distributed-shared-memory read, the barrier (its release waits for the atomics under way) and the list: about 3.5 us on a grid
-// of 90,601 nodes (595 rounds of 1,200 rows), where the two grid-wide launches took 11: 6.7 -> 2.2 ms per query; a grid of 1,600
+// distributed-shared-memory read, the barrier (its release waits for the atomics under way) and the list: about 3 us on a grid
+// of 90,601 nodes (595 rounds of 1,200 rows), where the two grid-wide launches took 12: 7.6 -> 1.8 ms per query; a grid of 1,600
 // nodes 2.2 us a round.  Tried and dropped: an mbarrier per CTA instead of the hardware barrier (its cluster-scope release
 // costs more than the barrier's), rows listed per warp without a block barrier (uneven warps), 1,024 threads.
 #pragma once
@@ -29,9 +32,14 @@ constexpr int kRcCtas = 8, kRcCtasLog = 3;       // the largest portable cluster
 constexpr int kRcBlock = 512;                    // 1024: 3 % faster on the 90,000-node grid, 6 - 9 % slower on grids of 1,600 and 10,000 nodes
 constexpr int kRcMinBits = 8, kRcMaxBits = 17;   // at least a bitmap word per CTA; two copies of 16384 slots in shared memory
 constexpr uint32_t kRcMaxRows = 8192;            // slots changed in a round (with repeats) up to which rounds stay in the cluster
-constexpr uint32_t kRcMaxCand = 65536;           // candidates of a round
+constexpr uint32_t kRcMaxCand = 65536;           // candidates of the first round, and of one whose degrees are not added up
+constexpr uint32_t kRcMaxCta = 8192;             // candidates of one CTA's keys, where they are: 8192 take 10 us, a grid-wide round 11
+constexpr uint32_t kRcMaxRun = 64;               // rows of the looked-up relation's longest run, unless it has at most kRcFewRows in all
+// grid-wide / in the cluster, us: R-MAT 11 with 13,898 edges 187 / 155, with 25,595 179 / 189, a star of 16,000 leaves 109 / 126, of
+// 32,000 113 / 147
+constexpr uint32_t kRcFewRows = 16384;
 constexpr uint32_t kRcWarpRow = 64, kRcBlockRow = 2048;      // rows with more matches are walked by a warp, by the block
-constexpr uint32_t kRcLong = 64;                 // such block rows per round (more: a warp each)
+constexpr uint32_t kRcLong = kRcMaxCand / kRcBlockRow;       // such block rows a round can have
 
 inline size_t res_cluster_smem(uint32_t slots) { const size_t sl = slots / kRcCtas; return sl * 8 + sl / 32 * 12 + sl * 2; }
 
@@ -52,6 +60,7 @@ __device__ __forceinline__ void dsm_improve(uint32_t a, int32_t v) {
 }
 __device__ __forceinline__ void dsm_or(uint32_t a, uint32_t v) { asm volatile("red.relaxed.cluster.shared::cluster.or.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
 __device__ __forceinline__ void dsm_add(uint32_t a, uint32_t v) { asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
+__device__ __forceinline__ void dsm_max(uint32_t a, uint32_t v) { asm volatile("red.relaxed.cluster.shared::cluster.max.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
 __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
@@ -66,14 +75,22 @@ struct ResCluster {
   ResState* st;
   unsigned long long* new_total;
   uint32_t key_max;
+  uint32_t longest;                // longest run of the looked-up relation
   uint32_t* err;
 };
+
+static __global__ void __launch_bounds__(256) k_longest_run(const uint32_t* __restrict__ off, int64_t domain, uint32_t* __restrict__ longest) {
+  uint32_t n = 0;
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < domain; v += (int64_t)gridDim.x * blockDim.x) n = max(n, off[v + 1] - off[v]);
+  n = __reduce_max_sync(0xffffffffu, n);
+  if (lane_id() == 0 && n) atomicMax(longest, n);
+}
 
 template <int SINK>
 __global__ void __launch_bounds__(kRcBlock, 1) k_res_cluster(const __grid_constant__ JoinSpec S, const __grid_constant__ ResCluster P) {
   extern __shared__ __align__(16) uint32_t rc_smem[];
-  __shared__ uint32_t s_sum[3][2];                   // per round modulo 3: slots improved anywhere in the cluster (with repeats), candidates
-  __shared__ uint32_t s_nd, s_nlong;                 // this CTA's rows of the delta; rows for the whole block
+  __shared__ uint32_t s_sum[3][2];                   // per round modulo 3: slots improved anywhere in the cluster (with repeats), most candidates of a CTA in the next
+  __shared__ uint32_t s_nd, s_nlong, s_next;         // this CTA's rows of the delta; rows for the whole block; candidates of its changed keys
   __shared__ uint4 s_long[kRcLong];                  // {first row of the run, length, tag bits, row part of the head key}
   ResState* const st = P.st;
   if (st->status != kResOk) return;
@@ -193,18 +210,39 @@ __global__ void __launch_bounds__(kRcBlock, 1) k_res_cluster(const __grid_consta
     __syncthreads();
     const uint32_t nlong = min(s_nlong, kRcLong);
     for (uint32_t q = 0; q < nlong; ++q) { const uint4 e = s_long[q]; walk(e.x, e.y, __uint_as_float(e.z), e.w, threadIdx.x, kRcBlock); }
-    // what changed and what it took, told to every CTA
-    const uint32_t w_imp = __reduce_add_sync(0xffffffffu, imp), w_cand = __reduce_add_sync(0xffffffffu, round_cand);
-    const uint32_t told = lane < kRcCtas ? w_imp : w_cand;
-    if (told && lane < 2 * kRcCtas) dsm_add(dsm_addr(&s_sum[par][lane / kRcCtas], lane % kRcCtas), told);
+    // what changed, told to every CTA
+    const uint32_t w_imp = __reduce_add_sync(0xffffffffu, imp);
+    if (w_imp && lane < kRcCtas) dsm_add(dsm_addr(&s_sum[par][0], lane), w_imp);
     const uint32_t par_next = par == 2 ? 0u : par + 1;
     if (threadIdx.x == 0) { s_sum[par_next][0] = s_sum[par_next][1] = 0u; s_nd = 0u; }
     cluster_barrier();
-    const uint32_t total_imp = s_sum[par][0], total_cand = s_sum[par][1];
+    const uint32_t total_imp = s_sum[par][0];
     { const uint32_t t = xcur; xcur = xnxt; xnxt = t; }        // the round's end is the next one's start
     if (total_imp == 0u) { cand += round_cand; round_cand = 0; ++closed; verdict = kResDone; break; }
     if (rounds0 + closed + 1 >= max_rounds) { cand += round_cand; round_cand = 0; ++closed; verdict = kResCap; break; }
-    if (total_imp > kRcMaxRows || total_cand > kRcMaxCand) break;        // the emit kernel closes this round
+    if (total_imp > kRcMaxRows) break;               // the emit kernel closes this round
+    if (total_imp * (uint64_t)P.longest > kRcMaxCand) {
+      // the changed keys' degrees, none counted for more than ends the matter
+      uint32_t next = 0;
+      for (uint32_t i = threadIdx.x; i < W; i += kRcBlock)
+        for (uint32_t m = rc_smem[chg + i]; m; m &= m - 1) {
+          const uint32_t key = key_of((i << 5) + __ffs(m) - 1);
+          uint32_t deg = 0;
+          if (plain) {
+            const uint32_t pv = (key >> S.s_probe_shift) & S.s_probe_mask;
+            if (pv < domain) deg = __ldg(S.inner_off + pv + 1) - __ldg(S.inner_off + pv);
+          } else deg = join_count_kv<uint32_t>(S, key, 0.f, 0, nullptr, P.err);
+          next += min(deg, kRcMaxCta + 1);
+        }
+      next = __reduce_add_sync(0xffffffffu, next);
+      if (threadIdx.x == 0) s_next = 0u;
+      __syncthreads();
+      if (lane == 0 && next) atomicAdd(&s_next, next);
+      __syncthreads();
+      if (threadIdx.x < kRcCtas && s_next) dsm_max(dsm_addr(&s_sum[par][1], threadIdx.x), s_next);
+      cluster_barrier();
+      if (s_sum[par][1] > kRcMaxCta) break;
+    }
     // close the round: this CTA's changed keys are its part of the next delta
     cand += round_cand; round_cand = 0; imp = 0; ++closed;
     if (threadIdx.x == 0) s_nlong = 0u;

@@ -108,3 +108,81 @@ def test_facts_beside_a_rule_without_an_atom_over_the_head_and_the_cap():
                 ctx.fixpoint()
             assert e.value.status == "CONVERGENCE_FAILURE"
         ctx.close()
+
+
+def profile(prog, **kw):
+    from paper_2609_27203_b200 import xlog
+    ctx, ids, _ = xlog.load_program(prog, arena_bytes=3 << 30, flags=xlog.FLAG_PROFILE, **kw)
+    ctx.fixpoint()
+    p = ctx.profile()
+    ctx.close()
+    return p
+
+
+def edges(n, deg, seed):
+    r = np.random.default_rng(seed)
+    key = np.unique(np.repeat(np.arange(n), deg) * n + r.integers(0, n, n * deg))
+    s, d = key // n, key % n
+    return s, d, (1 + 9 * r.random(len(s))).astype(np.float32)
+
+
+@pytest.mark.parametrize("sr", [W.MINPLUS, W.MAXPLUS])
+@pytest.mark.parametrize("n,deg", [(9000, 3), (60000, 8), (30000, 40), (8000, 64)])
+def test_short_runs_leave_with_the_candidates_and_come_back(sr, n, deg):
+    """Runs of at most 64: the rounds grow past what a CTA may have, some with few rows and many candidates, and shrink again."""
+    s, d, w = edges(n, deg, n)
+    w = w if sr == W.MINPLUS else -w
+    prog = W.sssp_program(s, d, w, 0, semiring=sr)
+    if sr == W.MAXPLUS:                                       # longest paths need a graph without cycles
+        keep = s < d
+        prog = W.sssp_program(s[keep], d[keep], w[keep], int(s[keep][0]), semiring=sr)
+    both(prog, "dist")
+
+
+def test_a_long_round_is_left_before_it_is_begun():
+    # 1, about 64 and about 3,200 rows: the third round has over 190,000 candidates though the second had 4,000
+    s, d, w = edges(8000, 64, 3)
+    prog = W.sssp_program(s, d, w, 0)
+    p, total = profile(prog), both(prog, "dist", check_oracle=False)["candidates"]
+    assert "k_res_cluster" in p and p["k_res_expand"]["bytes"] > (total - 50000) * 12
+
+
+def test_a_first_round_with_many_candidates_is_not_taken():
+    # the loaded facts are the first delta: 8,000 rows of 64 matches
+    s, d, w = edges(8000, 64, 4)
+    prog = W.sssp_program(s, d, w, 0)
+    prog.facts["dist"] = ([np.arange(8000, dtype=np.int32)], (np.arange(8000) % 97 + 1).astype(np.float32))
+    p = profile(prog)
+    assert p["k_res_expand"]["bytes"] > 450000 * 12 and "k_res_count_scan" in p
+    both(prog, "dist")
+
+
+@pytest.mark.parametrize("n,taken", [(16385, True), (16386, False)])
+def test_long_runs_only_in_small_relations(n, taken):
+    # a star: one run of n - 1 rows, walked by the block
+    prog = W.sssp_program(np.zeros(n - 1, np.int32), np.arange(1, n, dtype=np.int32), np.random.default_rng(n).random(n - 1).astype(np.float32) + 1, 0)
+    assert ("k_res_cluster" in profile(prog)) == taken
+    both(prog, "dist")
+
+
+@pytest.mark.parametrize("run,taken", [(64, True), (65, False)])
+def test_the_longest_run_decides(run, taken):
+    s, d, w = edges(20000, 3, run)
+    s, d, w = np.append(s, np.zeros(run, int)), np.append(d, 100 + np.arange(run)), np.append(w, np.ones(run, np.float32))
+    keep = np.ones(len(s), bool)
+    keep[:-run] = s[:-run] != 0                               # node 0 has exactly these
+    prog = W.sssp_program(s[keep], d[keep], w[keep], 0)
+    assert ("k_res_cluster" in profile(prog)) == taken
+    both(prog, "dist", check_oracle=False)
+
+
+def test_as_many_block_rows_as_a_round_can_have():
+    # 7 sources with edges to 4 hubs of 2,300 matches: the second round has 28 rows that the block walks and 64,400 candidates
+    hub, leaf = 100 + np.arange(4), 9000 + np.arange(2300)
+    s = np.concatenate([np.repeat(np.arange(7), 4), np.repeat(hub, len(leaf))])
+    d = np.concatenate([np.tile(hub, 7), np.tile(leaf, 4)])
+    w = (1 + np.random.default_rng(1).random(len(s))).astype(np.float32)
+    prog = W.reach_program(s.astype(np.int32), d.astype(np.int32), w, np.arange(7, dtype=np.int32))
+    p = profile(prog)
+    assert "k_res_cluster" in p and p["k_res_expand"]["bytes"] == 0
+    both(prog, "reach")
