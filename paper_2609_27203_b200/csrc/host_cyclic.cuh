@@ -47,14 +47,6 @@ void append_count_column(Ctx* c, Relation& H, KeyTags& u, const KeyLayout& cl) {
 constexpr int kSlotTrk = 48;               // the kTrkTotals control words
 static_assert(kSlotTrk + kTrkTotals <= 64, "control words overlap the resident state block");
 
-void exclusive_scan_u32(Ctx* c, const uint32_t* in, int64_t n, uint32_t* out, uint32_t* total) {
-  const unsigned tiles = (unsigned)((n + kScanTile - 1) / kScanTile);
-  DevBuf sums(c, (size_t)tiles * 4);
-  XLOG_LAUNCH(c, (k_scan_tile_sums<uint32_t, uint32_t>), tiles, kScanBlock, 0, in, n, sums.as<uint32_t>());
-  XLOG_LAUNCH(c, (k_scan_spine<uint32_t>), 1, 1024, 0, sums.as<uint32_t>(), (int64_t)tiles, total);
-  XLOG_LAUNCH(c, (k_scan_apply<uint32_t, uint32_t>), tiles, kScanBlock, 0, in, n, (const uint32_t*)sums.as<uint32_t>(), out);
-}
-
 TriRankLists tri_rank_lists(const TriRankIndex& X, int o) {
   return TriRankLists{X.off[o].as<uint32_t>(), X.split[o].as<uint32_t>(), X.nbr[o].as<uint32_t>(), X.num[o].as<float>(), o == 1 ? X.other.as<uint32_t>() : nullptr};
 }

@@ -286,8 +286,11 @@ void row_sums_rounds(Ctx* c, Relation& H, const std::vector<RowSumRule>& rules, 
 // ---- row-local fixpoint of short rows (sparse_rows.cuh) --------------------------------------------------------------------
 constexpr int kSlotSparse = 48;            // the kSpTotals control words (after the deferred counts of a component of one head)
 static_assert(kSlotSparse + kSpTotals <= kSlotResState, "control words overlap");
-// Worth trying when the rows are many (each is worked on by a few lanes) and their values of c too many for dense rows.  A try
-// that fails costs the launch until an eighth of the rows have outgrown the first table: tens of microseconds.
+// Worth trying when the rows are many (each is worked on by a few lanes) and their values of c too many for dense rows: the
+// ancestors of 4,200 / 8,000 values in a forest of 32,768 nodes 0.27 / 0.26 ms, over the mirror 3.3 / 3.4.  The line could lie lower:
+// of 500 / 2,000 0.25 / 0.26, over the mirror 0.76 / 2.3.
+// What a try costs that comes to nothing because an eighth of the rows outgrow the first table: the launch until then, 0.2 to 0.4 ms of
+// 8.4 (paths of 60 nodes, 16,000 in all: the seed round is evaluated a second time, over the mirror) and of 13.9 (200,000).
 constexpr int64_t kSparseMinRows = 4096, kSparseMaxRows = (int64_t)1 << 22;
 
 bool sparse_rows_applies(Ctx* c, const std::vector<int>& comp, const std::vector<const RuleC*>& rs, JoinSpec& S, int& r_rel) {
@@ -321,27 +324,48 @@ void launch_sparse_tier(Ctx* c, SparseRows& P, int tier, uint32_t rows, uint32_t
 // The tiers: lanes per row and slots per table.  Measured on 300,000 rows of 17 tuples (us for all tiers): 4 lanes and 32 slots
 // 613, 2 and 32 777, 8 and 32 739, 4 and 64 677: a longer first table costs rows in flight, wider groups cost lanes that idle.
 template <typename K, int SINK>
-void launch_sparse_tiers(Ctx* c, SparseRows& P, uint32_t* q0, uint32_t* q1) {
+void launch_sparse_tiers(Ctx* c, SparseRows& P, uint32_t* q0, uint32_t* q1, uint32_t* q2) {
   const uint32_t n = P.n_rows;
   P.rows_in = nullptr; P.rows_out = q0;
   launch_sparse_tier<K, SINK, 4, 32>(c, P, 0, n, n / 8 + 1024);
   P.rows_in = q0; P.rows_out = q1;
   launch_sparse_tier<K, SINK, 8, 128>(c, P, 1, n / 8 + 1024, n / 64 + 128);
-  P.rows_in = q1; P.rows_out = nullptr;
-  launch_sparse_tier<K, SINK, 32, (int)kSparseLongest>(c, P, 2, n / 64 + 128, 0);
+  P.rows_in = q1; P.rows_out = q2;
+  launch_sparse_tier<K, SINK, 32, (int)kSparseLongest>(c, P, 2, n / 64 + 128, n / 64 + 128);
 }
 
-// The rounds after the seed round: H holds the relation, (dkeys, dtags, dn) its delta.  False: some row is too long, or the
-// staging area too small; nothing has changed.
-bool sparse_rows_rounds(Ctx* c, Relation& H, const JoinSpec& S, uint32_t r_rows, const void* dkeys, const float* dtags, uint32_t dn) {
+// The tuples of the marked rows of a sorted list; *n_at: control slot of their number, valid at the next control read.
+DevBuf sparse_keep(Ctx* c, const void* keys, int key_bytes, uint32_t n, int c_bits, const DevBuf& mark, int n_at) {
+  DevBuf at(c, ((size_t)n + 1) * 4);
+  DISPATCH_K(key_bytes, XLOG_LAUNCH(c, (k_sparse_keep<K>), grid_for((uint64_t)n + 1, 256), 256, 0, (const K*)keys, n, c_bits, (const uint32_t*)mark.as<uint32_t>(), at.as<uint32_t>()));
+  exclusive_scan_u32(c, at.as<uint32_t>(), (int64_t)n + 1, at.as<uint32_t>(), ctrl_u32(c, n_at));
+  return at;
+}
+KeyTags sparse_take(Ctx* c, const void* keys, const float* tags, int key_bytes, uint32_t n, const DevBuf& at, uint32_t n_out) {
+  KeyTags out;
+  out.n = n_out;
+  out.keys = DevBuf(c, (size_t)std::max(n_out, 1u) * key_bytes);
+  out.tags = DevBuf(c, (size_t)std::max(n_out, 1u) * 4);
+  DISPATCH_K(key_bytes, XLOG_LAUNCH(c, (k_sparse_take<K>), grid_for(n, 256), 256, 0, (const K*)keys, tags, n, (const uint32_t*)at.as<uint32_t>(), out.keys.as<K>(), out.tags.as<float>()));
+  return out;
+}
+
+// The rounds after the seed round: H holds the relation, `delta` its delta.  kSparseDone: H is finished.  kSparseRest: `done` holds
+// the finished rows, *rounds their rounds, H and `delta` what there was of the others.  kSparseFailed: too many rows are long, or
+// the staging area is too small; nothing has changed.
+enum SparseOutcome { kSparseFailed, kSparseDone, kSparseRest };
+SparseOutcome sparse_rows_rounds(Ctx* c, Relation& H, const JoinSpec& S, uint32_t r_rows, KeyTags& delta, KeyTags& done, int64_t* rounds) {
+  const void* dkeys = delta.keys.p;
+  const float* dtags = delta.tags.as<float>();
+  const uint32_t dn = delta.n;
   const int c_bits = H.layout.shift[0];
   const uint32_t n_rows = (uint32_t)H.col_max[0] + 1;
   const uint32_t max_q0 = n_rows / 8 + 1024, max_q1 = n_rows / 64 + 128;
-  const size_t fixed = (size_t)n_rows * 44 + (size_t)r_rows * 16 + (size_t)(max_q0 + max_q1) * 4 + (1u << 20);
-  if (fixed > c->arena.largest_free() / 2) return false;
+  const size_t fixed = (size_t)n_rows * 44 + (size_t)r_rows * 16 + (size_t)(max_q0 + 2 * max_q1) * 4 + (1u << 20);
+  if (fixed > c->arena.largest_free() / 2) return kSparseFailed;
   const bool same = dn == H.n;              // the delta is a subset of the relation: of one size, they are the same rows
   DevBuf rec(c, (size_t)n_rows * 16), rec_run(c, (size_t)n_rows * 8), drec(c, same ? 8 : (size_t)n_rows * 8), adj(c, (size_t)r_rows * 16), row_pos(c, (size_t)n_rows * 4),
-      row_len(c, (size_t)n_rows * 4), row_off(c, (size_t)n_rows * 4), q0(c, (size_t)max_q0 * 4), q1(c, (size_t)max_q1 * 4);
+      row_len(c, (size_t)n_rows * 4), row_off(c, (size_t)n_rows * 4), q0(c, (size_t)max_q0 * 4), q1(c, (size_t)max_q1 * 4), q2(c, (size_t)max_q1 * 4);
   const size_t free_bytes = c->arena.largest_free();
   const uint64_t cap = std::min<uint64_t>(free_bytes / 24, (uint64_t)kSortMaxN);      // 8 bytes staged and up to 12 in the relation
   DevBuf st_c(c, cap * 4), st_t(c, cap * 4);
@@ -367,8 +391,8 @@ bool sparse_rows_rounds(Ctx* c, Relation& H, const JoinSpec& S, uint32_t r_rows,
   P.totals = (unsigned long long*)(c->d_ctrl + kSlotSparse); P.err = ctrl_u32(c, kSlotErr);
   const bool is_max = H.sr == XLOG_SR_MAXPLUS;
   DISPATCH_K(H.key_bytes, {
-    if (is_max) launch_sparse_tiers<K, kSinkMax>(c, P, q0.as<uint32_t>(), q1.as<uint32_t>());
-    else launch_sparse_tiers<K, kSinkMin>(c, P, q0.as<uint32_t>(), q1.as<uint32_t>());
+    if (is_max) launch_sparse_tiers<K, kSinkMax>(c, P, q0.as<uint32_t>(), q1.as<uint32_t>(), q2.as<uint32_t>());
+    else launch_sparse_tiers<K, kSinkMin>(c, P, q0.as<uint32_t>(), q1.as<uint32_t>(), q2.as<uint32_t>());
   });
   const unsigned tiles = (n_rows + kScanTile - 1) / kScanTile;
   DevBuf sums(c, (size_t)tiles * 4);
@@ -378,12 +402,14 @@ bool sparse_rows_rounds(Ctx* c, Relation& H, const JoinSpec& S, uint32_t r_rows,
               row_off.as<uint32_t>());
   sync_ctrl(c);
   const uint64_t* w = c->h_ctrl + kSlotSparse;
-  if (w[kSpStatus]) return false;
+  if (w[kSpStatus]) return kSparseFailed;
   c->r_candidates += (int64_t)w[kSpCandidates];
   c->r_unique += (int64_t)w[kSpUnique];
   c->r_new += (int64_t)w[kSpNew];
   c->r_improved += (int64_t)(w[kSpChanged] - w[kSpNew]);
-  c->r_iterations += (int64_t)w[kSpRounds];
+  *rounds = (int64_t)w[kSpRounds];
+  const uint32_t n_long = (uint32_t)w[kSpQueued + 2];
+  if (!n_long) c->r_iterations += *rounds;
   if (w[kSpCapped]) fail(XLOG_ERR_CONVERGENCE_FAILURE, "iteration cap reached before the fixpoint");
   KeyTags full;
   full.n = (uint32_t)c->h_ctrl[kSlotA];
@@ -393,12 +419,25 @@ bool sparse_rows_rounds(Ctx* c, Relation& H, const JoinSpec& S, uint32_t r_rows,
   DISPATCH_K(H.key_bytes, XLOG_LAUNCH(c, (k_sparse_emit<K>), grid_for((uint64_t)n_rows * 8, 256), 256, 0, (const uint32_t*)row_pos.as<uint32_t>(), (const uint32_t*)row_len.as<uint32_t>(),
                                        (const uint32_t*)row_off.as<uint32_t>(), n_rows, c_bits, (const uint32_t*)st_c.as<uint32_t>(), (const float*)st_t.as<float>(),
                                        full.keys.as<K>(), full.tags.as<float>()));
+  if (n_long) {
+    st_c.reset(); st_t.reset();
+    XLOG_CUDA(cudaMemsetAsync(row_pos.p, 0, (size_t)n_rows * 4, c->stream));
+    XLOG_LAUNCH(c, k_sparse_mark, grid_for(n_long, 256), 256, 0, (const uint32_t*)q2.as<uint32_t>(), n_long, row_pos.as<uint32_t>());
+    const DevBuf at = sparse_keep(c, H.keys(), H.key_bytes, H.n, c_bits, row_pos, kSlotA), dat = sparse_keep(c, dkeys, H.key_bytes, dn, c_bits, row_pos, kSlotB);
+    sync_ctrl(c);
+    KeyTags part = sparse_take(c, H.keys(), H.tags(), H.key_bytes, H.n, at, (uint32_t)c->h_ctrl[kSlotA]);
+    KeyTags dpart = sparse_take(c, dkeys, dtags, H.key_bytes, dn, dat, (uint32_t)c->h_ctrl[kSlotB]);
+    set_current(H, std::move(part));
+    delta = std::move(dpart);
+    done = std::move(full);
+    return kSparseRest;
+  }
   set_current(H, std::move(full));
   if (c->flags & XLOG_FLAG_CHECK_INVARIANTS) {
     DISPATCH_K(H.key_bytes, XLOG_LAUNCH(c, (k_check_sorted<K>), grid_for(H.n, 256), 256, 0, (const K*)H.keys(), (int64_t)H.n, ctrl_u32(c, kSlotErr)));
     sync_ctrl(c);
   }
-  return true;
+  return kSparseDone;
 }
 
 }  // namespace

@@ -42,6 +42,14 @@ void set_current(Relation& R, KeyTags&& kt) {
   drop_indices(R);
 }
 
+void exclusive_scan_u32(Ctx* c, const uint32_t* in, int64_t n, uint32_t* out, uint32_t* total) {
+  const unsigned tiles = (unsigned)((n + kScanTile - 1) / kScanTile);
+  DevBuf sums(c, (size_t)tiles * 4);
+  XLOG_LAUNCH(c, (k_scan_tile_sums<uint32_t, uint32_t>), tiles, kScanBlock, 0, in, n, sums.as<uint32_t>());
+  XLOG_LAUNCH(c, (k_scan_spine<uint32_t>), 1, 1024, 0, sums.as<uint32_t>(), (int64_t)tiles, total);
+  XLOG_LAUNCH(c, (k_scan_apply<uint32_t, uint32_t>), tiles, kScanBlock, 0, in, n, (const uint32_t*)sums.as<uint32_t>(), out);
+}
+
 // Column-major int32 view of the current contents.
 void ensure_soa(Ctx* c, Relation& R) {
   if (R.soa_valid) return;

@@ -135,12 +135,14 @@ void stratum_recursive(Ctx* c, const std::vector<int>& comp, const std::vector<c
   }
   const int64_t before[5] = {c->r_candidates, c->r_unique, c->r_new, c->r_improved, c->r_iterations};
   std::vector<KeyTags> delta(c->rels.size());
+  KeyTags done;                            // rows that are finished while the rounds of the others go on
+  int64_t done_rounds = 0;
   for (int64_t round = 0;; ++round) {
     if (round == 1 && try_rows) {
       Relation& H = *c->rels[comp[0]];
-      const KeyTags& d = delta[comp[0]];
-      if (sparse_rows_rounds(c, H, row_spec, c->rels[row_rel]->n, d.keys.p, d.tags.as<float>(), d.n)) return;
-      if (mirror_applies(c, comp, rs)) {                     // some row is long: over the mirror instead, from the start
+      const SparseOutcome got = sparse_rows_rounds(c, H, row_spec, c->rels[row_rel]->n, delta[comp[0]], done, &done_rounds);
+      if (got == kSparseDone) return;
+      if (got == kSparseFailed && mirror_applies(c, comp, rs)) {      // many rows are long: over the mirror instead, from the start
         delta.clear();
         drop_current(H);
         c->r_candidates = before[0]; c->r_unique = before[1]; c->r_new = before[2]; c->r_improved = before[3]; c->r_iterations = before[4];
@@ -227,6 +229,13 @@ void stratum_recursive(Ctx* c, const std::vector<int>& comp, const std::vector<c
       }
     }
     if (changed == 0) break;
+  }
+  if (done.n) {
+    Relation& H = *c->rels[comp[0]];
+    MergeResult m;
+    DISPATCH_K(H.key_bytes, m = merge<K>(c, H.sr, done.keys.as<K>(), done.tags.as<float>(), done.n, -1, (const K*)H.keys(), H.tags(), H.n, false, false));
+    set_current(H, std::move(m.full));
+    c->r_iterations = std::max(c->r_iterations, before[4] + 1 + done_rounds);
   }
 }
 

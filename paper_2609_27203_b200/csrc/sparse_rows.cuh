@@ -6,14 +6,18 @@
 // lanes takes a value of a and runs that row's rounds to the end on an open-addressed hash table of T slots in shared
 // memory: delta list with the tags set aside, candidates laid out in a line per G delta rows, one atomic max / min per
 // candidate.  The groups of a warp run their rounds in lockstep, each at its own row; a group that finishes writes the row to
-// a staging area and takes the next one.  A row that outgrows its table (7/8 full) is left alone and its a queued for the next
-// launch, with longer tables and wider groups; one that outgrows the last tier, a first tier in which every eighth row
-// outgrows its table, or a full staging area sets the status word, and the stratum goes on as if nothing had been tried (the
-// relation and its delta are only read here).
+// a staging area and takes the next one.  A row of more tuples than its table has slots is left alone at the first candidate that finds
+// no room and its a queued for the next launch, with longer tables and wider groups.  The rows that outgrow the last tier are few:
+// the stratum goes on with them alone, round by round, and the finished rows join them at its end (k_sparse_keep, k_sparse_take).
+// A first tier in which every eighth row outgrows its table (a second in which every 64th does), or a full staging area, sets
+// the status word, and the stratum goes on as if nothing had been tried (the relation and its delta are only read here).
 //
 // What bounds it: instruction issue (half of the slots) and the latency of one dependent L2 read per row and round, over as
 // many rows as shared memory holds at a time.  300,000 rows of 17 tuples and 13 rounds on average (5.06 M tuples, 28 rounds):
-// 7.22 ms on the sorting route, 0.89 ms here, of which 0.48 in the first tier and 0.12 in the second (5 % of the rows).
+// 7.22 ms on the sorting route, 0.89 ms here, of which 0.47 in the first tier and 0.15 in the second (5 % of the rows).
+// Rows of every length (the descendants in such forests, ms, sorting route or mirror / here): 9,000 nodes 2.80 / 3.16, 60,000 2.92 /
+// 4.18, 300,000 6.64 / 7.70, a node in 1,024 going on alone for all of the rounds; one row of 1,500 tuples that is done in two
+// rounds among 200,000: 2.63 / 0.42.
 // r is therefore read through 16-byte entries (c, tag, where c's own run begins, its length), so that a round needs no
 // look-up of offsets; a row's first key comes with its record, so that taking a row needs no chain of reads either; and rows
 // leave unordered (k_sparse_emit ranks them, at full occupancy).  See the tiers in host_mirror_rows.cuh.
@@ -105,7 +109,9 @@ __global__ void __launch_bounds__(256) k_sparse_records(const K* __restrict__ ke
   }
 }
 
-// Slot of c in the table, inserted if absent (is_new); T if there is no room.
+// Slot of c in the table, inserted if absent (is_new); T if there is no room.  Tables fill to the last slot; in the longer ones the
+// steps grow by one (1 + 2 + ... meets every slot of a power of two), or the last keys of a row would each look at most of the
+// table.
 template <int T>
 __device__ __forceinline__ uint32_t sparse_slot(SparseRow<T>& R, uint32_t c, bool& is_new) {
   constexpr int LOG = T == 32 ? 5 : T == 64 ? 6 : T == 128 ? 7 : T == 256 ? 8 : T == 512 ? 9 : 10;
@@ -120,7 +126,7 @@ __device__ __forceinline__ uint32_t sparse_slot(SparseRow<T>& R, uint32_t c, boo
       if (k == kSparseEmpty) { is_new = true; return h; }
     }
     if (k == c) return h;
-    h = (h + 1) & (T - 1);
+    h = (h + (T <= 32 ? 1 : probe + 1)) & (T - 1);
   }
   return T;
 }
@@ -133,7 +139,6 @@ __global__ void __launch_bounds__(kSparseBlock) k_sparse_rows(const __grid_const
   constexpr uint32_t kMaskB = B == 32 ? 0xffffffffu : (1u << (B & 31)) - 1u;
   constexpr unsigned kGroups = 32 / G;
   constexpr int kBatch = kGroups >= 4 ? 4 : 1;     // groups that leave together
-  constexpr uint32_t kChunk = G == 4 ? 32 : kGroups;      // rows a warp draws at a time
   extern __shared__ __align__(16) unsigned char sp_smem[];
   SparseRow<T>& R = reinterpret_cast<SparseRow<T>*>(sp_smem)[threadIdx.x / G];
   const unsigned lane = lane_id(), sub = lane % G, grp = lane / G;
@@ -143,6 +148,8 @@ __global__ void __launch_bounds__(kSparseBlock) k_sparse_rows(const __grid_const
   const K* dkeys = (const K*)P.dkeys;
   const K cmask = ((K)1 << P.c_bits) - 1;
   const uint32_t n_todo = P.rows_in ? min((uint32_t)P.totals[kSpQueued + P.tier - 1], P.max_in) : P.n_rows;
+  // rows a warp draws at a time: one a group, fewer where there are few (neighbouring rows may all be long)
+  const uint32_t per_draw = max(1u, min(kGroups, n_todo / (gridDim.x * (kSparseBlock / 32))));
   unsigned long long* const queued = P.totals + kSpQueued + P.tier;
   unsigned long long cand = 0;
   uint32_t uniq = 0, n_changed = 0, n_new = 0, max_rounds_seen = 0, capped = 0;
@@ -204,6 +211,7 @@ __global__ void __launch_bounds__(kSparseBlock) k_sparse_rows(const __grid_const
         if (active && outgrown && sub == 0) {
           const unsigned long long q = atomicAdd(queued, 1ull);
           if (q < P.max_queued) P.rows_out[q] = a; else atomicExch(P.totals + kSpStatus, 1ull);
+          P.row_len[a] = 0u;
         }
         if (emit) { max_rounds_seen = max(max_rounds_seen, rounds); cand += row_cand; uniq += row_uniq; n_changed += row_changed; n_new += row_new; }
         if (waits) active = false;
@@ -215,10 +223,10 @@ __global__ void __launch_bounds__(kSparseBlock) k_sparse_rows(const __grid_const
           uint32_t t = 0;
           if (lane == 0) {
             const bool stop = *reinterpret_cast<volatile unsigned long long*>(P.totals + kSpStatus) != 0ull;
-            t = stop ? n_todo : (uint32_t)atomicAdd(P.totals + kSpTicket + P.tier, (unsigned long long)kChunk);
+            t = stop ? n_todo : (uint32_t)atomicAdd(P.totals + kSpTicket + P.tier, (unsigned long long)per_draw);
           }
           chunk = __shfl_sync(0xffffffffu, t, 0);
-          chunk_end = min(chunk + kChunk, n_todo);
+          chunk_end = min(chunk + per_draw, n_todo);
           if (chunk >= n_todo) { dry = true; chunk = chunk_end = 0; }
         }
         const unsigned idle = __ballot_sync(0xffffffffu, !active && sub == 0);
@@ -303,11 +311,11 @@ __global__ void __launch_bounds__(kSparseBlock) k_sparse_rows(const __grid_const
     __syncwarp();
     if (go) for (int i = sub; i < T / 32; i += G) { R.seen[i] = 0u; R.chg[i] = 0u; }
     __syncwarp();
-    bool full = false;
-    for (uint32_t r0 = 0; __any_sync(0xffffffffu, go && r0 < nd); r0 += G) {
+    bool full = false, stop = false;                         // stop: some lane of the group found the table full; the round's rest is not looked at
+    for (uint32_t r0 = 0; __any_sync(0xffffffffu, go && !stop && r0 < nd); r0 += G) {
       uint32_t lo = 0, dg = 0;
       float t = 0.f;
-      if (go && r0 + sub < nd) {
+      if (go && !stop && r0 + sub < nd) {
         const uint2 run = R.hrun[R.list[r0 + sub]];
         t = R.dtag[r0 + sub];
         lo = run.x; dg = run.y;
@@ -317,14 +325,14 @@ __global__ void __launch_bounds__(kSparseBlock) k_sparse_rows(const __grid_const
       for (int d = 1; d < G; d <<= 1) { const uint32_t o = __shfl_up_sync(0xffffffffu, end, d, G); if ((int)sub >= d) end += o; }
       const uint32_t total = __shfl_sync(0xffffffffu, end, G - 1, G);
       row_cand += dg;
-      for (uint32_t p0 = 0; __any_sync(0xffffffffu, p0 < total); p0 += G) {
+      for (uint32_t p0 = 0; __any_sync(0xffffffffu, !stop && p0 < total); p0 += G) {
         const uint32_t p = p0 + sub;
         uint32_t owner = 0;                                  // first lane of the group whose inclusive prefix exceeds p
 #pragma unroll
         for (int d = G / 2; d; d >>= 1) { const uint32_t v = __shfl_sync(0xffffffffu, end, owner + d - 1, G); if (v <= p) owner += d; }
         const uint32_t from = __shfl_sync(0xffffffffu, lo + dg - end, owner, G);        // the owner's run, less the candidates before it
         const float ot = __shfl_sync(0xffffffffu, t, owner, G);
-        if (p < total) {
+        if (!stop && p < total) {
           const uint4 q = P.adj[from + p];
           const uint32_t c = q.x;
           const int32_t v = f2ord(ot + __uint_as_float(q.y));
@@ -342,6 +350,9 @@ __global__ void __launch_bounds__(kSparseBlock) k_sparse_rows(const __grid_const
             }
           }
         }
+        // once one candidate has found no room none is looked for any more
+        const unsigned none = __ballot_sync(0xffffffffu, full);      // by every lane, stopped or not
+        stop = (none & gmask) != 0u;
       }
     }
     __syncwarp();
@@ -430,6 +441,22 @@ __global__ void __launch_bounds__(256) k_sparse_emit(const uint32_t* __restrict_
     }
     __syncwarp();
   }
+}
+
+// The rows (of first column) on a list, marked; the tuples of marked rows in a list of keys, flagged; and copied to the places that
+// a scan of the flags gives.
+static __global__ void __launch_bounds__(256) k_sparse_mark(const uint32_t* __restrict__ rows, uint32_t n, uint32_t* __restrict__ mark) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) mark[rows[i]] = 1u;
+}
+template <typename K>
+__global__ void __launch_bounds__(256) k_sparse_keep(const K* __restrict__ keys, uint32_t n, int c_bits, const uint32_t* __restrict__ mark, uint32_t* __restrict__ flag) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i <= n; i += gridDim.x * blockDim.x) flag[i] = i < n ? mark[(uint32_t)(keys[i] >> c_bits)] : 0u;
+}
+template <typename K>
+__global__ void __launch_bounds__(256) k_sparse_take(const K* __restrict__ keys, const float* __restrict__ tags, uint32_t n, const uint32_t* __restrict__ at,
+                                                     K* __restrict__ out_keys, float* __restrict__ out_tags) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+    if (at[i] != at[i + 1]) { out_keys[at[i]] = keys[i]; out_tags[at[i]] = tags[i]; }
 }
 
 }  // namespace xlog
