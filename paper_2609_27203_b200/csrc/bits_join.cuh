@@ -12,7 +12,7 @@
 // 1.55 -> 0.37 ms; a lane per word and the hits of a path written as they fell: 0.23 and 0.75.  Triangle join, 65,536 rows over
 // 406 values, 4.2 M rows: 62 -> 9 us and 84 -> 61 us.
 //
-//   k_bits_rows    list entries -> bits;  k_bits_ranks   running counts per word
+//   k_bits_lists   list entries -> bits, and running counts per word
 //   k_bits_count   matches per path
 //   k_bits_emit    the rows: hits are queued per warp with their place in the output and worked off 32 at a time, so that
 //                  the two tag reads and the writes use every lane though a path has few hits
@@ -27,22 +27,26 @@ constexpr int kBitsLanes = 4;                    // lanes per path
 inline uint32_t bits_padded(uint32_t words) { return words <= 16 ? 16u : (words + 31) / 32 * 32; }
 constexpr uint32_t kBitsQueue = 256;             // hits a warp holds before it works them off
 
-static __global__ void __launch_bounds__(256) k_bits_rows(const uint32_t* __restrict__ off, int64_t domain, const int32_t* __restrict__ col, uint32_t words, uint32_t* __restrict__ bits) {
-  // a warp per list
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < domain; v += nwarps)
-    for (uint32_t i = off[v] + lane_id(); i < off[v + 1]; i += 32) { const uint32_t w = (uint32_t)col[i]; atomicOr(bits + (size_t)v * words + (w >> 5), 1u << (w & 31)); }
-}
-static __global__ void __launch_bounds__(256) k_bits_ranks(const uint32_t* __restrict__ bits, int64_t domain, uint32_t words, uint16_t* __restrict__ rank) {
+// A warp per list: its entries' bits are set in shared memory, then every word is written with the number of entries before it.
+static __global__ void __launch_bounds__(256) k_bits_lists(const uint32_t* __restrict__ off, int64_t domain, const int32_t* __restrict__ col, uint32_t words, uint32_t* __restrict__ bits,
+                                                           uint16_t* __restrict__ rank) {
+  __shared__ uint32_t s_bits[8][kBitsMaxWords];
+  uint32_t* const row = s_bits[warp_id()];
+  const unsigned lane = lane_id();
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < domain; v += nwarps) {
+    for (uint32_t k = lane; k < words; k += 32) row[k] = 0u;
+    __syncwarp();
+    for (uint32_t i = off[v] + lane; i < off[v + 1]; i += 32) { const uint32_t w = (uint32_t)col[i]; atomicOr(row + (w >> 5), 1u << (w & 31)); }
+    __syncwarp();
     uint32_t run = 0;
     for (uint32_t k = 0; k < words; k += 32) {
-      const uint32_t n = k + lane_id() < words ? (uint32_t)__popc(bits[(size_t)v * words + k + lane_id()]) : 0u;
-      const uint32_t incl = warp_scan_incl(n);
-      if (k + lane_id() < words) rank[(size_t)v * words + k + lane_id()] = (uint16_t)(run + incl - n);
+      const bool in = k + lane < words;
+      const uint32_t b = in ? row[k + lane] : 0u, n = (uint32_t)__popc(b), incl = warp_scan_incl(n);
+      if (in) { bits[(size_t)v * words + k + lane] = b; rank[(size_t)v * words + k + lane] = (uint16_t)(run + incl - n); }
       run += __shfl_sync(0xffffffffu, incl, 31);
     }
+    __syncwarp();
   }
 }
 

@@ -306,10 +306,8 @@ bool bits_join_applies(Ctx* c, const Relation& A, const Index& aix, const Relati
 BitsLists ensure_bits(Ctx* c, Index& ix, uint32_t words) {
   if (ix.bit_words != words) {
     ix.bits = DevBuf(c, (size_t)ix.domain * words * 4); ix.bit_rank = DevBuf(c, (size_t)ix.domain * words * 2);
-    XLOG_CUDA(cudaMemsetAsync(ix.bits.p, 0, (size_t)ix.domain * words * 4, c->stream));
-    const unsigned g = grid_for((uint64_t)ix.domain * 32, 256);
-    XLOG_LAUNCH(c, k_bits_rows, g, 256, 0, (const uint32_t*)ix.off.as<uint32_t>(), ix.domain, ix.other[0], words, ix.bits.as<uint32_t>());
-    XLOG_LAUNCH(c, k_bits_ranks, g, 256, 0, (const uint32_t*)ix.bits.as<uint32_t>(), ix.domain, words, ix.bit_rank.as<uint16_t>());
+    XLOG_LAUNCH(c, k_bits_lists, grid_for((uint64_t)ix.domain * 32, 256), 256, 0, (const uint32_t*)ix.off.as<uint32_t>(), ix.domain, ix.other[0], words, ix.bits.as<uint32_t>(),
+                ix.bit_rank.as<uint16_t>());
     ix.bit_words = words;
   }
   return BitsLists{ix.bits.as<uint32_t>(), ix.bit_rank.as<uint16_t>(), ix.off.as<uint32_t>(), ix.tags, (uint32_t)ix.domain};

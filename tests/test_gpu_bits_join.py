@@ -76,3 +76,30 @@ def test_sparse_lists_and_wide_values_keep_the_list_kernels(dom):
     assert H.compare_relations(got, ctx.read(ids["c4"]))["bit_unequal"] == 0
     ctx.close()
     assert ran == (dom == 16384)
+
+
+@pytest.mark.parametrize("w_dom", [33, 1024, 2111])
+def test_new_relations_have_new_bitmaps(w_dom):
+    """Relations loaded again, longer, shorter and over other values, through one context: a list's bits and counts are those of the
+    rows that are there now (one launch a list, which leaves nothing to be cleared)."""
+    from paper_2609_27203_b200 import xlog
+    prog = None
+    ctx = None
+    for seed, density in ((1, 0.3), (2, 0.9), (3, 0.15)):
+        r = np.random.default_rng(seed)
+        full = max(0.1, density * 8 / w_dom)
+        prog = W.triangle_join_program(pairs(r, 70, 130, 0.5), pairs(r, 130, w_dom, full), _turn(pairs(r, 70, w_dom, full)), semiring=W.MAXPLUS)
+        if ctx is None:
+            ctx, ids, _ = xlog.load_program(prog, arena_bytes=4 << 30, flags=xlog.FLAG_FORCE_WCOJ | xlog.FLAG_CHECK_INVARIANTS | xlog.FLAG_PROFILE)
+        else:
+            for name in ("r", "s", "t"):
+                ctx.load(ids[name], *prog.facts[name])
+        ctx.profile_reset()
+        ctx.fixpoint()
+        assert ctx.profile()["k_bits_lists"]["launches"] == 2
+        got = ctx.read(ids["tri"])
+        other, oids, _ = xlog.load_program(prog, arena_bytes=4 << 30, flags=xlog.FLAG_FORCE_CHAIN)
+        other.fixpoint()
+        assert H.compare_relations(got, other.read(oids["tri"]), what=f"seed {seed}")["bit_unequal"] == 0
+        other.close()
+    ctx.close()
