@@ -62,9 +62,31 @@ void ensure_soa(Ctx* c, Relation& R) {
   R.soa_valid = true;
 }
 
-// The current contents into device columns and tags of the caller's (null: not wanted), in stored order.
+// May a kernel on this device store 4-byte values there?  Memory of the device, managed memory, and host memory that is mapped for
+// it; anything else, and addresses that are no multiple of 4, is left to a copy, which finds out what it has before it.
+bool kernel_can_store(Ctx* c, const void* p) {
+  if (!p) return true;
+  if ((uintptr_t)p & 3u) return false;
+  cudaPointerAttributes a{};
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) { cudaGetLastError(); return false; }
+  if (a.type == cudaMemoryTypeDevice) return a.device == c->device;
+  return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeHost && a.devicePointer == p);
+}
+
+// The current contents into columns and tags of the caller's (null: not wanted) by copies from the column view, in stored order.
+void copy_out(Ctx* c, Relation& R, int32_t* const* cols, float* tags, cudaMemcpyKind kind) {
+  if (R.n == 0) return;
+  ensure_soa(c, R);
+  if (cols) for (int i = 0; i < R.arity; ++i) if (cols[i]) XLOG_CUDA(cudaMemcpyAsync(cols[i], R.cols[i].p, (size_t)R.n * 4, kind, c->stream));
+  if (tags) XLOG_CUDA(cudaMemcpyAsync(tags, R.tags(), (size_t)R.n * 4, kind, c->stream));
+}
+
+// The same into device memory, in one launch.
 void read_out(Ctx* c, Relation& R, int32_t* const* cols, float* tags) {
   if (R.n == 0) return;
+  bool direct = kernel_can_store(c, tags);
+  for (int i = 0; i < R.arity && direct; ++i) direct = !cols || kernel_can_store(c, cols[i]);
+  if (!direct) { copy_out(c, R, cols, tags, cudaMemcpyDeviceToDevice); return; }
   ReadOut out{};
   uintptr_t low = (uintptr_t)R.keys() | (uintptr_t)R.tags() | (uintptr_t)tags;
   for (int i = 0; i < R.arity; ++i) { out.c[i] = cols ? cols[i] : nullptr; low |= (uintptr_t)out.c[i]; }

@@ -141,11 +141,7 @@ xlog_status xlog_relation_read(xlog_ctx* c, xlog_rel rel, int32_t* const* cols_o
     if (R.is_head && c->idb_dirty) { reset_idb(c); c->idb_dirty = false; }
     if ((int64_t)R.n > capacity) { if (n_out) *n_out = R.n; fail(XLOG_ERR_BUFFER_TOO_SMALL, "capacity smaller than the relation"); }
     if (space == XLOG_MEM_DEVICE) read_out(c, R, cols_out, tags_out);
-    else if (R.n) {
-      ensure_soa(c, R);
-      if (cols_out) for (int i = 0; i < R.arity; ++i) if (cols_out[i]) XLOG_CUDA(cudaMemcpyAsync(cols_out[i], R.cols[i].p, (size_t)R.n * 4, cudaMemcpyDeviceToHost, c->stream));
-      if (tags_out) XLOG_CUDA(cudaMemcpyAsync(tags_out, R.tags(), (size_t)R.n * 4, cudaMemcpyDeviceToHost, c->stream));
-    }
+    else copy_out(c, R, cols_out, tags_out, cudaMemcpyDeviceToHost);
     XLOG_CUDA(cudaStreamSynchronize(c->stream));
     if (space == XLOG_MEM_HOST) c->d2h_bytes += (int64_t)R.n * 4 * (R.arity + 1);
     if (n_out) *n_out = R.n;

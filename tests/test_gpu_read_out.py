@@ -45,3 +45,29 @@ def test_dictionary_column():
     assert all(np.array_equal(a, b.cpu().numpy()) for a, b in zip(hc, dc)) and np.array_equal(ht, dt.cpu().numpy())
     assert set(np.unique(hc[0])) <= set(p.facts["src"][0][0].tolist())
     ctx.close()
+
+
+@pytest.mark.parametrize("where", ["pinned", "odd address"])
+def test_destinations_that_only_a_copy_or_a_mapping_reaches(where):
+    """Buffers handed in as device memory that are page-locked host memory (written through its mapping), or that begin between two
+    multiples of 4 (copied): as a copy would have it."""
+    import torch
+    from paper_2609_27203_b200 import xlog
+    r = np.random.default_rng(3)
+    ctx = xlog.Context(arena_bytes=1 << 24, flags=xlog.FLAG_PROFILE)
+    rel = ctx.relation(3, "maxplus")
+    ctx.load(rel, [r.integers(0, 1 << 20, 777).astype(np.int32) for _ in range(3)], r.random(777).astype(np.float32))
+    hc, ht = ctx.read(rel)
+    n = len(ht)
+    raw = torch.zeros(4, 4 * n + 16, dtype=torch.uint8, **(dict(pin_memory=True) if where == "pinned" else dict(device="cuda")))
+    at = 4 if where == "pinned" else 2
+    ptrs = (C.c_void_p * 3)(*[raw[i, at:].data_ptr() for i in range(3)])
+    got = C.c_int64()
+    torch.cuda.synchronize()
+    assert ctx._L.xlog_relation_read(ctx._h, rel, ptrs, raw[3, at:].data_ptr(), n, C.byref(got), xlog.MEM_DEVICE) == 0 and got.value == n
+    assert ("k_read_out" in ctx.profile()) == (where == "pinned")
+    out = raw.cpu().numpy()
+    for i in range(3):
+        assert np.array_equal(out[i, at:at + 4 * n].copy().view(np.int32), hc[i])
+    assert np.array_equal(out[3, at:at + 4 * n].copy().view(np.float32), ht) and (out[:, :at] == 0).all() and (out[:, at + 4 * n:] == 0).all()
+    ctx.close()
