@@ -399,6 +399,7 @@ bool group_rule_applies(Ctx* c, const Variant& v, const Relation& H, GroupRule& 
   const int64_t groups = ((int64_t)RA.val_max[0] - a0.add) / a0.mul + 1;
   if (groups > 2 * (int64_t)v.outer.n + 1024) return false;
   const uint32_t slots = (uint32_t)H.col_max[1] + 1;
+  if ((uint64_t)groups * slots > kSortMaxN) return false;      // no relation holds more rows: the join says so where this has them
   if (c->arena.largest_free() < (size_t)groups * (slots * 12 + 4) * 2 + ((size_t)1 << 20)) return false;
   Index& ia = ensure_index(c, RA, 0);
   Index& ib = ensure_index(c, RB, 0);
