@@ -210,6 +210,20 @@ def run_oracle_once(program, mode="seminaive"):
 
 # ------------------------------------------------------------------------------------------------
 MIRROR_JOIN_KERNELS = ("k_res_expand", "k_seg_expand", "k_bm_expand")
+# Kernels whose bytes cross HBM once or hardly at all: what bounds them instead, and why the byte rate beside it says nothing.
+ON_CHIP_KERNELS = {
+    "k_row_fixpoint": ("latency", "every round runs out of shared memory with the looked-up relation in L2: two barriers, a look-up and a candidate read one after the other"),
+    "k_dense_round": ("latency", "every round runs out of shared memory; the rows cross HBM once"),
+    "k_row_sums": ("latency", "every round runs out of shared memory: a chain of dependent L1 / L2 reads and two barriers"),
+    "k_sparse_rows": ("issue", "hash tables in shared memory: half of the issue slots, and one dependent L2 read per row and round"),
+    "k_res_cluster": ("latency", "rounds inside one thread-block cluster: two L2 reads, a distributed-shared-memory read and a cluster barrier a round"),
+    "k_tri_rank": ("issue", "list entries served by L2 and tested against a bitmap in shared memory: 75 % of the issue slots"),
+    "k_tri_rank_small": ("issue", "list entries served by L2, searched in shared memory"),
+    "k_bits_emit": ("issue", "bitmaps of the lists served by L2; the rows cross HBM once"),
+    "k_bits_count": ("issue", "bitmaps of the lists served by L2"),
+    "k_group_rule": ("issue", "an exponential and a dozen instructions per candidate, none of which reaches memory"),
+    "k_group_backward": ("issue", "an exponential and a dozen instructions per candidate, none of which reaches memory"),
+}
 
 
 L2_PEAK_SOURCE = ("measured here: xlog_device_gather, random 4-byte reads of a 64 MB table (L2-resident), 32 bytes per read: the kernels held "
@@ -237,7 +251,7 @@ def roofline_of(program, prof_all, steps, sorting_route):
     achieved = d["bytes"] / (d["ms"] / 1e3) / 1e9 if d["ms"] > 0 else 0.0
     mirror_kernel = dom in MIRROR_JOIN_KERNELS or (dom == "k_join_expand" and not sorting_route and "k_sort_pass" not in prof)
     ratio = traffic_ratios().get((dom, "mirror" if mirror_kernel else "sorting"))
-    bound = "hbm"
+    bound = ON_CHIP_KERNELS[dom][0] if dom in ON_CHIP_KERNELS else "hbm"
     l2 = None
     probes = None
     if dom == "k_tri_edges" and "n_edges" in program.info:
@@ -309,9 +323,8 @@ def roofline_of(program, prof_all, steps, sorting_route):
                         probes_per_s=l2["probes_per_s"], l2_bytes_per_probe=l2["l2_bytes_per_probe"])
         if "issue" in l2:
             roofline["issue"] = l2["issue"]
-    if dom in ("k_row_fixpoint", "k_dense_round"):
-        roofline["limiter"] = ("every round runs out of shared memory with the looked-up relation in L2; the rows cross HBM once, so the HBM "
-                               "fraction says nothing: read ms_per_step and the metric")
+    if dom in ON_CHIP_KERNELS:
+        roofline["limiter"] = ON_CHIP_KERNELS[dom][1] + ": the HBM fraction says nothing, read ms_per_step and the metric"
     if mirror_kernel:
         # the tag-mirror joins move few bytes per candidate by construction; what limits them is said here
         roofline["limiter"] = ("instruction issue; the table, too large for L2, is read from HBM one 128-byte line per (changed unit of 32 keys, neighbour)"
@@ -424,7 +437,8 @@ def config_of(args_workload, m, world):
             "derived_tuples": m["derived"], "rounds": receipt["iterations"], "candidates": receipt["candidates"],
             "triangle_plan": {0: None, 1: "wcoj", 2: "chain"}[receipt["triangle_plan"]],
             "unique_candidates": receipt["unique_candidates"], "l2": "flushed between steps (256 MB fill)",
-            "parallelism": "replicas only" if world > 1 else "1 gpu", "facts": "resident and indexed before timing"}
+            "parallelism": "replicas only" if world > 1 else "1 gpu", "facts": "resident and indexed before timing",
+            "step": "xlog_fixpoint: the derived relation is left as packed sorted keys and tags; unpacking it into columns belongs to reading it (in e2e)"}
 
 
 def run_ours(args):

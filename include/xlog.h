@@ -82,12 +82,13 @@ typedef struct {
 #define XLOG_FLAG_NO_GROUPED_JOIN 128u  /* tag mirror: always the row-wise join, never the grouped one (see csrc/group_join.cuh) */
 #define XLOG_FLAG_NO_BITMAP_JOIN  256u  /* tag mirror, grouped join: always from a delta row list, never straight from the changed bitmap (see csrc/bitmap_join.cuh) */
 #define XLOG_FLAG_NO_DENSE_DOUBLING 512u /* tag mirror: the path-doubling rule h(x,z) :- h(x,y), h(y,z) goes through the sorting route, not the dense rounds */
-#define XLOG_FLAG_NO_TRIANGLE_BITMAP 1024u /* fused triangle aggregate: always search the longer list, never mark in(x) in a shared-memory bitmap (see csrc/triangle.cuh) */
-#define XLOG_FLAG_NO_ROW_FIXPOINT 2048u /* tag mirror, h(a,c) :- h(a,b), r(b,c): never run the rounds of each a on their own in shared memory (see csrc/row_fixpoint.cuh) */
+#define XLOG_FLAG_NO_TRIANGLE_BITMAP 1024u /* fused triangle aggregate: always search the longer list, never mark in(x) in a shared-memory bitmap (see csrc/triangle.cuh), never order the graph by degree (csrc/tri_rank.cuh) */
+#define XLOG_FLAG_NO_ROW_FIXPOINT 2048u /* h(a,c) :- h(a,b), r(b,c): never run the rounds of each a on their own in shared memory (see csrc/row_fixpoint.cuh, csrc/sparse_rows.cuh, csrc/row_sums.cuh) */
 #define XLOG_FLAG_NO_GRAPH        16u  /* resident rounds are launched one by one instead of as one graph with a WHILE node */
 
 /* Evaluation routes of a recursive component (Algorithm 1).  All of them derive the same relation,
- * bit for bit, and the same receipt counters (unique_candidates excepted, see xlog_receipt).
+ * bit for bit, and the same receipt counters (unique_candidates excepted, see xlog_receipt).  (Under LOGSUMEXP and SUMPROD
+ * the routes agree to rounding; each of them repeats its own results bit for bit.)
  *  - Sorting route: join -> sort -> reduce-by-key -> merge-path difference, as in the paper's kernel table.
  *  - Tag mirror (default where it applies: one MAXPLUS/MINPLUS head relation, every rule with at most one
  *    atom over it and that atom scanned, packed key <= 30 bits, table fits the arena): the relation is a
@@ -106,13 +107,23 @@ typedef struct {
  *    of c): the rule never changes a, so the rounds of each a are independent; after the seed round one launch runs every
  *    a's rounds to the end, a thread block per a with that a's slots in shared memory; several mutually recursive heads
  *    whose rules all read h_i(a, c) :- h_j(a, b), r(b, c) and that share one key layout are handled alike (csrc/row_fixpoint.cuh;
- *    XLOG_FLAG_NO_ROW_FIXPOINT, and the flags that select the routes below, switch it off).
+ *    XLOG_FLAG_NO_ROW_FIXPOINT, and the flags that select the routes below, switch it off).  With more than 8192 possible values
+ *    of c, of any key width, and 4096 to 2^22 of a, each row is kept in a hash table of up to 1024 tuples instead; the few rows
+ *    that are longer go on round by round on the sorting route and are merged with the others, and a relation most of whose
+ *    rows are long is evaluated on another route after all (csrc/sparse_rows.cuh).  LOGSUMEXP / SUMPROD components of this
+ *    shape with one head, at most 8192 possible values of c and 2^27 possible keys run their rounds likewise (csrc/row_sums.cuh).
  *  - Resident rounds (tag mirror with <= 2^24 possible keys): the delta rounds run as one CUDA graph with a
  *    conditional WHILE node and fixed-capacity buffers (Section "GPU-Native Symbolic Substrate": resident
  *    conditional graph, no host reads inside the loop).  The buffers (about 36 bytes per possible key
  *    plus 12 MB) and the instantiated graph stay allocated in the arena from the first such xlog_fixpoint
  *    until the context is destroyed or the relation's key layout changes.  The first call also
- *    creates a private stream that records the graph; nothing else ever runs on it. */
+ *    creates a private stream that records the graph; nothing else ever runs on it.  Up to 2^17 keys, with one rule over the
+ *    head and a looked-up relation that has no run of more than 64 rows (or at most 16384 rows), small rounds run inside one
+ *    thread-block cluster that holds the mirror in shared memory (csrc/res_cluster.cuh).
+ * Outside recursion: a rule h(p', c0 + k1*a + k2*b) :- d(m*p + s, a), e(m'*p + s', b) whose second head column and whose a have
+ * at most 32 values is evaluated and differentiated group by group (csrc/group_rule.cuh); materialised triangle and
+ * four-cycle joins over lists that are dense in a small domain meet them as bitmaps (csrc/bits_join.cuh).  Bitmaps and the
+ * degree-ordered copy of a graph stay in the arena until the relation changes, as join indices do. */
 
 /* ---- context --------------------------------------------------------------- */
 xlog_status xlog_ctx_create(const xlog_config* cfg, xlog_ctx** out);
@@ -136,13 +147,16 @@ xlog_status xlog_relation_load(xlog_ctx* ctx, xlog_rel rel, const int32_t* const
 xlog_status xlog_relation_size(xlog_ctx* ctx, xlog_rel rel, int64_t* n);
 
 /* Copy the relation out in ascending lexicographic key order.  cols_out[c] and
- * tags_out each hold `capacity` elements in `space`; BUFFER_TOO_SMALL if n > capacity. */
+ * tags_out each hold `capacity` elements in `space`; BUFFER_TOO_SMALL if n > capacity.  NULL pointers are left out.  Into HOST
+ * memory, a relation that was derived since is first unpacked into the column view (see below): RESOURCE_EXHAUSTED if
+ * the arena has no room for it. */
 xlog_status xlog_relation_read(xlog_ctx* ctx, xlog_rel rel, int32_t* const* cols_out, float* tags_out,
                                int64_t capacity, int64_t* n_out, xlog_memspace space);
 
 /* Zero-copy DEVICE pointers to the stored columns (Section "Zero-copy
  * interoperability"); borrowed, valid until the relation next changes.  The store keeps packed keys; the column
- * view is built when it is first asked for.  xlog_relation_read into DEVICE memory does not need it. */
+ * view (4 bytes a row and column) is built when it is first asked for, which fails with RESOURCE_EXHAUSTED if the arena has
+ * no room for it.  xlog_relation_read into DEVICE memory does not need it. */
 xlog_status xlog_relation_view(xlog_ctx* ctx, xlog_rel rel, const int32_t** cols /*[arity]*/, const float** tags, int64_t* n);
 
 /* ---- rules: a compiled conjunctive plan ---------------------------------------
@@ -222,7 +236,8 @@ typedef struct {
   int64_t  strata;                 /* components evaluated */
   int64_t  iterations;             /* join rounds over all components, seed rounds included */
   int64_t  derived_tuples;         /* sum over rule heads of rows - loaded facts */
-  int64_t  candidates;             /* join outputs before aggregation */
+  int64_t  candidates;             /* join outputs before aggregation; for the fused triangle aggregate the list entries walked,
+                                      which depend on the kernels that the graph gets */
   int64_t  unique_candidates;      /* after reduce-by-key; -1 if a component was evaluated through a tag mirror,
                                       which never forms the list of distinct candidate keys */
   int64_t  new_tuples;
@@ -230,7 +245,8 @@ typedef struct {
   int64_t  h2d_bytes, d2h_bytes;   /* control traffic of this call (counters only) */
   int64_t  kernel_launches;
   int64_t  peak_arena_bytes;
-  double   device_ms;              /* CUDA-event time of the whole call on the ctx stream */
+  double   device_ms;              /* CUDA-event time of the call on the ctx stream.  Neither it nor peak_arena_bytes holds the column
+                                      views of the derived relations, which are built by the read or view that asks for them */
   int32_t  triangle_plan;          /* XLOG_PLAN_*: how the last materialised triangle or four-cycle join of this call was evaluated */
   int32_t  index_builds;           /* join indices (offsets over a column, permuted sorted copies) built during this call: indices
                                       of relations that did not change since an earlier call are reused, not rebuilt

@@ -272,7 +272,8 @@ inline unsigned grid_for(uint64_t n, int block, int cap = kSMs * 16) {
 }
 
 // Stores to the pinned block instead of a copy command: the copy engine's turn costs 7 us more, and every read waits for it
-// (closure of 1,000 nodes 255 -> 237 us, reachability from 7 sources 685 -> 667 us, 64 digit pairs' evaluation 52 -> 45 us).
+// (reachability from 7 sources 685 -> 667 us, 64 digit pairs' evaluation 52 -> 45 us; closure of 1,000 nodes 278 -> 255 us together with
+// the one wait at an evaluation's end, see sync_ctrl_end).
 static __global__ void k_ctrl_out(const uint64_t* __restrict__ d, uint64_t* __restrict__ h) { h[threadIdx.x] = d[threadIdx.x]; }
 
 // Copy the control block to pinned host memory and wait: the bounded control read of an iteration.

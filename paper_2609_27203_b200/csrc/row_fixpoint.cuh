@@ -20,7 +20,7 @@
 // holds.  Closing a round a lane per bit and laying the candidates out warp by warp, without a barrier: 1,000 nodes and 4,000
 // edges 122 -> 97 us, 300 nodes 43 -> 35 us, 2,400 nodes 536 -> 392 us (before: a thread per bitmap word, one prefix over
 // the whole block, ten steps of search per candidate).  Registers for 6 blocks an SM: with as many as the compiler
-// likes 134, 31 and 567 us; with 8 blocks 92, 37 and 407 us.
+// likes 134, 31 and 567 us; with 8 blocks 92, 37 and 407 us (6 is ahead on the small and the large graph, 8 on the middle one only).
 #pragma once
 #include "common.cuh"
 #include "join.cuh"

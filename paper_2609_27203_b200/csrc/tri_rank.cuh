@@ -3,7 +3,8 @@
 //
 // triangle.cuh finds every directed triangle three times, once from each of its corners, and walks 8.4e8 list entries on
 // an R-MAT 18 graph to do so.  Here the nodes are numbered by degree and a triangle v -> a -> b -> v is found from its lowest
-// corner v, whose lists are short (at most a few hundred entries whatever the hubs): 1.2e8 entries for the same graph.  Its
+// corner v, of whose lists only the higher part is walked (at most sqrt(2 m) entries whatever the hubs; a few hundred on R-MAT
+// graphs): 1.2e8 entries for the same graph.  Its
 // term goes to all three corners.  The tags make that cheap: the term's weight exp(w_va + w_ab + w_bv) is the product of three
 // numbers kept with the edges, and the sums are plain sums in fp64 (for sum-product the tags are such numbers already).
 // Usable while no product of two or three can leave the normal fp32 range, in whatever order a corner sees its factors: |w| <=
@@ -16,9 +17,8 @@
 // A corner a with little to walk is handled by one warp that searches out(a) instead (k_tri_rank_small).  k_tri_rank_groups then
 // adds up each node's parts: its units' sums of both launches and its edges' sums.
 //
-// R-MAT 18 (3.9 M edges, 39 M triangles): 5.51 -> 1.17 ms per evaluation, 0.88 ms of it the two bitmap launches (bound by instruction
-// issue: 75 % of the slots), 0.11 the searched corners; the first one on a
-// new relation, which orders the graph, 5.84 -> 2.59.
+// R-MAT 18 (3.9 M edges, 39 M triangles): 5.47 -> 1.12 ms per evaluation, 0.88 ms of it the two bitmap launches (bound by instruction
+// issue: 75 % of the slots), 0.11 the searched corners; the first one on a new relation, which orders the graph, 5.82 -> 2.42.
 #pragma once
 #include "common.cuh"
 
