@@ -79,6 +79,23 @@ struct ResCluster {
   uint32_t* err;
 };
 
+// This thread's part of the degrees of the keys that changed in a CTA's words, none counted for more than ends the matter.  Out of
+// line: the rounds of short rows never come here, and run 1 % slower with it among them.
+__device__ __noinline__ uint32_t rc_next_candidates(const JoinSpec& S, const uint32_t* words, uint32_t W, uint32_t rank, bool plain, uint32_t domain, uint32_t* err) {
+  uint32_t next = 0;
+  for (uint32_t i = threadIdx.x; i < W; i += kRcBlock)
+    for (uint32_t m = words[i]; m; m &= m - 1) {
+      const uint32_t key = (((i << kRcCtasLog) | rank) << 5) + __ffs(m) - 1;
+      uint32_t deg = 0;
+      if (plain) {
+        const uint32_t pv = (key >> S.s_probe_shift) & S.s_probe_mask;
+        if (pv < domain) deg = __ldg(S.inner_off + pv + 1) - __ldg(S.inner_off + pv);
+      } else deg = join_count_kv<uint32_t>(S, key, 0.f, 0, nullptr, err);
+      next += min(deg, kRcMaxCta + 1);
+    }
+  return next;
+}
+
 static __global__ void __launch_bounds__(256) k_longest_run(const uint32_t* __restrict__ off, int64_t domain, uint32_t* __restrict__ longest) {
   uint32_t n = 0;
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < domain; v += (int64_t)gridDim.x * blockDim.x) n = max(n, off[v + 1] - off[v]);
@@ -123,6 +140,7 @@ __global__ void __launch_bounds__(kRcBlock, 1) k_res_cluster(const __grid_consta
   unsigned long long cand = 0;                       // closed rounds'
   uint32_t round_cand = 0, n_changed = 0, n_new = 0, closed = 0;
   uint32_t verdict = kResOk, par = 0;
+  const uint32_t sure = kRcMaxCand / P.longest;      // rows that have no more candidates than that, whatever their degrees
   bool first = true;
   const uint32_t sm0 = (uint32_t)__cvta_generic_to_shared(rc_smem), mult = (uint32_t)S.inner_mult[0];
   // the usual row: no constants in the scanned atom, the probed column taken as it is, at most one head column copied from the
@@ -221,20 +239,8 @@ __global__ void __launch_bounds__(kRcBlock, 1) k_res_cluster(const __grid_consta
     if (total_imp == 0u) { cand += round_cand; round_cand = 0; ++closed; verdict = kResDone; break; }
     if (rounds0 + closed + 1 >= max_rounds) { cand += round_cand; round_cand = 0; ++closed; verdict = kResCap; break; }
     if (total_imp > kRcMaxRows) break;               // the emit kernel closes this round
-    if (total_imp * (uint64_t)P.longest > kRcMaxCand) {
-      // the changed keys' degrees, none counted for more than ends the matter
-      uint32_t next = 0;
-      for (uint32_t i = threadIdx.x; i < W; i += kRcBlock)
-        for (uint32_t m = rc_smem[chg + i]; m; m &= m - 1) {
-          const uint32_t key = key_of((i << 5) + __ffs(m) - 1);
-          uint32_t deg = 0;
-          if (plain) {
-            const uint32_t pv = (key >> S.s_probe_shift) & S.s_probe_mask;
-            if (pv < domain) deg = __ldg(S.inner_off + pv + 1) - __ldg(S.inner_off + pv);
-          } else deg = join_count_kv<uint32_t>(S, key, 0.f, 0, nullptr, P.err);
-          next += min(deg, kRcMaxCta + 1);
-        }
-      next = __reduce_add_sync(0xffffffffu, next);
+    if (__builtin_expect(total_imp > sure, 0)) {
+      const uint32_t next = __reduce_add_sync(0xffffffffu, rc_next_candidates(S, rc_smem + chg, W, rank, plain, domain, P.err));
       if (threadIdx.x == 0) s_next = 0u;
       __syncthreads();
       if (lane == 0 && next) atomicAdd(&s_next, next);
