@@ -43,7 +43,7 @@ def program(sr, groups, a_top, b_top, c0, k0, k1, mul, more, seed):
     (300, 9, 9, 0, 1, 1, 2, True),
     (40, 14, 16, 1, 1, 1, 1, False),                          # 32 slots, runs of up to 17: a whole warp per row
     (40, 15, 15, 0, 1, 1, 3, True),                           # runs of up to 16: half a warp per row
-    (33, 80, 31, 0, 0, 1, 1, False),                          # d's column does not reach the head: runs of over 32 rows
+    (33, 80, 31, 0, 0, 1, 1, False),                          # d's column does not reach the head: runs of over 32 rows, the join
     (33, 4, 9, 0, 1, 3, 1, True),                             # slots that only some rows reach
     (33, 10, 11, 10, 1, 1, 1, False),                         # 32 slots with a constant
     (33, 11, 11, 10, 1, 1, 1, False),                         # 33: the sorting route

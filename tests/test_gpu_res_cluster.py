@@ -75,7 +75,7 @@ def test_fan_out_of_one_row(deg):
     both(W.sssp_program(s, d, w, source=0), "dist")
 
 
-def test_many_hubs_in_one_round():                            # more block rows than are queued for the block
+def test_many_hubs_in_one_round():                            # long runs in a large relation: grid-wide rounds
     hubs, deg = 600, 2100
     s = np.concatenate([np.zeros(hubs, np.int64), np.repeat(1 + np.arange(hubs), deg)])
     d = np.concatenate([1 + np.arange(hubs), 1000 + (np.repeat(np.arange(hubs), deg) * 7 + np.tile(np.arange(deg), hubs)) % 90000])
