@@ -1,0 +1,341 @@
+// Heavy rounds of the bitmap-driven grouped join (bitmap_join.cuh) as a gather.  In a round that changes most nodes the join
+// relaxes nearly every row of r, and pushing each changed key along r's runs costs a step of a warp, a slot read and a compare per
+// (node, neighbour).  Turned round, every target c takes the minimum (maximum) over the rows r(b, c) that lead to it of the tags of b
+// plus the row's, a column per carried value, in registers; the slots of c are looked at once per run of rows, not once per row.
+//
+//   k_bm_count   totals of the round to come (changed, new keys, candidates, items, neighbour rows), nothing else: the host
+//                chooses between the two directions by them (host_mirror_strata.cuh)
+//   k_bm_snap    closes the round as k_bm_plan does and copies the rows of the nodes with a changed key out of the table: the tags
+//                as they stood when the round began, the carried values that can still derive anything packed together
+//   k_bm_pull    the gather
+//
+// Bound by instruction issue (57 % of the slots) and the reads' latency together; L2 serves 240 G sectors/s of it.  R-MAT 22, 64 sources, a
+// round over 65 million rows of r: 1.08 - 1.18 ms and 0.14 for the copy, pushed 1.4 - 2.0 and 0.2 - 0.3 for the plan; the fixpoint 9.1 -> 7.2.
+// Measured on the way: rows of whole sectors (28 columns in 112 bytes: 1.48), groups that read different banks (1.25), targets' slots a
+// target later (1.32), four rows under way per lane (2 blocks of 256 more per SM, or rows through a ring of cp.async: no gain); a warp
+// to one target with the groups' results shuffled together at its end 1.8: nine instructions a row more.
+//
+// A row of the copy holds all tags of its node, those that did not change in the last round too: what they lead to has been applied
+// in an earlier round and improves nothing now, so relation, rounds and counters are those of the push.
+#pragma once
+#include "bitmap_join.cuh"
+
+namespace xlog {
+
+constexpr int kBpMaxWordsLog2 = 3;                // at most 8 bitmap words (256 carried values) per node
+constexpr int kBpMaxCols = 256;
+constexpr int kBpBlock = 128;
+constexpr int kBpSweeps = 8;                      // rows of r per lane and chunk
+constexpr int kBpChunk = 32 * kBpSweeps;
+constexpr int kBpUnroll = 4;                      // rows of the copy a group has under way
+constexpr int kBpBlocks = 9;                      // resident blocks per SM
+
+// The looked-up relation by its other column: rows (b, tag), those of one target together, in no order among themselves.  Counted,
+// placed by an exclusive scan and dealt out with atomics on one counter per target: 65 million rows over 4.2 million targets in
+// 3.4 ms (0.7 to count, 2.7 to deal out: scattered stores), a sort of (target, row number) and a gather 3.8.
+// A place in `counter[z]`; the lanes that share the target of the first or the second lane left draw together, so that a target
+// that most rows lead to does not serialise them.
+__device__ __forceinline__ uint32_t rev_draw(uint32_t* __restrict__ counter, uint32_t z, bool in) {
+  uint32_t at = 0;
+  unsigned todo = __ballot_sync(0xffffffffu, in);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    if (todo == 0u) break;                         // uniform
+    const int first = __ffs(todo) - 1;
+    const uint32_t zf = __shfl_sync(0xffffffffu, z, first);
+    const bool mine = in && z == zf;
+    const unsigned same = __ballot_sync(0xffffffffu, mine);
+    uint32_t base = 0;
+    if ((int)lane_id() == first) base = atomicAdd(counter + zf, (uint32_t)__popc(same));
+    base = __shfl_sync(0xffffffffu, base, first);
+    if (mine) { at = base + __popc(same & lanemask_lt()); in = false; }
+    todo &= ~same;
+  }
+  if (in) at = atomicAdd(counter + z, 1u);
+  return at;
+}
+constexpr int kRevRows = 4;                       // rows per thread
+static __global__ void __launch_bounds__(256) k_rev_count(uint32_t n, const int32_t* __restrict__ col, uint32_t* __restrict__ counter) {
+  const uint32_t base = blockIdx.x * (256 * kRevRows) + threadIdx.x;
+#pragma unroll
+  for (int i = 0; i < kRevRows; ++i) {
+    const uint32_t r = base + i * 256;
+    rev_draw(counter, r < n ? (uint32_t)col[r] : 0u, r < n);
+  }
+}
+static __global__ void __launch_bounds__(256) k_rev_fill(uint32_t n, const int32_t* __restrict__ b, const int32_t* __restrict__ col, const float* __restrict__ tag, uint32_t* __restrict__ counter,
+                                                         uint2* __restrict__ rows, uint32_t* __restrict__ target) {
+  const uint32_t base = blockIdx.x * (256 * kRevRows) + threadIdx.x;
+  uint32_t z[kRevRows], at[kRevRows];
+#pragma unroll
+  for (int i = 0; i < kRevRows; ++i) { const uint32_t r = base + i * 256; z[i] = r < n ? (uint32_t)col[r] : 0u; }
+#pragma unroll
+  for (int i = 0; i < kRevRows; ++i) at[i] = rev_draw(counter, z[i], base + i * 256 < n);
+#pragma unroll
+  for (int i = 0; i < kRevRows; ++i) {
+    const uint32_t r = base + i * 256;
+    if (r < n) { rows[at[i]] = make_uint2((uint32_t)b[r], __float_as_uint(tag[r])); target[at[i]] = z[i]; }
+  }
+}
+
+struct BmCount {
+  const uint32_t* words;
+  const uint32_t* present;
+  uint32_t n_units;                // a unit: the bitmap words of one thread, max(4, W) of them
+  const uint32_t* off;
+  uint32_t domain;
+  unsigned long long* totals;      // as k_bm_plan's
+  uint32_t* live;                  // W words: carried values with a changed key that has matches
+};
+
+template <int WL>
+__global__ void __launch_bounds__(256) k_bm_count(BmCount P) {
+  constexpr int W = 1 << WL, U = W < 4 ? 4 : W, NB = U / W;
+  __shared__ unsigned long long s_tot[kBmTotals];
+  __shared__ uint32_t s_live[W];
+  if (threadIdx.x < kBmTotals) s_tot[threadIdx.x] = 0;
+  if (threadIdx.x < W) s_live[threadIdx.x] = 0;
+  __syncthreads();
+  uint32_t changed = 0, fresh = 0, live[W];
+  unsigned long long cand = 0, nbrs = 0, items = 0;
+#pragma unroll
+  for (int j = 0; j < W; ++j) live[j] = 0;
+  for (uint32_t u = blockIdx.x * 256 + threadIdx.x; u < P.n_units; u += gridDim.x * 256) {
+    uint32_t m[U];
+#pragma unroll
+    for (int q = 0; q < U / 4; ++q) {
+      const uint4 v = reinterpret_cast<const uint4*>(P.words)[(size_t)u * (U / 4) + q];
+      m[4 * q] = v.x; m[4 * q + 1] = v.y; m[4 * q + 2] = v.z; m[4 * q + 3] = v.w;
+    }
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      uint32_t k = 0;
+#pragma unroll
+      for (int j = 0; j < W; ++j) k += __popc(m[i * W + j]);
+      if (!k) continue;
+      changed += k;
+      const uint32_t b = u * NB + i;
+#pragma unroll
+      for (int j = 0; j < W; ++j) if (m[i * W + j]) fresh += __popc(m[i * W + j] & ~P.present[(size_t)b * W + j]);
+      const uint32_t dg = b < P.domain ? P.off[b + 1] - P.off[b] : 0u;
+      if (!dg) continue;
+      cand += (unsigned long long)k * dg;
+      nbrs += dg;
+      items += (unsigned long long)((dg + kBmSlice - 1) / kBmSlice) * ((k + 31) / 32);
+#pragma unroll
+      for (int j = 0; j < W; ++j) live[j] |= m[i * W + j];
+    }
+  }
+  changed = __reduce_add_sync(0xffffffffu, changed);
+  if (changed) {
+    fresh = __reduce_add_sync(0xffffffffu, fresh);
+#pragma unroll
+    for (int s = 16; s; s >>= 1) { cand += __shfl_down_sync(0xffffffffu, cand, s); nbrs += __shfl_down_sync(0xffffffffu, nbrs, s); items += __shfl_down_sync(0xffffffffu, items, s); }
+#pragma unroll
+    for (int j = 0; j < W; ++j) { live[j] = __reduce_or_sync(0xffffffffu, live[j]); if (lane_id() == 0 && live[j]) atomicOr(&s_live[j], live[j]); }
+    if (lane_id() == 0) {
+      atomicAdd(&s_tot[kBmChanged], (unsigned long long)changed); atomicAdd(&s_tot[kBmNew], (unsigned long long)fresh); atomicAdd(&s_tot[kBmCandidates], cand);
+      atomicAdd(&s_tot[kBmNeighbours], nbrs); atomicAdd(&s_tot[kBmReserve], items << 32);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < kBmTotals && s_tot[threadIdx.x]) atomicAdd(P.totals + threadIdx.x, s_tot[threadIdx.x]);
+  if (threadIdx.x < W) { const uint32_t v = s_live[threadIdx.x]; if (v & ~P.live[threadIdx.x]) atomicOr(P.live + threadIdx.x, v); }
+}
+
+// Columns of the copy: position 4 l + k of part y holds live carried value number (4 y + k) lanes + l, so that the k-th slots of the
+// lanes of a row lie side by side in the table.
+struct BpColumns {
+  int lanes, parts;                // lanes to a row of a part, four columns each
+  int16_t at[kBpMaxCols];          // carried value at a position, -1: none
+};
+
+struct BmSnap {
+  uint32_t* words;
+  uint32_t* present;
+  uint32_t n_units;
+  const uint32_t* off;
+  uint32_t domain;
+  const int32_t* table;
+  int carried_bits;
+  uint32_t* any;                   // out: bitmap of the nodes with a changed key that has matches
+  float* copy;                     // out: their rows
+};
+
+template <int WL>
+__global__ void __launch_bounds__(256) k_bm_snap(const __grid_constant__ BmSnap P, const __grid_constant__ BpColumns C) {
+  constexpr int W = 1 << WL, U = W < 4 ? 4 : W, NB = U / W;
+  constexpr int kAnyWords = 256 * NB / 32;
+  __shared__ uint32_t s_any[kAnyWords], s_node[256 * NB], s_n;
+  if (threadIdx.x < kAnyWords) s_any[threadIdx.x] = 0;
+  if (threadIdx.x == 0) s_n = 0;
+  __syncthreads();
+  const uint32_t u = blockIdx.x * 256 + threadIdx.x;
+  if (u < P.n_units) {
+    uint32_t m[U];
+    uint32_t some = 0;
+#pragma unroll
+    for (int q = 0; q < U / 4; ++q) {
+      const uint4 v = reinterpret_cast<const uint4*>(P.words)[(size_t)u * (U / 4) + q];
+      m[4 * q] = v.x; m[4 * q + 1] = v.y; m[4 * q + 2] = v.z; m[4 * q + 3] = v.w;
+      some |= v.x | v.y | v.z | v.w;
+    }
+    if (some) {
+#pragma unroll
+      for (int q = 0; q < U / 4; ++q) {
+        uint4* pp = reinterpret_cast<uint4*>(P.present) + (size_t)u * (U / 4) + q;
+        uint4 p = *pp;
+        p.x |= m[4 * q]; p.y |= m[4 * q + 1]; p.z |= m[4 * q + 2]; p.w |= m[4 * q + 3];
+        *pp = p;
+        reinterpret_cast<uint4*>(P.words)[(size_t)u * (U / 4) + q] = make_uint4(0u, 0u, 0u, 0u);
+      }
+#pragma unroll
+      for (int i = 0; i < NB; ++i) {
+        uint32_t k = 0;
+#pragma unroll
+        for (int j = 0; j < W; ++j) k |= m[i * W + j];
+        const uint32_t b = u * NB + i;
+        if (k && b < P.domain && P.off[b + 1] != P.off[b]) {
+          const uint32_t local = threadIdx.x * NB + i;
+          atomicOr(&s_any[local >> 5], 1u << (local & 31));
+          s_node[atomicAdd(&s_n, 1u)] = b;
+        }
+      }
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < kAnyWords) P.any[(size_t)blockIdx.x * kAnyWords + threadIdx.x] = s_any[threadIdx.x];
+  const uint32_t quads = (uint32_t)(C.lanes * C.parts), work = s_n * quads;
+  for (uint32_t i = threadIdx.x; i < work; i += 256) {
+    const uint32_t r = i / quads, q = i - r * quads, b = s_node[r];
+    const int32_t* row = P.table + ((size_t)b << P.carried_bits);
+    float v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) { const int a = C.at[4 * q + k]; v[k] = a >= 0 ? ord2f(__ldcg(row + a)) : __int_as_float(0x7fffffff); }
+    reinterpret_cast<float4*>(P.copy)[(size_t)b * quads + q] = make_float4(v[0], v[1], v[2], v[3]);
+  }
+}
+
+struct BmPull {
+  const uint2* rows;               // (b, tag) by target
+  const uint32_t* target;
+  uint32_t n_rows;
+  const uint32_t* any;
+  uint32_t n_nodes;                // nodes that the mirror has slots for
+  const float4* copy;
+  uint32_t z_max;                  // largest value the head's second column may take
+  int carried_bits;
+  int32_t* table;
+  uint32_t* changed;
+  uint32_t* err;
+};
+
+// A warp takes kBpChunk rows of r (neighbours in the order of targets; blockIdx.y: a part of the columns) and splits them among its
+// groups of lanes, a row of the copy to a group and step.  A target's slots are read when its last row has been met and looked at when
+// the next target's has.  An empty slot is a NaN in the copy, and min / max pass a NaN over.  FILTER: rows whose b has not changed are
+// dropped first; without it they take part with what the copy last held of b (empty, or tags that have been applied), which is
+// cheaper where few would be dropped: the look at the bitmap is a wavefront a row, as much as fetching the row.
+template <int SINK, bool FILTER>
+__global__ void __launch_bounds__(kBpBlock, kBpBlocks) k_bm_pull(const __grid_constant__ BmPull P, const __grid_constant__ BpColumns C) {
+  __shared__ uint2 s_row[kBpBlock / 32][kBpChunk];
+  __shared__ uint32_t s_target[kBpBlock / 32][kBpChunk];
+  const unsigned lane = lane_id(), wid = warp_id();
+  const uint32_t base = (blockIdx.x * (kBpBlock / 32) + wid) * kBpChunk;
+  if (base >= P.n_rows) return;
+  const uint32_t G = (uint32_t)C.lanes, quads = G * (uint32_t)C.parts, first_quad = blockIdx.y * G;
+  uint2* const rows = s_row[wid];
+  uint32_t* const target = s_target[wid];
+  uint32_t n = 0;
+  {
+    uint2 r[kBpSweeps];
+    uint32_t z[kBpSweeps], bits[kBpSweeps];
+#pragma unroll
+    for (int i = 0; i < kBpSweeps; ++i) {
+      const uint32_t e = base + i * 32 + lane;
+      r[i] = e < P.n_rows ? __ldcs(P.rows + e) : make_uint2(0xffffffffu, 0u);
+      z[i] = e < P.n_rows ? __ldcs(P.target + e) : 0u;
+    }
+#pragma unroll
+    for (int i = 0; i < kBpSweeps; ++i) bits[i] = r[i].x < P.n_nodes ? (FILTER ? __ldg(P.any + (r[i].x >> 5)) : 0xffffffffu) : 0u;
+#pragma unroll
+    for (int i = 0; i < kBpSweeps; ++i) {
+      bool in = (bits[i] >> (r[i].x & 31)) & 1u;
+      if (in && z[i] > P.z_max) {                  // a candidate there ends the fixpoint
+        if (FILTER || ((P.any[r[i].x >> 5] >> (r[i].x & 31)) & 1u)) atomicOr(P.err, kErrHeadRange);
+        in = false;
+      }
+      const unsigned bal = __ballot_sync(0xffffffffu, in);
+      if (in) {
+        const uint32_t at = n + __popc(bal & lanemask_lt());
+        rows[at] = make_uint2(r[i].x * quads + first_quad, r[i].y);
+        target[at] = z[i];
+      }
+      n += __popc(bal);
+    }
+  }
+  __syncwarp();
+  if (n == 0) return;
+  const uint32_t groups = 32 / G, g = lane / G, l = lane - g * G;
+  const uint32_t per = ((n + groups - 1) / groups) | 1u;                // odd: the groups read different banks
+  const uint32_t e0 = g < groups ? min(g * per, n) : n, e1 = min(e0 + per, n);
+  if (e0 >= e1) return;
+  int col[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) col[k] = max((int)C.at[4 * (first_quad + l) + k], 0);
+  const float none = __int_as_float(0x7fffffff);
+  const int32_t never = SINK == kSinkMin ? 0x7fffffff : (int32_t)0x80000000;
+  auto better = [](float a, float b) { return SINK == kSinkMin ? fminf(a, b) : fmaxf(a, b); };
+  float acc[4] = {none, none, none, none};
+  int32_t met[4], old[4];                          // the target before: its result and its slots
+#pragma unroll
+  for (int k = 0; k < 4; ++k) met[k] = old[k] = never;
+  uint32_t cur = target[e0], before = cur;
+  auto settle = [&]() {                            // the target before
+    bool up[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) up[k] = SINK == kSinkMin ? met[k] < old[k] : met[k] > old[k];
+    if (!(up[0] | up[1] | up[2] | up[3])) return;
+    const uint32_t zq = before << P.carried_bits;
+    int32_t* const slots = P.table + zq;
+    uint32_t* const words = P.changed + (zq >> 5);
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (up[k]) {
+        if (SINK == kSinkMin) atomicMin(slots + col[k], met[k]); else atomicMax(slots + col[k], met[k]);
+        atomicOr(words + (col[k] >> 5), 1u << (col[k] & 31));
+      }
+  };
+  auto turn = [&]() {                              // cur is complete: it becomes the target before, its slots on their way
+    const int32_t* const slots = P.table + (cur << P.carried_bits);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      met[k] = acc[k] == acc[k] ? f2ord(acc[k]) : never;      // a column that is none has met nothing
+      old[k] = __ldcg(slots + col[k]);
+      acc[k] = none;
+    }
+    before = cur;
+  };
+  const float4* const copy = P.copy + l;
+  for (uint32_t e = e0; e < e1; e += kBpUnroll) {
+    uint2 r[kBpUnroll];
+    float4 s[kBpUnroll];
+#pragma unroll
+    for (int u = 0; u < kBpUnroll; ++u) {
+      r[u] = rows[min(e + u, e1 - 1)];
+      s[u] = __ldcg(copy + r[u].x);
+    }
+#pragma unroll
+    for (int u = 0; u < kBpUnroll; ++u) {
+      if (e + u >= e1) break;
+      const uint32_t z = target[e + u];
+      if (z != cur) { settle(); turn(); cur = z; }
+      const float w = __uint_as_float(r[u].y);
+      acc[0] = better(acc[0], s[u].x + w); acc[1] = better(acc[1], s[u].y + w); acc[2] = better(acc[2], s[u].z + w); acc[3] = better(acc[3], s[u].w + w);
+    }
+  }
+  settle();
+  turn();
+  settle();
+}
+
+}  // namespace xlog

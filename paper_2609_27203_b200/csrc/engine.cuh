@@ -89,6 +89,15 @@ struct TriRankIndex {
   DevBuf rank, off[2], split[2], nbr[2], num[2], other, unit_off[2], unit[2];      // [0] out-lists, [1] in-lists; units of the launch by a, by b
 };
 
+// The rows of a binary relation by their second column, for the gather of bitmap_pull.cuh.  Made by the second evaluation that
+// wants them (they cost two evaluations' gain), kept with the relation while the arena has room to spare: whatever else does not fit
+// takes their place (DevBuf, free_block).
+struct RevLists {
+  bool valid = false, in_use = false;
+  int64_t wanted = 0;                   // number of the evaluation that first did
+  DevBuf rows, target;
+};
+
 struct Relation {
   int arity = 0, sr = 0;
   std::string name;
@@ -111,6 +120,7 @@ struct Relation {
   bool soa_valid = false;
   Index idx[kMaxArity];
   TriRankIndex tri;
+  RevLists rev;
   bool is_head = false;
 
   DictSet dicts() const {
@@ -169,6 +179,7 @@ struct Ctx {
   uint64_t* d_ctrl = nullptr;
   uint64_t* h_ctrl = nullptr;
   int64_t launches = 0, d2h_bytes = 0, h2d_bytes = 0;
+  int64_t evaluations = 0;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   int64_t ended_at = -1;                  // launch count at the last sync_ctrl_end
   // receipt counters of the running fixpoint
@@ -188,8 +199,23 @@ struct Ctx {
   std::vector<char> stratum_done;         // per relation: its stratum has been evaluated in the running fixpoint
 };
 
+// Give back what is only kept to save time.  Work that reads it is ahead of whatever reuses the memory on the context's one stream.
+inline bool drop_spare(Ctx* c) {
+  bool any = false;
+  for (Relation* R : c->rels)
+    if (R->rev.valid && !R->rev.in_use) { const int64_t w = R->rev.wanted; R->rev = RevLists(); R->rev.wanted = w; any = true; }
+  return any;
+}
+// The largest free block, for a choice that wants `wanted` bytes: as large as if nothing were kept, where that matters.
+inline size_t free_block(Ctx* c, uint64_t wanted) {
+  size_t n = c->arena.largest_free();
+  if (n < wanted && drop_spare(c)) n = c->arena.largest_free();
+  return n;
+}
+
 inline DevBuf::DevBuf(Ctx* ctx, size_t n) : c(ctx), bytes(n) {
   p = ctx->arena.alloc(n);
+  if (!p && drop_spare(ctx)) p = ctx->arena.alloc(n);
   if (!p) {
     char m[160];
     snprintf(m, sizeof m, "arena exhausted: need %zu bytes, %zu of %zu in use, largest free block %zu", n,

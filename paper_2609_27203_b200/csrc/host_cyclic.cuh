@@ -88,7 +88,8 @@ bool ensure_tri_rank(Ctx* c, Relation& E, Index& out_ix, Index& in_ix, bool lse)
   if (!X.checked) check_tri_rank(c, E, out_ix, in_ix, lse);
   if (!X.fit) return false;
   const uint32_t N = (uint32_t)std::max(out_ix.domain, in_ix.domain), m = E.n;
-  if ((size_t)m * 64 + (size_t)N * 64 + (4u << 20) > c->arena.largest_free() / 2) return false;
+  const size_t order_bytes = (size_t)m * 64 + (size_t)N * 64 + (4u << 20);
+  if (order_bytes > free_block(c, order_bytes * 2) / 2) return false;
   const int32_t* src = E.cols[0].as<int32_t>(); const int32_t* dst = E.cols[1].as<int32_t>();
   unsigned long long* tot = (unsigned long long*)(c->d_ctrl + kSlotTrk);
   zero_ctrl(c, kSlotTrk, kTrkTotals);
@@ -301,7 +302,7 @@ bool bits_join_applies(Ctx* c, const Relation& A, const Index& aix, const Relati
   if (words > kBitsMaxWords) return false;
   if ((uint64_t)A.n * kBitsSparsest < (uint64_t)aix.domain * words * 32 || (uint64_t)B.n * kBitsSparsest < (uint64_t)bix.domain * words * 32) return false;
   const size_t bytes = (size_t)(aix.domain + bix.domain) * words * 6;
-  return bytes <= kBitsMaxBytes && bytes <= c->arena.largest_free() / 4;
+  return bytes <= kBitsMaxBytes && bytes <= free_block(c, bytes * 4) / 4;
 }
 BitsLists ensure_bits(Ctx* c, Index& ix, uint32_t words) {
   if (ix.bit_words != words) {
@@ -434,7 +435,7 @@ void triangle_materialise(Ctx* c, Relation& H, const RuleC& r) {
     q.deg.reset(); q.sums.reset();
     const uint64_t biggest = std::max<uint64_t>(R.n, std::max<uint64_t>(S.n, T.n));
     const size_t need = (size_t)q.total * (H2.key_bytes + 4 + 12) + (16u << 20);
-    const bool fits = q.total <= kSortMaxN && need <= c->arena.largest_free() / 2;
+    const bool fits = q.total <= kSortMaxN && need <= free_block(c, need * 2) / 2;
     if (!(c->flags & XLOG_FLAG_FORCE_CHAIN)) chain = fits && q.total <= kChainMaxBlowup * biggest;
     else if (!fits) fail(XLOG_ERR_RESOURCE_EXHAUSTED, "triangle chain: the two-path intermediate does not fit the arena");
     if (chain) {
@@ -524,7 +525,7 @@ void cycle4_materialise(Ctx* c, Relation& H, const RuleC& r) {
   const int ckb = H2.key_bytes;
   const size_t need = (size_t)n2 * (ckb + 4 + 12) + (16u << 20);
   if (n2 > kSortMaxN) fail(XLOG_ERR_CAPACITY_EXCEEDED, "four-cycle: more than 2^30 - 1 two-paths");
-  if (need > c->arena.largest_free() / 2) fail(XLOG_ERR_RESOURCE_EXHAUSTED, "four-cycle: the two-paths do not fit the arena");
+  if (need > free_block(c, need * 2) / 2) fail(XLOG_ERR_RESOURCE_EXHAUSTED, "four-cycle: the two-paths do not fit the arena");
   c->r_candidates += (int64_t)n2;
   if (n2 == 0) { KeyTags empty; set_current(H, std::move(empty)); return; }
   c->last_triangle_plan = XLOG_PLAN_WCOJ;
@@ -560,7 +561,7 @@ void cycle4_materialise(Ctx* c, Relation& H, const RuleC& r) {
     const uint64_t n3 = c->h_ctrl[kSlotTotals];
     const uint64_t biggest = std::max<uint64_t>(std::max<uint64_t>(R.n, S.n), std::max<uint64_t>(T.n, U.n));
     const size_t need3 = (size_t)n3 * (kb3 + 4 + 12) + (16u << 20);
-    const bool fits = L3.total_bits <= 64 && n3 <= kSortMaxN && need3 <= c->arena.largest_free() / 2;
+    const bool fits = L3.total_bits <= 64 && n3 <= kSortMaxN && need3 <= free_block(c, need3 * 2) / 2;
     bool chain = fits && n3 <= kChainMaxBlowup * biggest;
     if (c->flags & XLOG_FLAG_FORCE_CHAIN) {
       if (!fits) fail(XLOG_ERR_RESOURCE_EXHAUSTED, "four-cycle chain: the three-path intermediate does not fit the arena");

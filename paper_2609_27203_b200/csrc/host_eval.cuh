@@ -312,7 +312,7 @@ KeyTags evaluate(Ctx* c, Relation& H, std::vector<Variant>& variants, const Sour
   {
     // besides the two candidate buffers a batch needs sort status words (1/4 B per row), the reduce's
     // spill tables (up to 2 B per row) and a few MB of per-group arrays
-    const size_t free_bytes = c->arena.largest_free();
+    const size_t free_bytes = free_block(c, cap * (per + 3) + (6u << 20));
     const uint64_t fit = free_bytes > (6u << 20) ? (free_bytes - (6u << 20)) / (per + 3) : 1;
     if (fit < cap) cap = std::max<uint64_t>(fit, 1);
   }
@@ -400,7 +400,8 @@ bool group_rule_applies(Ctx* c, const Variant& v, const Relation& H, GroupRule& 
   if (groups > 2 * (int64_t)v.outer.n + 1024) return false;
   const uint32_t slots = (uint32_t)H.col_max[1] + 1;
   if ((uint64_t)groups * slots > kSortMaxN) return false;      // no relation holds more rows: the join says so where this has them
-  if (c->arena.largest_free() < (size_t)groups * (slots * 12 + 4) * 2 + ((size_t)1 << 20)) return false;
+  const size_t rule_bytes = (size_t)groups * (slots * 12 + 4) * 2 + ((size_t)1 << 20);
+  if (free_block(c, rule_bytes) < rule_bytes) return false;
   Index& ia = ensure_index(c, RA, 0);
   Index& ib = ensure_index(c, RB, 0);
   P = GroupRule{};

@@ -3,7 +3,7 @@
 // Host-side driver code of the engine; included by xlog_api.cu only (one translation unit).
 #pragma once
 #include "host_eval.cuh"
-#include "bitmap_join.cuh"
+#include "bitmap_pull.cuh"
 #include "dense_closure.cuh"
 #include "group_join.cuh"
 #include "mirror.cuh"
@@ -72,7 +72,7 @@ bool mirror_applies(Ctx* c, const std::vector<int>& comp, const std::vector<cons
   }
   uint64_t need = ((uint64_t)4 << H.layout.total_bits) + ((uint64_t)1 << H.layout.total_bits) / 4 + (1u << 20);
   if (doubling_rule_of(c, comp[0], rs)) need += (uint64_t)4 << H.layout.total_bits;       // the snapshot of the matrix
-  return need <= c->arena.largest_free() / 2;
+  return need <= free_block(c, need * 2) / 2;
 }
 
 // ---- resident rounds (resident.cuh) --------------------------------------------------------------------
@@ -93,7 +93,7 @@ Resident* resident_for(Ctx* c, int h, int bits, uint64_t slots, uint32_t bm_quad
   c->resident.erase(h);
   const uint64_t dom = (uint64_t)1 << bits;
   const uint64_t need = slots * 4 + (uint64_t)bm_quads * 32 + dom * 32 + (uint64_t)max_tiles * 8 + (4u << 20);
-  if (need > c->arena.largest_free() / 3) return nullptr;
+  if (need > free_block(c, need * 3) / 3) return nullptr;
   std::unique_ptr<Resident> R(new Resident());
   R->slots = slots; R->max_tiles = max_tiles;
   R->table = DevBuf(c, slots * 4);
@@ -434,6 +434,7 @@ struct BitmapJoin {
   JoinSpec spec;
   DevBuf pairs, items;
   int carried_bits = 0;
+  Relation* rel = nullptr;                                // the looked-up relation
 };
 
 // Applicable when exactly one rule has an atom over h (so a round is one join), that rule has the grouped shape with the
@@ -453,18 +454,117 @@ void bitmap_join_setup(Ctx* c, int h, const std::vector<const RuleC*>& rs, const
   if (!S.fast || !S.has_inner || S.inner_free != 1 || S.outer_decode[0] || S.outer_decode[1] || S.head_encode[0] || S.head_encode[1] ||
       S.inner_mult[0] != ((uint64_t)1 << carried_bits))
     return;
-  const Relation& RB = *c->rels[rule->plan.atoms[1 - pos].rel];
+  Relation& RB = *c->rels[rule->plan.atoms[1 - pos].rel];
   const uint64_t passes = (uint64_t)1 << (carried_bits - 5);             // at most one pass per 32 carried values
   const uint64_t values = std::min<uint64_t>((uint64_t)S.inner_domain, slots >> carried_bits);
   const uint64_t max_items = ((uint64_t)RB.n / kBmSlice + values + 1) * passes;
   if (max_items >= ((uint64_t)1 << 32)) return;
   const uint64_t need = slots * 8 + max_items * 16 + (1u << 20);          // a round can change every key: one (tag, carried value) pair each
-  if (need > c->arena.largest_free() / 2) return;
+  if (need > free_block(c, need * 2) / 2) return;
   bj.pairs = DevBuf(c, slots * 8);
   bj.items = DevBuf(c, max_items * 16);
   bj.spec = S;
   bj.carried_bits = carried_bits;
+  bj.rel = &RB;
   bj.valid = true;
+}
+
+// The rows of a binary relation by their second column (bitmap_pull.cuh).
+void build_rev_lists(Ctx* c, Relation& R) {
+  ensure_soa(c, R);
+  RevLists L;
+  const uint32_t domain = (uint32_t)R.val_max[1] + 1u;
+  L.rows = DevBuf(c, (size_t)R.n * 8);
+  L.target = DevBuf(c, (size_t)R.n * 4);
+  DevBuf cnt(c, (size_t)domain * 4), at(c, (size_t)domain * 4);
+  const unsigned grid = (R.n + 256 * kRevRows - 1) / (256 * kRevRows);
+  XLOG_CUDA(cudaMemsetAsync(cnt.p, 0, (size_t)domain * 4, c->stream));
+  XLOG_LAUNCH(c, k_rev_count, grid, 256, 0, R.n, (const int32_t*)R.cols[1].as<int32_t>(), cnt.as<uint32_t>());
+  exclusive_scan_u32(c, cnt.as<uint32_t>(), domain, at.as<uint32_t>(), ctrl_u32(c, kSlotA));
+  XLOG_LAUNCH(c, k_rev_fill, grid, 256, 0, R.n, (const int32_t*)R.cols[0].as<int32_t>(), (const int32_t*)R.cols[1].as<int32_t>(), (const float*)R.tags(), at.as<uint32_t>(),
+              L.rows.as<uint2>(), L.target.as<uint32_t>());
+  L.valid = true;
+  L.wanted = R.rev.wanted;
+  R.rev = std::move(L);
+}
+
+// The gather of a stratum's heavy rounds: the copy of the changed nodes' rows, their bitmap, the columns in use.
+constexpr int kSlotBmLive = 91;            // the carried values that can derive anything, one bit each
+static_assert((1 << kBpMaxWordsLog2) * 4 <= (kCtrlSlots - kSlotBmLive) * 8, "control block too small");
+
+struct BitmapPull {
+  bool usable = false;
+  int words_log2 = 0;
+  uint32_t n_units = 0, blocks = 0;
+  int n_cols = -1;
+  BpColumns cols{};
+  DevBuf copy, any;
+  RevLists* lists = nullptr;
+  ~BitmapPull() { if (lists) lists->in_use = false; }
+};
+
+template <int WL> void launch_bm_count_w(Ctx* c, const BmCount& P) { XLOG_LAUNCH(c, k_bm_count<WL>, grid_for(P.n_units, 256, kSMs * 8), 256, 0, P); }
+void launch_bm_count(Ctx* c, int words_log2, const BmCount& P) {
+  switch (words_log2) {
+    case 0: launch_bm_count_w<0>(c, P); break;
+    case 1: launch_bm_count_w<1>(c, P); break;
+    case 2: launch_bm_count_w<2>(c, P); break;
+    default: launch_bm_count_w<3>(c, P); break;
+  }
+}
+template <int WL> void launch_bm_snap_w(Ctx* c, unsigned blocks, const BmSnap& P, const BpColumns& C) { XLOG_LAUNCH(c, k_bm_snap<WL>, blocks, 256, 0, P, C); }
+void launch_bm_snap(Ctx* c, int words_log2, unsigned blocks, const BmSnap& P, const BpColumns& C) {
+  switch (words_log2) {
+    case 0: launch_bm_snap_w<0>(c, blocks, P, C); break;
+    case 1: launch_bm_snap_w<1>(c, blocks, P, C); break;
+    case 2: launch_bm_snap_w<2>(c, blocks, P, C); break;
+    default: launch_bm_snap_w<3>(c, blocks, P, C); break;
+  }
+}
+
+template <int SINK> void launch_bm_pull_s(Ctx* c, bool filter, dim3 grid, const BmPull& P, const BpColumns& C) {
+  if (filter) XLOG_LAUNCH(c, (k_bm_pull<SINK, true>), grid, kBpBlock, 0, P, C);
+  else XLOG_LAUNCH(c, (k_bm_pull<SINK, false>), grid, kBpBlock, 0, P, C);
+}
+void launch_bm_pull(Ctx* c, bool is_max, bool filter, dim3 grid, const BmPull& P, const BpColumns& C) {
+  if (is_max) launch_bm_pull_s<kSinkMax>(c, filter, grid, P, C); else launch_bm_pull_s<kSinkMin>(c, filter, grid, P, C);
+}
+
+// Which carried values the copy holds, from the bits of kSlotBmLive (read with the totals): the values of the keys changed in the
+// seed round that have matches, and every later key carries one of them.
+void bitmap_pull_columns(Ctx* c, BitmapPull& bp) {
+  const uint32_t* live = reinterpret_cast<const uint32_t*>(c->h_ctrl + kSlotBmLive);
+  std::vector<int16_t> a;
+  for (int i = 0; i < (32 << bp.words_log2); ++i) if ((live[i >> 5] >> (i & 31)) & 1u) a.push_back((int16_t)i);
+  bp.n_cols = (int)a.size();
+  bp.cols.parts = std::max(1, (bp.n_cols + 127) / 128);
+  bp.cols.lanes = std::max(2, (bp.n_cols + 8 * bp.cols.parts - 1) / (8 * bp.cols.parts) * 2);      // rows of whole 32-byte sectors
+  const int G = bp.cols.lanes;
+  for (int i = 0; i < kBpMaxCols; ++i) bp.cols.at[i] = -1;
+  for (int y = 0; y < bp.cols.parts; ++y)
+    for (int l = 0; l < G; ++l)
+      for (int k = 0; k < 4; ++k) {
+        const int j = (4 * y + k) * G + l;
+        if (j < bp.n_cols) bp.cols.at[4 * (y * G + l) + k] = a[j];
+      }
+}
+
+// Buffers and lists for the gather, once a round wants it.  False: it is the first evaluation that does, or they do not fit with room to
+// spare; the rounds stay as they are.
+bool bitmap_pull_begin(Ctx* c, BitmapJoin& bj, BitmapPull& bp, uint64_t n_nodes) {
+  if (bp.lists) return true;
+  Relation& R = *bj.rel;
+  if (!R.rev.valid && (R.rev.wanted == 0 || R.rev.wanted == c->evaluations)) { R.rev.wanted = c->evaluations; bp.usable = false; return false; }
+  const uint64_t copy = (n_nodes + 1) * 16 * (uint64_t)(bp.cols.lanes * bp.cols.parts);
+  const uint64_t need = copy + (uint64_t)bp.blocks * 128 + (R.rev.valid ? 0 : (uint64_t)R.n * 12 + (uint64_t)R.val_max[1] * 8) + (4u << 20);
+  if (need > c->arena.largest_free() / 2 || copy / 16 > 0xffffffffull) { bp.usable = false; return false; }
+  if (!R.rev.valid) build_rev_lists(c, R);
+  R.rev.in_use = true;
+  bp.lists = &R.rev;
+  bp.copy = DevBuf(c, copy);
+  bp.any = DevBuf(c, (size_t)bp.blocks * 128);
+  XLOG_CUDA(cudaMemsetAsync(bp.copy.p, 0xff, copy, c->stream));          // no tags
+  return true;
 }
 
 }  // namespace

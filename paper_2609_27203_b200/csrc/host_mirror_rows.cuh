@@ -74,7 +74,7 @@ bool row_fixpoint_applies(Ctx* c, const std::vector<int>& comp, const std::vecto
   if (rules.empty() || rules.size() > (size_t)kRowMaxRules) return false;
   uint64_t need = 1u << 20;
   for (int h : comp) need += ((uint64_t)4 << c->rels[h]->layout.total_bits) + ((uint64_t)1 << c->rels[h]->layout.total_bits) / 4 + (1u << 16);
-  return need <= c->arena.largest_free() / 2;
+  return need <= free_block(c, need * 2) / 2;
 }
 
 // The stratum by the row-local route: the seed round from the host (every rule over the full relations, into the tables),
@@ -213,7 +213,7 @@ bool row_sums_applies(Ctx* c, const std::vector<int>& comp, const std::vector<co
   const Relation& H = *c->rels[comp[0]];
   if (H.arity != 2 || H.key_bytes != 4 || H.dict_n[1] || H.layout.shift[1] != 0) return false;
   if (H.layout.shift[0] > kRowMaxBits || H.layout.total_bits > kRowSumMaxBits) return false;
-  if (((uint64_t)16 << H.layout.total_bits) > c->arena.largest_free()) return false;       // the table, and a relation as large as it
+  if (((uint64_t)16 << H.layout.total_bits) > free_block(c, (uint64_t)16 << H.layout.total_bits)) return false;       // the table, and a relation as large as it
   rules.clear();
   for (const RuleC* r : rs) {
     int pos = -1, in = 0;
@@ -362,11 +362,11 @@ SparseOutcome sparse_rows_rounds(Ctx* c, Relation& H, const JoinSpec& S, uint32_
   const uint32_t n_rows = (uint32_t)H.col_max[0] + 1;
   const uint32_t max_q0 = n_rows / 8 + 1024, max_q1 = n_rows / 64 + 128;
   const size_t fixed = (size_t)n_rows * 44 + (size_t)r_rows * 16 + (size_t)(max_q0 + 2 * max_q1) * 4 + (1u << 20);
-  if (fixed > c->arena.largest_free() / 2) return kSparseFailed;
+  if (fixed > free_block(c, fixed * 2) / 2) return kSparseFailed;
   const bool same = dn == H.n;              // the delta is a subset of the relation: of one size, they are the same rows
   DevBuf rec(c, (size_t)n_rows * 16), rec_run(c, (size_t)n_rows * 8), drec(c, same ? 8 : (size_t)n_rows * 8), adj(c, (size_t)r_rows * 16), row_pos(c, (size_t)n_rows * 4),
       row_len(c, (size_t)n_rows * 4), row_off(c, (size_t)n_rows * 4), q0(c, (size_t)max_q0 * 4), q1(c, (size_t)max_q1 * 4), q2(c, (size_t)max_q1 * 4);
-  const size_t free_bytes = c->arena.largest_free();
+  const size_t free_bytes = free_block(c, (uint64_t)kSortMaxN * 24);
   const uint64_t cap = std::min<uint64_t>(free_bytes / 24, (uint64_t)kSortMaxN);      // 8 bytes staged and up to 12 in the relation
   DevBuf st_c(c, cap * 4), st_t(c, cap * 4);
   zero_ctrl(c, kSlotSparse, kSpTotals);

@@ -22,6 +22,7 @@ float one_of(int sr) { return sr == XLOG_SR_SUMPROD ? 1.f : 0.f; }
 void drop_indices(Relation& R) {
   for (int i = 0; i < kMaxArity; ++i) R.idx[i] = Index();
   R.tri = TriRankIndex();
+  R.rev = RevLists();
 }
 
 void drop_current(Relation& R) {

@@ -1,0 +1,89 @@
+"""Heavy rounds of the bitmap-driven join as a gather: one to eight bitmap words per node, one and two parts of columns, carried values
+that derive nothing, both directions of the order, targets of one row and of many chunks; against the sorting route (relations
+bit for bit, counters equal) and the oracle."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2609_27203_b200 import synth
+from paper_2609_27203_b200 import workloads as W
+from tests import helpers as H
+
+pytestmark = pytest.mark.gpu
+COUNTERS = ("iterations", "derived_tuples", "candidates", "new_tuples", "improved_tags")
+
+
+def check(s, d, w, sources, sr, pulls=True, check_oracle=True):
+    from paper_2609_27203_b200 import xlog
+    prog = W.reach_program(s, d, w, sources, semiring=sr)
+    got = []
+    for f in (xlog.FLAG_NO_RESIDENT_LOOP, xlog.FLAG_NO_RESIDENT_LOOP | xlog.FLAG_PROFILE, xlog.FLAG_NO_TAG_MIRROR):
+        ctx, ids, _ = xlog.load_program(prog, arena_bytes=2 << 30, flags=f | xlog.FLAG_CHECK_INVARIANTS)
+        recs = []
+        for _ in range(2):
+            recs.append(ctx.fixpoint())
+            rel = ctx.read(ids["reach"])
+            ctx.reset_idb()
+        assert [recs[0][k] for k in COUNTERS] == [recs[1][k] for k in COUNTERS]
+        if f & xlog.FLAG_PROFILE:
+            assert ("k_bm_pull" in ctx.profile()) == pulls
+        got.append((rel, recs[0]))
+        ctx.close()
+    for g in got[:2]:
+        assert H.compare_relations(g[0], got[2][0], what="gather vs sorting route")["bit_unequal"] == 0
+        assert [g[1][k] for k in COUNTERS] == [got[2][1][k] for k in COUNTERS]
+    if check_oracle:
+        o, oids, _ = oracle.load_program(prog)
+        o.run("seminaive")
+        assert H.compare_relations(got[0][0], o.read(oids["reach"]), what="gather vs oracle")["bit_unequal"] == 0
+
+
+@pytest.mark.parametrize("sr", [W.MINPLUS, W.MAXPLUS])
+@pytest.mark.parametrize("n,deg,n_src", [(500, 16, 17), (500, 16, 32), (700, 12, 33), (1000, 24, 64), (600, 16, 70), (600, 20, 128), (600, 30, 200), (600, 30, 256), (500, 16, 300)])
+def test_even_graphs(sr, n, deg, n_src):
+    s, d = synth.uniform_digraph(n, n * deg, 40 + n_src)
+    w = (1 + 9 * np.random.default_rng(n_src).random(len(s))).astype(np.float32)
+    sources = np.sort(np.random.default_rng(n_src).permutation(n)[:n_src]).astype(np.int32)
+    check(s, d, w if sr == W.MINPLUS else -w, sources, sr, pulls=n_src <= 256, check_oracle=n < 1000)
+
+
+@pytest.mark.parametrize("scale,ef,n_src", [(9, 16, 20), (9, 16, 33), (10, 24, 64), (9, 16, 100)])
+def test_skewed_graphs(scale, ef, n_src):                     # sources that lead nowhere: fewer columns than carried values
+    s, d, w = synth.rmat_graph(scale, ef, 40 + n_src, "u1_10")
+    sources = np.sort(np.random.default_rng(n_src).permutation(1 << scale)[:n_src]).astype(np.int32)
+    check(s, d, w, sources, W.MINPLUS, check_oracle=scale < 10)
+
+
+@pytest.mark.parametrize("n,deg", [(1, 1), (255, 3), (256, 3), (257, 40), (1000, 300)])
+def test_one_target_and_many(n, deg):
+    # all of a layer lead to node 0 (a run of many chunks), which leads to `deg` leaves of one row each; dense enough to be pulled
+    rng = np.random.default_rng(n + deg)
+    src = np.arange(1, n + 1)
+    extra = rng.integers(1, n + 1, (2, 12 * n))
+    s = np.concatenate([src, np.zeros(deg, np.int64), extra[0]])
+    d = np.concatenate([np.zeros(n, np.int64), n + 1 + np.arange(deg), extra[1]])
+    key = np.unique(s * (n + deg + 1) + d)
+    s, d = key // (n + deg + 1), key % (n + deg + 1)
+    w = (1 + 9 * rng.random(len(s))).astype(np.float32)
+    check(s.astype(np.int32), d.astype(np.int32), w, np.arange(min(n + 1, 40), dtype=np.int32), W.MINPLUS, pulls=n > 1)
+
+
+def test_overflowing_tags():                                  # sums past the fp32 range are tuples, in the gather as elsewhere
+    s, d, w = synth.rmat_graph(8, 16, 3, "u1_10")
+    check(s, d, w * np.float32(3e37), np.arange(40, dtype=np.int32), W.MINPLUS)
+
+
+def test_lists_give_way():                                    # an arena with little to spare: the same relation, gathered or not
+    from paper_2609_27203_b200 import xlog
+    s, d, w = synth.rmat_graph(10, 16, 5, "u1_10")
+    prog = W.reach_program(s, d, w, np.arange(64, dtype=np.int32))
+    want = None
+    for arena in (1 << 28, 1 << 24, 1 << 23, 3 << 21, 5 << 20, 4 << 20):
+        ctx, ids, _ = xlog.load_program(prog, arena_bytes=arena, flags=xlog.FLAG_NO_RESIDENT_LOOP)
+        for _ in range(3):
+            ctx.fixpoint()
+            rel = ctx.read(ids["reach"])
+            want = want or rel
+            assert H.compare_relations(rel, want, what=f"arena of {arena}")["bit_unequal"] == 0
+            ctx.reset_idb()
+        ctx.close()
