@@ -8,14 +8,14 @@
 // place in the list of its first entry, so that a hit's place (for its tag) is that plus popcounts.  The bitmaps are made
 // from a join index when first wanted and kept with it.
 //
-// Bound by instruction issue.  Four-cycle join, 4.2 M two-paths over 1,024 values, 16.8 M rows: count 0.55 -> 0.07 ms, write
-// 1.55 -> 0.37 ms; a lane per word and the hits of a path written as they fell: 0.23 and 0.75.  Triangle join, 65,536 rows over
-// 406 values, 4.2 M rows: 62 -> 9 us and 84 -> 61 us.
+// Bound by the load / store path (81 % of its wavefronts: the words and places of A's lists, two tags, a search in shared memory a hit).
+// Four-cycle join, 4.2 M two-paths over 1,024 values, 16.8 M rows: count 0.06 ms, write 0.26 ms (hits queued per lane as they fell,
+// each lane going through its words: 0.07 and 0.37, and a place per path to be scanned: 0.03).  Triangle join, 65,536 rows over 406
+// values, 4.2 M rows: write 60 -> 38 us; with 32 paths to a warp instead of 8 there 73.
 //
 //   k_bits_lists   list entries -> bits, and running counts per word
-//   k_bits_count   matches per path
-//   k_bits_emit    the rows: hits are queued per warp with their place in the output and worked off 32 at a time, so that
-//                  the two tag reads and the writes use every lane though a path has few hits
+//   k_bits_count   matches per group of paths that a warp of the next kernel takes
+//   k_bits_emit    the rows
 #pragma once
 #include "common.cuh"
 
@@ -25,7 +25,6 @@ constexpr uint32_t kBitsMaxWords = 512;          // w below 2^14
 constexpr int kBitsLanes = 4;                    // lanes per path
 // words of a list: a lane takes 4 (short lists) or 8 words of every stretch of 16 or 32
 inline uint32_t bits_padded(uint32_t words) { return words <= 16 ? 16u : (words + 31) / 32 * 32; }
-constexpr uint32_t kBitsQueue = 256;             // hits a warp holds before it works them off
 
 // A warp per list: its entries' bits are set in shared memory, then every word is written with the number of entries before it.
 static __global__ void __launch_bounds__(256) k_bits_lists(const uint32_t* __restrict__ off, int64_t domain, const int32_t* __restrict__ col, uint32_t words, uint32_t* __restrict__ bits,
@@ -85,113 +84,147 @@ __device__ __forceinline__ void bits_words_of(const uint32_t* __restrict__ row, 
   }
 }
 
-// A warp takes 32 paths, eight per step.
-template <typename K2, int WB>
+// Matches per group of 8 J paths (J = 1 or 4).  A warp takes 32 paths, eight per step.
+template <typename K2, int WB, int J>
 __global__ void __launch_bounds__(256) k_bits_count(const __grid_constant__ BitsJoin P, const K2* __restrict__ keys, uint64_t n, uint32_t* __restrict__ cnt) {
   const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
   const unsigned lane = lane_id(), sub = lane % kBitsLanes;
   for (uint64_t base = (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; base < n; base += nwarps * 32) {
-    uint32_t a = 0, b = 0, mine = 0;
-    const bool ok = base + lane < n && bits_path<K2>(P, keys[base + lane], a, b);
+    uint32_t a = 0, b = 0, s = 0;
+    const uint32_t ok = base + lane < n && bits_path<K2>(P, keys[base + lane], a, b) ? 1u : 0u;
 #pragma unroll
-    for (int j = 0; j < kBitsLanes; ++j) {
+    for (int j = 0; j < 4; ++j) {
       const int p = j * 8 + lane / kBitsLanes;
       const uint32_t* ra = P.A.bits + (size_t)(__shfl_sync(0xffffffffu, a, p) * P.words) + sub * WB;
       const uint32_t* rb = P.B.bits + (size_t)(__shfl_sync(0xffffffffu, b, p) * P.words) + sub * WB;
-      uint32_t s = 0;
+      const bool live = __shfl_sync(0xffffffffu, ok, p) != 0u;
       for (uint32_t k = 0; k < P.words; k += WB * kBitsLanes) {
         uint32_t wa[WB], wb[WB];
-        bits_words_of<WB>(ra + k, true, wa);
-        bits_words_of<WB>(rb + k, true, wb);
+        bits_words_of<WB>(ra + k, live, wa);
+        bits_words_of<WB>(rb + k, live, wb);
 #pragma unroll
         for (int q = 0; q < WB; ++q) s += __popc(wa[q] & wb[q]);
       }
-#pragma unroll
-      for (int d = kBitsLanes / 2; d; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-      const uint32_t got = __shfl_sync(0xffffffffu, s, (lane % 8) * kBitsLanes);
-      if ((int)lane / 8 == j) mine = got;
+      if (J == 1) {
+        s = __reduce_add_sync(0xffffffffu, s);
+        if (lane == 0 && base + j * 8 < n) cnt[base / 8 + j] = s;
+        s = 0;
+      }
     }
-    if (base + lane < n) cnt[base + lane] = ok ? mine : 0u;
+    if (J == 4) {
+      s = __reduce_add_sync(0xffffffffu, s);
+      if (lane == 0) cnt[base / 32] = s;
+    }
   }
 }
 
-template <typename K2, typename K, int WB>
-__global__ void __launch_bounds__(256) k_bits_emit(const __grid_constant__ BitsJoin P, const K2* __restrict__ keys, const float* __restrict__ tags, uint64_t n,
-                                                   const uint64_t* __restrict__ off, K* __restrict__ out_keys, float* __restrict__ out_tags) {
-  __shared__ uint4 s_queue[8][kBitsQueue];         // {output row, w | path << 14, place in A's list, in B's}
-  uint4* queue = s_queue[warp_id()];
+// A warp takes 8 J paths.  Four lanes AND a path's words; A's words and, per lane, the running counts of the hits go to shared memory,
+// and the hits of all the paths, laid out in a line, are then worked off 32 at a time: a lane finds the unit (path, lane) that its hit
+// falls to, the word and the bit by counts alone.  Where the lists are one stretch long, that is the order of the rows.
+constexpr int kBitsEmitWarps = 4;
+template <typename K2, typename K, int WB, int J>
+__global__ void __launch_bounds__(32 * kBitsEmitWarps) k_bits_emit(const __grid_constant__ BitsJoin P, const K2* __restrict__ keys, const float* __restrict__ tags, uint64_t n,
+                                                                   const uint64_t* __restrict__ off, K* __restrict__ out_keys, float* __restrict__ out_tags) {
+  constexpr int kPaths = 8 * J, kUnits = kPaths * kBitsLanes;
+  __shared__ uint4 s_word[kBitsEmitWarps][WB / 4][kUnits];       // A's words, four at a time
+  __shared__ uint2 s_below[kBitsEmitWarps][kUnits];             // byte q: hits in the words before word q of the unit (at most 224)
+  __shared__ uint32_t s_from[kBitsEmitWarps][kUnits + 1];       // hits of the units before
+  __shared__ uint4 s_lists[kBitsEmitWarps][kPaths];             // per path: rows of its two bitmaps, where its two lists start
+  __shared__ uint4 s_path[kBitsEmitWarps][kPaths];              // head key without w (low, high), tag, output row of the stretch's first hit
+  const unsigned lane = lane_id(), sub = lane % kBitsLanes, wid = warp_id();
   const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-  const unsigned lane = lane_id(), sub = lane % kBitsLanes, first = lane - sub;
-  for (uint64_t base = (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; base < n; base += nwarps * 32) {
-    uint32_t a = 0, b = 0, to = 0, ok = 0;
-    K prefix = 0;
-    float tag = 0.f;
-    if (base + lane < n) {
-      const K2 k2 = keys[base + lane];
-      ok = bits_path<K2>(P, k2, a, b) ? 1u : 0u;
-      to = (uint32_t)off[base + lane];
-      tag = tags[base + lane];
+  const bool one = P.words <= WB * kBitsLanes;     // one stretch
+  for (uint64_t base = (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kPaths; base < n; base += nwarps * kPaths) {
+    const uint32_t row0 = (uint32_t)off[base / kPaths];
+    uint32_t a = 0, b = 0, ok = 0;
+    {
+      K prefix = 0;
+      float tag = 0.f;
+      if (lane < kPaths && base + lane < n) {
+        const K2 k2 = keys[base + lane];
+        ok = bits_path<K2>(P, k2, a, b) ? 1u : 0u;
+        tag = tags[base + lane];
 #pragma unroll
-      for (int c = 0; c < kMaxArity; ++c) if (c < P.path.arity) prefix |= (K)(uint32_t)key_col<K2>(P.path, k2, c) << P.head.shift[c];
-    }
-    auto write = [&](const uint4 h, const K pre, const float tg) {
-      const float ta = P.A.tag[h.z], tb = P.B.tag[h.w];
-      out_keys[h.x] = pre | ((K)(h.y & 0x3fffu) << P.head.shift[P.path.arity]);
-      out_tags[h.x] = P.times ? (tg * ta) * tb : (tg + ta) + tb;
-    };
-    uint32_t qn = 0;                               // queued hits (uniform)
-    auto flush = [&]() {
-      __syncwarp();
-      for (uint32_t i = 0; i < qn; i += 32) {
-        const uint4 h = i + lane < qn ? queue[i + lane] : make_uint4(0u, 0u, 0u, 0u);
-        const int p = h.y >> 14;
-        const K pre = (K)__shfl_sync(0xffffffffu, prefix, p);
-        const float tg = __shfl_sync(0xffffffffu, tag, p);
-        if (i + lane < qn) write(h, pre, tg);
+        for (int c = 0; c < kMaxArity; ++c) if (c < P.path.arity) prefix |= (K)(uint32_t)key_col<K2>(P.path, k2, c) << P.head.shift[c];
       }
-      qn = 0;
       __syncwarp();
-    };
-#pragma unroll 1
-    for (int j = 0; j < kBitsLanes; ++j) {
-      const uint32_t p = j * 8 + lane / kBitsLanes;
-      const uint32_t pa = __shfl_sync(0xffffffffu, a, p), pb = __shfl_sync(0xffffffffu, b, p);
-      const bool live = __shfl_sync(0xffffffffu, ok, p) != 0u;
-      uint32_t at = __shfl_sync(0xffffffffu, to, p);
-      for (uint32_t k0 = sub * WB; k0 < P.words; k0 += WB * kBitsLanes) {
-        const uint32_t ra = pa * P.words + k0, rb = pb * P.words + k0;
-        uint32_t wa[WB], wb[WB];
-        bits_words_of<WB>(P.A.bits + ra, live, wa);
-        bits_words_of<WB>(P.B.bits + rb, live, wb);
-        uint32_t mine = 0;
+      if (lane < kPaths) {
+        s_lists[wid][lane] = make_uint4(a * P.words, b * P.words, ok ? P.A.off[a] : 0u, ok ? P.B.off[b] : 0u);
+        s_path[wid][lane] = make_uint4((uint32_t)prefix, sizeof(K) == 8 ? (uint32_t)((uint64_t)prefix >> 32) : 0u, __float_as_uint(tag), row0);
+      }
+      __syncwarp();
+    }
+    if (!one) {                                    // where every path's rows begin
+      for (int j = 0; j < J; ++j) {
+        const uint32_t p = j * 8 + lane / kBitsLanes;
+        const uint4 rows = s_lists[wid][p];
+        const bool live = __shfl_sync(0xffffffffu, ok, p) != 0u;
+        uint32_t s = 0;
+        for (uint32_t k = sub * WB; k < P.words; k += WB * kBitsLanes) {
+          uint32_t wa[WB], wb[WB];
+          bits_words_of<WB>(P.A.bits + rows.x + k, live, wa);
+          bits_words_of<WB>(P.B.bits + rows.y + k, live, wb);
 #pragma unroll
-        for (int q = 0; q < WB; ++q) mine += __popc(wa[q] & wb[q]);
-        const uint32_t incl = warp_scan_incl(mine), total = __shfl_sync(0xffffffffu, incl, 31);
-        if (total == 0u) continue;                 // uniform
-        const uint32_t before = __shfl_sync(0xffffffffu, incl - mine, first);
-        uint32_t row = at + incl - mine - before;  // output row of the lane's next hit
-        at += __shfl_sync(0xffffffffu, incl, first + kBitsLanes - 1) - before;
-        if (qn + total > kBitsQueue) flush();
-        const bool queued = total <= kBitsQueue;   // else the lanes have many hits each and write them themselves
-        uint32_t pos = qn + incl - mine, from_a = 0, from_b = 0;
-        K pre = 0;
-        float tg = 0.f;
-        if (mine) { from_a = P.A.off[pa] + P.A.rank[ra]; from_b = P.B.off[pb] + P.B.rank[rb]; }
-        if (!queued) { pre = (K)__shfl_sync(0xffffffffu, prefix, p); tg = __shfl_sync(0xffffffffu, tag, p); }
-#pragma unroll
-        for (int q = 0; q < WB; ++q) {
-          for (uint32_t m = wa[q] & wb[q]; m; m &= m - 1) {
-            const uint32_t bit = __ffs(m) - 1, below = (1u << bit) - 1u;
-            const uint4 h = make_uint4(row++, ((k0 + q) << 5) | bit | p << 14, from_a + __popc(wa[q] & below), from_b + __popc(wb[q] & below));
-            if (queued) queue[pos++] = h; else write(h, pre, tg);
-          }
-          from_a += __popc(wa[q]); from_b += __popc(wb[q]);
+          for (int q = 0; q < WB; ++q) s += __popc(wa[q] & wb[q]);
         }
-        if (queued) qn += total;
+#pragma unroll
+        for (int d = kBitsLanes / 2; d; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+        if (sub == 0) s_from[wid][p] = s;
+      }
+      __syncwarp();
+      const uint32_t mine = lane < kPaths ? s_from[wid][lane] : 0u, incl = warp_scan_incl(mine);
+      if (lane < kPaths) s_path[wid][lane].w += incl - mine;
+      __syncwarp();
+    }
+    for (uint32_t k0 = 0; k0 < P.words; k0 += WB * kBitsLanes) {
+      uint32_t total = 0;                          // uniform
+#pragma unroll 1
+      for (int j = 0; j < J; ++j) {
+        const uint32_t p = j * 8 + lane / kBitsLanes;
+        const uint4 rows = s_lists[wid][p];
+        const bool live = __shfl_sync(0xffffffffu, ok, p) != 0u;
+        uint32_t wa[WB], wb[WB];
+        bits_words_of<WB>(P.A.bits + rows.x + k0 + sub * WB, live, wa);
+        bits_words_of<WB>(P.B.bits + rows.y + k0 + sub * WB, live, wb);
+#pragma unroll
+        for (int q = 0; q < WB / 4; ++q) s_word[wid][q][j * 32 + lane] = make_uint4(wa[4 * q], wa[4 * q + 1], wa[4 * q + 2], wa[4 * q + 3]);
+        uint32_t mine = 0, below[2] = {0u, 0u};
+#pragma unroll
+        for (int q = 0; q < WB; ++q) { below[q / 4] |= mine << (8 * (q % 4)); mine += __popc(wa[q] & wb[q]); }
+        const uint32_t incl = warp_scan_incl(mine);
+        s_below[wid][j * 32 + lane] = make_uint2(below[0], below[1]);
+        s_from[wid][j * 32 + lane] = total + incl - mine;
+        total += __shfl_sync(0xffffffffu, incl, 31);
+      }
+      if (lane == 0) s_from[wid][kUnits] = total;
+      __syncwarp();
+      for (uint32_t h = lane; h < total; h += 32) {
+        uint32_t u = 0;                            // last unit that starts at or before h
+#pragma unroll
+        for (int d = kUnits / 2; d; d >>= 1) if (s_from[wid][u + d] <= h) u += d;
+        const uint32_t r = h - s_from[wid][u], p = u / kBitsLanes;
+        const uint2 bl = s_below[wid][u];
+        const uint32_t r4 = r * 0x01010101u;       // r is at most 255
+        const uint32_t q = (uint32_t)__popc(__vcmpleu4(bl.x, r4) & 0x01010101u) + (WB == 8 ? (uint32_t)__popc(__vcmpleu4(bl.y, r4) & 0x01010101u) : 0u) - 1u;
+        const uint32_t w = k0 + (u % kBitsLanes) * WB + q;
+        const uint4 rows = s_lists[wid][p], path = s_path[wid][p];
+        const uint32_t ia = rows.x + w, ib = rows.y + w, wa = reinterpret_cast<const uint32_t*>(&s_word[wid][q / 4][u])[q % 4], wb = P.B.bits[ib];
+        uint32_t m = wa & wb;
+        for (uint32_t i = r - (((q < 4 ? bl.x : bl.y) >> (8 * (q % 4))) & 0xffu); i; --i) m &= m - 1;
+        const uint32_t bit = __ffs(m) - 1, mask = (1u << bit) - 1u;
+        const float ta = P.A.tag[rows.z + P.A.rank[ia] + __popc(wa & mask)], tb = P.B.tag[rows.w + P.B.rank[ib] + __popc(wb & mask)];
+        const float tg = __uint_as_float(path.z);
+        const uint32_t row = one ? row0 + h : path.w + h - s_from[wid][p * kBitsLanes];
+        const K pre = sizeof(K) == 8 ? (K)(((uint64_t)path.y << 32) | path.x) : (K)path.x;
+        out_keys[row] = pre | ((K)((w << 5) | bit) << P.head.shift[P.path.arity]);
+        out_tags[row] = P.times ? (tg * ta) * tb : (tg + ta) + tb;
+      }
+      __syncwarp();
+      if (!one) {                                  // the paths' next rows
+        if (lane < kPaths) s_path[wid][lane].w += s_from[wid][(lane + 1) * kBitsLanes] - s_from[wid][lane * kBitsLanes];
         __syncwarp();
       }
     }
-    flush();
   }
 }
 

@@ -313,25 +313,38 @@ BitsLists ensure_bits(Ctx* c, Index& ix, uint32_t words) {
   }
   return BitsLists{ix.bits.as<uint32_t>(), ix.bit_rank.as<uint16_t>(), ix.off.as<uint32_t>(), ix.tags, (uint32_t)ix.domain};
 }
+template <typename K2, typename K, int J>
+void bits_emit_j(Ctx* c, const BitsJoin& P, const void* keys, const float* tags, uint64_t n, const uint64_t* off, void* ok, float* ot) {
+  const unsigned g = grid_for(n, 8 * J * kBitsEmitWarps);
+  if (P.words > 16) XLOG_LAUNCH(c, (k_bits_emit<K2, K, 8, J>), g, 32 * kBitsEmitWarps, 0, P, (const K2*)keys, tags, n, off, (K*)ok, ot);
+  else XLOG_LAUNCH(c, (k_bits_emit<K2, K, 4, J>), g, 32 * kBitsEmitWarps, 0, P, (const K2*)keys, tags, n, off, (K*)ok, ot);
+}
+template <typename K2, int J>
+void bits_count_j(Ctx* c, const BitsJoin& P, const void* keys, uint64_t n, uint32_t* cnt) {
+  if (P.words > 16) XLOG_LAUNCH(c, (k_bits_count<K2, 8, J>), grid_for(n, 256), 256, 0, P, (const K2*)keys, n, cnt);
+  else XLOG_LAUNCH(c, (k_bits_count<K2, 4, J>), grid_for(n, 256), 256, 0, P, (const K2*)keys, n, cnt);
+}
+// With fewer paths than this a warp takes eight of them instead of 32, so that there are warps enough.
+constexpr uint64_t kBitsManyPaths = (uint64_t)kSMs * 64 * 32;
 template <typename K2, typename K>
 void bits_emit(Ctx* c, const BitsJoin& P, const void* keys, const float* tags, uint64_t n, const uint64_t* off, void* ok, float* ot) {
-  const unsigned g = grid_for(n, 256);
-  if (P.words > 16) XLOG_LAUNCH(c, (k_bits_emit<K2, K, 8>), g, 256, 0, P, (const K2*)keys, tags, n, off, (K*)ok, ot);
-  else XLOG_LAUNCH(c, (k_bits_emit<K2, K, 4>), g, 256, 0, P, (const K2*)keys, tags, n, off, (K*)ok, ot);
+  if (n >= kBitsManyPaths) bits_emit_j<K2, K, 4>(c, P, keys, tags, n, off, ok, ot);
+  else bits_emit_j<K2, K, 1>(c, P, keys, tags, n, off, ok, ot);
 }
 // All rows of the join of n paths: count -> scan -> one control read -> write.
 KeyTags bits_join(Ctx* c, const BitsJoin& P, const void* keys, int key_bytes, const float* tags, uint64_t n, int head_bytes, const char* what) {
-  DevBuf cnt(c, n * 4), off(c, n * 8);
-  const unsigned tiles = (unsigned)((n + kScanTile - 1) / kScanTile);
+  const uint64_t ng = n >= kBitsManyPaths ? (n + 31) / 32 : (n + 7) / 8;       // groups of paths
+  DevBuf cnt(c, std::max<uint64_t>(ng, 1) * 4), off(c, std::max<uint64_t>(ng, 1) * 8);
+  const unsigned tiles = (unsigned)((ng + kScanTile - 1) / kScanTile);
   DevBuf sums(c, (size_t)tiles * 8);
   c->note_bytes = (int64_t)n * (key_bytes + 4);
   DISPATCH_K(key_bytes, {
-    if (P.words > 16) XLOG_LAUNCH(c, (k_bits_count<K, 8>), grid_for(n, 256), 256, 0, P, (const K*)keys, n, cnt.as<uint32_t>());
-    else XLOG_LAUNCH(c, (k_bits_count<K, 4>), grid_for(n, 256), 256, 0, P, (const K*)keys, n, cnt.as<uint32_t>());
+    if (n >= kBitsManyPaths) bits_count_j<K, 4>(c, P, keys, n, cnt.as<uint32_t>());
+    else bits_count_j<K, 1>(c, P, keys, n, cnt.as<uint32_t>());
   });
-  XLOG_LAUNCH(c, (k_scan_tile_sums<uint32_t, uint64_t>), tiles, kScanBlock, 0, (const uint32_t*)cnt.as<uint32_t>(), (int64_t)n, sums.as<uint64_t>());
+  XLOG_LAUNCH(c, (k_scan_tile_sums<uint32_t, uint64_t>), tiles, kScanBlock, 0, (const uint32_t*)cnt.as<uint32_t>(), (int64_t)ng, sums.as<uint64_t>());
   XLOG_LAUNCH(c, (k_scan_spine<uint64_t>), 1, 1024, 0, sums.as<uint64_t>(), (int64_t)tiles, (uint64_t*)(c->d_ctrl + kSlotTotals));
-  XLOG_LAUNCH(c, (k_scan_apply<uint32_t, uint64_t>), tiles, kScanBlock, 0, (const uint32_t*)cnt.as<uint32_t>(), (int64_t)n, (const uint64_t*)sums.as<uint64_t>(), off.as<uint64_t>());
+  XLOG_LAUNCH(c, (k_scan_apply<uint32_t, uint64_t>), tiles, kScanBlock, 0, (const uint32_t*)cnt.as<uint32_t>(), (int64_t)ng, (const uint64_t*)sums.as<uint64_t>(), off.as<uint64_t>());
   sync_ctrl(c);                                            // the one small metadata read that sizes the output
   const uint64_t total = c->h_ctrl[kSlotTotals];
   if (total > kSortMaxN) fail(XLOG_ERR_CAPACITY_EXCEEDED, std::string("materialised ") + what + " relation exceeds 2^30 - 1 rows");
