@@ -23,7 +23,7 @@
 namespace xlog {
 
 constexpr int kBpMaxWordsLog2 = 3;                // at most 8 bitmap words (256 carried values) per node
-constexpr int kBpMaxCols = 256;
+constexpr int kBpMaxCols = 128;                  // carried values that can derive anything: four columns a lane of a warp
 constexpr int kBpBlock = 128;
 constexpr int kBpSweeps = 8;                      // rows of r per lane and chunk
 constexpr int kBpChunk = 32 * kBpSweeps;
@@ -143,10 +143,10 @@ __global__ void __launch_bounds__(256) k_bm_count(BmCount P) {
   if (threadIdx.x < W) { const uint32_t v = s_live[threadIdx.x]; if (v & ~P.live[threadIdx.x]) atomicOr(P.live + threadIdx.x, v); }
 }
 
-// Columns of the copy: position 4 l + k of part y holds live carried value number (4 y + k) lanes + l, so that the k-th slots of the
-// lanes of a row lie side by side in the table.
+// Columns of the copy: position 4 l + k holds live carried value number k lanes + l, so that the k-th slots of the lanes of a row lie
+// side by side in the table.
 struct BpColumns {
-  int lanes, parts;                // lanes to a row of a part, four columns each
+  int lanes;                       // lanes to a row, four columns each
   int16_t at[kBpMaxCols];          // carried value at a position, -1: none
 };
 
@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(256) k_bm_snap(const __grid_constant__ BmSnap 
   }
   __syncthreads();
   if (threadIdx.x < kAnyWords) P.any[(size_t)blockIdx.x * kAnyWords + threadIdx.x] = s_any[threadIdx.x];
-  const uint32_t quads = (uint32_t)(C.lanes * C.parts), work = s_n * quads;
+  const uint32_t quads = (uint32_t)C.lanes, work = s_n * quads;
   for (uint32_t i = threadIdx.x; i < work; i += 256) {
     const uint32_t r = i / quads, q = i - r * quads, b = s_node[r];
     const int32_t* row = P.table + ((size_t)b << P.carried_bits);
@@ -230,7 +230,7 @@ struct BmPull {
   uint32_t* err;
 };
 
-// A warp takes kBpChunk rows of r (neighbours in the order of targets; blockIdx.y: a part of the columns) and splits them among its
+// A warp takes kBpChunk rows of r (neighbours in the order of targets) and splits them among its
 // groups of lanes, a row of the copy to a group and step.  A target's slots are read when its last row has been met and looked at when
 // the next target's has.  An empty slot is a NaN in the copy, and min / max pass a NaN over.  FILTER: rows whose b has not changed are
 // dropped first; without it they take part with what the copy last held of b (empty, or tags that have been applied), which is
@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(kBpBlock, kBpBlocks) k_bm_pull(const __grid_co
   const unsigned lane = lane_id(), wid = warp_id();
   const uint32_t base = (blockIdx.x * (kBpBlock / 32) + wid) * kBpChunk;
   if (base >= P.n_rows) return;
-  const uint32_t G = (uint32_t)C.lanes, quads = G * (uint32_t)C.parts, first_quad = blockIdx.y * G;
+  const uint32_t G = (uint32_t)C.lanes;
   uint2* const rows = s_row[wid];
   uint32_t* const target = s_target[wid];
   uint32_t n = 0;
@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(kBpBlock, kBpBlocks) k_bm_pull(const __grid_co
       const unsigned bal = __ballot_sync(0xffffffffu, in);
       if (in) {
         const uint32_t at = n + __popc(bal & lanemask_lt());
-        rows[at] = make_uint2(r[i].x * quads + first_quad, r[i].y);
+        rows[at] = make_uint2(r[i].x * G, r[i].y);
         target[at] = z[i];
       }
       n += __popc(bal);
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(kBpBlock, kBpBlocks) k_bm_pull(const __grid_co
   if (e0 >= e1) return;
   int col[4];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) col[k] = max((int)C.at[4 * (first_quad + l) + k], 0);
+  for (int k = 0; k < 4; ++k) col[k] = max((int)C.at[4 * l + k], 0);
   const float none = __int_as_float(0x7fffffff);
   const int32_t never = SINK == kSinkMin ? 0x7fffffff : (int32_t)0x80000000;
   auto better = [](float a, float b) { return SINK == kSinkMin ? fminf(a, b) : fmaxf(a, b); };

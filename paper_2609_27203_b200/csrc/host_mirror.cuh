@@ -79,6 +79,9 @@ bool mirror_applies(Ctx* c, const std::vector<int>& comp, const std::vector<cons
 constexpr int kResidentMaxBits = 24;
 constexpr uint32_t kResidentMaxTiles = 1u << 20;
 
+#ifndef XLOG_RES_UNROLL
+#define XLOG_RES_UNROLL 4
+#endif
 ResState* res_state(Ctx* c) { return reinterpret_cast<ResState*>(c->d_ctrl + kSlotResState); }
 static_assert(sizeof(ResState) <= (kCtrlSlots - kSlotResState) * sizeof(uint64_t), "state block must fit the control words");
 
@@ -254,13 +257,16 @@ ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*
     sync_ctrl(c);
     memcpy(&out, c->h_ctrl + kSlotResState, sizeof out);
   };
+  // Going round the WHILE node costs 9 to 10 us, a round's launches after the end 4: the body holds several rounds, except where the
+  // cluster kernel runs most of them in one go.
+  const int rounds_per_body = longest ? 1 : XLOG_RES_UNROLL;
   if (use_graph) {
     std::vector<char> sig;
     for (const JoinSpec& S : specs) sig_add(sig, S);
     sig_add(sig, mr.table); sig_add(sig, mr.changed); sig_add(sig, mr.n_new); sig_add(sig, mr.key_max); sig_add(sig, mr.err); sig_add(sig, R.present.p);
     sig_add(sig, longest);
     if (longest) sig_add(sig, res_cluster_slots(H));
-    sig_add(sig, is_max); sig_add(sig, bm_quads); sig_add(sig, ch_tiles); sig_add(sig, c->d_ctrl); sig_add(sig, c->spin_limit);
+    sig_add(sig, rounds_per_body); sig_add(sig, is_max); sig_add(sig, bm_quads); sig_add(sig, ch_tiles); sig_add(sig, c->d_ctrl); sig_add(sig, c->spin_limit);
     if (!R.exec || sig != R.sig) {
       if (R.exec) { cudaGraphExecDestroy(R.exec); R.exec = nullptr; }
       if (R.graph) { cudaGraphDestroy(R.graph); R.graph = nullptr; }
@@ -283,7 +289,7 @@ ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*
       c->stream = c->capture_stream;
       const int64_t b0 = c->launches;
       try {
-        resident_body(c, R, specs, H, is_max, mr, bm_quads, ch_tiles, longest, handle, 1);
+        for (int i = 0; i < rounds_per_body; ++i) resident_body(c, R, specs, H, is_max, mr, bm_quads, ch_tiles, longest, handle, 1);
       } catch (...) {
         c->stream = caller;
         cudaGraph_t dummy = nullptr;
@@ -291,7 +297,7 @@ ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*
         throw;
       }
       c->stream = caller;
-      R.body_launches = c->launches - b0;
+      R.body_launches = (c->launches - b0) / rounds_per_body;
       XLOG_CUDA(cudaStreamEndCapture(c->capture_stream, nullptr));
       XLOG_CUDA(cudaGraphInstantiate(&R.exec, R.graph, 0));
       R.sig = std::move(sig);
@@ -522,11 +528,11 @@ void launch_bm_snap(Ctx* c, int words_log2, unsigned blocks, const BmSnap& P, co
   }
 }
 
-template <int SINK> void launch_bm_pull_s(Ctx* c, bool filter, dim3 grid, const BmPull& P, const BpColumns& C) {
+template <int SINK> void launch_bm_pull_s(Ctx* c, bool filter, unsigned grid, const BmPull& P, const BpColumns& C) {
   if (filter) XLOG_LAUNCH(c, (k_bm_pull<SINK, true>), grid, kBpBlock, 0, P, C);
   else XLOG_LAUNCH(c, (k_bm_pull<SINK, false>), grid, kBpBlock, 0, P, C);
 }
-void launch_bm_pull(Ctx* c, bool is_max, bool filter, dim3 grid, const BmPull& P, const BpColumns& C) {
+void launch_bm_pull(Ctx* c, bool is_max, bool filter, unsigned grid, const BmPull& P, const BpColumns& C) {
   if (is_max) launch_bm_pull_s<kSinkMax>(c, filter, grid, P, C); else launch_bm_pull_s<kSinkMin>(c, filter, grid, P, C);
 }
 
@@ -537,16 +543,10 @@ void bitmap_pull_columns(Ctx* c, BitmapPull& bp) {
   std::vector<int16_t> a;
   for (int i = 0; i < (32 << bp.words_log2); ++i) if ((live[i >> 5] >> (i & 31)) & 1u) a.push_back((int16_t)i);
   bp.n_cols = (int)a.size();
-  bp.cols.parts = std::max(1, (bp.n_cols + 127) / 128);
-  bp.cols.lanes = std::max(2, (bp.n_cols + 8 * bp.cols.parts - 1) / (8 * bp.cols.parts) * 2);      // rows of whole 32-byte sectors
-  const int G = bp.cols.lanes;
+  if (bp.n_cols > kBpMaxCols) { bp.usable = false; return; }
+  bp.cols.lanes = std::max(2, (bp.n_cols + 7) / 8 * 2);                  // rows of whole 32-byte sectors
   for (int i = 0; i < kBpMaxCols; ++i) bp.cols.at[i] = -1;
-  for (int y = 0; y < bp.cols.parts; ++y)
-    for (int l = 0; l < G; ++l)
-      for (int k = 0; k < 4; ++k) {
-        const int j = (4 * y + k) * G + l;
-        if (j < bp.n_cols) bp.cols.at[4 * (y * G + l) + k] = a[j];
-      }
+  for (int j = 0; j < bp.n_cols; ++j) bp.cols.at[4 * (j % bp.cols.lanes) + j / bp.cols.lanes] = a[j];
 }
 
 // Buffers and lists for the gather, once a round wants it.  False: it is the first evaluation that does, or they do not fit with room to
@@ -555,7 +555,7 @@ bool bitmap_pull_begin(Ctx* c, BitmapJoin& bj, BitmapPull& bp, uint64_t n_nodes)
   if (bp.lists) return true;
   Relation& R = *bj.rel;
   if (!R.rev.valid && (R.rev.wanted == 0 || R.rev.wanted == c->evaluations)) { R.rev.wanted = c->evaluations; bp.usable = false; return false; }
-  const uint64_t copy = (n_nodes + 1) * 16 * (uint64_t)(bp.cols.lanes * bp.cols.parts);
+  const uint64_t copy = (n_nodes + 1) * 16 * (uint64_t)bp.cols.lanes;
   const uint64_t need = copy + (uint64_t)bp.blocks * 128 + (R.rev.valid ? 0 : (uint64_t)R.n * 12 + (uint64_t)R.val_max[1] * 8) + (4u << 20);
   if (need > c->arena.largest_free() / 2 || copy / 16 > 0xffffffffull) { bp.usable = false; return false; }
   if (!R.rev.valid) build_rev_lists(c, R);

@@ -220,15 +220,15 @@ void stratum_recursive_mirror(Ctx* c, int h, const std::vector<const RuleC*>& rs
         // Which way, in twentieths of a picosecond (R-MAT 22, 27 of 64 sources with edges): the push takes 17 a neighbour row and 0.55 a
         // candidate, the gather 2.5 a row of r and 2.05 a lane and neighbour row.  Rounds of 524, 1581, 961 and 185 million candidates over
         // 54 to 65 million neighbour rows: 1.65, 2.31, 1.91 and 1.17 ms pushed (with the plan), 1.32, 1.34, 1.31 and 1.18 gathered.
-        const bool pull = count_first && cand * 11 + nbrs * 340 > (uint64_t)bj.rel->n * 50 + nbrs * 41 * (uint64_t)(bp.cols.lanes * bp.cols.parts);
+        const bool pull = count_first && bp.usable && cand * 11 + nbrs * 340 > (uint64_t)bj.rel->n * 50 + nbrs * 41 * (uint64_t)bp.cols.lanes;
         if (pull && bitmap_pull_begin(c, bj, bp, n_nodes)) {
           const BmSnap N{reinterpret_cast<uint32_t*>(bitmap), present, bp.n_units, bj.spec.inner_off, P.domain, table, carried_bits, bp.any.as<uint32_t>(), bp.copy.as<float>()};
           launch_bm_snap(c, bp.words_log2, bp.blocks, N, bp.cols);
           const BmPull L{bp.lists->rows.as<uint2>(), bp.lists->target.as<uint32_t>(), bj.rel->n, bp.any.as<uint32_t>(), n_nodes, bp.copy.as<float4>(), H.layout.mask[1], carried_bits,
                          table, reinterpret_cast<uint32_t*>(bitmap), ctrl_u32(c, kSlotErr)};
-          const dim3 grid((unsigned)((bj.rel->n + kBpChunk * (kBpBlock / 32) - 1) / (kBpChunk * (kBpBlock / 32))), (unsigned)bp.cols.parts);
+          const unsigned grid = (bj.rel->n + kBpChunk * (kBpBlock / 32) - 1) / (kBpChunk * (kBpBlock / 32));
           // per row of r its node, tag and target; per (b, neighbour) with a changed b a row of the copy
-          c->note_bytes = (int64_t)bj.rel->n * 12 + (int64_t)nbrs * 16 * bp.cols.lanes * bp.cols.parts;
+          c->note_bytes = (int64_t)bj.rel->n * 12 + (int64_t)nbrs * 16 * bp.cols.lanes;
           launch_bm_pull(c, is_max, nbrs < (uint64_t)bj.rel->n / 8 * 7, grid, L, bp.cols);
           continue;
         }

@@ -23,7 +23,7 @@
 
 namespace xlog {
 
-enum { kResOk = 0, kResCap = 1, kResOverflow = 2, kResError = 3, kResDone = 4 };      // kResDone: finished inside the cluster kernel (res_cluster.cuh)
+enum { kResOk = 0, kResCap = 1, kResOverflow = 2, kResError = 3, kResDone = 4 };      // kResDone: the delta ran empty
 
 struct ResState {
   uint32_t n_delta;                  // rows of the current delta
@@ -39,7 +39,7 @@ struct ResState {
   unsigned long long n_new;          // new tuples / improved tags of all completed rounds
   unsigned long long n_improved;
   unsigned long long small_cand;     // candidates of rounds run by the cluster kernel (res_cluster.cuh)
-  uint32_t bodies;                   // times the loop body ran
+  uint32_t bodies;                   // times a round's launches ran
   uint32_t pad;
 };
 
@@ -217,6 +217,10 @@ __device__ __forceinline__ void res_close_round(const bool live, ResState* __res
                                                 const unsigned long long* __restrict__ new_counter, uint32_t* __restrict__ ctr,
                                                 cudaGraphConditionalHandle handle, int use_handle, uint32_t& s_last,
                                                 unsigned long long* __restrict__ reserve, uint2* __restrict__ tile_rows) {
+  if (!live) {                                           // the loop is over (or abandoned): its books stay as they are
+    if (blockIdx.x == 0 && threadIdx.x == 0) { st->bodies += 1; if (use_handle) cudaGraphSetConditional(handle, 0u); }
+    return;
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
@@ -227,14 +231,14 @@ __device__ __forceinline__ void res_close_round(const bool live, ResState* __res
   __threadfence();
   unsigned long long next_total = 0;
   uint32_t changed = 0;
-  if (live) {
+  {
     if (reserve) {
       const unsigned long long r = ld_volatile_u64(reserve);
       changed = (uint32_t)(r & ((1ull << kResRowBits) - 1));
       next_total = r >> kResRowBits;
     } else changed = *reinterpret_cast<volatile uint32_t*>(&ctr[0]);
   }
-  if (live && !reserve) {
+  if (!reserve) {
     const uint32_t tiles = (st->n_delta + kResScanTile - 1) / kResScanTile + 1;
     for (uint32_t v = 0; v < n_variants; ++v)
       for (uint32_t i = threadIdx.x; i < tiles && i < sc.scan_tiles_cap; i += blockDim.x) sc.scan_status[(size_t)v * sc.scan_tiles_cap + i] = 0;
@@ -244,7 +248,7 @@ __device__ __forceinline__ void res_close_round(const bool live, ResState* __res
   if (threadIdx.x == 0) {
     unsigned again = 0;
     st->bodies += 1;
-    if (live) {
+    {
       const unsigned long long seen = *new_counter;
       const unsigned long long fresh = seen - st->new_seen;
       st->new_seen = seen;
@@ -254,9 +258,9 @@ __device__ __forceinline__ void res_close_round(const bool live, ResState* __res
       st->round_cand = 0;
       st->n_delta = changed;
       st->rounds += 1;
-      if (changed > 0) {
-        if (st->rounds >= st->max_rounds) st->status = kResCap; else again = 1;
-      }
+      if (changed == 0) st->status = kResDone;
+      else if (st->rounds >= st->max_rounds) st->status = kResCap;
+      else again = 1;
       if (reserve) {                                     // the next round's join, as k_res_count_scan's last tile would announce it
         const unsigned long long nt = (next_total + kExpTileMirror - 1) / kExpTileMirror;
         st->total = next_total;
