@@ -300,11 +300,15 @@ inline unsigned grid_for(uint64_t n, int block, int cap = kSMs * 16) {
 // Stores to the pinned block instead of a copy command: the copy engine's turn costs 7 us more, and every read waits for it
 // (reachability from 7 sources 685 -> 667 us, 64 digit pairs' evaluation 52 -> 45 us; closure of 1,000 nodes 278 -> 255 us together with
 // the one wait at an evaluation's end, see sync_ctrl_end).
-static __global__ void k_ctrl_out(const uint64_t* __restrict__ d, uint64_t* __restrict__ h) { h[threadIdx.x] = d[threadIdx.x]; }
+static __global__ void k_ctrl_out(uint64_t* __restrict__ d, uint64_t* __restrict__ h, uint32_t clear, uint32_t n_clear) {
+  h[threadIdx.x] = d[threadIdx.x];
+  if (threadIdx.x - clear < n_clear) d[threadIdx.x] = 0ull;
+}
 
-// Copy the control block to pinned host memory and wait: the bounded control read of an iteration.
-inline void sync_ctrl(Ctx* c) {
-  k_ctrl_out<<<1, kCtrlSlots, 0, c->stream>>>((const uint64_t*)c->d_ctrl, c->h_ctrl);
+// Copy the control block to pinned host memory and wait: the bounded control read of an iteration.  n_clear > 0: that many words from
+// `clear` on are zero afterwards.
+inline void sync_ctrl(Ctx* c, uint32_t clear = 0, uint32_t n_clear = 0) {
+  k_ctrl_out<<<1, kCtrlSlots, 0, c->stream>>>(c->d_ctrl, c->h_ctrl, clear, n_clear);
   XLOG_CUDA(cudaGetLastError());
   XLOG_CUDA(cudaStreamSynchronize(c->stream));
   if (!c->prof_pending.empty()) prof_collect(c);

@@ -274,6 +274,42 @@ void launch_expand_mirror(Ctx* c, Counted& q, bool is_max, const MirrorArgs& mr)
 
 constexpr int kSlotTotals = 16;          // uint64 candidate totals of the variants of a round
 
+// A rule of one atom over distinct plain variables: every row of the atom's relation matches, once.
+bool matches_every_row(const xlog_plan& p, int arity) {
+  if (p.n_atoms != 1 || p.atoms[0].negated || p.emit_count_column) return false;
+  for (int i = 0; i < arity; ++i) {
+    if (!is_plain_var(p.atoms[0].args[i])) return false;
+    for (int j = 0; j < i; ++j) if (p.atoms[0].args[j].var == p.atoms[0].args[i].var) return false;
+  }
+  return true;
+}
+// Such a rule whose head is the atom, column for column: the candidates are the atom's rows, ordered and each key once.
+bool copies_rows(Ctx* c, const Variant& v, const Relation& H, const KeyLayout& head) {
+  const xlog_plan& p = v.rule->plan;
+  const Relation& R = *c->rels[p.atoms[0].rel];
+  if (v.rule->kind != 1 || p.n_head_cols != R.arity || H.arity != R.arity || head.arity != R.arity || v.outer.layout.arity != R.arity || !matches_every_row(p, R.arity)) return false;
+  for (int i = 0; i < R.arity; ++i) {
+    if (H.dict_n[i] || R.dict_n[i] || p.head[i].c0 != 0 || v.outer.layout.mask[i] > head.mask[i]) return false;
+    for (int k = 0; k < XLOG_MAX_VARS; ++k) if (p.head[i].coef[k] != (k == p.atoms[0].args[i].var ? 1 : 0)) return false;
+  }
+  return true;
+}
+// A variant every row of which is one candidate for a mirror, applied in one launch: no count, no scan, no control read.  False:
+// some other rule, nothing done.
+bool mirror_rows(Ctx* c, const Variant& v, const Relation& H, const KeyLayout* head_layout, bool is_max, const MirrorArgs& mr) {
+  const xlog_plan& p = v.rule->plan;
+  if (v.rule->kind != 1 || v.outer.n == 0 || !matches_every_row(p, c->rels[p.atoms[0].rel]->arity)) return false;
+  const JoinSpec S = make_spec(c, v, H, head_layout);
+  if (!S.fast || S.has_inner) return false;
+  c->note_bytes = (int64_t)v.outer.n * (v.outer.key_bytes + 8);
+  DISPATCH_K(v.outer.key_bytes, {
+    if (is_max) XLOG_LAUNCH(c, (k_mirror_rows<K, kSinkMax>), (v.outer.n + 255) / 256, 256, 0, S, (const K*)v.outer.keys, v.outer.tags, v.outer.n, mr);
+    else XLOG_LAUNCH(c, (k_mirror_rows<K, kSinkMin>), (v.outer.n + 255) / 256, 256, 0, S, (const K*)v.outer.keys, v.outer.tags, v.outer.n, mr);
+  });
+  c->r_candidates += v.outer.n;
+  return true;
+}
+
 // Evaluate the variants, all deriving head relation H: join, project, sort, reduce by key.
 // `extra` (optional) is appended to the candidates before the sort (loaded facts of H in a
 // non-recursive stratum).  Returns the sorted unique candidates.
@@ -282,6 +318,25 @@ constexpr int kSlotTotals = 16;          // uint64 candidate totals of the varia
 KeyTags evaluate(Ctx* c, Relation& H, std::vector<Variant>& variants, const Source* extra, const KeyLayout& cand_layout,
                  bool want_head_pos, int defer_slot = -1) {
   const int ckb = cand_layout.total_bits <= 32 ? 4 : 8;
+  const Variant* only = nullptr;           // the one variant with rows to scan
+  for (const Variant& v : variants) if (v.outer.n) { if (only) { only = nullptr; break; } only = &v; }
+  if (only && !extra && !want_head_pos && copies_rows(c, *only, H, cand_layout)) {
+    // the rows of another relation as they are: nothing to count, sort or reduce
+    const Source& o = only->outer;
+    KeyTags out;
+    out.n = o.n;
+    out.keys = DevBuf(c, (size_t)o.n * ckb);
+    out.tags = DevBuf(c, (size_t)o.n * 4);
+    c->note_bytes = (int64_t)o.n * (o.key_bytes + ckb + 8);
+    const unsigned g = grid_for(o.n, 256);
+    if (o.key_bytes == 4 && ckb == 4) XLOG_LAUNCH(c, (k_copy_rows<uint32_t, uint32_t>), g, 256, 0, (const uint32_t*)o.keys, o.tags, o.n, o.layout, cand_layout, out.keys.as<uint32_t>(), out.tags.as<float>());
+    else if (o.key_bytes == 4) XLOG_LAUNCH(c, (k_copy_rows<uint32_t, uint64_t>), g, 256, 0, (const uint32_t*)o.keys, o.tags, o.n, o.layout, cand_layout, out.keys.as<uint64_t>(), out.tags.as<float>());
+    else if (ckb == 4) XLOG_LAUNCH(c, (k_copy_rows<uint64_t, uint32_t>), g, 256, 0, (const uint64_t*)o.keys, o.tags, o.n, o.layout, cand_layout, out.keys.as<uint32_t>(), out.tags.as<float>());
+    else XLOG_LAUNCH(c, (k_copy_rows<uint64_t, uint64_t>), g, 256, 0, (const uint64_t*)o.keys, o.tags, o.n, o.layout, cand_layout, out.keys.as<uint64_t>(), out.tags.as<float>());
+    c->r_candidates += o.n;
+    c->r_unique += o.n;
+    return out;
+  }
   std::vector<Counted> counted;
   counted.reserve(variants.size());
   if (variants.size() > 16) fail(XLOG_ERR_UNSUPPORTED, "too many rule variants for one head");

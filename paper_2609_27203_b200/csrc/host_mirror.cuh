@@ -128,6 +128,37 @@ void launch_changed_emit(Ctx* c, uint32_t* words, uint32_t nwords, unsigned tile
   else XLOG_LAUNCH(c, (k_mirror_changed_emit<uint32_t, 4>), tiles, kMirBlock, 0, words, nwords, base, table, keys, tags, skip);
 }
 
+// A mirror with nothing in it: every slot empty, no key changed or present, the counters n0 words from slot0 (and n1 from slot1) zero.
+void clear_mirror(Ctx* c, void* table, uint64_t slots, int32_t empty, void* changed, void* present, uint32_t word_quads, int slot0, int n0, int slot1 = 0, int n1 = 0) {
+  const MirrorClear P{(int4*)table, slots / 4, empty, {(uint4*)changed, (uint4*)present}, word_quads,
+                      {(unsigned long long*)(c->d_ctrl + slot0), (unsigned long long*)(c->d_ctrl + slot1)}, {n0, n1}};
+  XLOG_LAUNCH(c, k_mirror_clear, grid_for(std::max<uint64_t>(P.nquads, 2ull * word_quads), 256 * 2), 256, 0, P);
+}
+
+// The occupied slots of a table, in slot order, as (key, tag) rows of the relation: count, prefix, write.  `out` has room for all of them;
+// their number is left in kSlotA.
+void emit_mirror(Ctx* c, const int32_t* table, uint64_t slots, int32_t empty, const KeyLayout& from, const KeyLayout& to, int64_t rows, KeyTags& out) {
+  const uint64_t nquads = slots / 4;
+  const unsigned tiles = (unsigned)((slots + kMirSlotsPerTile - 1) / kMirSlotsPerTile);
+  DevBuf sums(c, (size_t)tiles * 4);
+  c->note_bytes = (int64_t)slots * 4;
+  XLOG_LAUNCH(c, k_mirror_full_count, tiles, kMirBlock, 0, reinterpret_cast<const int4*>(table), nquads, empty, sums.as<uint32_t>());
+  XLOG_LAUNCH(c, (k_scan_spine<uint32_t>), 1, 1024, 0, sums.as<uint32_t>(), (int64_t)tiles, ctrl_u32(c, kSlotA));
+  c->note_bytes = (int64_t)slots * 4 + rows * 8;
+  XLOG_LAUNCH(c, (k_mirror_full_emit<uint32_t>), tiles, kMirBlock, 0, reinterpret_cast<const int4*>(table), nquads, empty, (const uint32_t*)sums.as<uint32_t>(), from, to,
+              out.keys.as<uint32_t>(), out.tags.as<float>());
+}
+KeyTags mirror_rows_buffer(Ctx* c, uint64_t rows) {
+  KeyTags k;
+  k.n = (uint32_t)rows;
+  k.keys = DevBuf(c, (size_t)std::max<uint64_t>(rows, 1) * 4);
+  k.tags = DevBuf(c, (size_t)std::max<uint64_t>(rows, 1) * 4);
+  return k;
+}
+// A relation of a small key space is written out at its upper bound, every key, behind the rounds that derive it: the read of their
+// counters is then the evaluation's last wait instead of one in the middle (13 to 15 us).  Only where that is little of what is free.
+bool emits_ahead(Ctx* c, uint64_t slots) { return slots * 8 <= kDeferBytes && slots * 8 <= c->arena.largest_free() / 16; }
+
 template <typename T> void sig_add(std::vector<char>& sig, const T& v) {
   const char* p = reinterpret_cast<const char*>(&v);
   sig.insert(sig.end(), p, p + sizeof(T));
@@ -230,8 +261,9 @@ void resident_body(Ctx* c, Resident& R, const std::vector<JoinSpec>& specs, cons
 
 // Run rounds on the device until the delta is empty, the round budget is used up or a round needs more tiles than
 // planned.  Returns the final state block (read once, after the loop).
+// `behind` (may be empty) issues what is to run behind the loop's one launch, before the state is read.
 ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*>& rs, bool is_max, const MirrorArgs& mr_host, uint32_t bm_quads,
-                      unsigned ch_tiles, uint32_t n_delta, int64_t rounds_left, uint64_t new_seen) {
+                      unsigned ch_tiles, uint32_t n_delta, int64_t rounds_left, uint64_t new_seen, const std::function<void()>& behind) {
   Relation& H = *c->rels[h];
   std::vector<JoinSpec> specs;
   for (const RuleC* r : rs)
@@ -303,8 +335,14 @@ ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*
       R.sig = std::move(sig);
     }
     XLOG_CUDA(cudaGraphLaunch(R.exec, c->stream));
-    read_state();
-    c->launches = l0 + R.body_launches * (int64_t)out.bodies;
+    const int64_t l1 = c->launches;
+    if (behind) {
+      behind();
+      sync_ctrl_end(c);
+      memcpy(&out, c->h_ctrl + kSlotResState, sizeof out);
+    } else read_state();
+    c->launches += R.body_launches * (int64_t)out.bodies - (l1 - l0);
+    if (behind) c->ended_at = c->launches;
   } else {
     unsigned long long seen = 0;
     uint32_t rows = n_delta;

@@ -86,8 +86,6 @@ void stratum_row_fixpoint(Ctx* c, const std::vector<int>& comp, const std::vecto
   const uint64_t dom = (uint64_t)1 << bits, slots = dom;
   const uint32_t nwords = (uint32_t)(dom / 32);
   std::vector<Head> heads(comp.size());
-  zero_ctrl(c, kSlotMultiNew, kMultiMaxHeads);
-  zero_ctrl(c, kSlotRow, kRowTotals);
   for (size_t i = 0; i < comp.size(); ++i) {
     Head& X = heads[i];
     X.H = c->rels[comp[i]];
@@ -95,13 +93,11 @@ void stratum_row_fixpoint(Ctx* c, const std::vector<int>& comp, const std::vecto
     X.is_max = H.sr == XLOG_SR_MAXPLUS;
     X.empty = X.is_max ? kMirrorEmptyMax : kMirrorEmptyMin;
     X.table = DevBuf(c, slots * 4); X.bitmap = DevBuf(c, (size_t)nwords * 4); X.present = DevBuf(c, (size_t)nwords * 4);
-    XLOG_LAUNCH(c, k_fill_i32, grid_for(slots, 256 * 8), 256, 0, X.table.as<int32_t>(), slots, X.empty);
-    XLOG_CUDA(cudaMemsetAsync(X.bitmap.p, 0, (size_t)nwords * 4, c->stream));
-    XLOG_CUDA(cudaMemsetAsync(X.present.p, 0, (size_t)nwords * 4, c->stream));
+    clear_mirror(c, X.table.p, slots, X.empty, X.bitmap.p, X.present.p, (nwords + 3) / 4, kSlotMultiNew, i == 0 ? kMultiMaxHeads : 0, kSlotRow, i == 0 ? kRowTotals : 0);
     X.n_start = H.n;
     if (X.n_start)
       XLOG_LAUNCH(c, (k_mirror_scatter<uint32_t>), grid_for(X.n_start, 256, 1 << 30), 256, 0, (const uint32_t*)H.keys(), (const float*)H.tags(), X.n_start, H.layout,
-                  H.layout, X.table.as<int32_t>(), X.present.as<uint32_t>());
+                  H.layout, X.table.as<int32_t>(), X.present.as<uint32_t>(), (uint32_t*)nullptr, (float*)nullptr);
     X.mr = MirrorArgs{X.table.as<int32_t>(), X.bitmap.as<uint32_t>(), (unsigned long long*)(c->d_ctrl + kSlotMultiNew + i), (uint32_t)(dom - 1), ctrl_u32(c, kSlotErr)};
   }
   c->unique_untracked = true;
@@ -120,6 +116,7 @@ void stratum_row_fixpoint(Ctx* c, const std::vector<int>& comp, const std::vecto
         if (vs[v].outer.n == 0) continue;
         Head* T = nullptr;
         for (size_t i = 0; i < comp.size(); ++i) if (comp[i] == vs[v].rule->plan.head_rel) T = &heads[i];
+        if (mirror_rows(c, vs[v], *T->H, nullptr, T->is_max, T->mr)) { seed_total += vs[v].outer.n; continue; }
         counted.emplace_back();
         count_variant(c, vs[v], *T->H, counted.back(), kSlotTotals + (int)counted.size() - 1);
         target.push_back(T);
@@ -140,6 +137,7 @@ void stratum_row_fixpoint(Ctx* c, const std::vector<int>& comp, const std::vecto
     }
   }
   uint64_t total_new = 0;
+  KeyTags ahead;                           // the relation, if it has been written out behind the rounds
   if (seed_total) {
     RowFix P{};
     P.n_heads = (int)heads.size(); P.n_rules = (int)rules.size();
@@ -164,7 +162,11 @@ void stratum_row_fixpoint(Ctx* c, const std::vector<int>& comp, const std::vecto
       default: XLOG_ROW_FIX(4); break;
     }
 #undef XLOG_ROW_FIX
-    sync_ctrl(c);
+    if (heads.size() == 1 && emits_ahead(c, slots)) {
+      ahead = mirror_rows_buffer(c, slots);
+      emit_mirror(c, heads[0].table.as<int32_t>(), slots, heads[0].empty, H0.layout, H0.layout, (int64_t)slots, ahead);
+      sync_ctrl_end(c);
+    } else sync_ctrl(c);
     const uint64_t cand = c->h_ctrl[kSlotRow + kRowCandidates], changed = c->h_ctrl[kSlotRow + kRowChanged], n_new = c->h_ctrl[kSlotRow + kRowNew];
     c->r_candidates += (int64_t)cand;
     c->r_new += (int64_t)n_new; c->r_improved += (int64_t)changed - (int64_t)n_new;
@@ -176,24 +178,22 @@ void stratum_row_fixpoint(Ctx* c, const std::vector<int>& comp, const std::vecto
   // come with the count (one control read per head), with one head it is what was there plus what was new
   for (Head& X : heads) {
     Relation& H = *X.H;
-    const uint64_t nquads = slots / 4;
-    const unsigned tiles = (unsigned)((slots + kMirSlotsPerTile - 1) / kMirSlotsPerTile);
-    DevBuf sums(c, (size_t)tiles * 4);
-    c->note_bytes = (int64_t)slots * 4;
-    XLOG_LAUNCH(c, k_mirror_full_count, tiles, kMirBlock, 0, (const int4*)X.table.as<int4>(), nquads, X.empty, sums.as<uint32_t>());
-    XLOG_LAUNCH(c, (k_scan_spine<uint32_t>), 1, 1024, 0, sums.as<uint32_t>(), (int64_t)tiles, ctrl_u32(c, kSlotA));
     uint64_t n_out = (uint64_t)X.n_start + total_new;
-    if (heads.size() > 1) { sync_ctrl(c); n_out = (uint32_t)c->h_ctrl[kSlotA]; }
-    KeyTags full;
-    full.n = (uint32_t)n_out;
-    full.keys = DevBuf(c, (size_t)std::max<uint64_t>(n_out, 1) * 4);
-    full.tags = DevBuf(c, (size_t)std::max<uint64_t>(n_out, 1) * 4);
-    if (n_out) {
-      c->note_bytes = (int64_t)slots * 4 + (int64_t)n_out * 8;
-      XLOG_LAUNCH(c, (k_mirror_full_emit<uint32_t>), tiles, kMirBlock, 0, (const int4*)X.table.as<int4>(), nquads, X.empty, (const uint32_t*)sums.as<uint32_t>(), H.layout,
-                  H.layout, full.keys.as<uint32_t>(), full.tags.as<float>());
+    if (heads.size() > 1) {
+      const unsigned tiles = (unsigned)((slots + kMirSlotsPerTile - 1) / kMirSlotsPerTile);
+      DevBuf sums(c, (size_t)tiles * 4);
+      c->note_bytes = (int64_t)slots * 4;
+      XLOG_LAUNCH(c, k_mirror_full_count, tiles, kMirBlock, 0, (const int4*)X.table.as<int4>(), slots / 4, X.empty, sums.as<uint32_t>());
+      XLOG_LAUNCH(c, (k_scan_spine<uint32_t>), 1, 1024, 0, sums.as<uint32_t>(), (int64_t)tiles, ctrl_u32(c, kSlotA));
+      sync_ctrl(c);
+      n_out = (uint32_t)c->h_ctrl[kSlotA];
     }
-    set_current(H, std::move(full));
+    if (!ahead.keys.p) {
+      ahead = mirror_rows_buffer(c, n_out);
+      if (n_out) emit_mirror(c, X.table.as<int32_t>(), slots, X.empty, H.layout, H.layout, (int64_t)n_out, ahead);
+    }
+    ahead.n = (uint32_t)n_out;
+    set_current(H, std::move(ahead));
     X.table.reset(); X.bitmap.reset(); X.present.reset();
     if (c->flags & XLOG_FLAG_CHECK_INVARIANTS) {
       XLOG_LAUNCH(c, (k_check_sorted<uint32_t>), grid_for(H.n, 256), 256, 0, (const uint32_t*)H.keys(), (int64_t)H.n, ctrl_u32(c, kSlotErr));
@@ -259,13 +259,12 @@ void row_sums_rounds(Ctx* c, Relation& H, const std::vector<RowSumRule>& rules, 
   } while (0)
   if (H.sr == XLOG_SR_SUMPROD) XLOG_ROW_SUMS(OpSum); else XLOG_ROW_SUMS(OpLse);
 #undef XLOG_ROW_SUMS
-  const uint64_t nquads = slots / 4;
-  const unsigned tiles = (unsigned)((slots + kMirSlotsPerTile - 1) / kMirSlotsPerTile);
-  DevBuf sums(c, (size_t)tiles * 4);
-  c->note_bytes = (int64_t)slots * 4;
-  XLOG_LAUNCH(c, k_mirror_full_count, tiles, kMirBlock, 0, (const int4*)table.as<int4>(), nquads, kMirrorEmptyMin, sums.as<uint32_t>());
-  XLOG_LAUNCH(c, (k_scan_spine<uint32_t>), 1, 1024, 0, sums.as<uint32_t>(), (int64_t)tiles, ctrl_u32(c, kSlotA));
-  sync_ctrl(c);
+  KeyTags full;
+  if (emits_ahead(c, slots)) {
+    full = mirror_rows_buffer(c, slots);
+    emit_mirror(c, table.as<int32_t>(), slots, kMirrorEmptyMin, H.layout, H.layout, (int64_t)slots, full);
+    sync_ctrl_end(c);
+  } else sync_ctrl(c);
   c->r_candidates += (int64_t)c->h_ctrl[kSlotRow + kRsCandidates];
   c->r_unique += (int64_t)c->h_ctrl[kSlotRow + kRsUnique];
   c->r_new += (int64_t)c->h_ctrl[kSlotRow + kRsNew];
@@ -273,13 +272,12 @@ void row_sums_rounds(Ctx* c, Relation& H, const std::vector<RowSumRule>& rules, 
   c->r_iterations += (int64_t)c->h_ctrl[kSlotRow + kRsRounds];
   if (c->h_ctrl[kSlotRow + kRsCapped])
     fail(XLOG_ERR_CONVERGENCE_FAILURE, "iteration cap reached before the fixpoint (cyclic derivations under a non-idempotent oplus never end)");
-  KeyTags full;
-  full.n = (uint32_t)c->h_ctrl[kSlotA];
-  full.keys = DevBuf(c, (size_t)std::max(full.n, 1u) * 4);
-  full.tags = DevBuf(c, (size_t)std::max(full.n, 1u) * 4);
-  c->note_bytes = (int64_t)slots * 4 + (int64_t)full.n * 8;
-  XLOG_LAUNCH(c, (k_mirror_full_emit<uint32_t>), tiles, kMirBlock, 0, (const int4*)table.as<int4>(), nquads, kMirrorEmptyMin, (const uint32_t*)sums.as<uint32_t>(), H.layout,
-              H.layout, full.keys.as<uint32_t>(), full.tags.as<float>());
+  const uint32_t n_out = H.n + (uint32_t)c->h_ctrl[kSlotRow + kRsNew];       // what the seed round derived, and what was new after it
+  if (!full.keys.p) {
+    full = mirror_rows_buffer(c, n_out);
+    emit_mirror(c, table.as<int32_t>(), slots, kMirrorEmptyMin, H.layout, H.layout, (int64_t)n_out, full);
+  }
+  full.n = n_out;
   set_current(H, std::move(full));
 }
 

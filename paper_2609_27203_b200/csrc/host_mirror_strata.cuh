@@ -54,14 +54,12 @@ void stratum_recursive_mirror(Ctx* c, int h, const std::vector<const RuleC*>& rs
   int32_t* table = R ? R->table.as<int32_t>() : table_own.as<int32_t>();
   uint4* bitmap = R ? R->bitmap.as<uint4>() : bitmap_own.as<uint4>();
   uint32_t* ch_sums = R ? R->ch_sums.as<uint32_t>() : ch_sums_own.as<uint32_t>();
-  XLOG_LAUNCH(c, k_fill_i32, grid_for(slots, 256 * 8), 256, 0, table, slots, empty);
-  XLOG_CUDA(cudaMemsetAsync(bitmap, 0, (size_t)bm_quads * 16, c->stream));
-  XLOG_CUDA(cudaMemsetAsync(present, 0, (size_t)bm_quads * 16, c->stream));
+  clear_mirror(c, table, slots, empty, bitmap, present, bm_quads, kSlotMirNew, 2);
   // what the relation holds now (its loaded facts, or the result of an earlier fixpoint) is the starting state
   const uint32_t n_start = H.n;
   if (n_start)
-    XLOG_LAUNCH(c, (k_mirror_scatter<uint32_t>), grid_for(n_start, 256, 1 << 30), 256, 0, (const uint32_t*)H.keys(), (const float*)H.tags(), n_start, H.layout, M, table, present);
-  zero_ctrl(c, kSlotMirNew, 2);
+    XLOG_LAUNCH(c, (k_mirror_scatter<uint32_t>), grid_for(n_start, 256, 1 << 30), 256, 0, (const uint32_t*)H.keys(), (const float*)H.tags(), n_start, H.layout, M, table, present,
+                R ? R->dkeys.as<uint32_t>() : (uint32_t*)nullptr, R ? R->dtags.as<float>() : (float*)nullptr);
   const MirrorArgs mr{table, reinterpret_cast<uint32_t*>(bitmap), (unsigned long long*)(c->d_ctrl + kSlotMirNew), (uint32_t)(dom - 1),
                       ctrl_u32(c, kSlotErr)};
   c->unique_untracked = true;
@@ -76,6 +74,7 @@ void stratum_recursive_mirror(Ctx* c, int h, const std::vector<const RuleC*>& rs
     uint64_t total = 0;
     for (Variant& v : vs) {
       if (v.outer.n == 0) continue;
+      if (mirror_rows(c, v, H, ML, is_max, mr)) { total += v.outer.n; continue; }
       if (grouped && v.outer.keys == dk && v.rule->plan.atoms[v.outer_atom].rel == h) {
         // a delta variant of the grouped shape: the delta is ordered by the probed column
         const uint64_t t = grouped_apply(c, v, H, M, carried_bits, is_max, mr);
@@ -104,6 +103,7 @@ void stratum_recursive_mirror(Ctx* c, int h, const std::vector<const RuleC*>& rs
     return false;
   };
 
+  KeyTags ahead;                           // the relation, if it has been written out behind the rounds
   int64_t round = 0;
   bool plain_rules_done = false;           // the rules without an atom over H have had their one evaluation
   bool converged = false;
@@ -116,11 +116,12 @@ void stratum_recursive_mirror(Ctx* c, int h, const std::vector<const RuleC*>& rs
       if (!over_h(r)) { const int outer = seed_outer(comp, r); plain.push_back(Variant{r, outer, full_source(*c->rels[r->plan.atoms[outer].rel])}); }
     host_apply(plain);
     plain_rules_done = true;
-    if (n_start) {
-      XLOG_CUDA(cudaMemcpyAsync(R->dkeys.p, H.keys(), (size_t)n_start * 4, cudaMemcpyDeviceToDevice, c->stream));
-      XLOG_CUDA(cudaMemcpyAsync(R->dtags.p, H.tags(), (size_t)n_start * 4, cudaMemcpyDeviceToDevice, c->stream));
+    std::function<void()> behind;
+    if (emits_ahead(c, slots)) {
+      ahead = mirror_rows_buffer(c, slots);
+      behind = [&]() { emit_mirror(c, table, slots, empty, M, H.layout, (int64_t)slots, ahead); };
     }
-    const ResState s = run_resident(c, *R, h, rs, is_max, mr, bm_quads, ch_tiles, n_start, c->max_iter, 0);
+    const ResState s = run_resident(c, *R, h, rs, is_max, mr, bm_quads, ch_tiles, n_start, c->max_iter, 0, behind);
     round = s.rounds;
     c->r_iterations += s.rounds; c->r_candidates += (int64_t)s.candidates;
     c->r_new += (int64_t)s.n_new; c->r_improved += (int64_t)s.n_improved;
@@ -129,6 +130,7 @@ void stratum_recursive_mirror(Ctx* c, int h, const std::vector<const RuleC*>& rs
     if (s.status == kResCap) fail(XLOG_ERR_CONVERGENCE_FAILURE, "iteration cap reached before the fixpoint");
     if (s.status == kResOk || s.status == kResDone) converged = true;      // the delta ran empty
     // kResOverflow: a round needs more expand tiles than planned; the host redoes that round and finishes the job
+    if (!converged || c->ended_at != c->launches) ahead = KeyTags();      // not the relation, or not written (rounds launched one by one)
   }
   for (; !converged; ++round) {
     if (round >= c->max_iter) fail(XLOG_ERR_CONVERGENCE_FAILURE, "iteration cap reached before the fixpoint");
@@ -265,12 +267,12 @@ void stratum_recursive_mirror(Ctx* c, int h, const std::vector<const RuleC*>& rs
   }
   // the relation in sorted form: every occupied slot, in slot order
   const uint64_t n_out = (uint64_t)n_start + total_new;
-  KeyTags full;
+  const bool written = ahead.keys.p != nullptr;
+  KeyTags full = written ? std::move(ahead) : mirror_rows_buffer(c, n_out);
   full.n = (uint32_t)n_out;
-  full.keys = DevBuf(c, (size_t)std::max<uint64_t>(n_out, 1) * 4);
-  full.tags = DevBuf(c, (size_t)std::max<uint64_t>(n_out, 1) * 4);
-  bool counted_slots = false;              // kSlotA holds the number of occupied slots (for the invariant check)
-  if (n_out && grouped && carried_bits <= 6) {
+  bool counted_slots = written;            // kSlotA holds the number of occupied slots (for the invariant check)
+  if (written) {
+  } else if (n_out && grouped && carried_bits <= 6) {
     // the mirror is ordered (column 1, column 0) and column 0 has at most 64 values: every row goes straight to its place
     // in the relation's order (mirror.cuh), found from the bitmap of present keys; no pass over empty slots, no sort
     const int per_node = 1 << carried_bits;
@@ -290,15 +292,7 @@ void stratum_recursive_mirror(Ctx* c, int h, const std::vector<const RuleC*>& rs
                 (const uint32_t*)base.as<uint32_t>(), H.layout.shift[0], H.layout.shift[1], full.keys.as<uint32_t>(), full.tags.as<float>());
     counted_slots = true;
   } else if (n_out) {
-    const uint64_t nquads = slots / 4;
-    const unsigned tiles = (unsigned)((slots + kMirSlotsPerTile - 1) / kMirSlotsPerTile);
-    DevBuf sums(c, (size_t)tiles * 4);
-    c->note_bytes = (int64_t)slots * 4;
-    XLOG_LAUNCH(c, k_mirror_full_count, tiles, kMirBlock, 0, (const int4*)table, nquads, empty, sums.as<uint32_t>());
-    XLOG_LAUNCH(c, (k_scan_spine<uint32_t>), 1, 1024, 0, sums.as<uint32_t>(), (int64_t)tiles, ctrl_u32(c, kSlotA));
-    c->note_bytes = (int64_t)slots * 4 + (int64_t)n_out * 8;
-    XLOG_LAUNCH(c, (k_mirror_full_emit<uint32_t>), tiles, kMirBlock, 0, (const int4*)table, nquads, empty, (const uint32_t*)sums.as<uint32_t>(), M, H.layout,
-                full.keys.as<uint32_t>(), full.tags.as<float>());
+    emit_mirror(c, table, slots, empty, M, H.layout, (int64_t)n_out, full);
     counted_slots = true;
     if (grouped && n_out > 1) {
       // rows came out in the mirror's order, (column 1, column 0) ascending: a stable sort on column 0's bits alone puts
@@ -378,7 +372,7 @@ void stratum_recursive_mirror_multi(Ctx* c, const std::vector<int>& comp, const 
     XLOG_CUDA(cudaMemsetAsync(X.present.p, 0, (size_t)X.bm_quads * 16, c->stream));
     if (X.n_start)
       XLOG_LAUNCH(c, (k_mirror_scatter<uint32_t>), grid_for(X.n_start, 256, 1 << 30), 256, 0, (const uint32_t*)H.keys(), (const float*)H.tags(), X.n_start, H.layout,
-                  H.layout, X.table.as<int32_t>(), X.present.as<uint32_t>());
+                  H.layout, X.table.as<int32_t>(), X.present.as<uint32_t>(), (uint32_t*)nullptr, (float*)nullptr);
     X.mr = MirrorArgs{X.table.as<int32_t>(), X.bitmap.as<uint32_t>(), (unsigned long long*)(c->d_ctrl + kSlotMultiNew + i), (uint32_t)(dom - 1),
                       ctrl_u32(c, kSlotErr)};
   }

@@ -166,11 +166,10 @@ void load_relation(Ctx* c, Relation& R, const int32_t* const* cols, const float*
     XLOG_LAUNCH(c, k_col_stats, grid_for(n, 256, kSMs * 8), 256, 0, in, dtags, n, R.arity, R.sr,
                 reinterpret_cast<int32_t*>(c->d_ctrl + kSlotA), ctrl_u32(c, kSlotErr), ctrl_u32(c, kSlotC));
   }
-  sync_ctrl(c);
+  sync_ctrl(c, kSlotA, 4);                                    // and the words are clear again
   const bool in_order = (uint32_t)c->h_ctrl[kSlotC] == 0;     // rows arrived strictly increasing: nothing to sort or combine
   const int32_t* mx = reinterpret_cast<const int32_t*>(c->h_ctrl + kSlotA);
   for (int i = 0; i < R.arity; ++i) R.col_max[i] = R.fact_max[i] = R.val_max[i] = mx[i];
-  zero_ctrl(c, kSlotA, 4);
   R.layout = make_layout(R.arity, R.col_max);
   if (R.layout.total_bits > 64) fail(XLOG_ERR_CAPACITY_EXCEEDED, "packed key of relation '" + R.name + "' needs more than 64 bits");
   R.key_bytes = R.layout.total_bits <= 32 ? 4 : 8;
@@ -210,10 +209,17 @@ Index& ensure_index(Ctx* c, Relation& R, int col) {
   Index& ix = R.idx[col];
   if (ix.valid) return ix;
   ++c->r_index_builds;
-  ensure_soa(c, R);
   ix = Index();
   ix.domain = (int64_t)R.val_max[col] + 1;
   ix.n_other = R.arity - 1;
+  if (col == 0 && !R.soa_valid && R.n) {                      // columns and offsets in one launch
+    ColPtrsMut out{};
+    for (int i = 0; i < R.arity; ++i) { R.cols[i] = DevBuf(c, (size_t)R.n * 4); out.c[i] = R.cols[i].as<int32_t>(); }
+    ix.off = DevBuf(c, ((size_t)ix.domain + 1) * 4);
+    DISPATCH_K(R.key_bytes, XLOG_LAUNCH(c, (k_unpack_offsets<K>), grid_for(std::max<int64_t>(R.n, ix.domain + 1), 256), 256, 0, (const K*)R.keys(), R.n, R.layout, R.dicts(), out,
+                                         ix.domain, ix.off.as<uint32_t>()));
+    R.soa_valid = true;
+  } else ensure_soa(c, R);
   const int32_t* lead = nullptr;
   if (col == 0 || R.n == 0) {
     lead = R.cols[col].as<int32_t>();
@@ -253,8 +259,10 @@ Index& ensure_index(Ctx* c, Relation& R, int col) {
     ix.valid = true;
     return ix;
   }
-  ix.off = DevBuf(c, ((size_t)ix.domain + 1) * 4);
-  XLOG_LAUNCH(c, k_build_offsets, grid_for(ix.domain + 1, 256), 256, 0, lead, R.n, ix.domain, ix.off.as<uint32_t>());
+  if (!ix.off.p) {
+    ix.off = DevBuf(c, ((size_t)ix.domain + 1) * 4);
+    XLOG_LAUNCH(c, k_build_offsets, grid_for(ix.domain + 1, 256), 256, 0, lead, R.n, ix.domain, ix.off.as<uint32_t>());
+  }
   ix.valid = true;
   return ix;
 }

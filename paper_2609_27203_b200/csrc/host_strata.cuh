@@ -41,6 +41,16 @@ void stratum_once(Ctx* c, int head, const std::vector<const RuleC*>& rs) {
   c->r_new += (int64_t)H.n - H.n_facts;
 }
 
+// The same rows, owned by somebody else: a delta that is the whole relation, which stays as it is until the delta has been joined (every
+// round drops its deltas before it changes a relation).
+KeyTags borrowed(const KeyTags& u) {
+  KeyTags b;
+  b.n = u.n;
+  b.keys.p = u.keys.p; b.keys.bytes = u.keys.bytes;
+  b.tags.p = u.tags.p; b.tags.bytes = u.tags.bytes;
+  return b;
+}
+
 // Recursive component under a non-idempotent oplus (logsumexp / sum): the tag of a tuple is the oplus over all of its
 // derivations, which is finite when the tuples' dependencies form a DAG (path counting, path-probability sums on an
 // acyclic graph).  Algorithm 1 with the delta carrying tag DIFFERENCES: the rules are linear in the component's relations
@@ -93,13 +103,9 @@ void stratum_recursive_additive(Ctx* c, const std::vector<int>& comp, const std:
       if (u.n == 0) continue;
       derived += u.n;
       if (H.n == 0) {                                       // nothing to merge with: I is Delta
-        KeyTags copy; copy.n = u.n;
-        copy.keys = DevBuf(c, (size_t)u.n * H.key_bytes); copy.tags = DevBuf(c, (size_t)u.n * 4);
-        XLOG_CUDA(cudaMemcpyAsync(copy.keys.p, u.keys.p, (size_t)u.n * H.key_bytes, cudaMemcpyDeviceToDevice, c->stream));
-        XLOG_CUDA(cudaMemcpyAsync(copy.tags.p, u.tags.p, (size_t)u.n * 4, cudaMemcpyDeviceToDevice, c->stream));
         c->r_new += u.n;
-        set_current(H, std::move(copy));
-        delta[pr.first] = std::move(u);
+        delta[pr.first] = borrowed(u);
+        set_current(H, std::move(u));
         continue;
       }
       MergeResult m;
@@ -187,13 +193,9 @@ void stratum_recursive(Ctx* c, const std::vector<int>& comp, const std::vector<c
       KeyTags& u = produced[i].second;
       if (u.n == 0) continue;
       if (H.n == 0) {                                       // nothing to merge with: the relation and its delta are the list
-        KeyTags copy; copy.n = u.n;
-        copy.keys = DevBuf(c, (size_t)u.n * H.key_bytes); copy.tags = DevBuf(c, (size_t)u.n * 4);
-        XLOG_CUDA(cudaMemcpyAsync(copy.keys.p, u.keys.p, (size_t)u.n * H.key_bytes, cudaMemcpyDeviceToDevice, c->stream));
-        XLOG_CUDA(cudaMemcpyAsync(copy.tags.p, u.tags.p, (size_t)u.n * 4, cudaMemcpyDeviceToDevice, c->stream));
         merged[i].n_new = u.n;
-        merged[i].full = std::move(copy);
-        merged[i].delta = std::move(u);                     // (the count stays behind for the loop below)
+        merged[i].delta = borrowed(u);
+        merged[i].full = std::move(u);                      // (the count stays behind for the loop below)
         continue;
       }
       if (!H.cur_owned && H.n_facts) {
@@ -245,7 +247,6 @@ void run_fixpoint(Ctx* c) {
   if (c->poisoned) fail(XLOG_ERR_INVALID_STATE, "derived relations are poisoned by an earlier failure; call xlog_ctx_reset_idb");
   c->poisoned = true;                      // cleared on success
   c->ended_at = -1;
-  zero_ctrl(c, kSlotErr);
   propagate_bounds(c);
   for (const std::vector<int>& comp : components(c)) {
     std::vector<const RuleC*> rs;

@@ -272,6 +272,16 @@ __device__ __forceinline__ void mirror_apply(const MirrorArgs& m, uint32_t key, 
   if (SINK == kSinkMin ? v < cur : v > cur) mirror_commit<SINK>(m, key, v);
 }
 
+// A rule of one atom whose rows all match: every row is one candidate, straight into the mirror.
+template <typename KO, int SINK>
+__global__ void __launch_bounds__(256) k_mirror_rows(const __grid_constant__ JoinSpec S, const KO* __restrict__ okeys, const float* __restrict__ otags, uint32_t n, MirrorArgs m) {
+  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  uint4 info = make_uint4(0, 0, 0, 0);
+  const float tag = otags[i];
+  if (join_count_kv<KO>(S, okeys[i], tag, 0, &info, m.err)) mirror_apply<SINK>(m, info.z, tag);
+}
+
 // One thread per tile: the first and last outer row that contribute candidates to the tile
 // (r_lo = last row with start <= tile begin, r_hi = last row with start < tile end).  Done for all
 // tiles at once so that the dependent binary-search loads of one tile overlap with those of the others.

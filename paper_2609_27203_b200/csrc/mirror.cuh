@@ -30,13 +30,34 @@ __device__ __forceinline__ uint32_t relayout_key(const KeyLayout& from, const Ke
   return out;
 }
 
+// An empty mirror: table, both bitmaps, and the control words that count in it, in one launch.
+struct MirrorClear {
+  int4* table;                     // slots / 4 vectors
+  uint64_t nquads;
+  int32_t empty;
+  uint4* words[2];                 // the bitmaps
+  uint32_t word_quads;
+  unsigned long long* ctrl[2];
+  int n_ctrl[2];
+};
+static __global__ void __launch_bounds__(256) k_mirror_clear(const __grid_constant__ MirrorClear P) {
+  const uint64_t t = (uint64_t)blockIdx.x * 256 + threadIdx.x, step = (uint64_t)gridDim.x * 256;
+  const int4 e = make_int4(P.empty, P.empty, P.empty, P.empty);
+  for (uint64_t i = t; i < P.nquads; i += step) P.table[i] = e;
+  for (uint64_t i = t; i < 2ull * P.word_quads; i += step) P.words[i >= P.word_quads][i >= P.word_quads ? i - P.word_quads : i] = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) if (t < (uint64_t)P.n_ctrl[k]) P.ctrl[k][t] = 0ull;
+}
+
 template <typename K>
 __global__ void __launch_bounds__(256) k_mirror_scatter(const K* __restrict__ keys, const float* __restrict__ tags, uint32_t n,
-                                                        KeyLayout from, KeyLayout to, int32_t* __restrict__ table, uint32_t* __restrict__ present) {
+                                                        KeyLayout from, KeyLayout to, int32_t* __restrict__ table, uint32_t* __restrict__ present,
+                                                        uint32_t* __restrict__ dkeys, float* __restrict__ dtags) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) {
     const uint32_t key = relayout_key(from, to, (uint32_t)keys[i]);
     table[key] = f2ord(tags[i]);
+    if (dkeys) { dkeys[i] = key; dtags[i] = tags[i]; }     // the first delta, where it is all that is there
     atomicOr(present + (key >> 5), 1u << (key & 31));
   }
 }

@@ -205,6 +205,29 @@ static __global__ void __launch_bounds__(256) k_build_offsets(const int32_t* __r
   }
 }
 
+// k_unpack and, over column 0, k_build_offsets in one launch.
+template <typename K>
+__global__ void __launch_bounds__(256) k_unpack_offsets(const K* __restrict__ keys, uint32_t n, KeyLayout L, DictSet D, ColPtrsMut cols, int64_t domain, uint32_t* __restrict__ off) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+  auto value = [&](K k, int c) {
+    const int32_t code = key_col<K>(L, k, c);
+    return D.n[c] ? D.v[c][min((uint32_t)code, D.n[c] - 1)] : code;
+  };
+  for (int64_t v = t; v <= domain; v += step) {
+    uint32_t lo = 0, hi = n;
+    while (lo < hi) {
+      const uint32_t mid = lo + ((hi - lo) >> 1);
+      if ((int64_t)value(keys[mid], 0) < v) lo = mid + 1; else hi = mid;
+    }
+    off[v] = lo;
+  }
+  for (int64_t i = t; i < n; i += step) {
+    const K k = keys[i];
+#pragma unroll
+    for (int c = 0; c < kMaxArity; ++c) if (c < L.arity) cols.c[c][i] = value(k, c);
+  }
+}
+
 template <typename K>
 __global__ void __launch_bounds__(256) k_check_sorted(const K* __restrict__ keys, int64_t n, uint32_t* __restrict__ err) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x + 1; i < n; i += (int64_t)gridDim.x * blockDim.x)
@@ -558,6 +581,20 @@ __global__ void __launch_bounds__(kMrgBlock) k_merge(const K* __restrict__ A, co
       }
       ++pf; ++y;
     }
+  }
+}
+
+// Rows under another layout of the same columns.
+template <typename KI, typename KO>
+__global__ void __launch_bounds__(256) k_copy_rows(const KI* __restrict__ keys, const float* __restrict__ tags, uint32_t n, KeyLayout from, KeyLayout to, KO* __restrict__ out_keys,
+                                                   float* __restrict__ out_tags) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const KI k = keys[i];
+    KO o = 0;
+#pragma unroll
+    for (int c = 0; c < kMaxArity; ++c) if (c < from.arity) o |= (KO)(uint32_t)key_col<KI>(from, k, c) << to.shift[c];
+    out_keys[i] = o;
+    out_tags[i] = tags[i];
   }
 }
 

@@ -11,6 +11,7 @@ namespace {
 template <typename F>
 xlog_status guarded(xlog_ctx* c, F&& f) {
   if (!c) return XLOG_ERR_INVALID_ARGUMENT;
+  xlog_status st;
   try {
     cudaSetDevice(c->device);
     f();
@@ -18,11 +19,14 @@ xlog_status guarded(xlog_ctx* c, F&& f) {
     return XLOG_OK;
   } catch (const Fail& e) {
     c->err = e.msg;
-    return e.st;
+    st = e.st;
   } catch (const std::exception& e) {
     c->err = e.what();
-    return XLOG_ERR_INTERNAL;
+    st = XLOG_ERR_INTERNAL;
   }
+  // a call that ended early leaves no error flag to the next: the flag word is clear whenever a call begins
+  if (c->d_ctrl) cudaMemsetAsync(c->d_ctrl + kSlotErr, 0, sizeof(uint64_t), c->stream);
+  return st;
 }
 
 // the sort pass needs more than 48 KB of dynamic shared memory and the largest carve-out

@@ -1,0 +1,82 @@
+"""Rules of one atom: heads that copy the atom (no count, sort or reduce), heads that permute or repeat its columns, atoms that filter;
+32- and 64-bit keys, every semiring, as rules of their own and as seeds of a recursion; against the oracle, counters included."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2609_27203_b200 import workloads as W
+from paper_2609_27203_b200.workloads import Atom, Program, Rule, V, Var
+from tests import helpers as H
+
+pytestmark = pytest.mark.gpu
+SEMIRINGS = (W.MAXPLUS, W.MINPLUS, W.LOGSUMEXP, W.SUMPROD)
+
+
+def rows(n, top, seed):
+    rng = np.random.default_rng(seed)
+    cols = [rng.integers(0, t + 1, n).astype(np.int32) for t in top]
+    if n:
+        for c, t in zip(cols, top):
+            c[0] = t                                          # the columns' widths
+    key = np.unique(np.stack(cols, 1), axis=0) if n else np.zeros((0, len(top)), np.int32)
+    key = rng.permutation(key)
+    return [np.ascontiguousarray(key[:, i]) for i in range(len(top))], (0.25 + rng.random(len(key))).astype(np.float32)
+
+
+def check(prog, flags=0, tol=0.0):
+    from paper_2609_27203_b200 import xlog
+    o, oids, _ = oracle.load_program(prog)
+    o.run("seminaive")
+    ctx, ids, _ = xlog.load_program(prog, arena_bytes=1 << 29, flags=flags | xlog.FLAG_CHECK_INVARIANTS)
+    for _ in range(2):
+        rec = ctx.fixpoint()
+        for name in prog.outputs:
+            H.compare_relations(ctx.read(ids[name]), o.read(oids[name]), abs_tol=tol, what=name)
+        ctx.reset_idb()
+    ctx.close()
+    return rec
+
+
+@pytest.mark.parametrize("sr", SEMIRINGS)
+@pytest.mark.parametrize("n,top", [(0, (9,)), (1, (0,)), (255, (300,)), (5000, (99, 77)), (3000, (1 << 20, 1 << 19)), (2000, (7, 1 << 30, 5)), (4097, (1 << 15, 1 << 15, 3))])
+def test_heads_of_one_atom(sr, n, top):
+    cols, tags = rows(n, top, len(top) + n)
+    k = len(top)
+    x = tuple(Var(i) for i in range(k))
+    rules = [Rule("same", tuple(V(i) for i in range(k)), (Atom("e", x),)),
+             Rule("turned", tuple(V(k - 1 - i) for i in range(k)), (Atom("e", x),)),
+             Rule("first", (V(0), V(0)), (Atom("e", x),)),
+             Rule("again", tuple(V(i) for i in range(k)), (Atom("same", x),))]
+    rel = {"e": (k, sr), "same": (k, sr), "turned": (k, sr), "first": (2, sr), "again": (k, sr)}
+    if k == 2:
+        rules.append(Rule("loops", (V(0),), (Atom("e", (Var(0), Var(0))),)))
+        rel["loops"] = (1, sr)
+    prog = Program(name="one_atom", relations=rel, rules=rules, facts={"e": (cols, tags)}, outputs=tuple(r for r in rel if r != "e"))
+    rec = check(prog, tol=0.0 if sr in (W.MAXPLUS, W.MINPLUS) else 1e-5)      # sums of up to a few hundred tags below 1.25 in another order
+    assert rec["candidates"] >= 4 * len(tags)
+
+
+@pytest.mark.parametrize("sr", SEMIRINGS)
+@pytest.mark.parametrize("n,scale", [(2, 1), (40, 1), (300, 1), (40, 1 << 14), (300, 1 << 13)])
+def test_seeds_of_a_recursion(sr, n, scale):                  # acyclic, so that sums end; ids far apart for 64-bit keys
+    from paper_2609_27203_b200 import xlog
+    rng = np.random.default_rng(n)
+    a, b = rng.integers(0, n, 3 * n), rng.integers(0, n, 3 * n)
+    key = np.unique(np.minimum(a, b) * n + np.maximum(a, b))
+    s, d = key // n, key % n
+    s, d = s[s != d], d[s != d]
+    if len(s) == 0:
+        s, d = np.array([0]), np.array([1])
+    w = (0.25 + rng.random(len(s))).astype(np.float32)
+    prog = W.closure_program((s * scale).astype(np.int32), (d * scale).astype(np.int32), np.log(w) if sr == W.LOGSUMEXP else (-w if sr == W.MAXPLUS else w), semiring=sr)
+    exact = sr in (W.MAXPLUS, W.MINPLUS)
+    for flags in (0, xlog.FLAG_NO_ROW_FIXPOINT, xlog.FLAG_NO_TAG_MIRROR, xlog.FLAG_NO_RESIDENT_LOOP):
+        o, oids, _ = oracle.load_program(prog)
+        o.run("seminaive")
+        ctx, ids, _ = xlog.load_program(prog, arena_bytes=1 << 29, flags=flags | xlog.FLAG_CHECK_INVARIANTS)
+        for _ in range(2):
+            ctx.fixpoint()
+            # path sums grow with the number of paths: relative, as the two sides round at other places (fp32 per round)
+            H.compare_relations(ctx.read(ids["path"]), o.read(oids["path"]), rel_tol=0.0 if exact else 1e-5, abs_tol=0.0 if exact else 1e-4, what=f"{sr} {flags}")
+            ctx.reset_idb()
+        ctx.close()
