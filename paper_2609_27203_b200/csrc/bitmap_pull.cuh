@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(256) k_bm_count(BmCount P) {
 // side by side in the table.
 struct BpColumns {
   int lanes;                       // lanes to a row, four columns each
-  int16_t at[kBpMaxCols];          // carried value at a position, -1: none
+  int32_t at[kBpMaxCols];          // what the carried value at a position adds to a slot's number, -1: none
 };
 
 struct BmSnap {
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(256) k_bm_snap(const __grid_constant__ BmSnap 
     const int32_t* row = P.table + ((size_t)b << P.carried_bits);
     float v[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) { const int a = C.at[4 * q + k]; v[k] = a >= 0 ? ord2f(__ldcg(row + a)) : __int_as_float(0x7fffffff); }
+    for (int k = 0; k < 4; ++k) { const int32_t a = C.at[4 * q + k]; v[k] = a >= 0 ? ord2f(__ldcg(row + a)) : __int_as_float(0x7fffffff); }
     reinterpret_cast<float4*>(P.copy)[(size_t)b * quads + q] = make_float4(v[0], v[1], v[2], v[3]);
   }
 }
@@ -224,7 +224,7 @@ struct BmPull {
   uint32_t n_nodes;                // nodes that the mirror has slots for
   const float4* copy;
   uint32_t z_max;                  // largest value the head's second column may take
-  int carried_bits;
+  int z_shift;                     // a slot's number: (target << z_shift) + what the carried value adds
   int32_t* table;
   uint32_t* changed;
   uint32_t* err;
@@ -236,15 +236,9 @@ struct BmPull {
 // dropped first; without it they take part with what the copy last held of b (empty, or tags that have been applied), which is
 // cheaper where few would be dropped: the look at the bitmap is a wavefront a row, as much as fetching the row.
 template <int SINK, bool FILTER>
-__global__ void __launch_bounds__(kBpBlock, kBpBlocks) k_bm_pull(const __grid_constant__ BmPull P, const __grid_constant__ BpColumns C) {
-  __shared__ uint2 s_row[kBpBlock / 32][kBpChunk];
-  __shared__ uint32_t s_target[kBpBlock / 32][kBpChunk];
-  const unsigned lane = lane_id(), wid = warp_id();
-  const uint32_t base = (blockIdx.x * (kBpBlock / 32) + wid) * kBpChunk;
-  if (base >= P.n_rows) return;
+__device__ __forceinline__ void bm_pull_chunk(const BmPull& P, const BpColumns& C, const uint32_t base, uint2* const rows, uint32_t* const target) {
+  const unsigned lane = lane_id();
   const uint32_t G = (uint32_t)C.lanes;
-  uint2* const rows = s_row[wid];
-  uint32_t* const target = s_target[wid];
   uint32_t n = 0;
   {
     uint2 r[kBpSweeps];
@@ -261,7 +255,7 @@ __global__ void __launch_bounds__(kBpBlock, kBpBlocks) k_bm_pull(const __grid_co
     for (int i = 0; i < kBpSweeps; ++i) {
       bool in = (bits[i] >> (r[i].x & 31)) & 1u;
       if (in && z[i] > P.z_max) {                  // a candidate there ends the fixpoint
-        if (FILTER || ((P.any[r[i].x >> 5] >> (r[i].x & 31)) & 1u)) atomicOr(P.err, kErrHeadRange);
+        if (FILTER || (P.any && ((P.any[r[i].x >> 5] >> (r[i].x & 31)) & 1u))) atomicOr(P.err, kErrHeadRange);
         in = false;
       }
       const unsigned bal = __ballot_sync(0xffffffffu, in);
@@ -279,9 +273,9 @@ __global__ void __launch_bounds__(kBpBlock, kBpBlocks) k_bm_pull(const __grid_co
   const uint32_t per = ((n + groups - 1) / groups) | 1u;                // odd: the groups read different banks
   const uint32_t e0 = g < groups ? min(g * per, n) : n, e1 = min(e0 + per, n);
   if (e0 >= e1) return;
-  int col[4];
+  uint32_t col[4];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) col[k] = max((int)C.at[4 * l + k], 0);
+  for (int k = 0; k < 4; ++k) col[k] = (uint32_t)max(C.at[4 * l + k], 0);
   const float none = __int_as_float(0x7fffffff);
   const int32_t never = SINK == kSinkMin ? 0x7fffffff : (int32_t)0x80000000;
   auto better = [](float a, float b) { return SINK == kSinkMin ? fminf(a, b) : fmaxf(a, b); };
@@ -295,18 +289,17 @@ __global__ void __launch_bounds__(kBpBlock, kBpBlocks) k_bm_pull(const __grid_co
 #pragma unroll
     for (int k = 0; k < 4; ++k) up[k] = SINK == kSinkMin ? met[k] < old[k] : met[k] > old[k];
     if (!(up[0] | up[1] | up[2] | up[3])) return;
-    const uint32_t zq = before << P.carried_bits;
-    int32_t* const slots = P.table + zq;
-    uint32_t* const words = P.changed + (zq >> 5);
+    const uint32_t zq = before << P.z_shift;
 #pragma unroll
     for (int k = 0; k < 4; ++k)
       if (up[k]) {
-        if (SINK == kSinkMin) atomicMin(slots + col[k], met[k]); else atomicMax(slots + col[k], met[k]);
-        atomicOr(words + (col[k] >> 5), 1u << (col[k] & 31));
+        const uint32_t slot = zq + col[k];
+        if (SINK == kSinkMin) atomicMin(P.table + slot, met[k]); else atomicMax(P.table + slot, met[k]);
+        atomicOr(P.changed + (slot >> 5), 1u << (slot & 31));
       }
   };
   auto turn = [&]() {                              // cur is complete: it becomes the target before, its slots on their way
-    const int32_t* const slots = P.table + (cur << P.carried_bits);
+    const int32_t* const slots = P.table + (cur << P.z_shift);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       met[k] = acc[k] == acc[k] ? f2ord(acc[k]) : never;      // a column that is none has met nothing
@@ -336,6 +329,14 @@ __global__ void __launch_bounds__(kBpBlock, kBpBlocks) k_bm_pull(const __grid_co
   settle();
   turn();
   settle();
+}
+
+template <int SINK, bool FILTER>
+__global__ void __launch_bounds__(kBpBlock, kBpBlocks) k_bm_pull(const __grid_constant__ BmPull P, const __grid_constant__ BpColumns C) {
+  __shared__ uint2 s_row[kBpBlock / 32][kBpChunk];
+  __shared__ uint32_t s_target[kBpBlock / 32][kBpChunk];
+  const uint32_t base = (blockIdx.x * (kBpBlock / 32) + warp_id()) * kBpChunk;
+  if (base < P.n_rows) bm_pull_chunk<SINK, FILTER>(P, C, base, s_row[warp_id()], s_target[warp_id()]);
 }
 
 }  // namespace xlog

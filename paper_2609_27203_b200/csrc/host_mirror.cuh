@@ -216,14 +216,29 @@ void launch_res_cluster(Ctx* c, const JoinSpec& S, const ResCluster& P) {
   check_launch(c, "k_res_cluster");
 }
 
+// The gather of a head's heavy resident rounds: over the shape h(a, c) :- h(a, b), r(b, c) with two to 32 values of a, where a round
+// of many candidates reads a sector per (row of r, few values of a) instead of one per candidate.
+struct ResPull {
+  bool on = false;
+  unsigned long long min = ~0ull;        // candidates from which a round is gathered
+  BmPull args{};
+  BpColumns cols{};
+  int shift = 0;
+  RevLists* lists = nullptr;
+  ~ResPull() { if (lists) lists->in_use = false; }
+};
+ResScratch res_scratch(Resident& R, const ResPull& p) {
+  return ResScratch{R.scan_status.as<unsigned long long>(), R.scan_tiles_cap, R.tickets.as<uint32_t>(), p.on ? p.min : ~0ull, p.on ? R.copy.as<float>() : nullptr, p.shift, (uint32_t)p.cols.lanes};
+}
+
 // One round's launches.  Nothing here allocates, copies or waits: the same calls are either captured into the WHILE
 // body or issued directly (host-driven rounds, used when launches are being timed one by one).
 void resident_body(Ctx* c, Resident& R, const std::vector<JoinSpec>& specs, const Relation& H, bool is_max, const MirrorArgs& mr, uint32_t bm_quads, unsigned ch_tiles,
-                   uint32_t longest, cudaGraphConditionalHandle handle, int use_handle) {
+                   uint32_t longest, const ResPull& pull, cudaGraphConditionalHandle handle, int use_handle) {
   ResState* st = res_state(c);
   uint32_t* err = ctrl_u32(c, kSlotErr);
   const uint32_t* dk = R.dkeys.as<uint32_t>();
-  const ResScratch sc{R.scan_status.as<unsigned long long>(), R.scan_tiles_cap, R.tickets.as<uint32_t>()};
+  const ResScratch sc = res_scratch(R, pull);
   const bool fused = specs.size() == 1;                  // the count of the next round rides on the emit kernel; the first round's is launched before the loop
   if (longest) {
     const uint32_t slots = res_cluster_slots(H);
@@ -240,6 +255,11 @@ void resident_body(Ctx* c, Resident& R, const std::vector<JoinSpec>& specs, cons
     if (S.fast) { if (is_max) XLOG_RES_EXPAND(kExpFast, kSinkMax); else XLOG_RES_EXPAND(kExpFast, kSinkMin); }
     else { if (is_max) XLOG_RES_EXPAND(kExpGeneric, kSinkMax); else XLOG_RES_EXPAND(kExpGeneric, kSinkMin); }
 #undef XLOG_RES_EXPAND
+  }
+  if (pull.on) {
+    const unsigned g = (unsigned)std::min<uint64_t>(((uint64_t)pull.args.n_rows + kBpChunk * (kBpBlock / 32) - 1) / (kBpChunk * (kBpBlock / 32)), (uint64_t)kSMs * kBpBlocks);
+    if (is_max) XLOG_LAUNCH(c, (k_res_pull<kSinkMax>), g, kBpBlock, 0, (const ResState*)st, pull.args, pull.cols);
+    else XLOG_LAUNCH(c, (k_res_pull<kSinkMin>), g, kBpBlock, 0, (const ResState*)st, pull.args, pull.cols);
   }
   uint32_t* ctr = sc.tickets + kResTkEmit;
   if (fused) {
@@ -263,7 +283,7 @@ void resident_body(Ctx* c, Resident& R, const std::vector<JoinSpec>& specs, cons
 // planned.  Returns the final state block (read once, after the loop).
 // `behind` (may be empty) issues what is to run behind the loop's one launch, before the state is read.
 ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*>& rs, bool is_max, const MirrorArgs& mr_host, uint32_t bm_quads,
-                      unsigned ch_tiles, uint32_t n_delta, int64_t rounds_left, uint64_t new_seen, const std::function<void()>& behind) {
+                      unsigned ch_tiles, uint32_t n_delta, int64_t rounds_left, uint64_t new_seen, const ResPull& pull, const std::function<void()>& behind) {
   Relation& H = *c->rels[h];
   std::vector<JoinSpec> specs;
   for (const RuleC* r : rs)
@@ -274,7 +294,7 @@ ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*
       }
   if (specs.size() > 16) fail(XLOG_ERR_UNSUPPORTED, "too many rule variants for one head");
   const uint32_t budget = (uint32_t)std::min<int64_t>(rounds_left, 0x7fffffff);
-  const ResScratch sc{R.scan_status.as<unsigned long long>(), R.scan_tiles_cap, R.tickets.as<uint32_t>()};
+  const ResScratch sc = res_scratch(R, pull);
   const uint32_t longest = res_cluster_longest(c, h, rs, specs, H.layout.total_bits);
   XLOG_LAUNCH(c, k_res_init, 1, 1024, 0, res_state(c), sc, (uint32_t)specs.size(), n_delta, budget, R.max_tiles, (unsigned long long)new_seen);
   const MirrorArgs& mr = mr_host;
@@ -298,6 +318,8 @@ ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*
     sig_add(sig, mr.table); sig_add(sig, mr.changed); sig_add(sig, mr.n_new); sig_add(sig, mr.key_max); sig_add(sig, mr.err); sig_add(sig, R.present.p);
     sig_add(sig, longest);
     if (longest) sig_add(sig, res_cluster_slots(H));
+    sig_add(sig, pull.on);
+    if (pull.on) { sig_add(sig, pull.args); sig_add(sig, pull.cols); sig_add(sig, sc); }
     sig_add(sig, rounds_per_body); sig_add(sig, is_max); sig_add(sig, bm_quads); sig_add(sig, ch_tiles); sig_add(sig, c->d_ctrl); sig_add(sig, c->spin_limit);
     if (!R.exec || sig != R.sig) {
       if (R.exec) { cudaGraphExecDestroy(R.exec); R.exec = nullptr; }
@@ -321,7 +343,7 @@ ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*
       c->stream = c->capture_stream;
       const int64_t b0 = c->launches;
       try {
-        for (int i = 0; i < rounds_per_body; ++i) resident_body(c, R, specs, H, is_max, mr, bm_quads, ch_tiles, longest, handle, 1);
+        for (int i = 0; i < rounds_per_body; ++i) resident_body(c, R, specs, H, is_max, mr, bm_quads, ch_tiles, longest, pull, handle, 1);
       } catch (...) {
         c->stream = caller;
         cudaGraph_t dummy = nullptr;
@@ -348,12 +370,13 @@ ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*
     uint32_t rows = n_delta;
     double expand_ms_seen = 0.0;
     int64_t expand_launches_seen = 0;
+    bool pulled = false;
     {
       auto it0 = c->prof_index.find("k_res_expand");
       if (it0 != c->prof_index.end()) { expand_ms_seen = c->prof[it0->second].ms; expand_launches_seen = c->prof[it0->second].launches; }
     }
     for (;;) {
-      resident_body(c, R, specs, H, is_max, mr, bm_quads, ch_tiles, longest, cudaGraphConditionalHandle{}, 0);
+      resident_body(c, R, specs, H, is_max, mr, bm_quads, ch_tiles, longest, pull, cudaGraphConditionalHandle{}, 0);
       read_state();
       if (c->flags & XLOG_FLAG_PROFILE) {
         // per delta row and rule: key and tag read, two offsets probed, 16-byte row record and 8-byte start offset written
@@ -363,7 +386,7 @@ ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*
         // algorithmic bytes of the round's expand launches (per candidate: the looked-up columns and tag, and the slot)
         auto it = c->prof_index.find("k_res_expand");
         if (it != c->prof_index.end()) {
-          const int64_t bytes = (int64_t)(out.candidates - out.small_cand - seen) * (4 + (specs[0].has_inner ? 4 * (specs[0].inner_free + 1) : 0));
+          const int64_t bytes = pulled ? 0 : (int64_t)(out.candidates - out.small_cand - seen) * (4 + (specs[0].has_inner ? 4 * (specs[0].inner_free + 1) : 0));
           Ctx::ProfEntry& pe = c->prof[it->second];
           pe.bytes += bytes;
           if (bytes >= kProfLargeBytes) {                // this round's launches, totalled on their own like any large launch
@@ -380,6 +403,7 @@ ResState run_resident(Ctx* c, Resident& R, int h, const std::vector<const RuleC*
           expand_ms_seen = c->prof[it->second].ms; expand_launches_seen = c->prof[it->second].launches;
         }
         seen = out.candidates - out.small_cand;
+        pulled = out.pull != 0;
       }
       if (out.status != kResOk || out.n_delta == 0) break;
     }
@@ -532,6 +556,41 @@ void build_rev_lists(Ctx* c, Relation& R) {
   R.rev = std::move(L);
 }
 
+// Whether and from where on the resident rounds of head h are gathered; `rel`: the looked-up relation, where the rule has the shape.
+constexpr uint32_t kResPullRows = 1u << 20;       // rows of r below which the launch that looks whether it is wanted costs what it brings
+void resident_pull_setup(Ctx* c, int h, const std::vector<const RuleC*>& rs, Resident& R, bool is_max, const MirrorArgs& mr, ResPull& pull, Relation*& rel) {
+  const Relation& H = *c->rels[h];
+  rel = nullptr;
+  if ((c->flags & (XLOG_FLAG_NO_GROUPED_JOIN | XLOG_FLAG_NO_BITMAP_JOIN)) || H.arity != 2 || H.dict_n[1] || H.layout.shift[1] != 0 || !grouped_shape(c, h, rs)) return;
+  const int n_cols = H.col_max[0] + 1;
+  if (n_cols < 2 || n_cols > 32) return;
+  int over = 0;
+  Relation* RB = nullptr;
+  for (const RuleC* r : rs)
+    for (int j = 0; j < r->plan.n_atoms; ++j) if (r->plan.atoms[j].rel == h) { ++over; RB = c->rels[r->plan.atoms[1 - j].rel]; }
+  if (over != 1 || RB->n < kResPullRows || RB->val_max[1] > (int32_t)H.layout.mask[1]) return;
+  rel = RB;
+  const int lanes = std::max(2, (n_cols + 7) / 8 * 2);
+  // the join takes 7 ps a candidate, the gather about 12 a row of r and two lanes
+  pull.min = (unsigned long long)RB->n * 8 / 5 * (lanes / 2);
+  // lists by the second evaluation that has such a round
+  if (!RB->rev.valid && (RB->rev.wanted == 0 || RB->rev.wanted == c->evaluations)) return;
+  const uint64_t n_nodes = (uint64_t)1 << H.layout.shift[0], copy = (n_nodes + 1) * 16 * lanes;
+  const bool have = R.copy.p && R.copy.bytes == copy;
+  if ((have ? 0 : copy) + (RB->rev.valid ? 0 : (uint64_t)RB->n * 12 + (uint64_t)RB->val_max[1] * 8) + (4u << 20) > c->arena.largest_free() / 2) return;
+  if (!RB->rev.valid) build_rev_lists(c, *RB);
+  if (!have) { R.copy.reset(); R.copy = DevBuf(c, copy); }
+  XLOG_CUDA(cudaMemsetAsync(R.copy.p, 0xff, copy, c->stream));
+  RB->rev.in_use = true;
+  pull.lists = &RB->rev;
+  pull.shift = H.layout.shift[0];
+  pull.cols.lanes = lanes;
+  for (int i = 0; i < kBpMaxCols; ++i) pull.cols.at[i] = -1;
+  for (int a = 0; a < n_cols; ++a) pull.cols.at[4 * (a % lanes) + a / lanes] = a << pull.shift;
+  pull.args = BmPull{RB->rev.rows.as<uint2>(), RB->rev.target.as<uint32_t>(), RB->n, nullptr, (uint32_t)n_nodes, R.copy.as<float4>(), H.layout.mask[1], 0, mr.table, mr.changed, mr.err};
+  pull.on = true;
+}
+
 // The gather of a stratum's heavy rounds: the copy of the changed nodes' rows, their bitmap, the columns in use.
 constexpr int kSlotBmLive = 91;            // the carried values that can derive anything, one bit each
 static_assert((1 << kBpMaxWordsLog2) * 4 <= (kCtrlSlots - kSlotBmLive) * 8, "control block too small");
@@ -578,8 +637,8 @@ void launch_bm_pull(Ctx* c, bool is_max, bool filter, unsigned grid, const BmPul
 // seed round that have matches, and every later key carries one of them.
 void bitmap_pull_columns(Ctx* c, BitmapPull& bp) {
   const uint32_t* live = reinterpret_cast<const uint32_t*>(c->h_ctrl + kSlotBmLive);
-  std::vector<int16_t> a;
-  for (int i = 0; i < (32 << bp.words_log2); ++i) if ((live[i >> 5] >> (i & 31)) & 1u) a.push_back((int16_t)i);
+  std::vector<int32_t> a;
+  for (int i = 0; i < (32 << bp.words_log2); ++i) if ((live[i >> 5] >> (i & 31)) & 1u) a.push_back(i);
   bp.n_cols = (int)a.size();
   if (bp.n_cols > kBpMaxCols) { bp.usable = false; return; }
   bp.cols.lanes = std::max(2, (bp.n_cols + 7) / 8 * 2);                  // rows of whole 32-byte sectors

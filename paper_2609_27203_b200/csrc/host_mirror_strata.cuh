@@ -121,7 +121,11 @@ void stratum_recursive_mirror(Ctx* c, int h, const std::vector<const RuleC*>& rs
       ahead = mirror_rows_buffer(c, slots);
       behind = [&]() { emit_mirror(c, table, slots, empty, M, H.layout, (int64_t)slots, ahead); };
     }
-    const ResState s = run_resident(c, *R, h, rs, is_max, mr, bm_quads, ch_tiles, n_start, c->max_iter, 0, behind);
+    ResPull pull;
+    Relation* pull_rel = nullptr;
+    if (n_start == 0) resident_pull_setup(c, h, rs, *R, is_max, mr, pull, pull_rel);
+    const ResState s = run_resident(c, *R, h, rs, is_max, mr, bm_quads, ch_tiles, n_start, c->max_iter, 0, pull, behind);
+    if (pull_rel && !pull_rel->rev.wanted && s.most >= pull.min) pull_rel->rev.wanted = c->evaluations;
     round = s.rounds;
     c->r_iterations += s.rounds; c->r_candidates += (int64_t)s.candidates;
     c->r_new += (int64_t)s.n_new; c->r_improved += (int64_t)s.n_improved;

@@ -16,6 +16,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "bitmap_pull.cuh"
 #include "common.cuh"
 #include "join.cuh"
 #include "mirror.cuh"
@@ -40,7 +41,8 @@ struct ResState {
   unsigned long long n_improved;
   unsigned long long small_cand;     // candidates of rounds run by the cluster kernel (res_cluster.cuh)
   uint32_t bodies;                   // times a round's launches ran
-  uint32_t pad;
+  uint32_t pull;                     // the round to come is a gather (k_res_pull), not a push
+  unsigned long long most;           // candidates of the largest round
 };
 
 constexpr int kResMaxVariants = 16;
@@ -66,7 +68,17 @@ struct ResScratch {
   unsigned long long* scan_status;   // [kResMaxVariants][scan_tiles_cap]
   uint32_t scan_tiles_cap;
   uint32_t* tickets;                 // [kResMaxVariants], then the emit kernel's two counters
+  // rounds of at least that many candidates are gathered (~0: none); the tags that the gather reads are kept up to date by the emit
+  // kernel: a row of 4 lanes floats per target value, carried value a at 4 (a % lanes) + a / lanes
+  unsigned long long pull_min;
+  float* copy;
+  int copy_shift;                    // key: carried value << copy_shift | value
+  uint32_t copy_lanes;
 };
+__device__ __forceinline__ size_t res_copy_at(const ResScratch& sc, uint32_t key) {
+  const uint32_t a = key >> sc.copy_shift, z = key & ((1u << sc.copy_shift) - 1u);
+  return (size_t)z * (4 * sc.copy_lanes) + 4 * (a % sc.copy_lanes) + a / sc.copy_lanes;
+}
 
 static __global__ void __launch_bounds__(1024) k_res_init(ResState* st, ResScratch sc, uint32_t n_variants, uint32_t n_delta, uint32_t max_rounds,
                                                           uint32_t max_tiles, unsigned long long new_seen) {
@@ -194,7 +206,7 @@ __global__ void __launch_bounds__(kExpBlock, kExpMirrorBlocksPerSM) k_res_expand
                                                           const uint64_t* __restrict__ start, const uint4* __restrict__ rowinfo,
                                                           const uint2* __restrict__ tile_rows, uint32_t* __restrict__ err, MirrorArgs mr) {
   __shared__ ExpSmem<ExpShapeT<true>> sm;
-  if (st->status != kResOk) return;
+  if (st->status != kResOk || st->pull) return;
   const uint32_t ntiles = st->ntiles, n = st->n_delta;
   const uint64_t total = st->total;
   const BwdArgs bw{};
@@ -206,6 +218,20 @@ __global__ void __launch_bounds__(kExpBlock, kExpMirrorBlocksPerSM) k_res_expand
     __syncthreads();
   }
   if (e) atomicOr(err, e);
+}
+
+// A heavy round as a gather (bitmap_pull.cuh), where the state block says so: eight carried values of a node are one sector of the copy,
+// where the row-wise join reads a sector a candidate.  Reachability from 7 sources on R-MAT 18 (3.8 M rows), the two largest rounds: 100 and
+// 72 -> 52 and 46 us; a launch that is not wanted 2 us a round; 656 -> 616 us per evaluation and read.
+template <int SINK>
+__global__ void __launch_bounds__(kBpBlock, kBpBlocks) k_res_pull(const ResState* __restrict__ st, const __grid_constant__ BmPull P, const __grid_constant__ BpColumns C) {
+  __shared__ uint2 s_row[kBpBlock / 32][kBpChunk];
+  __shared__ uint32_t s_target[kBpBlock / 32][kBpChunk];
+  if (st->status != kResOk || !st->pull) return;
+  for (uint64_t base = (uint64_t)(blockIdx.x * (kBpBlock / 32) + warp_id()) * kBpChunk; base < P.n_rows; base += (uint64_t)gridDim.x * (kBpBlock / 32) * kBpChunk) {
+    __syncwarp();
+    bm_pull_chunk<SINK, false>(P, C, (uint32_t)base, s_row[warp_id()], s_target[warp_id()]);
+  }
 }
 
 // Tail of a round's last kernel, called by every thread of every block: the block that finishes last closes the
@@ -265,6 +291,8 @@ __device__ __forceinline__ void res_close_round(const bool live, ResState* __res
         const unsigned long long nt = (next_total + kExpTileMirror - 1) / kExpTileMirror;
         st->total = next_total;
         st->ntiles = 0;
+        st->pull = again && next_total >= sc.pull_min ? 1u : 0u;
+        st->most = max(st->most, next_total);
         if (again) {
           if (nt > st->max_tiles) { st->status = kResOverflow; again = 0; }
           else {
@@ -422,6 +450,7 @@ __global__ void __launch_bounds__(kMirBlock) k_res_emit_count(uint32_t* __restri
             const uint32_t row = row0 + ib + k;
             keys[row] = key[k];
             tags[row] = tag[k];
+            if (sc.copy) sc.copy[res_copy_at(sc, key[k])] = tag[k];
             d[k] = join_count_kv<uint32_t>(S, key[k], tag[k], row, rowinfo, err);
           }
           mine += d[k];

@@ -87,3 +87,32 @@ def test_lists_give_way():                                    # an arena with li
             assert H.compare_relations(rel, want, what=f"arena of {arena}")["bit_unequal"] == 0
             ctx.reset_idb()
         ctx.close()
+
+
+@pytest.mark.parametrize("sr,n_src", [(W.MINPLUS, 2), (W.MINPLUS, 7), (W.MAXPLUS, 8), (W.MINPLUS, 9), (W.MINPLUS, 20), (W.MAXPLUS, 32), (W.MINPLUS, 33)])
+def test_resident_rounds(sr, n_src):                          # few sources over a large relation: the resident loop's heavy rounds
+    from paper_2609_27203_b200 import xlog
+    rng = np.random.default_rng(n_src)
+    n = 20000
+    key = np.unique(rng.integers(0, n, 1200000) * n + (n * rng.random(1200000) ** 2).astype(np.int64))
+    s, d = (key // n).astype(np.int32), (key % n).astype(np.int32)
+    w = (1 + 9 * rng.random(len(s))).astype(np.float32) * np.float32(1 if sr == W.MINPLUS else -1)
+    prog = W.reach_program(s, d, w, np.sort(rng.permutation(n)[:n_src]).astype(np.int32), semiring=sr)
+    got = []
+    for f in (0, xlog.FLAG_NO_GRAPH, xlog.FLAG_PROFILE, xlog.FLAG_NO_TAG_MIRROR):
+        ctx, ids, _ = xlog.load_program(prog, arena_bytes=3 << 30, flags=f | xlog.FLAG_CHECK_INVARIANTS)
+        recs, rels = [], []
+        for _ in range(1 if f & xlog.FLAG_NO_TAG_MIRROR else 3):
+            recs.append(ctx.fixpoint())
+            rels.append(ctx.read(ids["reach"]))
+            ctx.reset_idb()
+        for r, rel in zip(recs, rels):
+            assert [r[k] for k in COUNTERS] == [recs[0][k] for k in COUNTERS]
+            assert H.compare_relations(rel, rels[0], what="one evaluation vs another")["bit_unequal"] == 0
+        if f & xlog.FLAG_PROFILE:
+            assert ("k_res_pull" in ctx.profile()) == (n_src <= 32)
+        got.append((rels[0], recs[0]))
+        ctx.close()
+    for g in got[:3]:
+        assert H.compare_relations(g[0], got[3][0], what="resident vs sorting route")["bit_unequal"] == 0
+        assert [g[1][k] for k in COUNTERS] == [got[3][1][k] for k in COUNTERS]
