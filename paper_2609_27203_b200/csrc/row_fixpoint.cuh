@@ -20,7 +20,7 @@
 // holds.  Closing a round a lane per bit and laying the candidates out warp by warp, without a barrier: 1,000 nodes and 4,000
 // edges 122 -> 97 us, 300 nodes 43 -> 35 us, 2,400 nodes 536 -> 392 us (before: a thread per bitmap word, one prefix over
 // the whole block, ten steps of search per candidate).  Registers for 6 blocks an SM: with as many as the compiler
-// likes 134, 31 and 567 us; with 8 blocks 92, 37 and 407 us (6 is ahead on the small and the large graph, 8 on the middle one only).
+// likes 134, 31 and 567 us; for 8 blocks 88, 37 and 407 us, which is taken where it saves a wave of rows.
 #pragma once
 #include "common.cuh"
 #include "join.cuh"
@@ -29,9 +29,7 @@ namespace xlog {
 
 constexpr int kRowMaxBits = 13;                  // keys per value of a: at most 8192 (row, tags set aside and delta list: 80 KB)
 constexpr int kRowBlock = 256;
-#ifndef XLOG_ROW_BLOCKS
-#define XLOG_ROW_BLOCKS 6
-#endif
+constexpr int kRowBlocks = 6, kRowBlocksMany = 8;       // blocks an SM of one head's kernel is built for
 constexpr int kRowUnroll = 2;                    // candidates a lane looks up at a time
 
 // Totals of the launch, in the control words.
@@ -69,8 +67,8 @@ struct RowFix {
 // per head: row tags (4 B per slot), delta tags (4 B), delta slots (2 B), changed and present bits
 inline size_t row_fix_smem(int c_bits, int n_heads) { return (size_t)n_heads * (((size_t)10 << c_bits) + ((size_t)2 << c_bits) / 8); }
 
-template <int NH>
-__global__ void __launch_bounds__(kRowBlock, NH == 1 ? XLOG_ROW_BLOCKS : 1) k_row_fixpoint(const __grid_constant__ RowFix P) {
+template <int NH, int BLOCKS>
+__global__ void __launch_bounds__(kRowBlock, BLOCKS) k_row_fixpoint(const __grid_constant__ RowFix P) {
   extern __shared__ uint32_t row_smem[];
   __shared__ uint32_t s_nd[2][NH];                                   // delta rows of every head in the running round, and in the next
   const uint32_t S = 1u << P.c_bits, W = S >> 5;
