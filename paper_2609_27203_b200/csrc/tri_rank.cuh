@@ -17,8 +17,9 @@
 // A corner a with little to walk is handled by one warp that searches out(a) instead (k_tri_rank_small).  k_tri_rank_groups then
 // adds up each node's parts: its units' sums of both launches and its edges' sums.
 //
-// R-MAT 18 (3.9 M edges, 39 M triangles): 5.47 -> 1.12 ms per evaluation, 0.88 ms of it the two bitmap launches (bound by instruction
-// issue: 75 % of the slots), 0.11 the searched corners; the first one on a new relation, which orders the graph, 5.82 -> 2.42.
+// R-MAT 18 (3.9 M edges, 39 M triangles): 5.47 -> 1.03 ms per evaluation, 0.83 ms of it the two bitmap launches (bound by instruction
+// issue: 75 % of the slots; 0.88 with a chain of reads ahead of every item's list), 0.11 the searched corners; the first one on a new
+// relation, which orders the graph, 5.82 -> 2.42.
 #pragma once
 #include "common.cuh"
 
@@ -232,33 +233,40 @@ __global__ void __launch_bounds__(kTriRankBlock) k_tri_rank(const __grid_constan
   const uint32_t it0 = un.y, it1 = min(it0 + trk_unit_items(m1 - m0), P.I.split[a]);
   double sum = 0.0;
   uint32_t cnt = 0;
-  for (uint32_t it = it0 + wid; it < it1; it += kTriRankBlock / 32) {
-    const uint32_t v = P.I.nbr[it];
-    const float ev = P.I.e[it];
-    const uint32_t w0 = P.I.split[v], w1 = P.I.off[v + 1];
-    double isum = 0.0;
-    uint32_t icnt = 0;
-    for (uint32_t i0 = w0; i0 < w1; i0 += 32 * kTriRankSweeps) {
-      uint32_t z[kTriRankSweeps], wd[kTriRankSweeps];
+  // a warp takes one in sixteen of the unit's items (neighbours have lists of like length), and a lane each fetches the next 32 items' bounds
+  for (uint32_t b0 = it0 + wid; b0 < it1; b0 += kTriRankBlock) {
+    const uint32_t ib = b0 + lane * (kTriRankBlock / 32);
+    uint32_t first = 0, end = 0;
+    float e = 0.f;
+    if (ib < it1) { const uint32_t v = P.I.nbr[ib]; e = P.I.e[ib]; first = P.I.split[v]; end = P.I.off[v + 1]; }
+#pragma unroll 1
+    for (uint32_t j = 0, it = b0; it < it1 && j < 32; ++j, it += kTriRankBlock / 32) {
+      const uint32_t w0 = __shfl_sync(0xffffffffu, first, j), w1 = __shfl_sync(0xffffffffu, end, j);
+      const float ev = __shfl_sync(0xffffffffu, e, j);
+      double isum = 0.0;
+      uint32_t icnt = 0;
+      for (uint32_t i0 = w0; i0 < w1; i0 += 32 * kTriRankSweeps) {
+        uint32_t z[kTriRankSweeps], wd[kTriRankSweeps];
 #pragma unroll
-      for (int k = 0; k < kTriRankSweeps; ++k) { const uint32_t i = i0 + k * 32 + lane; z[k] = i < w1 ? P.I.nbr[i] : 0xffffffffu; }
+        for (int k = 0; k < kTriRankSweeps; ++k) { const uint32_t i = i0 + k * 32 + lane; z[k] = i < w1 ? P.I.nbr[i] : 0xffffffffu; }
 #pragma unroll
-      for (int k = 0; k < kTriRankSweeps; ++k) wd[k] = z[k] != 0xffffffffu ? bits[z[k] >> 5] : 0u;
+        for (int k = 0; k < kTriRankSweeps; ++k) wd[k] = z[k] != 0xffffffffu ? bits[z[k] >> 5] : 0u;
 #pragma unroll
-      for (int k = 0; k < kTriRankSweeps; ++k)
-        if ((wd[k] >> (z[k] & 31)) & 1u) {
-          const uint32_t at = before[z[k] >> 5] + __popc(wd[k] & ((1u << (z[k] & 31)) - 1u));
-          isum += (double)((ev * P.M.e[at]) * P.I.e[i0 + k * 32 + lane]);
-          ++icnt;
-        }
-    }
-    sum += isum; cnt += icnt;
-    if (EDGES) {
-      icnt = __reduce_add_sync(0xffffffffu, icnt);
-      if (icnt)
+        for (int k = 0; k < kTriRankSweeps; ++k)
+          if ((wd[k] >> (z[k] & 31)) & 1u) {
+            const uint32_t at = before[z[k] >> 5] + __popc(wd[k] & ((1u << (z[k] & 31)) - 1u));
+            isum += (double)((ev * P.M.e[at]) * P.I.e[i0 + k * 32 + lane]);
+            ++icnt;
+          }
+      }
+      sum += isum; cnt += icnt;
+      if (EDGES) {
+        icnt = __reduce_add_sync(0xffffffffu, icnt);
+        if (icnt)
 #pragma unroll
-        for (int d = 16; d; d >>= 1) isum += __shfl_xor_sync(0xffffffffu, isum, d);
-      if (lane == 0) { const uint32_t o = P.I.other[it]; P.edge_sum[o] = isum; P.edge_cnt[o] = icnt; }
+          for (int d = 16; d; d >>= 1) isum += __shfl_xor_sync(0xffffffffu, isum, d);
+        if (lane == 0) { const uint32_t o = P.I.other[it]; P.edge_sum[o] = isum; P.edge_cnt[o] = icnt; }
+      }
     }
   }
   cnt = __reduce_add_sync(0xffffffffu, cnt);
@@ -342,37 +350,45 @@ __global__ void __launch_bounds__(256) k_tri_rank_small(const __grid_constant__ 
   }
 }
 
-// A warp per node of the relation: its parts from both launches and from its edges to higher corners, in a fixed order.
+// Eight lanes a node of the relation: its parts from both launches and from its edges to higher corners, in a fixed order.  A chain of
+// reads (rank, bounds, sums) and few of them a node: R-MAT 18 51 us, a warp a node 88.
+constexpr int kTrkGroupLanes = 8;
 template <bool LSE>
 __global__ void __launch_bounds__(256) k_tri_rank_groups(TriRankPass A, TriRankPass B, const uint32_t* __restrict__ rank, int64_t domain, uint32_t* __restrict__ grp_cnt,
                                                          float* __restrict__ grp_tag, uint32_t* __restrict__ flag, uint32_t* __restrict__ max_cnt, uint32_t* __restrict__ err) {
-  const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-  const unsigned lane = lane_id();
-  for (int64_t x = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < domain; x += nwarps) {
-    const uint32_t v = rank[x];
+  constexpr int G = kTrkGroupLanes;
+  const int64_t step = (int64_t)gridDim.x * 256 / G;
+  const unsigned sub = threadIdx.x % G;
+  uint32_t top = 0;
+  for (int64_t x0 = ((int64_t)blockIdx.x * 256 + threadIdx.x) / 32 * (32 / G); x0 < domain; x0 += step) {      // uniform over the warp
+    const int64_t x = x0 + lane_id() / G;
+    const uint32_t v = x < domain ? rank[x] : 0xffffffffu;
     double sum = 0.0;
     uint64_t cnt = 0;
     if (v < A.n_nodes) {
+      const uint32_t e0 = A.M.split[v] + sub, e1 = A.M.off[v + 1];
 #pragma unroll
       for (int p = 0; p < 2; ++p) {
         const TriRankPass& Q = p ? B : A;
         const uint32_t u0 = Q.unit_off[v], u1 = Q.unit_off[v + 1];
-        for (uint32_t u = u0 + lane; u < u1; u += 32) { sum += Q.unit_sum[u]; cnt += Q.unit_cnt[u]; }
-        if (u0 == u1 && lane == 0) { sum += Q.unit_sum[Q.n_units + v]; cnt += Q.unit_cnt[Q.n_units + v]; }
+        for (uint32_t u = u0 + sub; u < u1; u += G) { sum += Q.unit_sum[u]; cnt += Q.unit_cnt[u]; }
+        if (u0 == u1 && sub == 0) { sum += Q.unit_sum[Q.n_units + v]; cnt += Q.unit_cnt[Q.n_units + v]; }
       }
-      const uint32_t e1 = A.M.off[v + 1];
-      for (uint32_t i = A.M.split[v] + lane; i < e1; i += 32) { sum += A.edge_sum[i]; cnt += A.edge_cnt[i]; }
+#pragma unroll 4
+      for (uint32_t i = e0; i < e1; i += G) { sum += A.edge_sum[i]; cnt += A.edge_cnt[i]; }
     }
 #pragma unroll
-    for (int d = 16; d; d >>= 1) { sum += __shfl_xor_sync(0xffffffffu, sum, d); cnt += __shfl_xor_sync(0xffffffffu, cnt, d); }
-    if (lane == 0) {
+    for (int d = G / 2; d; d >>= 1) { sum += __shfl_xor_sync(0xffffffffu, sum, d); cnt += __shfl_xor_sync(0xffffffffu, cnt, d); }
+    if (sub == 0 && x < domain) {
       if (cnt > 0x7fffffffull) { atomicOr(err, kErrCountOverflow); cnt = 0x7fffffffull; }
       grp_cnt[x] = (uint32_t)cnt;
       grp_tag[x] = cnt ? (LSE ? (float)log(sum) : (float)sum) : 0.f;
       flag[x] = cnt ? 1u : 0u;
-      if (cnt) atomicMax(max_cnt, (uint32_t)cnt);
+      top = max(top, (uint32_t)cnt);
     }
   }
+  top = __reduce_max_sync(0xffffffffu, top);
+  if (lane_id() == 0 && top) atomicMax(max_cnt, top);
 }
 
 }  // namespace xlog
