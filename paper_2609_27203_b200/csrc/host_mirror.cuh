@@ -579,10 +579,10 @@ void resident_pull_setup(Ctx* c, int h, const std::vector<const RuleC*>& rs, Res
   const bool have = R.copy.p && R.copy.bytes == copy;
   if ((have ? 0 : copy) + (RB->rev.valid ? 0 : (uint64_t)RB->n * 12 + (uint64_t)RB->val_max[1] * 8) + (4u << 20) > c->arena.largest_free() / 2) return;
   if (!RB->rev.valid) build_rev_lists(c, *RB);
-  if (!have) { R.copy.reset(); R.copy = DevBuf(c, copy); }
-  XLOG_CUDA(cudaMemsetAsync(R.copy.p, 0xff, copy, c->stream));
   RB->rev.in_use = true;
   pull.lists = &RB->rev;
+  if (!have) { R.copy.reset(); R.copy = DevBuf(c, copy); }
+  XLOG_CUDA(cudaMemsetAsync(R.copy.p, 0xff, copy, c->stream));
   pull.shift = H.layout.shift[0];
   pull.cols.lanes = lanes;
   for (int i = 0; i < kBpMaxCols; ++i) pull.cols.at[i] = -1;
