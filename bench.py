@@ -209,7 +209,7 @@ def run_oracle_once(program, mode="seminaive"):
 
 
 # ------------------------------------------------------------------------------------------------
-MIRROR_JOIN_KERNELS = ("k_res_expand", "k_seg_expand", "k_bm_expand")
+MIRROR_JOIN_KERNELS = ("k_res_expand", "k_seg_expand", "k_bm_expand", "k_bm_pull", "k_res_pull")
 # Kernels whose bytes cross HBM once or hardly at all: what bounds them instead, and why the byte rate beside it says nothing.
 ON_CHIP_KERNELS = {
     "k_row_fixpoint": ("latency", "every round runs out of shared memory with the looked-up relation in L2: two barriers, a look-up and a candidate read one after the other"),
@@ -219,7 +219,7 @@ ON_CHIP_KERNELS = {
     "k_res_cluster": ("latency", "rounds inside one thread-block cluster: two L2 reads, a distributed-shared-memory read and a cluster barrier a round"),
     "k_tri_rank": ("issue", "list entries served by L2 and tested against a bitmap in shared memory: 75 % of the issue slots"),
     "k_tri_rank_small": ("issue", "list entries served by L2, searched in shared memory"),
-    "k_bits_emit": ("issue", "bitmaps of the lists served by L2; the rows cross HBM once"),
+    "k_bits_emit": ("l1", "four fifths of the load / store path's wavefronts: words and tags of the lists served by L1 and L2; the rows cross HBM once"),
     "k_bits_count": ("issue", "bitmaps of the lists served by L2"),
     "k_group_rule": ("issue", "an exponential and a dozen instructions per candidate, none of which reaches memory"),
     "k_group_backward": ("issue", "an exponential and a dozen instructions per candidate, none of which reaches memory"),
@@ -329,8 +329,10 @@ def roofline_of(program, prof_all, steps, sorting_route):
         # the tag-mirror joins move few bytes per candidate by construction; what limits them is said here
         roofline["limiter"] = ("instruction issue; the table, too large for L2, is read from HBM one 128-byte line per (changed unit of 32 keys, neighbour)"
                                if dom in ("k_seg_expand", "k_bm_expand") else
+                               "instruction issue and the latency of a row of tags per (row of the relation, target), three quarters of them from L2"
+                               if dom in ("k_bm_pull", "k_res_pull") else
                                "L2 random sector access (one tag-mirror slot per candidate); HBM carries about 8 B per candidate")
-        if dom not in ("k_seg_expand", "k_bm_expand"):
+        if dom not in ("k_seg_expand", "k_bm_expand", "k_bm_pull", "k_res_pull"):
             roofline["candidates_per_s"] = achieved * 1e9 / 12.0
     return roofline
 
