@@ -216,6 +216,8 @@ ON_CHIP_KERNELS = {
     "k_dense_round": ("latency", "every round runs out of shared memory; the rows cross HBM once"),
     "k_row_sums": ("latency", "every round runs out of shared memory: a chain of dependent L1 / L2 reads and two barriers"),
     "k_sparse_rows": ("issue", "hash tables in shared memory: half of the issue slots, and one dependent L2 read per row and round"),
+    "k_bm_pull": ("issue", "a row of tags per (row of the relation, target), three quarters of them from L2: 57 % of the issue slots, and the rows' latency"),
+    "k_res_pull": ("issue", "a sector of tags per (row of the relation, target), served by L2"),
     "k_res_cluster": ("latency", "rounds inside one thread-block cluster: two L2 reads, a distributed-shared-memory read and a cluster barrier a round"),
     "k_tri_rank": ("issue", "list entries served by L2 and tested against a bitmap in shared memory: 75 % of the issue slots"),
     "k_tri_rank_small": ("issue", "list entries served by L2, searched in shared memory"),
@@ -325,14 +327,12 @@ def roofline_of(program, prof_all, steps, sorting_route):
             roofline["issue"] = l2["issue"]
     if dom in ON_CHIP_KERNELS:
         roofline["limiter"] = ON_CHIP_KERNELS[dom][1] + ": the HBM fraction says nothing, read ms_per_step and the metric"
-    if mirror_kernel:
+    if mirror_kernel and dom not in ON_CHIP_KERNELS:
         # the tag-mirror joins move few bytes per candidate by construction; what limits them is said here
         roofline["limiter"] = ("instruction issue; the table, too large for L2, is read from HBM one 128-byte line per (changed unit of 32 keys, neighbour)"
                                if dom in ("k_seg_expand", "k_bm_expand") else
-                               "instruction issue and the latency of a row of tags per (row of the relation, target), three quarters of them from L2"
-                               if dom in ("k_bm_pull", "k_res_pull") else
                                "L2 random sector access (one tag-mirror slot per candidate); HBM carries about 8 B per candidate")
-        if dom not in ("k_seg_expand", "k_bm_expand", "k_bm_pull", "k_res_pull"):
+        if dom not in ("k_seg_expand", "k_bm_expand"):
             roofline["candidates_per_s"] = achieved * 1e9 / 12.0
     return roofline
 

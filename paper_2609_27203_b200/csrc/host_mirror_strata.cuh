@@ -233,8 +233,8 @@ void stratum_recursive_mirror(Ctx* c, int h, const std::vector<const RuleC*>& rs
           const BmPull L{bp.lists->rows.as<uint2>(), bp.lists->target.as<uint32_t>(), bj.rel->n, bp.any.as<uint32_t>(), n_nodes, bp.copy.as<float4>(), H.layout.mask[1], carried_bits,
                          table, reinterpret_cast<uint32_t*>(bitmap), ctrl_u32(c, kSlotErr)};
           const unsigned grid = (bj.rel->n + kBpChunk * (kBpBlock / 32) - 1) / (kBpChunk * (kBpBlock / 32));
-          // per row of r its node, tag and target; per (b, neighbour) with a changed b a row of the copy
-          c->note_bytes = (int64_t)bj.rel->n * 12 + (int64_t)nbrs * 16 * bp.cols.lanes;
+          // per row of r its node, tag and target; the changed keys' tags, once (a row of the copy per (b, neighbour) comes from L2)
+          c->note_bytes = (int64_t)bj.rel->n * 12 + (int64_t)changed * 4;
           launch_bm_pull(c, is_max, nbrs < (uint64_t)bj.rel->n / 8 * 7, grid, L, bp.cols);
           continue;
         }
